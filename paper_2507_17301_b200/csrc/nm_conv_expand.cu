@@ -144,7 +144,7 @@ k_conv_expand(const ConvParams p, const ExpandCfg cfg, const __grid_constant__ C
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
     const int NS = cfg.stages, n_sub = cfg.n_sub;
     const uint32_t wres = (smem_u32(smem_raw) + 1023u) & ~1023u;   // resident weight slice (may be empty)
     const uint32_t ring = wres + cfg.wres_bytes;
@@ -176,7 +176,7 @@ k_conv_expand(const ConvParams p, const ExpandCfg cfg, const __grid_constant__ C
 
     if (warp == 0) {
         // =========================== producer ===========================
-        if (lane == 0) {
+        if (elect_one()) {
             int issued = 0;
             const int hw = p.ho * p.wo;
             const uint32_t tx = static_cast<uint32_t>(KBLK) * (SUB_BYTES + (cfg.w_res ? 0u : static_cast<uint32_t>(cfg.bn) * 128u));
@@ -271,7 +271,7 @@ k_conv_expand(const ConvParams p, const ExpandCfg cfg, const __grid_constant__ C
         // earlier use of the slot, and with ownership by position inside the item a thread would skip uses of a slot
         // at the seams between items (found as a fault on the GPU, reproduced and fixed in a CPU model of the protocol).
         const int iss = warp >> 1;
-        if (lane == 0 && iss < cfg.n_iss) {
+        if (iss < cfg.n_iss && elect_one()) {
             const uint32_t idesc = umma_idesc_tf32(BM, cfg.bn);
             const bool shared_k = cfg.n_iss == 2;
             if (cfg.w_res && !mbar_wait(smem_u32(&s_wres), 0)) *abort_flag = 9;
@@ -465,7 +465,7 @@ k_conv_expand(const ConvParams p, const ExpandCfg cfg, const __grid_constant__ C
                     }
                 }
                 const uint32_t box = my_staging + (nb & box_toggle) * BOX_BYTES;
-                if (lane == 0) {
+                if (elect_one()) {
                     // the store that last read this box must be done with it
                     if (cfg.boxes == 2) { if (nb >= 2) tma_store_wait_read_n<1>(); }
                     else if (nb >= 1) tma_store_wait_read_n<0>();
@@ -500,7 +500,7 @@ k_conv_expand(const ConvParams p, const ExpandCfg cfg, const __grid_constant__ C
                 }
                 fence_proxy_async();
                 __syncwarp();
-                if (lane == 0) {
+                if (elect_one()) {
                     if (pix0 + q * 32 < p.pixels)
                         tma_store_2d(&tm_y, box, o0 + blk * 32, ks * cfg.p_pad + static_cast<int>(pix0) + q * 32);
                     tma_store_commit();
@@ -524,7 +524,7 @@ k_conv_expand(const ConvParams p, const ExpandCfg cfg, const __grid_constant__ C
                         flags[(gridDim.x - 1u - pos) * 8u + (warp - 4)] = 0u;
             }
         }
-        if (lane == 0) tma_store_wait_read();   // shared memory must outlive the stores' reads; the writes complete with the grid
+        if (elect_one()) tma_store_wait_read();   // shared memory must outlive the stores' reads; the writes complete with the grid
     }
 
     tc_fence_before();

@@ -30,7 +30,7 @@ __global__ void __launch_bounds__(128) k_conv_gather(const ConvParams p, const i
     __shared__ uint32_t s_tmem;
     __shared__ int s_row_n[BM], s_row_ih0[BM], s_row_iw0[BM];
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
     const int r = blockIdx.y;  // pruning tile
     const long long pix0 = static_cast<long long>(blockIdx.x) * BM;
 
@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(128) k_conv_gather(const ConvParams p, const i
         }
         fence_proxy_async();
         __syncthreads();
-        if (tid == 0) {
+        if (warp == 0 && elect_one()) {
             tc_fence_after();
 #pragma unroll
             for (int kq = 0; kq < NM_KCHUNK / 8; ++kq)

@@ -58,7 +58,7 @@ k_conv_pair(const ConvParams p, const PairCfg cfg, const __grid_constant__ CUten
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
     const uint32_t rank = cluster_ctarank();                  // 0: issues the MMAs
     const uint32_t pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
     const uint32_t n_work = static_cast<uint32_t>(cfg.n_work);
@@ -92,7 +92,7 @@ k_conv_pair(const ConvParams p, const PairCfg cfg, const __grid_constant__ CUten
 
     if (warp == 0) {
         // =========================== producer (both CTAs) ===========================
-        if (lane == 0) {
+        if (elect_one()) {
             int issued = 0;
             const int hw = p.ho * p.wo;
             const uint32_t w_bytes = static_cast<uint32_t>(cfg.half_rows) * 128u;
@@ -144,7 +144,7 @@ k_conv_pair(const ConvParams p, const PairCfg cfg, const __grid_constant__ CUten
         }
     } else if (warp == 1 && rank == 1) {
         // =========================== relay (second CTA) ===========================
-        if (lane == 0) {
+        if (elect_one()) {
             RingPos rp;
             for (uint32_t work = pair; work < n_work && !aborted(abort_flag); work += n_pairs) {
                 for (int c = 0; c < n_sub; ++c) {
@@ -156,7 +156,7 @@ k_conv_pair(const ConvParams p, const PairCfg cfg, const __grid_constant__ CUten
         }
     } else if (warp == 1) {
         // =========================== MMA issuer (first CTA) ===========================
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t idesc = umma_idesc_tf32(2 * BM, cfg.bn);
             RingPos rp;
             uint32_t ab = 0, acc_par = 0;
@@ -227,7 +227,7 @@ k_conv_pair(const ConvParams p, const PairCfg cfg, const __grid_constant__ CUten
                     if (lane == 0) mbar_arrive_cluster(accfree_remote);
                 }
                 const uint32_t box = my_staging + (nb & box_toggle) * BOX_BYTES;
-                if (lane == 0) {
+                if (elect_one()) {
                     if (cfg.boxes == 2) { if (nb >= 2) tma_store_wait_read_n<1>(); }
                     else if (nb >= 1) tma_store_wait_read_n<0>();
                 }
@@ -259,13 +259,13 @@ k_conv_pair(const ConvParams p, const PairCfg cfg, const __grid_constant__ CUten
                 }
                 fence_proxy_async();
                 __syncwarp();
-                if (lane == 0) {
+                if (elect_one()) {
                     if (pix0 + q * 32 < p.pixels) tma_store_2d(&tm_y, box, o0 + blk * 32, static_cast<int>(pix0) + q * 32);
                     tma_store_commit();
                 }
             }
         }
-        if (lane == 0) tma_store_wait_read();
+        if (elect_one()) tma_store_wait_read();
     }
 
     tc_fence_before();

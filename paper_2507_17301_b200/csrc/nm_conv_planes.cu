@@ -68,7 +68,7 @@ k_conv_planes(const ConvParams p, const PlaneCfg cfg, const __grid_constant__ CU
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
     const uint32_t n_work = static_cast<uint32_t>(cfg.n_work);   // below 2^31: per-item arithmetic stays 32-bit
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t w_smem = base;
@@ -100,11 +100,11 @@ k_conv_planes(const ConvParams p, const PlaneCfg cfg, const __grid_constant__ CU
 
     if (warp < 4) {
         // =========================== MMA issuers ===========================
-        if (lane == 0 && warp == 0) {
+        if (warp == 0 && elect_one()) {
             mbar_arrive_expect_tx(smem_u32(&s_wfull), static_cast<uint32_t>(cfg.w_bytes));
             bulk_load_1d(w_smem, p.ws, static_cast<uint32_t>(cfg.w_bytes), smem_u32(&s_wfull));
         }
-        if (lane == 0 && warp < cfg.r) {
+        if (warp < cfg.r && elect_one()) {
             const int mi = warp;
             const uint32_t idesc = umma_idesc_tf32(BM, p.c_out);
             const uint32_t lbo = S == 2 ? static_cast<uint32_t>(cfg.pe) * 16u : 16u;
@@ -165,7 +165,7 @@ k_conv_planes(const ConvParams p, const PlaneCfg cfg, const __grid_constant__ CU
                 tmem_ld32(tmem + lane_addr + ab * cfg.acc_cols + mi * p.c_out + blk * 32, v);
                 const float bias_cur = bias_next;
                 bias_next = bias_lane_load(p.bias, blk + 1 < n_blk ? (blk + 1) * 32 : 0, p.c_out, lane);
-                if (lane == 0 && nb >= 1) tma_store_wait_read();   // the store that last read the box is done with it
+                if (nb >= 1 && elect_one()) tma_store_wait_read();   // the store that last read the box is done with it
                 __syncwarp();
                 tmem_ld_wait();
                 if (blk == n_blk - 1) {
@@ -196,7 +196,7 @@ k_conv_planes(const ConvParams p, const PlaneCfg cfg, const __grid_constant__ CU
                 }
                 fence_proxy_async();
                 __syncwarp();
-                if (lane == 0) {
+                if (elect_one()) {
                     // output seen as (channel, ow, n * ho + oh): pixels past the row's end are clipped
                     if (box_ok) tma_store_3d(&tm_y, box, blk * 32, q * 32, n * p.ho + oh);
                     tma_store_commit();
@@ -208,7 +208,7 @@ k_conv_planes(const ConvParams p, const PlaneCfg cfg, const __grid_constant__ CU
                 if (lane == 0) mbar_arrive(smem_u32(&s_accfree[ab]));
             }
         }
-        if (lane == 0) tma_store_wait_read();   // shared memory must outlive the stores' reads; the writes complete with the grid
+        if (elect_one()) tma_store_wait_read();   // shared memory must outlive the stores' reads; the writes complete with the grid
     } else {
         // =========================== loaders ===========================
         // One thread per padded pixel: entry (row j, padded column pp) of the band goes to plane pp % S,

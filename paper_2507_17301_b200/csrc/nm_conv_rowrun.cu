@@ -63,7 +63,7 @@ k_conv_rowrun(const ConvParams p, const RowCfg cfg, const __grid_constant__ CUte
     __shared__ int s_koff[MAX_KB * 32];   // per column: kernel row << 24 | float offset inside the row set; -1 = padding
     __shared__ uint32_t s_range[MAX_KB * 32];   // per column: first valid output pixel << 16 | number of valid ones
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
     const uint32_t n_work = static_cast<uint32_t>(cfg.n_work);   // below 2^31: per-item arithmetic stays 32-bit
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t w_smem = base;
@@ -119,7 +119,7 @@ k_conv_rowrun(const ConvParams p, const RowCfg cfg, const __grid_constant__ CUte
 
     if (warp == 0) {
         // =========================== producer ===========================
-        if (lane == 0) {
+        if (elect_one()) {
             mbar_arrive_expect_tx(smem_u32(&s_wfull), static_cast<uint32_t>(cfg.w_bytes));
             bulk_load_1d(w_smem, p.wx, static_cast<uint32_t>(cfg.w_bytes), smem_u32(&s_wfull));
             RingPos rs;
@@ -168,7 +168,7 @@ k_conv_rowrun(const ConvParams p, const RowCfg cfg, const __grid_constant__ CUte
         }
     } else if (warp == 1) {
         // =========================== MMA issuer ===========================
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t idesc = umma_idesc_tf32(BM, cfg.bn);
             if (!mbar_wait(smem_u32(&s_wfull), 0)) *abort_flag = 9;
             RingPos rp;
@@ -219,7 +219,7 @@ k_conv_rowrun(const ConvParams p, const RowCfg cfg, const __grid_constant__ CUte
                     if (lane == 0) mbar_arrive(smem_u32(&s_accfree[ab]));
                 }
                 const uint32_t box = my_staging + (nb & 1u) * 4096;
-                if (lane == 0 && nb >= 2) tma_store_wait_read_n<1>();
+                if (nb >= 2 && elect_one()) tma_store_wait_read_n<1>();
                 __syncwarp();
                 const uint32_t stage_row = box + lane * 128;
                 // pixel of this thread: output row `work`, column q * 32 + lane (past the row's end: none)
@@ -245,14 +245,14 @@ k_conv_rowrun(const ConvParams p, const RowCfg cfg, const __grid_constant__ CUte
                 }
                 fence_proxy_async();
                 __syncwarp();
-                if (lane == 0) {
+                if (elect_one()) {
                     // output seen as (channel, ow, n * ho + oh): pixels past the row's end are clipped
                     if (q * 32 < p.wo) tma_store_3d(&tm_y, box, blk * 32, q * 32, static_cast<int>(work));
                     tma_store_commit();
                 }
             }
         }
-        if (lane == 0) tma_store_wait_read();   // shared memory must outlive the stores' reads; the writes complete with the grid
+        if (elect_one()) tma_store_wait_read();   // shared memory must outlive the stores' reads; the writes complete with the grid
     } else if (warp >= 8) {
         // =========================== builders ===========================
         // Two groups of eight warps build alternate sub-tiles, so that one group's barrier waits and

@@ -167,7 +167,7 @@ k_conv_select(const ConvParams p, const SelCfg cfg, const __grid_constant__ CUte
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
     const uint32_t n_work = static_cast<uint32_t>(cfg.n_work);   // below 2^31: per-item arithmetic stays 32-bit
     const int T = p.tile_t, g = cfg.g;
     const uint32_t p_ring = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -214,7 +214,7 @@ k_conv_select(const ConvParams p, const SelCfg cfg, const __grid_constant__ CUte
 
     if (warp == 0) {
         // =========================== activation producer ===========================
-        if (lane == 0) {
+        if (elect_one()) {
             const int hw = p.ho * p.wo;
             RingPos rp;
             int issued = 0;
@@ -269,7 +269,7 @@ k_conv_select(const ConvParams p, const SelCfg cfg, const __grid_constant__ CUte
         }
     } else if (warp == 1) {
         // =========================== weight producer ===========================
-        if (lane == 0) {
+        if (elect_one()) {
             RingPos rw;
             int issued = 0;
             const size_t chunk_floats = static_cast<size_t>(p.c_out) * 32;
@@ -309,7 +309,7 @@ k_conv_select(const ConvParams p, const SelCfg cfg, const __grid_constant__ CUte
     } else if (warp == 2 || warp == 3 || warp == 16 || warp == 17) {
         // =========================== MMA issuers ===========================
         const int iss = warp < 4 ? warp - 2 : warp - 14;
-        if (lane == 0 && iss < cfg.n_iss) {
+        if (iss < cfg.n_iss && elect_one()) {
             const uint32_t idesc = umma_idesc_tf32(BM, cfg.mma_n);
             const int units_per_tile = T / cfg.mma_n;
             RingPos rw;
@@ -403,7 +403,7 @@ k_conv_select(const ConvParams p, const SelCfg cfg, const __grid_constant__ CUte
                 }
                 // two boxes: the box's previous store (two blocks ago) has read it; a box per block: nothing to wait for
                 const uint32_t box = my_staging + (cfg.boxes == 2 ? (nb & 1u) : static_cast<uint32_t>(blk / ESTEP)) * 4096;
-                if (cfg.boxes == 2 && lane == 0 && nb >= 2) tma_store_wait_read_n<1>();
+                if (cfg.boxes == 2 && nb >= 2 && elect_one()) tma_store_wait_read_n<1>();
                 __syncwarp();
                 const uint32_t stage_row = box + lane * 128;
                 const bool res_pass = p.residual != nullptr && box_pix < p.pixels;
@@ -432,13 +432,13 @@ k_conv_select(const ConvParams p, const SelCfg cfg, const __grid_constant__ CUte
                 }
                 fence_proxy_async();
                 __syncwarp();
-                if (lane == 0) {
+                if (elect_one()) {
                     if (in_range) tma_store_2d(&tm_y, box, o0 + blk * 32, store_row);
                     tma_store_commit();
                 }
             }
         }
-        if (lane == 0) tma_store_wait_read();   // shared memory must outlive the stores' reads; the writes complete with the grid
+        if (elect_one()) tma_store_wait_read();   // shared memory must outlive the stores' reads; the writes complete with the grid
     } else if (warp >= 8 && warp < 16) {
         // =========================== compactors ===========================
         const uint32_t team = static_cast<uint32_t>(warp - 8) >> 2;   // chunks cg = team (mod 2) are this warp's
@@ -560,7 +560,7 @@ k_conv_select(const ConvParams p, const SelCfg cfg, const __grid_constant__ CUte
                     tmem_st_wait();
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) {
+                    if (elect_one()) {
                         mbar_arrive(aready);
                         mbar_arrive(wfree);
                         if (t + 2 >= cfg.taps) mbar_arrive(pfree);   // this team's last chunk of the stage

@@ -63,7 +63,7 @@ k_conv_slab(const ConvParams p, const SlabCfg cfg, const __grid_constant__ CUten
     __shared__ int s_rowoff[BM];
     __shared__ unsigned long long s_rowmask[BM];
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
     const int slice = blockIdx.x % cfg.n_slices;
     const long long pix0 = static_cast<long long>(blockIdx.x / cfg.n_slices) * BM;
     const int tile0 = slice * cfg.g_tiles;
@@ -119,7 +119,7 @@ k_conv_slab(const ConvParams p, const SlabCfg cfg, const __grid_constant__ CUten
     if (warp >= 4 && warp < 8) {
         if (TMA) {
             // =========================== TMA producer (one thread) ===========================
-            if (tid == 128) {
+            if (warp == 4 && elect_one()) {
                 const int hw = p.ho * p.wo;
                 const int n0 = static_cast<int>(pix0 / hw);
                 const int rem = static_cast<int>(pix0 - static_cast<long long>(n0) * hw);
@@ -330,7 +330,7 @@ k_conv_slab(const ConvParams p, const SlabCfg cfg, const __grid_constant__ CUten
                 }
             }
         }
-    } else if (tid == 256) {
+    } else if (warp == 8 && elect_one()) {
         // =========================== MMA issuer ===========================
         const uint32_t idesc = umma_idesc_tf32(BM, cfg.umma_n);
         int use = 0;

@@ -127,7 +127,7 @@ k_conv_stream(const ConvParams p, const StreamCfg cfg, const __grid_constant__ C
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
     const uint32_t n_work = static_cast<uint32_t>(cfg.n_work);   // below 2^31: per-item arithmetic stays 32-bit
     const int NS = cfg.stages, n_chunks = p.v2_chunks, g = cfg.g, T = p.tile_t;
     const uint32_t ring = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -162,7 +162,7 @@ k_conv_stream(const ConvParams p, const StreamCfg cfg, const __grid_constant__ C
 
     if (warp == 0) {
         // =========================== producer ===========================
-        if (lane == 0) {
+        if (elect_one()) {
             const int hw = p.ho * p.wo;
             const size_t rpitch = static_cast<size_t>(n_chunks) * 32;
             const uint32_t tx_fixed = static_cast<uint32_t>(cfg.bn) * 128u + static_cast<uint32_t>(g) * 32u;
@@ -215,7 +215,7 @@ k_conv_stream(const ConvParams p, const StreamCfg cfg, const __grid_constant__ C
         }
     } else if (warp == 1) {
         // =========================== MMA issuer ===========================
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t idesc = umma_idesc_tf32(BM, T);
             RingPos rp;
             uint32_t set = 0, set_par = 0;          // operand set of this chunk, parity of its current use
@@ -289,7 +289,7 @@ k_conv_stream(const ConvParams p, const StreamCfg cfg, const __grid_constant__ C
                     if (lane == 0) mbar_arrive(smem_u32(&s_accfree[ab]));
                 }
                 const uint32_t box = my_staging + (nb & 1u) * 4096;
-                if (lane == 0 && nb >= 2) tma_store_wait_read_n<1>();  // the box's previous store has read it
+                if (nb >= 2 && elect_one()) tma_store_wait_read_n<1>();  // the box's previous store has read it
                 __syncwarp();
                 const uint32_t stage_row = box + lane * 128;
                 // with a shortcut input the activation waits for the second pass below
@@ -321,14 +321,14 @@ k_conv_stream(const ConvParams p, const StreamCfg cfg, const __grid_constant__ C
                 }
                 fence_proxy_async();
                 __syncwarp();
-                if (lane == 0) {
+                if (elect_one()) {
                     if (pix0 + q * 32 < p.pixels)
                         tma_store_2d(&tm_y, box, o0 + blk * 32, static_cast<int>(pix0) + q * 32);
                     tma_store_commit();
                 }
             }
         }
-        if (lane == 0) tma_store_wait_read();   // shared memory must outlive the stores' reads; the writes complete with the grid
+        if (elect_one()) tma_store_wait_read();   // shared memory must outlive the stores' reads; the writes complete with the grid
     } else if (warp >= 8) {
         // =========================== compactors ===========================
         const int wg = (warp - 8) >> 2;   // which half of the chunk
@@ -390,7 +390,7 @@ k_conv_stream(const ConvParams p, const StreamCfg cfg, const __grid_constant__ C
                 tmem_st_wait();
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) {
+                if (elect_one()) {
                     mbar_arrive(smem_u32(&s_aready[set]));
                     mbar_arrive(smem_u32(&s_free[s]));
                 }

@@ -87,7 +87,7 @@ k_conv_window(const ConvParams p, const WinCfg cfg, const __grid_constant__ CUte
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
     const uint32_t n_work = static_cast<uint32_t>(cfg.n_work);   // below 2^31: per-item arithmetic stays 32-bit
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t p_ring = base;
@@ -116,7 +116,7 @@ k_conv_window(const ConvParams p, const WinCfg cfg, const __grid_constant__ CUte
 
     if (warp == 0) {
         // =========================== patch producer ===========================
-        if (lane == 0) {
+        if (elect_one()) {
             RingPos rp;
             int issued = 0;
             for (uint32_t work = blockIdx.x; work < n_work && !aborted(abort_flag); work += gridDim.x) {
@@ -141,7 +141,7 @@ k_conv_window(const ConvParams p, const WinCfg cfg, const __grid_constant__ CUte
         }
     } else if (warp == 1) {
         // =========================== weight producer ===========================
-        if (lane == 0) {
+        if (elect_one()) {
             RingPos rw;
             int issued = 0;
             const size_t blk_floats = static_cast<size_t>(p.c_out) * 32;
@@ -175,7 +175,7 @@ k_conv_window(const ConvParams p, const WinCfg cfg, const __grid_constant__ CUte
         // One thread per M-tile: a single thread cannot issue small MMAs as fast as the tensor core
         // retires them, and the M-tiles have separate accumulators, so each gets its own issuer.
         // Ring slots and accumulator hand-offs count one commit per issuer.
-        if (lane == 0) {
+        if (elect_one()) {
             const int mi = warp - 2;
             const uint32_t idesc = umma_idesc_tf32(BM, cfg.bn);
             // one tap to the right = dil_w patch rows of 128 bytes; after the last tap of a kernel row,
