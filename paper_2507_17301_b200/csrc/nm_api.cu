@@ -25,20 +25,11 @@ int kept_count(int k, int n_keep, int m_group)
     return full * n_keep + std::min(tail, n_keep);
 }
 
-void free_handle_memory(nm_weights* h)
+// `idle`: the device has been synchronised, so the block may serve the next handle.
+void free_handle_memory(nm_weights* h, bool idle)
 {
     if (!h) return;
-    cudaFree(h->values);
-    cudaFree(h->indices);
-    cudaFree(h->wt);
-    cudaFree(h->taps);
-    cudaFree(h->status);
-    cudaFree(h->wt2);
-    cudaFree(h->rel2);
-    cudaFree(h->wx);
-    cudaFree(h->w3);
-    cudaFree(h->sel3);
-    cudaFree(h->ws);
+    nmhost::device_block_free(h->block, h->block_bytes, h->device, idle);
     cudaFree(h->splitk);
     h->magic = 0;
     delete h;
@@ -77,18 +68,10 @@ nm_status_t make_handle(const char* who, int c_out, int kh, int kw, int c_in, in
     h->kk = kept_count(h->k, n_keep, m_group);
     h->n_tiles = (c_out + tile_t - 1) / tile_t;
     h->kk_pad = ((h->kk + NM_KCHUNK - 1) / NM_KCHUNK) * NM_KCHUNK;
-    const size_t nv = static_cast<size_t>(c_out) * std::max(h->kk, 1);
-    const size_t ni = static_cast<size_t>(h->n_tiles) * std::max(h->kk, 1);
-    const size_t nw = static_cast<size_t>(c_out) * h->kk_pad;
-    const size_t nt = static_cast<size_t>(h->n_tiles) * h->kk_pad;
-    if (cudaMalloc(&h->values, nv * sizeof(float)) != cudaSuccess ||
-        cudaMalloc(&h->indices, ni * sizeof(uint16_t)) != cudaSuccess ||
-        cudaMalloc(&h->wt, std::max<size_t>(nw, 1) * sizeof(float)) != cudaSuccess ||
-        cudaMalloc(&h->taps, std::max<size_t>(nt, 1) * sizeof(uint32_t)) != cudaSuccess ||
-        cudaMalloc(&h->status, 4 * sizeof(int)) != cudaSuccess || cudaMemset(h->status, 0, 4 * sizeof(int)) != cudaSuccess) {
-        const char* msg = cudaGetErrorString(cudaGetLastError());
-        free_handle_memory(h);
-        return nmhost::fail(NM_ERR_ALLOC, "%s: device allocation failed: %s", who, msg);
+    const nm_status_t s = nmhost::alloc_handle_memory(h, who);
+    if (s != NM_OK) {
+        delete h;
+        return s;
     }
     *out = h;
     return NM_OK;
@@ -312,12 +295,8 @@ nm_status_t nm_prune(const float* w_dense, int c_out, int kh, int kw, int c_in, 
     nm_status_t s = make_handle("nm_prune", c_out, kh, kw, c_in, n_keep, m_group, tile_t, &h);
     if (s != NM_OK) return s;
     s = nmhost::prune_on_device(w_dense, h, static_cast<cudaStream_t>(cuda_stream));
-    if (s == NM_OK) s = nmhost::build_slab_layout(h, static_cast<cudaStream_t>(cuda_stream));
-    if (s == NM_OK) s = nmhost::build_expanded_layout(h, static_cast<cudaStream_t>(cuda_stream));
-    if (s == NM_OK) s = nmhost::build_select_layout(h, static_cast<cudaStream_t>(cuda_stream));
-    if (s == NM_OK) s = nmhost::build_planes_layout(h, static_cast<cudaStream_t>(cuda_stream));
     if (s != NM_OK) {
-        free_handle_memory(h);
+        free_handle_memory(h, false);
         return s;
     }
     *out = h;
@@ -332,12 +311,8 @@ nm_status_t nm_weights_import(const float* values, const uint16_t* indices, int 
     nm_status_t s = make_handle("nm_weights_import", c_out, kh, kw, c_in, n_keep, m_group, tile_t, &h);
     if (s != NM_OK) return s;
     s = nmhost::build_from_compressed(values, indices, h, static_cast<cudaStream_t>(cuda_stream));
-    if (s == NM_OK) s = nmhost::build_slab_layout(h, static_cast<cudaStream_t>(cuda_stream));
-    if (s == NM_OK) s = nmhost::build_expanded_layout(h, static_cast<cudaStream_t>(cuda_stream));
-    if (s == NM_OK) s = nmhost::build_select_layout(h, static_cast<cudaStream_t>(cuda_stream));
-    if (s == NM_OK) s = nmhost::build_planes_layout(h, static_cast<cudaStream_t>(cuda_stream));
     if (s != NM_OK) {
-        free_handle_memory(h);
+        free_handle_memory(h, false);
         *out = nullptr;
         return s;
     }
@@ -443,8 +418,12 @@ nm_status_t nm_weights_free(nm_weights_t* w)
 {
     if (!w) return NM_OK;
     if (!valid(w)) return nmhost::fail(NM_ERR_INVALID_ARG, "nm_weights_free: bad weights handle");
-    cudaDeviceSynchronize();
-    free_handle_memory(w);
+    // the device the handle lives on, which need not be the current one
+    int dev = w->device;
+    const bool moved = cudaGetDevice(&dev) == cudaSuccess && dev != w->device && cudaSetDevice(w->device) == cudaSuccess;
+    const bool idle = cudaDeviceSynchronize() == cudaSuccess;
+    free_handle_memory(w, idle);
+    if (moved) cudaSetDevice(dev);
     return NM_OK;
 }
 

@@ -346,46 +346,9 @@ bool encode_y_rows(const ConvParams& p, CUtensorMap* tm)
                                   CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// The handle's weights for this kernel: ws[kh][c_out][32] TF32; a row holds the taps of one kernel row as
-// (kw, c) with c padded to 4 and kw to 8, its 16-byte pieces (one tap each) XOR-ed with (o % 8) (128-byte
-// swizzle); zeros in the padding and in pruned columns.
-__global__ void k_build_ws(const float* __restrict__ values, const uint16_t* __restrict__ indices, int c_out, int kk,
-                           int tile_t, int kw, int c_in, float* __restrict__ ws)
-{
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    const int o = blockIdx.y;
-    if (j >= kk) return;
-    const int k = indices[static_cast<size_t>(o / tile_t) * kk + j];
-    const int run = kw * c_in;
-    const int khi = k / run, r = k - khi * run;
-    const int kwi = r / c_in, c = r - kwi * c_in;
-    ws[(static_cast<size_t>(khi) * c_out + o) * 32 + ((kwi ^ (o & 7)) << 2) + c] = to_tf32(values[static_cast<size_t>(o) * kk + j]);
-}
-
 }  // namespace
 
 namespace nmhost {
-
-nm_status_t build_planes_layout(nm_weights* h, cudaStream_t st)
-{
-    h->ws = nullptr;
-    if (h->c_in > 4 || h->kw > 8 || h->c_out % 32 != 0 || h->c_out > 256 || h->kk == 0 || h->kh * h->c_out * 128 >= (1 << 20))
-        return NM_OK;
-    const size_t bytes = static_cast<size_t>(h->kh) * h->c_out * 32 * sizeof(float);
-    if (cudaMalloc(&h->ws, bytes) != cudaSuccess) {
-        (void)cudaGetLastError();
-        h->ws = nullptr;
-        return fail(NM_ERR_ALLOC, "cannot allocate the plane-kernel weights (%zu bytes)", bytes);
-    }
-    cudaError_t e = cudaMemsetAsync(h->ws, 0, bytes, st);
-    if (e != cudaSuccess) return fail(NM_ERR_CUDA, "plane layout memset: %s", cudaGetErrorString(e));
-    const dim3 grid((h->kk + 127) / 128, h->c_out);
-    k_build_ws<<<grid, 128, 0, st>>>(h->values, h->indices, h->c_out, h->kk, h->tile_t, h->kw, h->c_in, h->ws);
-    count_launch(1);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return fail(NM_ERR_CUDA, "plane layout kernel: %s", cudaGetErrorString(e));
-    return NM_OK;
-}
 
 bool planes_plan_ok(const ConvParams& p, const nm_plan_t* plan)
 {

@@ -783,80 +783,17 @@ nm_status_t launch(const ConvParams& p, const SelCfg& cfg, cudaStream_t st)
     return NM_OK;
 }
 
-// ---- the handle's copy of the compressed form for this kernel -------------------------------------------
-// Retained weights per chunk as the shared-memory image the tensor core reads: w3[chunk][o][32] TF32, of a row's
-// 32 slots the first KC used, the row's 16-byte pieces XOR-ed with (o % 8) (128-byte swizzle), so that the
-// rows of any run of tiles are one contiguous bulk copy.
-__global__ void k_build_w3(const float* __restrict__ values, const uint16_t* __restrict__ indices, int c_out, int kk,
-                           int tile_t, int s_cols, int kc, float* __restrict__ w3)
-{
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    const int o = blockIdx.y;
-    if (j >= kk) return;
-    const int col = indices[static_cast<size_t>(o / tile_t) * kk + j];
-    const int chunk = col / s_cols;
-    const int jj = j - chunk * kc;   // every group is full: a chunk holds exactly kc retained columns
-    w3[(static_cast<size_t>(chunk) * c_out + o) * 32 + ((((jj >> 2) ^ (o & 7)) << 2) | (jj & 3))] =
-        nmk::to_tf32(values[static_cast<size_t>(o) * kk + j]);
-}
-
-// Select masks: for retained column j (the jn-th of its group, at position pos in the group) the D = M - N words
-// m[i] = all ones iff pos == jn + i, i < D (all zero: the column is the last candidate, jn + D); `mw` bytes per tile and chunk.
-__global__ void k_build_sel3(const uint16_t* __restrict__ indices, int n_tiles, int kk, int n_keep, int m_group,
-                             int s_cols, int kc, int mw, uint8_t* __restrict__ sel3)
-{
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    const int r = blockIdx.y;
-    if (j >= kk) return;
-    const int d = m_group - n_keep;
-    const int col = indices[static_cast<size_t>(r) * kk + j];
-    const int chunk = col / s_cols;
-    const int jj = j - chunk * kc;           // slot within the chunk = group-in-chunk * N + jn
-    const int jn = jj % n_keep;
-    const int pos = col % m_group;
-    uint32_t* m = reinterpret_cast<uint32_t*>(sel3 + (static_cast<size_t>(chunk) * n_tiles + r) * mw) + static_cast<size_t>(jj) * d;
-    for (int i = 0; i < d; ++i) m[i] = (pos == jn + i) ? 0xFFFFFFFFu : 0u;
-}
-
 }  // namespace
 
 namespace nmhost {
 
-nm_status_t build_select_layout(nm_weights* h, cudaStream_t st)
+bool select_layout_dims(const nm_weights* h, int* s, int* kc, int* mw)
 {
-    h->w3 = nullptr;
-    h->sel3 = nullptr;
-    h->sel_s = h->sel_kc = h->sel_mw = 0;
     ConvParams probe = {};
     probe.n_keep = h->n_keep;
     probe.m_group = h->m_group;
-    int S = 0, KC = 0, MW = 0;
-    if (!dims_of(pattern_code(probe), &S, &KC, &MW)) return NM_OK;
-    if (h->kk == 0 || h->k % h->m_group != 0 || h->c_in % S != 0 || h->tile_t % 16 != 0 || h->c_out % h->tile_t != 0)
-        return NM_OK;
-    const int chunks = h->k / S;
-    const size_t wbytes = static_cast<size_t>(chunks) * h->c_out * 32 * sizeof(float);
-    const size_t mbytes = static_cast<size_t>(chunks) * h->n_tiles * MW;
-    if (cudaMalloc(&h->w3, wbytes) != cudaSuccess || cudaMalloc(&h->sel3, mbytes) != cudaSuccess) {
-        (void)cudaGetLastError();
-        cudaFree(h->w3);
-        h->w3 = nullptr;
-        h->sel3 = nullptr;
-        return fail(NM_ERR_ALLOC, "cannot allocate the select-kernel weights");
-    }
-    cudaError_t e = cudaMemsetAsync(h->w3, 0, wbytes, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->sel3, 0, mbytes, st);   // the padding bytes of a tile's masks
-    if (e != cudaSuccess) return fail(NM_ERR_CUDA, "select layout memset: %s", cudaGetErrorString(e));
-    const dim3 gw((h->kk + 127) / 128, h->c_out), gm((h->kk + 127) / 128, h->n_tiles);
-    k_build_w3<<<gw, 128, 0, st>>>(h->values, h->indices, h->c_out, h->kk, h->tile_t, S, KC, h->w3);
-    k_build_sel3<<<gm, 128, 0, st>>>(h->indices, h->n_tiles, h->kk, h->n_keep, h->m_group, S, KC, MW, h->sel3);
-    count_launch(2);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return fail(NM_ERR_CUDA, "select layout kernels: %s", cudaGetErrorString(e));
-    h->sel_s = S;
-    h->sel_kc = KC;
-    h->sel_mw = MW;
-    return NM_OK;
+    if (!dims_of(pattern_code(probe), s, kc, mw)) return false;
+    return h->kk > 0 && h->k % h->m_group == 0 && h->c_in % *s == 0 && h->tile_t % 16 == 0 && h->c_out % h->tile_t == 0;
 }
 
 bool select_plan_ok(const ConvParams& p, const nm_plan_t* plan)

@@ -14,6 +14,9 @@ constexpr int NM_KCHUNK = 32;               // kept columns per shared-memory op
 struct nm_weights {
     uint32_t magic;
     int device;
+    uint8_t* block;      // the handle's device memory: one allocation that every array below except `splitk` lies in
+    size_t block_bytes, block_used, zero_from;   // size of the block, bytes of it in use, first byte of the part that is cleared
+    double* mass;        // device double[2] + int: L1 sums of the pruning pass, validity of imported indices
     int c_out, kh, kw, c_in, k, kk, n_keep, m_group, tile_t, n_tiles;
     int kk_pad;          // kk rounded up to a multiple of NM_KCHUNK
     double l1_total, l1_kept;   // L1 mass of the dense weights / of the retained ones (l1_total < 0: not known)
@@ -31,15 +34,15 @@ struct nm_weights {
     // Expanded layout (variant 4): the pruned matrix back in dense shape, zeros in the pruned columns.
     float* splitk;       // scratch for split-K partial sums (variant 4), allocated by nm_autotune; may be NULL
     size_t splitk_bytes;
-    float* wx;           // [ceil(k / 32)][wx_rows][32] TF32, rows swizzled (see k_expand); NULL when the shape rules the variant out
+    float* wx;           // [ceil(k / 32)][wx_rows][32] TF32, rows swizzled (see k_build_layouts); NULL when the shape rules the variant out
     int wx_rows;         // c_out rounded up to a multiple of 32 (the rows past c_out are zero)
     // Select layout (variant 8): chunks of sel_s source columns of which every tile keeps sel_kc; NULL when the
     // pattern or the shape rules the variant out.
-    float* w3;           // [k / sel_s][c_out][32] TF32, rows swizzled (see k_build_w3)
-    uint8_t* sel3;       // [k / sel_s][n_tiles][sel_mw bytes] select masks, 32-bit words (see k_build_sel3)
+    float* w3;           // [k / sel_s][c_out][32] TF32, rows swizzled (see k_build_layouts)
+    uint8_t* sel3;       // [k / sel_s][n_tiles][sel_mw bytes] select masks, 32-bit words (see k_build_layouts)
     int sel_s, sel_kc, sel_mw;
     // Plane layout (variant 9): per kernel row a [c_out][32] tile of (kw, c) slots; NULL when the shape rules it out.
-    float* ws;           // [kh][c_out][32] TF32, rows swizzled (see k_build_ws)
+    float* ws;           // [kh][c_out][32] TF32, rows swizzled (see k_build_layouts)
 };
 
 // Geometry handed to the convolution kernels.
@@ -139,12 +142,18 @@ cudaError_t ensure_dynamic_smem(const void* kernel, size_t bytes);
 nm_status_t fail(nm_status_t s, const char* fmt, ...);
 void count_launch(int n = 1);
 
+// nm_layout.cu: the handles' device memory, and the kernel-side copies of the compressed form
+void* device_block_alloc(size_t bytes, int device, size_t* got);   // NULL when there is no memory; reuses blocks of freed handles
+void device_block_free(void* ptr, size_t bytes, int device, bool idle);   // idle: nothing on the device uses it any more
+nm_status_t alloc_handle_memory(nm_weights* h, const char* who);
+nm_status_t clear_handle_memory(nm_weights* h, cudaStream_t st);   // the part of the block that is not written in full
+// Values and layouts from the index array `idx` and the dense weights (import = false) or the retained values (true).
+nm_status_t build_layouts(nm_weights* h, const float* src, const uint16_t* idx, bool import, cudaStream_t st);
+nm_status_t finish_handle(nm_weights* h, cudaStream_t st, double* mass2, int* bad);   // synchronises `st`
+
 // nm_prune.cu
 nm_status_t prune_on_device(const float* w_dense, nm_weights* h, cudaStream_t st);
 nm_status_t build_from_compressed(const float* values, const uint16_t* indices, nm_weights* h, cudaStream_t st);
-
-nm_status_t build_slab_layout(nm_weights* h, cudaStream_t st);
-nm_status_t build_expanded_layout(nm_weights* h, cudaStream_t st);
 
 // nm_conv_gather.cu — variant 1
 nm_status_t launch_conv_gather(const ConvParams& p, cudaStream_t st);
@@ -180,13 +189,12 @@ bool stream_plan_ok(const ConvParams& p, const nm_plan_t* plan);
 nm_status_t launch_conv_stream(const ConvParams& p, const nm_plan_t* plan, cudaStream_t st);
 
 // nm_conv_select.cu — variant 8
-nm_status_t build_select_layout(nm_weights* h, cudaStream_t st);
+bool select_layout_dims(const nm_weights* h, int* s, int* kc, int* mw);   // false: the pattern or shape rules the kernel out
 bool select_plan_ok(const ConvParams& p, const nm_plan_t* plan);
 size_t select_splitk_bytes(const ConvParams& p, int splits);
 nm_status_t launch_conv_select(const ConvParams& p, const nm_plan_t* plan, cudaStream_t st);
 
 // nm_conv_planes.cu — variant 9
-nm_status_t build_planes_layout(nm_weights* h, cudaStream_t st);
 bool planes_plan_ok(const ConvParams& p, const nm_plan_t* plan);
 nm_status_t launch_conv_planes(const ConvParams& p, const nm_plan_t* plan, cudaStream_t st);
 }  // namespace nmhost
