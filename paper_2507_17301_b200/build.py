@@ -1,5 +1,8 @@
 """Builds ``libnm_b200.so`` (the C-ABI library) in-tree with nvcc for sm_100a.
 
+``_nm_binding`` (``csrc/nm_binding.cpp``), the CPython extension through which ``nm.py`` makes its per-layer calls, is
+built beside it with g++ against torch's headers.
+
 Every ``csrc/*.cu`` is compiled to its own object under ``_build/`` (in parallel, and only when the
 source or a header is newer than the object), then the objects are linked into the shared library.
 """
@@ -9,6 +12,7 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -16,6 +20,30 @@ CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libnm_b200.so")
 ARCH = ["-gencode", "arch=compute_100a,code=sm_100a"]
+
+
+BINDING_SRC = os.path.join(CSRC, "nm_binding.cpp")
+BINDING = os.path.join(HERE, "_nm_binding" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
+
+
+def build_binding(force: bool = False) -> str:
+    """Compiles the CPython extension; returns its path."""
+    deps = [BINDING_SRC, os.path.join(os.path.dirname(HERE), "include", "nm.h")]
+    if not force and os.path.exists(BINDING) and os.path.getmtime(BINDING) > max(os.path.getmtime(d) for d in deps):
+        return BINDING
+    import torch
+
+    root = os.path.dirname(torch.__file__)
+    inc = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
+           sysconfig.get_paths()["include"], os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")]
+    lib = os.path.join(root, "lib")
+    tmp = BINDING + f".tmp{os.getpid()}"
+    subprocess.check_call(
+        ["g++", "-O2", "-std=c++20", "-shared", "-fPIC", "-fvisibility=hidden", "-w",
+         f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", "-o", tmp, BINDING_SRC]
+        + [f"-I{d}" for d in inc] + [f"-L{lib}", f"-Wl,-rpath,{lib}", "-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10"])
+    os.replace(tmp, BINDING)
+    return BINDING
 
 
 def sources():
@@ -51,6 +79,8 @@ def build(force: bool = False, verbose: bool = False, defines=(), suffix: str = 
         raise ValueError("a build with extra macros needs a suffix of its own")
     lib = LIB[:-3] + suffix + ".so"
     objdir = OBJ + suffix
+    if not suffix:
+        build_binding(force)
     if not force and not _stale(lib):
         return lib
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")

@@ -1,4 +1,5 @@
-"""ctypes binding of the C-ABI library (``include/nm.h``): same names, argument marshalling only.
+"""Binding of the C-ABI library (``include/nm.h``): same names, argument marshalling only (ctypes; the calls a
+network makes per layer go through the CPython extension ``_nm_binding``, which does the same steps in native code).
 
 Every function takes torch CUDA tensors (used purely as device memory) and passes their
 ``data_ptr()`` plus ``torch.cuda.current_stream().cuda_stream`` to the library.  No step of the
@@ -95,6 +96,13 @@ def _load():
 
 _lib = _load()
 
+try:
+    from . import _nm_binding
+except ImportError as e:
+    raise ImportError("the CPython extension _nm_binding is not built; run `python -m paper_2507_17301_b200.build` "
+                      f"(there is no fallback path without it): {e}") from e
+_nm_binding.bind(*(ctypes.cast(f, ctypes.c_void_p).value for f in (_lib.nm_conv2d, _lib.nm_conv2d_res, _lib.nm_maxpool2d)))
+
 EXPORTS = ("nm_plan_key", "nm_plan_cache_store", "nm_plan_cache_lookup", "nm_selftest_wait_expiry", "nm_maxpool2d", "nm_weights_retained_l1", "nm_conv2d_res", "nm_plan_scratch_bytes", "nm_weights_reserve", "nm_prune", "nm_prune_noalloc", "nm_weights_dims", "nm_weights_export", "nm_weights_import", "nm_weights_check",
            "nm_weights_free", "nm_conv2d", "nm_conv2d_host", "nm_autotune", "nm_autotune_tile",
            "nm_status_string", "nm_last_error", "nm_launch_count")
@@ -117,8 +125,7 @@ def _check(status: int):
         raise NmError(status, nm_last_error())
 
 
-def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+_stream = _nm_binding.stream_ptr   # the current stream of the current device, as an address
 
 
 def _dev_f32(t: torch.Tensor, what: str) -> int:
@@ -136,6 +143,7 @@ class Weights:
 
     def __init__(self, handle: int):
         self._h = ctypes.c_void_p(handle)
+        self._addr = handle or 0
         dims = [ctypes.c_int() for _ in range(5)]
         _check(_lib.nm_weights_dims(self._h, *[ctypes.byref(d) for d in dims]))
         self.c_out, self.k, self.kk, self.n_tiles, self.tile_t = (d.value for d in dims)
@@ -148,6 +156,7 @@ class Weights:
         if self._h is not None and self._h.value:
             _lib.nm_weights_free(self._h)
         self._h = None
+        self._addr = 0
 
     def __del__(self):
         try:
@@ -231,14 +240,9 @@ def nm_weights_reserve(w: Weights, nbytes: int):
 
 def nm_maxpool2d(x: torch.Tensor, kernel=3, stride=2, pad=1, y: torch.Tensor | None = None) -> torch.Tensor:
     """Max pooling of CUDA fp32 NHWC activations; allocates ``y`` unless given."""
-    kernel, stride, pad = _pair(kernel), _pair(stride), _pair(pad)
-    b, h, wd, c = x.shape
-    if y is None:
-        ho = (h + 2 * pad[0] - kernel[0]) // stride[0] + 1
-        wo = (wd + 2 * pad[1] - kernel[1]) // stride[1] + 1
-        y = torch.empty((b, max(ho, 1), max(wo, 1), c), dtype=torch.float32, device=x.device)
-    _check(_lib.nm_maxpool2d(_dev_f32(x, "x"), b, h, wd, c, kernel[0], kernel[1], stride[0], stride[1], pad[0], pad[1],
-                             _dev_f32(y, "y"), _stream()))
+    y = _nm_binding.maxpool2d(x, kernel, stride, pad, y)
+    if y.__class__ is int:
+        _check(y)
     return y
 
 
@@ -295,26 +299,10 @@ def nm_conv2d(w: Weights, x: torch.Tensor, kh: int, kw: int, stride=1, pad=0, di
               residual: torch.Tensor | None = None) -> torch.Tensor:
     """``x``: CUDA fp32 NHWC.  Allocates ``y`` (NHWC) unless given.  Asynchronous on the current stream.
     With ``residual`` (NHWC, the output's shape) it calls ``nm_conv2d_res``: act(conv + bias + residual)."""
-    stride, pad, dil = _pair(stride), _pair(pad), _pair(dil)
-    xp = _dev_f32(x, "x")
-    b, h, wd, _ = x.shape
-    if y is None:
-        if min(stride) < 1 or min(dil) < 1:  # let the library report it
-            y = torch.empty(4, dtype=torch.float32, device=x.device)
-        else:
-            shape = out_shape(x.shape, kh, kw, w.c_out, stride, pad, dil)
-            y = torch.empty([max(d, 1) for d in shape], dtype=torch.float32, device=x.device)
-    yp = _dev_f32(y, "y")
-    bp = _dev_f32(bias, "bias") if bias is not None else None
-    pl = ctypes.byref(plan) if plan is not None else None
-    if residual is None:
-        _check(_lib.nm_conv2d(w.handle, xp, b, h, wd, stride[0], stride[1], pad[0], pad[1], dil[0], dil[1], bp,
-                              int(bool(relu)), yp, pl, _stream()))
-    else:
-        if tuple(residual.shape) != tuple(y.shape):
-            raise TypeError("residual must have the output's shape")
-        _check(_lib.nm_conv2d_res(w.handle, xp, b, h, wd, stride[0], stride[1], pad[0], pad[1], dil[0], dil[1], bp,
-                                  _dev_f32(residual, "residual"), int(bool(relu)), yp, pl, _stream()))
+    y = _nm_binding.conv2d(w._addr, w.c_out, x, kh, kw, stride, pad, dil, bias, relu, y,
+                           0 if plan is None else ctypes.addressof(plan), residual)
+    if y.__class__ is int:
+        _check(y)
     return y
 
 

@@ -1,0 +1,47 @@
+"""The per-call extension: argument checks (no GPU) and the output it allocates."""
+import pytest
+import torch
+
+from paper_2507_17301_b200 import nm
+
+
+def test_host_tensors_and_wrong_types_are_refused():
+    x = torch.zeros(1, 4, 4, 8)
+    w = nm.Weights.__new__(nm.Weights)
+    w._h, w._addr, w.c_out = None, 0, 8
+    for bad in (x, x.double(), None, 3):
+        with pytest.raises(TypeError, match="x must be a contiguous float32 CUDA tensor"):
+            nm.nm_conv2d(w, bad, 1, 1)
+        with pytest.raises(TypeError, match="x must be"):
+            nm.nm_maxpool2d(bad)
+    with pytest.raises((TypeError, IndexError)):
+        nm.nm_conv2d(w, x, 1, 1, stride=(1,))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("h,w,k,stride,pad,dil", [(7, 9, 3, (2, 1), (1, 0), (1, 2)), (5, 5, 5, 1, 0, 1), (8, 3, 1, 3, 0, 1)])
+def test_allocated_output_has_the_librarys_shape(h, w, k, stride, pad, dil):
+    x = torch.randn(2, h, w, 8, device="cuda")
+    hnd = nm.nm_prune(torch.randn(12, k, k, 8, device="cuda"), 2, 4, 4)
+    y = nm.nm_conv2d(hnd, x, k, k, stride, pad, dil)
+    assert tuple(y.shape) == nm.out_shape(x.shape, k, k, 12, nm._pair(stride), nm._pair(pad), nm._pair(dil))
+    given = torch.empty_like(y)
+    assert nm.nm_conv2d(hnd, x, k, k, stride, pad, dil, y=given) is given
+    assert torch.equal(given, y)
+    with pytest.raises(TypeError, match="residual must have the output's shape"):
+        nm.nm_conv2d(hnd, x, k, k, stride, pad, dil, residual=torch.zeros(1, 1, 1, 12, device="cuda"))
+    with pytest.raises(TypeError, match="y must be"):
+        nm.nm_conv2d(hnd, x, k, k, stride, pad, dil, y=given.double())
+    hnd.free()
+    with pytest.raises(nm.NmError):
+        nm.nm_conv2d(hnd, x, k, k, stride, pad, dil)
+
+
+@pytest.mark.gpu
+def test_calls_go_to_the_current_stream():
+    x = torch.randn(1, 6, 6, 8, device="cuda")
+    side = torch.cuda.Stream()
+    assert nm._stream() == torch.cuda.current_stream().cuda_stream
+    with torch.cuda.stream(side):
+        assert nm._stream() == side.cuda_stream
+    assert torch.equal(nm.nm_maxpool2d(x, 2, 2, 0), torch.nn.functional.max_pool2d(x.permute(0, 3, 1, 2), 2, 2).permute(0, 2, 3, 1))
