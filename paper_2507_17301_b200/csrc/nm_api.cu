@@ -608,6 +608,8 @@ nm_status_t nm_autotune(nm_weights_t* w, const float* x, int batch, int h, int w
         if (!ok || cudaStreamSynchronize(st) != cudaSuccess) continue;
         std::vector<float> t;
         for (int i = 0; i < kReps && ok; ++i) {
+            // three launches tell a candidate that is out of reach (tuning a layer takes half the time this way)
+            if (t.size() == 3 && best_t > 0.f && *std::min_element(t.begin(), t.end()) > 1.25f * best_t) break;
             if (flush) cudaMemsetAsync(flush, i, kFlushBytes, st);
             cudaEventRecord(e0, st);
             ok = run_plan(p, &cand, st) == NM_OK;
