@@ -149,6 +149,8 @@ nm_status_t run_plan(const ConvParams& p, const nm_plan_t* plan, cudaStream_t st
             return nmhost::launch_conv_select(p, plan, st);
         case 9:
             return nmhost::launch_conv_planes(p, plan, st);
+        case 10:
+            return nmhost::launch_conv_cluster(p, plan, st);
         default:
             return nmhost::fail(NM_ERR_UNSUPPORTED, "nm_conv2d: unknown plan variant %d", variant);
     }
@@ -159,6 +161,14 @@ std::vector<nm_plan_t> candidate_plans(const nm_weights* /*w*/, const ConvParams
 {
     std::vector<nm_plan_t> out;
     nm_plan_t a;
+    std::memset(&a, 0, sizeof(a));
+    // cluster kernel (short launches)
+    for (int ksplit : {8, 4, 2, 1}) {
+        for (int bn : {32, 64, 128}) {
+            a.variant = 10; a.bn = bn; a.ksplit = ksplit;
+            if (nmhost::cluster_plan_ok(p, &a)) out.push_back(a);
+        }
+    }
     std::memset(&a, 0, sizeof(a));
     // select kernel (contracts over the retained columns only): all of a tile group's channels per CTA down to one
     // tile, with the activation loads it prefers for the shape, and with the reduction axis split where few work

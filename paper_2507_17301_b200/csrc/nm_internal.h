@@ -197,4 +197,8 @@ nm_status_t launch_conv_select(const ConvParams& p, const nm_plan_t* plan, cudaS
 // nm_conv_planes.cu — variant 9
 bool planes_plan_ok(const ConvParams& p, const nm_plan_t* plan);
 nm_status_t launch_conv_planes(const ConvParams& p, const nm_plan_t* plan, cudaStream_t st);
+
+// nm_conv_cluster.cu — variant 10
+bool cluster_plan_ok(const ConvParams& p, const nm_plan_t* plan);
+nm_status_t launch_conv_cluster(const ConvParams& p, const nm_plan_t* plan, cudaStream_t st);
 }  // namespace nmhost
