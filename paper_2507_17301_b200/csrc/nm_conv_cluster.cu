@@ -7,9 +7,10 @@
 // cluster of S = 1, 2, 4 or 8 CTAs, each of which
 //   * accumulates its contiguous range of 32-column blocks in tensor memory (operands as in variant 4: dense activations
 //     by TMA, zero-expanded weights by bulk copy, SS MMA),
-//   * sends every row of its partial sums to the CTA that finishes the row (the rows of an item are dealt to the CTAs in S
-//     runs): asynchronous stores into that CTA's shared memory, counted by a barrier there, so that nobody waits for the
-//     whole cluster, and
+//   * sends every run of rows of its partial sums to the CTA that finishes the run (the rows of an item are dealt to the CTAs
+//     in S runs): one bulk copy from shared to distributed shared memory each, counted by a barrier there (with remote
+//     stores of 16 bytes each, plain or asynchronous, it took 1.3-1.9 us from the accumulator to the last arrival; 0.7 us with
+//     the copies, ResNet-50 at batch 1 343 -> 316 us), and
 //   * once its own rows are complete adds the S partial sums in the order of the ranges (the result does not depend on
 //     timing), adds bias and shortcut, applies the activation and writes whole 128-byte rows to NHWC.
 // No scratch memory, no second launch.  A CTA takes a quarter to a half of an SM's shared memory and BN tensor-memory columns, so
@@ -62,11 +63,11 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const void* tmap, uint
         ::"r"(dst), "l"(tmap), "r"(bar), "r"(c), "r"(w), "r"(h), "r"(n)
         : "memory");
 }
-// 16 bytes into the shared memory of a CTA of the cluster; their arrival is counted by a barrier of that CTA.
-__device__ __forceinline__ void st_async_v4(uint32_t addr, uint32_t bar, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
+// Shared memory of this CTA to that of a CTA of the cluster; the barrier is one of the receiving CTA.
+__device__ __forceinline__ void bulk_copy_cluster(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar)
 {
-    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%2, %3, %4, %5}, [%1];" ::"r"(addr), "r"(bar),
-                 "r"(a), "r"(b), "r"(c), "r"(d)
+    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "r"(src),
+                 "r"(bytes), "r"(bar)
                  : "memory");
 }
 __device__ __forceinline__ float4 ld_shared_f4(uint32_t addr)
@@ -255,41 +256,43 @@ k_conv_cluster(const ConvParams p, const ClusterCfg cfg, const __grid_constant__
         const bool ok = aborted(abort_flag) || mbar_wait(smem_u32(&s_acc), 0);
         if (!__all_sync(0xFFFFFFFFu, ok)) *abort_flag = 4;
         tc_fence_after();
-        // a row of partial sums per thread, to the CTA that finishes it; 16-byte pieces XOR-ed with the row, so that the 32
-        // rows of a warp do not meet in one bank
+        // A row of partial sums per thread, into this CTA's own shared memory: over the ring, which is idle now (with one CTA
+        // per item straight to where they are added up).  16-byte pieces are XOR-ed with the row inside its run, so that the
+        // 32 rows of a warp do not meet in one bank.
         const int q = warp & 3;        // tensor-memory lane quadrant this warp may read
         const int row = q * 32 + lane;
-        const int owner = row / cfg.rps, lrow = row - owner * cfg.rps;
-        const bool send = row < count;
-        uint32_t dst = part + (rank * cfg.rps + lrow) * (BN * 4), bar = smem_u32(&s_part);
-        if (CS > 1 && send) {
-            dst = mapa_shared(dst, static_cast<uint32_t>(owner));
-            bar = mapa_shared(bar, static_cast<uint32_t>(owner));
-        }
+        const int lrow = CS > 1 ? row % cfg.rps : row;
+        const uint32_t dst = (CS > 1 ? ring : part) + row * (BN * 4);
 #pragma unroll
         for (int blk = 0; blk < BN / 32; ++blk) {
             uint32_t v[32];
             tmem_ld32(tmem + (static_cast<uint32_t>(q * 32) << 16) + blk * 32, v);
             tmem_ld_wait();
-            if (send) {
+            if (row < count) {
 #pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    const uint32_t at = dst + blk * 128 + ((k ^ (lrow & 7)) << 4);
-                    if (CS > 1) st_async_v4(at, bar, v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
-                    else asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(v[4 * k]), "r"(v[4 * k + 1]),
-                                      "r"(v[4 * k + 2]), "r"(v[4 * k + 3]) : "memory");
-                }
+                for (int k = 0; k < 8; ++k)
+                    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst + blk * 128 + ((k ^ (lrow & 7)) << 4)), "r"(v[4 * k]),
+                                 "r"(v[4 * k + 1]), "r"(v[4 * k + 2]), "r"(v[4 * k + 3])
+                                 : "memory");
             }
         }
         tc_fence_before();
+        if (CS > 1) fence_proxy_async();
+        asm volatile("bar.sync 1, %0;" ::"n"(EPI) : "memory");
         if (CS > 1) {
-            // every partial sum of this CTA's rows has landed (and no other CTA writes to its shared memory after that); the
-            // limit is a multiple of the other waits', so that a CTA of the cluster that gave up on one of those has sent by then
+            for (int owner = q; owner < CS; owner += 4) {
+                const int rows = count - owner * cfg.rps < cfg.rps ? count - owner * cfg.rps : cfg.rps;
+                if (rows > 0 && elect_one())
+                    bulk_copy_cluster(mapa_shared(part + rank * cfg.rps * (BN * 4), static_cast<uint32_t>(owner)),
+                                      ring + owner * cfg.rps * (BN * 4), static_cast<uint32_t>(rows) * (BN * 4),
+                                      mapa_shared(smem_u32(&s_part), static_cast<uint32_t>(owner)));
+            }
+            // every partial sum of this CTA's rows has landed; the limit is a multiple of the other waits', so that a CTA of the
+            // cluster that gave up on one of those has sent by then
             const uint32_t bar_own = smem_u32(&s_part);
             const bool landed = mbar_wait_cluster(bar_own, 0) || mbar_wait_cluster(bar_own, 0) || mbar_wait_cluster(bar_own, 0);
             if (!__all_sync(0xFFFFFFFFu, landed)) *abort_flag = 5;
-        } else {
-            asm volatile("bar.sync 1, %0;" ::"n"(EPI) : "memory");
+            asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
         }
         if (!aborted(abort_flag)) {
             const uint32_t src_step = static_cast<uint32_t>(cfg.rps) * (BN * 4);
@@ -313,6 +316,11 @@ k_conv_cluster(const ConvParams p, const ClusterCfg cfg, const __grid_constant__
         }
     }
 
+    if (CS > 1) {
+        // a CTA leaves once every CTA of the cluster has what was sent to it: its copies have then been read
+        if (warp < 2) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
     tc_fence_before();
     __syncthreads();
     if (tid == 0 && s_abort != 0) {
@@ -385,9 +393,16 @@ bool make_cfg(const ConvParams& p, const nm_plan_t* plan, ClusterCfg* cfg, size_
     int stages = plan && plan->stages > 0 ? plan->stages : (range < NSTAGE_MAX ? range : NSTAGE_MAX);
     if (stages > NSTAGE_MAX) return false;
     while (stages > 1 && stages * cfg->stage_bytes > budget) --stages;
+    if (cfg->cs > 1 && stages * cfg->stage_bytes + 128 * 128 < cfg->rows * bn * 4) return false;   // the sums to send lie over the ring
     if (stages * cfg->stage_bytes > budget || (stages < 2 && range > 1)) return false;
     cfg->stages = stages;
     *smem = static_cast<size_t>(fixed) + static_cast<size_t>(stages) * cfg->stage_bytes;
+    // The CTAs of a cluster wait for one another, so none of them may be held up in its tensor-memory allocation by a CTA
+    // that waits in turn: a CTA takes at least its columns' share of the SM's shared memory (kernels that allocate all 512
+    // columns take NM_EXCLUSIVE_SMEM, next to which no CTA of this kernel fits).
+    const size_t share = static_cast<size_t>(bn) * (228 * 1024 / 512);
+    if (*smem < share) *smem = share;
+    if (*smem < NM_BESIDE_EXCLUSIVE) *smem = NM_BESIDE_EXCLUSIVE;
     // Short launches only: with many rounds of CTAs the persistent kernels keep the tensor core busier.
     return static_cast<long long>(cfg->tiles) * cfg->n_slices * cfg->cs <= 12ll * sm_count();
 }

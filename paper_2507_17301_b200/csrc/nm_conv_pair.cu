@@ -319,7 +319,7 @@ bool make_cfg(const ConvParams& p, const nm_plan_t* plan, PairCfg* cfg)
 size_t smem_bytes(const PairCfg& cfg)
 {
     size_t smem = 1024 + static_cast<size_t>(cfg.stages) * cfg.stage_bytes + 8 * cfg.boxes * BOX_BYTES;
-    return smem < 120 * 1024 ? 120 * 1024 : smem;   // one CTA per SM: the pair owns all 512 TMEM columns of both
+    return smem < NM_EXCLUSIVE_SMEM ? NM_EXCLUSIVE_SMEM : smem;   // one CTA per SM: the pair owns all 512 TMEM columns of both
 }
 
 // Pairs of SMs that can hold one cluster each at the same time (per device; 0 = clusters unavailable).

@@ -329,7 +329,7 @@ bool make_cfg(const ConvParams& p, const nm_plan_t* plan, PlaneCfg* cfg, size_t*
     if (n_slots < 2 || fixed + static_cast<size_t>(n_slots) * cfg->slot_bytes > budget) return false;
     cfg->n_slots = n_slots;
     const size_t smem = fixed + static_cast<size_t>(n_slots) * cfg->slot_bytes;
-    *smem_out = smem < 120 * 1024 ? 120 * 1024 : smem;   // one CTA per SM: it owns all of tensor memory
+    *smem_out = smem < NM_EXCLUSIVE_SMEM ? NM_EXCLUSIVE_SMEM : smem;   // one CTA per SM: it owns all of tensor memory
     return true;
 }
 

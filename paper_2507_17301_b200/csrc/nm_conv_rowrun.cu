@@ -382,7 +382,7 @@ bool make_cfg(const ConvParams& p, RowCfg* cfg, size_t* smem_out)
     while (cfg->n_sets > 2 && fixed + static_cast<size_t>(cfg->n_sets) * cfg->rowset_bytes > 227 * 1024 - 4096) --cfg->n_sets;
     const size_t smem = fixed + static_cast<size_t>(cfg->n_sets) * cfg->rowset_bytes;
     if (smem > 227 * 1024 - 4096) return false;
-    *smem_out = smem < 120 * 1024 ? 120 * 1024 : smem;
+    *smem_out = smem < NM_EXCLUSIVE_SMEM ? NM_EXCLUSIVE_SMEM : smem;
     return true;
 }
 

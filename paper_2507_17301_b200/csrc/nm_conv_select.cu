@@ -770,7 +770,7 @@ nm_status_t launch(const ConvParams& p, const SelCfg& cfg, cudaStream_t st)
     q.pixels = p.pixels;
     size_t smem = 1024 + static_cast<size_t>(cfg.n_p) * cfg.p_bytes + static_cast<size_t>(cfg.n_w) * cfg.wstage_bytes +
                   (cfg.alias_staging ? 0 : (cfg.epi8 ? 2 : 1) * STAGING_BYTES);
-    if (smem < 120 * 1024) smem = 120 * 1024;   // one CTA per SM: it owns all 512 TMEM columns
+    if (smem < NM_EXCLUSIVE_SMEM) smem = NM_EXCLUSIVE_SMEM;   // one CTA per SM: it owns all 512 TMEM columns
     const auto kernel = cfg.epi8 ? k_conv_select<NK, MG, 1> : k_conv_select<NK, MG, 0>;
     cudaError_t e = nmhost::ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), smem);
     if (e != cudaSuccess) return nmhost::fail(NM_ERR_CUDA, "cudaFuncSetAttribute (variant 8): %s", cudaGetErrorString(e));

@@ -352,7 +352,7 @@ bool make_cfg(const ConvParams& p, const nm_plan_t* plan, WinCfg* cfg, size_t* s
     cfg->n_p = n_p;
     cfg->n_w = n_w;
     size_t smem = 1024 + static_cast<size_t>(n_p) * cfg->pslot_bytes + static_cast<size_t>(n_w) * wslot;
-    *smem_out = smem < 120 * 1024 ? 120 * 1024 : smem;
+    *smem_out = smem < NM_EXCLUSIVE_SMEM ? NM_EXCLUSIVE_SMEM : smem;
     return true;
 }
 

@@ -9,6 +9,12 @@ constexpr uint32_t NM_MAGIC = 0x4E4D5754u;  // "NMWT"
 constexpr uint32_t NM_TAP_PAD = 0xFFFFFFFFu;  // tap-table entry of a padding column: gathers zero
 constexpr int NM_KCHUNK = 32;               // kept columns per shared-memory operand chunk (128 B of TF32)
 
+// Least dynamic shared memory of the kernels that allocate all of an SM's tensor memory, and of the cluster kernel, whose
+// CTAs wait for CTAs on other SMs: together more than an SM has, so that the two kinds are never resident on one SM and a
+// waiting CTA never stands between a cluster's CTA and its tensor memory.
+constexpr size_t NM_EXCLUSIVE_SMEM = 204 * 1024;
+constexpr size_t NM_BESIDE_EXCLUSIVE = 24 * 1024;
+
 // Compressed weights of one layer.  `values` / `indices` are the canonical, exportable form;
 // `wt` and `taps` are what the convolution kernels read.
 struct nm_weights {

@@ -2,7 +2,10 @@
 import pytest
 import torch
 
-from paper_2507_17301_b200 import nm
+from paper_2507_17301_b200 import build
+
+build.build()
+from paper_2507_17301_b200 import nm  # noqa: E402
 
 
 def test_host_tensors_and_wrong_types_are_refused():
