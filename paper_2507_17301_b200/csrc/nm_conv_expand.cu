@@ -12,16 +12,20 @@
 // bound by HBM and the tensor pipe has slack; the auto-tuner decides per layer by measurement.
 // The pruning tile width plays no role here, so any tile_t is accepted.
 //
-//   producer (1 thread)   TMA im2col load of the slab + one contiguous bulk copy of the weight block
-//                         (stored pre-swizzled, so it costs no per-row TMA requests) per stage; a
-//                         weight slice of at most 128 KB is instead fetched once and stays resident
+//   activation producer   TMA load of the slab per stage: im2col mode, or plain 2-D rows for pointwise layers of stride 1;
+//   (1 thread)
+//   weight producer       one contiguous bulk copy of the weight block per stage (stored pre-swizzled, so it costs no per-row
+//   (1 thread)            TMA requests); a weight slice of at most 128 KB is instead fetched once and stays resident
 //                         (the grid is then a multiple of the slice count, so a CTA keeps its slice)
 //   MMA issuer (1 thread) four 128 x BN x 8 TF32 tcgen05.mma (SS) per stage into one of two
 //                         accumulator buffers in tensor memory
 //   epilogue (8 warps)    TMEM -> registers, + bias, ReLU, swizzled staging, TMA store to NHWC;
 //                         overlaps the next work item's main loop
-// Work items (128 pixels x BN channels) are walked in a static persistent schedule; every wait is
+// Work items (up to 128 pixels x BN channels) are walked in a static persistent schedule; every wait is
 // bounded and reports through the handle's status word.
+// Pixels per item: as few as keep the number of rounds (items / CTAs, rounded up) what it is with 128.  A layer whose items
+// fill 1.32 rounds of the SMs takes two rounds either way, and with 128-pixel items it spends the second one with
+// a third of the SMs pulling in all of the bytes; equal items of 88 pixels spread them over all SMs.
 //
 // Balanced mode (plan.split = -1), for layers with fewer work items than would keep every SM busy:
 // the (item, stage) pairs of the whole layer are laid end to end and cut into one contiguous,
@@ -48,6 +52,7 @@ constexpr int NSTAGE_MAX = 10;
 constexpr int WRES_MAX = 128 * 1024;            // largest weight slice kept resident
 constexpr int THREADS = 384;                   // 4 service warps + 8 epilogue warps
 constexpr int BOX_BYTES = 4096;                // one 32-pixel x 32-channel output box
+constexpr int BOXES_MAX = 3;                   // staging boxes per epilogue warp
 
 struct ExpandCfg {
     int bn;           // output channels per work item
@@ -62,20 +67,65 @@ struct ExpandCfg {
     int n_iss;        // MMA issuer threads (1 or 2): two take alternate pipeline stages of an item, each into an accumulator of its own
     int n_acc;        // accumulator buffers (of n_iss accumulators each) in tensor memory: 2 when they fit, else 1
     int sub_bytes;    // bytes of one 32-column block inside a stage: activations (+ streamed weights)
+    int rows;         // pixels per work item
+    int flat;         // 1: activations as 2-D rows (pointwise, stride 1), 0: im2col
     int ksplit;       // K splits (1 = none): a work item covers one of them and stores raw partial sums
     int p_pad;        // pixel blocks * 128: rows of one split in the partial-sum scratch
-    int boxes;        // output staging boxes per epilogue warp: 2 for short reductions, 1 when the ring needs the room
+    int boxes;        // output staging boxes per epilogue warp: 2 for short reductions, 1 when the ring needs the room;
+                      // with a shortcut input, which is loaded into them ahead of time, 3 (2 when the ring needs the room)
+    int sl_shift;     // log2 of n_slices, -1 where it is no power of two
     int balanced;     // 1: contiguous (item, stage) ranges per CTA, partial sums through per-CTA scratch slots
     long long n_work;
 };
 
 __device__ __forceinline__ bool aborted(volatile int* flag) { return *flag != 0; }
 
+// Wait of a producer for a ring slot.  The abort flag is looked at only here, i.e. when the slot was not free at once: a
+// pipeline whose other end has given up comes to a halt, so nobody runs past this point for long.
+__device__ __forceinline__ bool wait_stage(uint32_t bar, uint32_t parity, volatile int* flag, int site)
+{
+    for (uint32_t i = 0; i < kWaitPolls; ++i) {
+        if (mbar_try_wait(bar, parity)) return true;
+        if ((i & 15u) == 0u && *flag != 0) return false;
+    }
+    *flag = site;
+    return false;
+}
+// After an abort: loads already issued still target this CTA's shared memory, let them land (bounded).
+__device__ __forceinline__ void drain_ring(RingPos rp, int issued, int n, uint64_t* full)
+{
+    for (int back = 0; back < n && back < issued; ++back) {
+        if (rp.s == 0) { rp.s = n; rp.parity ^= 1u; }
+        --rp.s;
+        (void)mbar_wait_polls(smem_u32(&full[rp.s]), rp.parity, 1u << 16);
+    }
+}
+
 // One piece of work of a CTA: stages [sb, se) of work item `work`.
 struct Seg {
     uint32_t work;
     int sb, se;
 };
+struct ItemPos {
+    uint32_t tile, slice, ks;   // pixel tile, channel slice, range of the reduction axis
+};
+__device__ __forceinline__ ItemPos item_of(uint32_t work, const ExpandCfg& cfg)
+{
+    ItemPos it = {work, 0u, 0u};
+    if (cfg.sl_shift > 0) {
+        it.tile = work >> cfg.sl_shift;
+        it.slice = work - (it.tile << cfg.sl_shift);
+    } else if (cfg.sl_shift < 0) {
+        it.tile = work / static_cast<uint32_t>(cfg.n_slices);
+        it.slice = work - it.tile * static_cast<uint32_t>(cfg.n_slices);
+    }
+    if (cfg.ksplit > 1) {
+        const uint32_t t = it.tile / static_cast<uint32_t>(cfg.ksplit);
+        it.ks = it.tile - t * static_cast<uint32_t>(cfg.ksplit);
+        it.tile = t;
+    }
+    return it;
+}
 // Walks a CTA's pieces: whole items `first, first + stride, ...` in the static schedule, or the
 // contiguous range of (item, stage) units of balanced mode.
 template <bool BAL>
@@ -137,10 +187,11 @@ __device__ __forceinline__ void st_release_gpu(uint32_t* ptr, uint32_t v)
 template <int KBLK, bool BAL>
 __global__ void __launch_bounds__(THREADS, 1)
 k_conv_expand(const ConvParams p, const ExpandCfg cfg, const __grid_constant__ CUtensorMap tm_x,
-              const __grid_constant__ CUtensorMap tm_y)
+              const __grid_constant__ CUtensorMap tm_y, const __grid_constant__ CUtensorMap tm_tail,
+              const __grid_constant__ CUtensorMap tm_res)
 {
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t s_full[NSTAGE_MAX], s_free[NSTAGE_MAX], s_accfull[2], s_accfree[2], s_wres;
+    __shared__ uint64_t s_full[NSTAGE_MAX], s_free[NSTAGE_MAX], s_accfull[2], s_accfree[2], s_wres, s_res[8][BOXES_MAX];
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
 
@@ -154,7 +205,7 @@ k_conv_expand(const ConvParams p, const ExpandCfg cfg, const __grid_constant__ C
     if (warp == 2) tmem_alloc(smem_u32(&s_tmem), 512);
     if (tid == 0) {
         for (int i = 0; i < NSTAGE_MAX; ++i) {
-            mbar_init(smem_u32(&s_full[i]), 1);   // producer's expect-tx arrival
+            mbar_init(smem_u32(&s_full[i]), cfg.w_res ? 1 : 2);   // the producers' expect-tx arrivals
             mbar_init(smem_u32(&s_free[i]), 1);   // the commit of the issuer that read the stage
         }
         for (int i = 0; i < 2; ++i) {
@@ -162,6 +213,7 @@ k_conv_expand(const ConvParams p, const ExpandCfg cfg, const __grid_constant__ C
             mbar_init(smem_u32(&s_accfree[i]), 8);   // epilogue warps
         }
         mbar_init(smem_u32(&s_wres), 1);
+        for (int i = 0; i < 8 * BOXES_MAX; ++i) mbar_init(smem_u32(&s_res[0][0] + i), 1);   // a shortcut box has landed
         mbar_fence_init();
         s_abort = 0;
         tma_prefetch_desc(&tm_x);
@@ -175,48 +227,30 @@ k_conv_expand(const ConvParams p, const ExpandCfg cfg, const __grid_constant__ C
     pdl_wait();                // from here on global memory written by the previous kernel is read
 
     if (warp == 0) {
-        // =========================== producer ===========================
+        // =========================== activation producer ===========================
         if (elect_one()) {
             int issued = 0;
             const int hw = p.ho * p.wo;
-            const uint32_t tx = static_cast<uint32_t>(KBLK) * (SUB_BYTES + (cfg.w_res ? 0u : static_cast<uint32_t>(cfg.bn) * 128u));
+            const uint32_t tx = static_cast<uint32_t>(KBLK) * static_cast<uint32_t>(cfg.rows) * 128u;
             const int n_blk32 = n_sub * KBLK;   // 32-column blocks per work item
-            if (cfg.w_res) {
-                // the grid is a multiple of the slice count, so every work item of this CTA has the
-                // same channel slice: its weights are fetched once
-                const int slice = static_cast<int>(blockIdx.x % static_cast<uint32_t>(cfg.n_slices));
-                mbar_arrive_expect_tx(smem_u32(&s_wres), static_cast<uint32_t>(n_blk32) * static_cast<uint32_t>(cfg.bn) * 128u);
-                for (int c = 0; c < n_blk32; ++c)
-                    bulk_load_1d(wres + c * cfg.b_bytes, p.wx + (static_cast<size_t>(c) * p.wx_rows + slice * cfg.bn) * 32,
-                                 static_cast<uint32_t>(cfg.bn) * 128u, smem_u32(&s_wres));
-            }
-            const uint32_t w_bytes = static_cast<uint32_t>(cfg.bn) * 128u;
-            const size_t w_step = static_cast<size_t>(p.wx_rows) * 32;   // floats between two 32-column blocks
             RingPos rp;
             SegIter<BAL> it = make_iter<BAL>(cfg);
             Seg seg;
-            while (!aborted(abort_flag) && it.next(seg)) {
-                // The item's coordinates, with the divisions the common cases do not need left out: this thread
-                // issues the kernel's first load only after them.
-                const uint32_t work = seg.work;
-                uint32_t slice = 0, rest = work, ks = 0;
-                if (cfg.n_slices > 1) {
-                    rest = work / static_cast<uint32_t>(cfg.n_slices);
-                    slice = work - rest * static_cast<uint32_t>(cfg.n_slices);
+            bool ok = true, free_now = true;   // free_now: the slot's release was seen while the stage before it was issued
+            while (ok && it.next(seg)) {
+                const ItemPos item = item_of(seg.work, cfg);
+                const uint32_t ks = item.ks;
+                const int pix0 = static_cast<int>(item.tile) * cfg.rows;
+                int n0 = 0, w0 = 0, h0 = 0;
+                if (!cfg.flat) {
+                    n0 = static_cast<int>(static_cast<uint32_t>(pix0) / static_cast<uint32_t>(hw));
+                    const int rem = pix0 - n0 * hw;
+                    const int oh0 = rem / p.wo, ow0 = rem - oh0 * p.wo;
+                    w0 = ow0 * p.stride_w - p.pad_w;
+                    h0 = oh0 * p.stride_h - p.pad_h;
                 }
-                if (cfg.ksplit > 1) {
-                    const uint32_t pb = rest / static_cast<uint32_t>(cfg.ksplit);
-                    ks = rest - pb * static_cast<uint32_t>(cfg.ksplit);
-                    rest = pb;
-                }
-                const uint32_t pix0 = rest * BM;
-                const int n0 = static_cast<int>(pix0 / static_cast<uint32_t>(hw));
-                const int rem = static_cast<int>(pix0 - static_cast<uint32_t>(n0) * static_cast<uint32_t>(hw));
-                const int oh0 = rem / p.wo, ow0 = rem - oh0 * p.wo;
-                const int w0 = ow0 * p.stride_w - p.pad_w, h0 = oh0 * p.stride_h - p.pad_h;
                 // first 32-column block of this item's share of the reduction axis
                 const int c0 = static_cast<int>(ks) * n_blk32 + seg.sb * KBLK;
-                const float* wsrc = p.wx + static_cast<size_t>(slice) * cfg.bn * 32 + static_cast<size_t>(c0) * w_step;
                 int ch = 0, tw = 0, off_w = 0, off_h = 0;
                 if (c0 != 0) {
                     const int tap0 = (c0 * 32) / p.c_in, th = tap0 / p.kw;
@@ -226,18 +260,20 @@ k_conv_expand(const ConvParams p, const ExpandCfg cfg, const __grid_constant__ C
                     off_h = th * p.dil_h;
                 }
                 for (int c = seg.sb; c < seg.se; ++c) {
-                    if (rp.wrapped && !mbar_wait_lone(smem_u32(&s_free[rp.s]), rp.parity ^ 1u)) *abort_flag = 2;
-                    if (aborted(abort_flag)) break;
+                    if (!free_now && !wait_stage(smem_u32(&s_free[rp.s]), rp.parity ^ 1u, abort_flag, 2)) { ok = false; break; }
                     uint32_t a_smem = ring + rp.s * cfg.stage_bytes;
                     const uint32_t bar = smem_u32(&s_full[rp.s]);
                     mbar_arrive_expect_tx(bar, tx);
+                    rp.advance(NS);
+                    free_now = !rp.wrapped || mbar_test_wait(smem_u32(&s_free[rp.s]), rp.parity ^ 1u);
 #pragma unroll
                     for (int j = 0; j < KBLK; ++j) {
-                        tma_load_im2col_4d(a_smem, &tm_x, bar, ch, w0, h0, n0, static_cast<uint16_t>(off_w),
-                                           static_cast<uint16_t>(off_h));
-                        if (!cfg.w_res) bulk_load_1d(a_smem + SUB_BYTES, wsrc, w_bytes, bar);
+                        if (cfg.flat)
+                            tma_load_2d(a_smem, &tm_x, bar, ch, pix0);
+                        else
+                            tma_load_im2col_4d(a_smem, &tm_x, bar, ch, w0, h0, n0, static_cast<uint16_t>(off_w),
+                                               static_cast<uint16_t>(off_h));
                         a_smem += cfg.sub_bytes;
-                        wsrc += w_step;
                         ch += 32;
                         if (ch >= p.c_in) {
                             ch = 0;
@@ -245,19 +281,55 @@ k_conv_expand(const ConvParams p, const ExpandCfg cfg, const __grid_constant__ C
                             if (++tw == p.kw) { tw = 0; off_w = 0; off_h += p.dil_h; }
                         }
                     }
-                    rp.advance(NS);
                     ++issued;
                 }
             }
-            if (aborted(abort_flag)) {
-                // loads already issued still target this CTA's shared memory: let them land
-                if (cfg.w_res) (void)mbar_wait(smem_u32(&s_wres), 0);
-                for (int back = 0; back < NS && back < issued; ++back) {
-                    if (rp.s == 0) { rp.s = NS; rp.parity ^= 1u; }
-                    --rp.s;
-                    (void)mbar_wait(smem_u32(&s_full[rp.s]), rp.parity);
+            if (aborted(abort_flag)) drain_ring(rp, issued, NS, s_full);
+        }
+    } else if (warp == 2) {
+        // =========================== weight producer ===========================
+        if (elect_one()) {
+            const int n_blk32 = n_sub * KBLK;
+            const uint32_t w_bytes = static_cast<uint32_t>(cfg.bn) * 128u;
+            const size_t w_step = static_cast<size_t>(p.wx_rows) * 32;   // floats between two 32-column blocks
+            if (cfg.w_res) {
+                // the grid is a multiple of the slice count, so every work item of this CTA has the
+                // same channel slice: its weights are fetched once
+                const int slice = static_cast<int>(blockIdx.x % static_cast<uint32_t>(cfg.n_slices));
+                mbar_arrive_expect_tx(smem_u32(&s_wres), static_cast<uint32_t>(n_blk32) * w_bytes);
+                for (int c = 0; c < n_blk32; ++c)
+                    bulk_load_1d(wres + c * cfg.b_bytes, p.wx + static_cast<size_t>(c) * w_step + static_cast<size_t>(slice) * cfg.bn * 32,
+                                 w_bytes, smem_u32(&s_wres));
+            } else {
+                int issued = 0;
+                RingPos rp;
+                SegIter<BAL> it = make_iter<BAL>(cfg);
+                Seg seg;
+                bool ok = true, free_now = true;
+                while (ok && it.next(seg)) {
+                    const ItemPos item = item_of(seg.work, cfg);
+                    const uint32_t slice = item.slice;
+                    const int c0 = static_cast<int>(item.ks) * n_blk32 + seg.sb * KBLK;
+                    const float* wsrc = p.wx + static_cast<size_t>(slice) * cfg.bn * 32 + static_cast<size_t>(c0) * w_step;
+                    for (int c = seg.sb; c < seg.se; ++c) {
+                        if (!free_now && !wait_stage(smem_u32(&s_free[rp.s]), rp.parity ^ 1u, abort_flag, 9)) { ok = false; break; }
+                        uint32_t b_smem = ring + rp.s * cfg.stage_bytes + SUB_BYTES;
+                        const uint32_t bar = smem_u32(&s_full[rp.s]);
+                        mbar_arrive_expect_tx(bar, static_cast<uint32_t>(KBLK) * w_bytes);
+                        rp.advance(NS);
+                        free_now = !rp.wrapped || mbar_test_wait(smem_u32(&s_free[rp.s]), rp.parity ^ 1u);
+#pragma unroll
+                        for (int j = 0; j < KBLK; ++j) {
+                            bulk_load_1d(b_smem, wsrc, w_bytes, bar);
+                            b_smem += cfg.sub_bytes;
+                            wsrc += w_step;
+                        }
+                        ++issued;
+                    }
                 }
+                if (aborted(abort_flag)) drain_ring(rp, issued, NS, s_full);
             }
+            if (cfg.w_res && aborted(abort_flag)) (void)mbar_wait(smem_u32(&s_wres), 0);
         }
     } else if (warp == 1 || warp == 3) {
         // =========================== MMA issuers ===========================
@@ -330,10 +402,10 @@ k_conv_expand(const ConvParams p, const ExpandCfg cfg, const __grid_constant__ C
         const int half = (warp - 4) >> 2;  // which channel blocks of 32: blk = 2 * i + half
         const uint32_t lane_addr = static_cast<uint32_t>(q * 32) << 16;
         const uint32_t my_staging = staging + (warp - 4) * cfg.boxes * BOX_BYTES;
-        const uint32_t box_toggle = cfg.boxes == 2 ? 1u : 0u;
         const uint32_t rx = static_cast<uint32_t>(lane & 7);
         const int n_blk = cfg.bn / 32;
-        uint32_t nb = 0, ti = 0;
+        const int box_rows = cfg.rows - q * 32 < 0 ? 0 : cfg.rows - q * 32 < 32 ? cfg.rows - q * 32 : 32;   // pixels of this warp's boxes
+        uint32_t ti = 0;
         uint32_t stage_count = 0;   // stages of all earlier pieces of this CTA
         // balanced mode: this CTA's partial-sum slot (128 rows x bn) and its warps' flags, in the handle's scratch
         const uint32_t units = static_cast<uint32_t>(cfg.n_work) * static_cast<uint32_t>(cfg.n_sub);
@@ -344,14 +416,44 @@ k_conv_expand(const ConvParams p, const ExpandCfg cfg, const __grid_constant__ C
         const int my_row = q * 32 + lane;
         SegIter<BAL> it = make_iter<BAL>(cfg);
         Seg seg;
+        // Shortcut input: the box of a block is loaded into the block's staging box, cfg.boxes - 1 blocks ahead (the walk
+        // `nit` runs ahead of `it` by that much), added there and stored from there.  (Held in registers a block
+        // ahead it cost two passes over the box and left too little in flight: 64 -> 256 at 56x56, batch 64, took 101-106 us,
+        // now 82-87 with the bytes' own time at 70; 256 -> 1024 at 14x14, batch 128, 58 -> 45 us.)
+        const bool res = p.residual != nullptr;
+        const uint32_t n_box = static_cast<uint32_t>(cfg.boxes);
+        uint32_t bx = 0, bpar = 0;      // this block's staging box, parity of its current use
+        uint32_t nbx = 0, asked = 0, taken = 0;
+        SegIter<BAL> nit = make_iter<BAL>(cfg);
+        Seg nseg;
+        int nblk = n_blk, no0 = 0, npix = 0;
+        auto request = [&]() {
+            while (nblk >= n_blk) {
+                if (!nit.next(nseg)) return;
+                const ItemPos item = item_of(nseg.work, cfg);
+                no0 = static_cast<int>(item.slice) * cfg.bn;
+                npix = static_cast<int>(item.tile) * cfg.rows + q * 32;
+                if (box_rows > 0 && npix < p.pixels && !(BAL && nseg.sb > 0)) nblk = half;
+            }
+            if (elect_one()) {
+                const uint32_t bar = smem_u32(&s_res[warp - 4][nbx]);
+                mbar_arrive_expect_tx(bar, BOX_BYTES);
+                tma_load_2d(my_staging + nbx * BOX_BYTES, &tm_res, bar, no0 + nblk * 32, npix);
+            }
+            nblk += 2;
+            nbx = nbx + 1 == n_box ? 0 : nbx + 1;
+            ++asked;
+        };
+        if (res)
+            for (uint32_t k = 1; k < n_box; ++k) request();
         for (; it.next(seg); ++ti) {
             const uint32_t work = seg.work;
             const bool publish = BAL && seg.sb > 0;                   // a later part of an item: store raw sums
             const bool finish = BAL && seg.sb == 0 && seg.se < n_sub;  // the first part: add the others' sums
-            const int slice = static_cast<int>(work % static_cast<uint32_t>(cfg.n_slices));
-            const uint32_t rest = work / static_cast<uint32_t>(cfg.n_slices);
-            const int ks = static_cast<int>(rest % static_cast<uint32_t>(cfg.ksplit));
-            const uint32_t pix0 = (rest / static_cast<uint32_t>(cfg.ksplit)) * BM;
+            const ItemPos item = item_of(work, cfg);
+            const int pix0 = static_cast<int>(item.tile) * cfg.rows + q * 32;   // first pixel of this warp's boxes
+            const int o0 = static_cast<int>(item.slice) * cfg.bn;
+            const bool live = box_rows > 0 && pix0 < p.pixels;
             const int ab = cfg.n_acc == 2 ? static_cast<int>(ti & 1u) : 0;
             // two issuers: stages went to them by ring slot, i.e. by the parity of the running stage count; a piece of
             // one stage is in the accumulator of that stage's owner, a longer one in both
@@ -359,23 +461,12 @@ k_conv_expand(const ConvParams p, const ExpandCfg cfg, const __grid_constant__ C
             stage_count += static_cast<uint32_t>(seg.se - seg.sb);
             const bool two_acc = cfg.n_iss == 2 && seg.se - seg.sb >= 2;
             const uint32_t acc_first = (cfg.n_iss == 2 && seg.se - seg.sb == 1) ? (piece_first & 1u) : 0u;
-            // the shortcut input does not depend on the accumulator: its first box is requested before the
-            // wait for the main loop, every later box while the one before it is being stored
-            const long long box_pix = static_cast<long long>(pix0) + q * 32;
-            const bool res_pass = p.residual != nullptr && box_pix < p.pixels && !publish;
-            const int res_rows = p.pixels - box_pix < 32 ? static_cast<int>(p.pixels - box_pix) : 32;
-            const float* res_base = res_pass ? p.residual + box_pix * p.c_out + slice * cfg.bn : nullptr;
-            float4 rv[8];
-            const int cols_left = p.c_out - slice * cfg.bn;   // channels of this slice that exist (may end inside a box)
-            const int o0 = slice * cfg.bn;
-            float bias_next = half < n_blk ? bias_lane_load(p.bias, o0 + half * 32, p.c_out, lane) : 0.f;   // first block's bias
-            if (res_pass && half < n_blk) load_residual_box(rv, res_base + half * 32, p.c_out, res_rows, lane, cols_left - half * 32);
             // positions (of the equal ranges) that hold the rest of this item: first_pos + 1 .. last_pos.  Their
             // partial sums were stored long ago (they are those CTAs' first piece of work), so the flags are
-            // checked and, where no shortcut input occupies the registers, the first counterpart's sums of
-            // this warp's first block are requested BEFORE the wait for this CTA's own accumulator.
+            // checked and the first counterpart's sums of this warp's first block are requested BEFORE the wait for this CTA's own accumulator.
             uint32_t first_pos = 0, last_pos = 0;
             bool ahead = false;
+            float4 rv[8];
             if (finish) {
                 first_pos = gridDim.x - 1u - blockIdx.x;
                 const uint32_t u_last = (work + 1u) * static_cast<uint32_t>(n_sub) - 1u;
@@ -389,7 +480,7 @@ k_conv_expand(const ConvParams p, const ExpandCfg cfg, const __grid_constant__ C
                     for (uint32_t poll = 0; poll < kWaitPolls && !seen; ++poll) seen = ld_acquire_gpu(f) == 1u;
                     if (!seen) *abort_flag = 10;
                 }
-                if (!res_pass && half < n_blk && !aborted(abort_flag)) {
+                if (half < n_blk && !aborted(abort_flag)) {
                     const float4* src = reinterpret_cast<const float4*>(slots + slot_floats * (gridDim.x - 2u - first_pos)) +
                                         static_cast<size_t>(half) * 8 * BM + my_row;
 #pragma unroll
@@ -397,11 +488,21 @@ k_conv_expand(const ConvParams p, const ExpandCfg cfg, const __grid_constant__ C
                     ahead = true;
                 }
             }
-            const bool ok = aborted(abort_flag) || mbar_wait(smem_u32(&s_accfull[ab]), (cfg.n_acc == 2 ? (ti >> 1) : ti) & 1u);
+            const bool ok = aborted(abort_flag) || mbar_wait_lone(smem_u32(&s_accfull[ab]), (cfg.n_acc == 2 ? (ti >> 1) : ti) & 1u);
             if (!__all_sync(0xFFFFFFFFu, ok)) *abort_flag = 8;
             if (__any_sync(0xFFFFFFFFu, aborted(abort_flag))) break;
             tc_fence_after();
-            for (int blk = half; blk < n_blk; blk += 2, ++nb) {
+            if (!BAL && !live) {   // an item of fewer pixels: this warp's quadrant of the accumulator holds nothing
+                if (lane == 0) mbar_arrive(smem_u32(&s_accfree[ab]));
+                continue;
+            }
+            for (int blk = half; blk < n_blk; blk += 2) {
+                float4 bias[8];
+#pragma unroll
+                for (int qq = 0; qq < 8; ++qq) {
+                    const int o = o0 + blk * 32 + qq * 4;
+                    bias[qq] = p.bias != nullptr && o < p.c_out ? __ldg(reinterpret_cast<const float4*>(p.bias + o)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                }
                 uint32_t v[32];
                 tmem_ld32(tmem + lane_addr + (ab * cfg.n_iss + acc_first) * cfg.bn + blk * 32, v);
                 if (two_acc) {
@@ -427,7 +528,6 @@ k_conv_expand(const ConvParams p, const ExpandCfg cfg, const __grid_constant__ C
                     for (int qq = 0; qq < 8; ++qq)
                         __stcg(dst + qq * BM, make_float4(__uint_as_float(v[qq * 4 + 0]), __uint_as_float(v[qq * 4 + 1]),
                                                      __uint_as_float(v[qq * 4 + 2]), __uint_as_float(v[qq * 4 + 3])));
-                    --nb;   // no staging box used
                     continue;
                 }
                 if (finish) {
@@ -464,47 +564,46 @@ k_conv_expand(const ConvParams p, const ExpandCfg cfg, const __grid_constant__ C
                         }
                     }
                 }
-                const uint32_t box = my_staging + (nb & box_toggle) * BOX_BYTES;
-                if (elect_one()) {
+                if (BAL && !live) continue;
+                const uint32_t box = my_staging + bx * BOX_BYTES;
+                if (res) {
+                    // the store of the block before this one must have read its box, the next one to be loaded
+                    if (elect_one()) tma_store_wait_read_n<0>();
+                    __syncwarp();
+                    request();
+                    const bool landed = mbar_wait_lone(smem_u32(&s_res[warp - 4][bx]), bpar);
+                    if (!__all_sync(0xFFFFFFFFu, landed)) *abort_flag = 11;
+                    ++taken;
+                } else {
                     // the store that last read this box must be done with it
-                    if (cfg.boxes == 2) { if (nb >= 2) tma_store_wait_read_n<1>(); }
-                    else if (nb >= 1) tma_store_wait_read_n<0>();
+                    if (elect_one()) {
+                        if (n_box >= 2) tma_store_wait_read_n<1>();
+                        else tma_store_wait_read_n<0>();
+                    }
+                    __syncwarp();
                 }
-                __syncwarp();
                 const uint32_t stage_row = box + lane * 128;
-                // with a shortcut input the activation waits for the second pass below
-                const int relu_now = res_pass ? 0 : p.relu;
-                const float bias_cur = bias_next;
-                if (blk + 2 < n_blk) bias_next = bias_lane_load(p.bias, o0 + (blk + 2) * 32, p.c_out, lane);   // a block ahead
 #pragma unroll
                 for (int qq = 0; qq < 8; ++qq) {
-                    float o[4];
-                    const float4 bv = bias_quad(bias_cur, qq);
-                    o[0] = __uint_as_float(v[qq * 4 + 0]) + bv.x;
-                    o[1] = __uint_as_float(v[qq * 4 + 1]) + bv.y;
-                    o[2] = __uint_as_float(v[qq * 4 + 2]) + bv.z;
-                    o[3] = __uint_as_float(v[qq * 4 + 3]) + bv.w;
-                    if (relu_now) {
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) o[e] = fmaxf(o[e], 0.f);
+                    const uint32_t at = stage_row + ((qq ^ rx) << 4);
+                    float4 o = make_float4(__uint_as_float(v[qq * 4 + 0]), __uint_as_float(v[qq * 4 + 1]), __uint_as_float(v[qq * 4 + 2]),
+                                           __uint_as_float(v[qq * 4 + 3]));
+                    nm_add4(o, bias[qq]);
+                    if (res) {
+                        float4 x;
+                        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(at) : "memory");
+                        nm_add4(o, x);
                     }
-                    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(stage_row + ((qq ^ rx) << 4)), "f"(o[0]),
-                                 "f"(o[1]), "f"(o[2]), "f"(o[3])
-                                 : "memory");
-                }
-                if (res_pass) {
-                    __syncwarp();
-                    apply_residual_box(box, rv, p.relu, lane);
-                    if (blk + 2 < n_blk)
-                        load_residual_box(rv, res_base + (blk + 2) * 32, p.c_out, res_rows, lane, cols_left - (blk + 2) * 32);
+                    if (p.relu) { o.x = fmaxf(o.x, 0.f); o.y = fmaxf(o.y, 0.f); o.z = fmaxf(o.z, 0.f); o.w = fmaxf(o.w, 0.f); }
+                    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(at), "f"(o.x), "f"(o.y), "f"(o.z), "f"(o.w) : "memory");
                 }
                 fence_proxy_async();
                 __syncwarp();
                 if (elect_one()) {
-                    if (pix0 + q * 32 < p.pixels)
-                        tma_store_2d(&tm_y, box, o0 + blk * 32, ks * cfg.p_pad + static_cast<int>(pix0) + q * 32);
+                    tma_store_2d(box_rows == 32 ? &tm_y : &tm_tail, box, o0 + blk * 32, static_cast<int>(item.ks) * cfg.p_pad + pix0);
                     tma_store_commit();
                 }
+                if (++bx == n_box) { bx = 0; bpar ^= 1u; }
             }
             if (n_blk == 1 && half == 1) {
                 // a single channel block: the second warp of the quadrant only releases the buffer
@@ -522,6 +621,12 @@ k_conv_expand(const ConvParams p, const ExpandCfg cfg, const __grid_constant__ C
                 if (lane == 0)
                     for (uint32_t pos = first_pos + 1u; pos <= last_pos; ++pos)
                         flags[(gridDim.x - 1u - pos) * 8u + (warp - 4)] = 0u;
+            }
+        }
+        if (aborted(abort_flag)) {   // shortcut boxes still on their way to this CTA's shared memory (bounded)
+            for (; taken != asked; ++taken) {
+                (void)mbar_wait_polls(smem_u32(&s_res[warp - 4][bx]), bpar, 1u << 16);
+                if (++bx == n_box) { bx = 0; bpar ^= 1u; }
             }
         }
         if (elect_one()) tma_store_wait_read();   // shared memory must outlive the stores' reads; the writes complete with the grid
@@ -598,6 +703,7 @@ bool make_cfg(const ConvParams& p, const nm_plan_t* plan, ExpandCfg* cfg)
     if (bn < 32 || bn > 256 || bn % 32 != 0 || p.wx_rows % bn != 0) return false;
     cfg->bn = bn;
     cfg->n_slices = p.wx_rows / bn;
+    cfg->sl_shift = (cfg->n_slices & (cfg->n_slices - 1)) == 0 ? __builtin_ctz(static_cast<unsigned>(cfg->n_slices)) : -1;
     cfg->b_bytes = ((bn * 128 + 1023) / 1024) * 1024;
     const int splits = plan && plan->split > 1 ? plan->split : 1;
     const bool balanced = plan && plan->split == -1;
@@ -632,7 +738,17 @@ bool make_cfg(const ConvParams& p, const nm_plan_t* plan, ExpandCfg* cfg)
     }
     cfg->sub_bytes = SUB_BYTES + (cfg->w_res ? 0 : cfg->b_bytes);
     cfg->stage_bytes = kblk * cfg->sub_bytes;
-    const int budget = 227 * 1024 - 1024 - 8 * cfg->boxes * BOX_BYTES - 1024 - cfg->wres_bytes;
+    const int room = 227 * 1024 - 1024 - 1024 - cfg->wres_bytes;
+    if (p.residual && splits == 1) {
+        // as many boxes as leave the ring four (three boxes) or three (two) blocks of 32 columns, or the stages asked for
+        const int want = plan && plan->stages > 0 ? plan->stages * cfg->stage_bytes : 0;
+        cfg->boxes = 1;
+        for (int b = BOXES_MAX; b >= 2 && cfg->boxes == 1; --b) {
+            const int ring = room - 8 * b * BOX_BYTES;
+            if (ring >= (want ? want : (b + 1) * cfg->sub_bytes) && ring >= 2 * cfg->stage_bytes) cfg->boxes = b;
+        }
+    }
+    const int budget = room - 8 * cfg->boxes * BOX_BYTES;
     int stages = plan && plan->stages > 0 ? plan->stages : NSTAGE_MAX;
     if (stages > NSTAGE_MAX) return false;
     if (plan && plan->stages > 0) {
@@ -644,7 +760,20 @@ bool make_cfg(const ConvParams& p, const nm_plan_t* plan, ExpandCfg* cfg)
         if (stages * cfg->stage_bytes > budget) return false;
     }
     cfg->stages = stages;
-    cfg->n_work = ((p.pixels + BM - 1) / BM) * cfg->n_slices * splits;
+    cfg->flat = pointwise && p.stride_h == 1 && p.stride_w == 1 && p.pad_h == 0 && p.pad_w == 0;
+    cfg->rows = BM;
+    long long tiles = (p.pixels + BM - 1) / BM;
+    if (splits == 1 && !balanced) {
+        // fewest pixels per item (in steps of 8) that the same number of rounds covers
+        const long long ctas = cfg->w_res ? sm_count() / cfg->n_slices * cfg->n_slices : sm_count();
+        const long long rounds = (tiles * cfg->n_slices + ctas - 1) / ctas;
+        const long long most = rounds * ctas / cfg->n_slices;   // pixel tiles that fit into them
+        cfg->rows = static_cast<int>(((p.pixels + most - 1) / most + 7) / 8 * 8);
+        if (cfg->rows > BM) cfg->rows = BM;
+        if (cfg->rows < 32) cfg->rows = 32;   // a whole box; below that the weights cost more than the pixels
+        tiles = (p.pixels + cfg->rows - 1) / cfg->rows;
+    }
+    cfg->n_work = tiles * cfg->n_slices * splits;
     if (cfg->n_work >= (1ll << 31)) return false;
     cfg->balanced = 0;
     if (balanced) {
@@ -689,13 +818,19 @@ nm_status_t launch_conv_expand(const ConvParams& p, const nm_plan_t* plan, cudaS
         q.residual = nullptr;
         q.relu = 0;
     }
-    alignas(64) CUtensorMap tm_x, tm_y;
-    if (!nmtm::encode_x_im2col(p, BM, &tm_x) || !nmtm::encode_y_tiled(q, &tm_y))
+    alignas(64) CUtensorMap tm_x, tm_y, tm_tail, tm_res;
+    if (!(cfg.flat ? nmtm::encode_x_rows(p, cfg.rows, &tm_x) : nmtm::encode_x_im2col(p, cfg.rows, &tm_x)) || !nmtm::encode_y_tiled(q, &tm_y))
+        return fail(NM_ERR_CUDA, "nm_conv2d: tensor-map encoding failed (variant 4)");
+    tm_res = tm_y;
+    if (q.residual && !nmtm::encode_y_tiled(q, &tm_res, 32, q.residual))
+        return fail(NM_ERR_CUDA, "nm_conv2d: tensor-map encoding failed (variant 4)");
+    tm_tail = tm_y;   // an item's last box, when its pixels are no multiple of 32
+    if (cfg.rows % 32 != 0 && !nmtm::encode_y_tiled(q, &tm_tail, cfg.rows % 32))
         return fail(NM_ERR_CUDA, "nm_conv2d: tensor-map encoding failed (variant 4)");
     q.pixels = p.pixels;
     size_t smem = 1024 + cfg.wres_bytes + static_cast<size_t>(cfg.stages) * cfg.stage_bytes + 8 * cfg.boxes * BOX_BYTES;
     if (smem < NM_EXCLUSIVE_SMEM) smem = NM_EXCLUSIVE_SMEM;   // one CTA per SM: it owns all 512 TMEM columns
-    using Kernel = void (*)(const ConvParams, const ExpandCfg, const CUtensorMap, const CUtensorMap);
+    using Kernel = void (*)(const ConvParams, const ExpandCfg, const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap);
     const Kernel kernel = cfg.balanced ? (cfg.kblk == 2 ? k_conv_expand<2, true> : k_conv_expand<1, true>)
                                        : (cfg.kblk == 2 ? k_conv_expand<2, false> : k_conv_expand<1, false>);
     cudaError_t e = nmhost::ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), smem);
@@ -703,7 +838,7 @@ nm_status_t launch_conv_expand(const ConvParams& p, const nm_plan_t* plan, cudaS
     long long grid = cfg.n_work < sm_count() ? cfg.n_work : sm_count();
     if (cfg.balanced) grid = sm_count();
     if (cfg.w_res) grid = (grid / cfg.n_slices) * cfg.n_slices;   // n_work is a multiple of n_slices, so grid >= n_slices
-    e = nmhost::launch_pdl(kernel, static_cast<unsigned>(grid), THREADS, smem, st, q, cfg, tm_x, tm_y);
+    e = nmhost::launch_pdl(kernel, static_cast<unsigned>(grid), THREADS, smem, st, q, cfg, tm_x, tm_y, tm_tail, tm_res);
     nmhost::count_launch(1);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return fail(NM_ERR_CUDA, "nm_conv2d launch (variant 4): %s", cudaGetErrorString(e));

@@ -84,14 +84,27 @@ inline bool encode_w_tiled(const ConvParams& p, int rows, CUtensorMap* tm)
                             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Output [pixels][c_out] as a tiled map with a 32-channel x 32-pixel box (one warp's share).
-inline bool encode_y_tiled(const ConvParams& p, CUtensorMap* tm)
+// Activations of a pointwise layer of stride 1: [pixels][c_in] as a tiled map with a 32-channel x `rows`-pixel box.
+inline bool encode_x_rows(const ConvParams& p, int rows, CUtensorMap* tm)
+{
+    const cuuint64_t dims[2] = {static_cast<cuuint64_t>(p.c_in), static_cast<cuuint64_t>(p.batch) * p.h * p.w};
+    const cuuint64_t strides[1] = {static_cast<cuuint64_t>(p.c_in) * 4};
+    const cuuint32_t box[2] = {32, static_cast<cuuint32_t>(rows)};
+    const cuuint32_t es[2] = {1, 1};
+    return encoders().tiled(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(p.x), dims, strides, box, es,
+                            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// Output [pixels][c_out] as a tiled map with a 32-channel x 32-pixel box (one warp's share), or fewer pixels; `base`: another
+// tensor of the output's shape (the shortcut input).
+inline bool encode_y_tiled(const ConvParams& p, CUtensorMap* tm, int rows = 32, const float* base = nullptr)
 {
     const cuuint64_t dims[2] = {static_cast<cuuint64_t>(p.c_out), static_cast<cuuint64_t>(p.pixels)};
     const cuuint64_t strides[1] = {static_cast<cuuint64_t>(p.c_out) * 4};
-    const cuuint32_t box[2] = {32, 32};
+    const cuuint32_t box[2] = {32, static_cast<cuuint32_t>(rows)};
     const cuuint32_t es[2] = {1, 1};
-    return encoders().tiled(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, p.y, dims, strides, box, es,
+    return encoders().tiled(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, base ? const_cast<float*>(base) : p.y, dims, strides, box, es,
                             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
