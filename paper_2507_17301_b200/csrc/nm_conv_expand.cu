@@ -32,7 +32,7 @@
 // equally long range per CTA, so an item may be shared by two or more CTAs.  A CTA whose range
 // begins inside an item handles that part FIRST, stores the raw partial accumulator to its own
 // slot of the handle's scratch and raises a per-warp flag; the CTA whose range holds the item's
-// first stage handles it LAST, waits (bounded) for the flags of the others, adds their partial sums
+// first stage handles it next, before its whole items, waits (bounded) for the flags of the others, adds their partial sums
 // to its accumulator, lowers the flags again (every flag has exactly one reader, so the scratch is
 // back in its cleared state when the launch ends and a recorded launch can be replayed) and runs
 // the normal epilogue.  Ranges are handed out from the end of the
@@ -127,25 +127,47 @@ __device__ __forceinline__ ItemPos item_of(uint32_t work, const ExpandCfg& cfg)
     return it;
 }
 // Walks a CTA's pieces: whole items `first, first + stride, ...` in the static schedule, or the
-// contiguous range of (item, stage) units of balanced mode.
+// contiguous range of (item, stage) units of balanced mode: the rest of an item begun elsewhere first, then the part of
+// the item that is continued elsewhere, then the whole items.  The part that waits for other CTAs' sums is so finished while
+// the main loop of a whole item runs, instead of after the last of them.
 template <bool BAL>
 struct SegIter {
-    uint32_t cur, end, stride;
+    uint32_t cur, end, stride;   // balanced: stride counts the phases done
     int stages;
     __device__ __forceinline__ bool next(Seg& g)
     {
-        if (cur >= end) return false;
         if (!BAL) {
+            if (cur >= end) return false;
             g.work = cur; g.sb = 0; g.se = stages;
             cur += stride;
             return true;
         }
-        g.work = cur / static_cast<uint32_t>(stages);
-        g.sb = static_cast<int>(cur - g.work * static_cast<uint32_t>(stages));
-        const uint32_t left = end - cur, room = static_cast<uint32_t>(stages - g.sb);
-        const int len = static_cast<int>(left < room ? left : room);
-        g.se = g.sb + len;
-        cur += static_cast<uint32_t>(len);
+        const uint32_t n = static_cast<uint32_t>(stages);
+        if (stride == 0) {
+            stride = 1;
+            g.work = cur / n;
+            g.sb = static_cast<int>(cur - g.work * n);
+            if (g.sb > 0 && cur < end) {
+                const uint32_t room = n - static_cast<uint32_t>(g.sb), len = end - cur < room ? end - cur : room;
+                g.se = g.sb + static_cast<int>(len);
+                cur += len;
+                return true;
+            }
+        }
+        if (stride == 1) {
+            stride = 2;
+            g.work = end / n;
+            const uint32_t part = end - g.work * n;
+            if (part > 0 && end - part >= cur) {
+                g.sb = 0;
+                g.se = static_cast<int>(part);
+                end -= part;
+                return true;
+            }
+        }
+        if (cur >= end) return false;
+        g.work = cur / n; g.sb = 0; g.se = stages;
+        cur += n;
         return true;
     }
 };
@@ -496,6 +518,11 @@ k_conv_expand(const ConvParams p, const ExpandCfg cfg, const __grid_constant__ C
                 if (lane == 0) mbar_arrive(smem_u32(&s_accfree[ab]));
                 continue;
             }
+            // The accumulator columns of a block are read while the block before it is finished (not in balanced mode, which
+            // has partial sums in those registers).
+            const uint32_t acc_addr = tmem + lane_addr + (ab * cfg.n_iss + acc_first) * cfg.bn;
+            uint32_t vn[32];
+            if (!BAL && half < n_blk) tmem_ld32(acc_addr + half * 32, vn);
             for (int blk = half; blk < n_blk; blk += 2) {
                 float4 bias[8];
 #pragma unroll
@@ -504,16 +531,20 @@ k_conv_expand(const ConvParams p, const ExpandCfg cfg, const __grid_constant__ C
                     bias[qq] = p.bias != nullptr && o < p.c_out ? __ldg(reinterpret_cast<const float4*>(p.bias + o)) : make_float4(0.f, 0.f, 0.f, 0.f);
                 }
                 uint32_t v[32];
-                tmem_ld32(tmem + lane_addr + (ab * cfg.n_iss + acc_first) * cfg.bn + blk * 32, v);
+                if (BAL) tmem_ld32(acc_addr + blk * 32, vn);
                 if (two_acc) {
                     uint32_t v2[32];
                     tmem_ld32(tmem + lane_addr + (ab * cfg.n_iss + 1) * cfg.bn + blk * 32, v2);
-                    tmem_ld_wait();
+                    tmem_ld_wait(v2);
+                    tmem_ld_wait(vn);
 #pragma unroll
-                    for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) + __uint_as_float(v2[e]));
+                    for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(__uint_as_float(vn[e]) + __uint_as_float(v2[e]));
                 } else {
-                    tmem_ld_wait();
+                    tmem_ld_wait(vn);
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) v[e] = vn[e];
                 }
+                if (!BAL && blk + 2 < n_blk) tmem_ld32(acc_addr + (blk + 2) * 32, vn);
                 if (blk + 2 >= n_blk) {
                     tc_fence_before();
                     __syncwarp();
