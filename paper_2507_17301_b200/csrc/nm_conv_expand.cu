@@ -38,6 +38,8 @@
 // the normal epilogue.  Ranges are handed out from the end of the
 // layer to CTA 0 upwards, so a CTA only ever waits for CTAs with a lower index, whose first action
 // is the store it waits for.
+#include <algorithm>
+
 #include "nm_internal.h"
 #include "nm_ptx.cuh"
 #include "nm_tmap.cuh"
@@ -47,8 +49,7 @@ namespace {
 using namespace nmk;
 
 constexpr int BM = 128;
-constexpr int SUB_BYTES = BM * 128;
-constexpr int NSTAGE_MAX = 10;
+constexpr int NSTAGE_MAX = 14;
 constexpr int WRES_MAX = 128 * 1024;            // largest weight slice kept resident
 constexpr int THREADS = 384;                   // 4 service warps + 8 epilogue warps
 constexpr int BOX_BYTES = 4096;                // one 32-pixel x 32-channel output box
@@ -57,16 +58,16 @@ constexpr int BOXES_MAX = 3;                   // staging boxes per epilogue war
 struct ExpandCfg {
     int bn;           // output channels per work item
     int n_slices;
-    int stages;
-    int b_bytes;      // weight bytes per stage (bn rows of 128 bytes)
-    int stage_bytes;
+    int stages;       // activation ring: slots
+    int w_stages;     // weight ring: slots, at most `stages` (0 with resident weights)
+    int b_bytes;      // bytes of a weight block (bn rows of 128 bytes)
+    int a_bytes;      // bytes a 32-column block of activations takes in a slot (rows of 128 bytes, rounded up to 1 KB)
     int w_res;        // 1: this CTA's weight slice stays resident in shared memory (it is loaded once)
     int wres_bytes;   // bytes of the resident slice: all 32-column blocks of bn rows
     int n_sub;        // pipeline stages one work item reduces over: (K / 32) / ksplit / kblk
     int kblk;         // 32-column blocks per stage (1 or 2): one barrier round trip then covers kblk * 4 MMAs
     int n_iss;        // MMA issuer threads (1 or 2): two take alternate pipeline stages of an item, each into an accumulator of its own
     int n_acc;        // accumulator buffers (of n_iss accumulators each) in tensor memory: 2 when they fit, else 1
-    int sub_bytes;    // bytes of one 32-column block inside a stage: activations (+ streamed weights)
     int rows;         // pixels per work item
     int flat;         // 1: activations as 2-D rows (pointwise, stride 1), 0: im2col
     int ksplit;       // K splits (1 = none): a work item covers one of them and stores raw partial sums
@@ -221,7 +222,11 @@ k_conv_expand(const ConvParams p, const ExpandCfg cfg, const __grid_constant__ C
     const int NS = cfg.stages, n_sub = cfg.n_sub;
     const uint32_t wres = (smem_u32(smem_raw) + 1023u) & ~1023u;   // resident weight slice (may be empty)
     const uint32_t ring = wres + cfg.wres_bytes;
-    const uint32_t staging = ring + NS * cfg.stage_bytes;
+    const uint32_t a_slot = static_cast<uint32_t>(KBLK * cfg.a_bytes), w_slot = static_cast<uint32_t>(KBLK * cfg.b_bytes);
+    // activation ring, weight ring, output staging; an MMA reads 128 rows from an activation slot's start, rows past the
+    // item's come from whatever lies behind and end in accumulator rows nobody reads
+    const uint32_t w_ring = ring + NS * a_slot;
+    const uint32_t staging = w_ring + cfg.w_stages * w_slot;
     volatile int* abort_flag = &s_abort;
 
     if (warp == 2) tmem_alloc(smem_u32(&s_tmem), 512);
@@ -283,7 +288,7 @@ k_conv_expand(const ConvParams p, const ExpandCfg cfg, const __grid_constant__ C
                 }
                 for (int c = seg.sb; c < seg.se; ++c) {
                     if (!free_now && !wait_stage(smem_u32(&s_free[rp.s]), rp.parity ^ 1u, abort_flag, 2)) { ok = false; break; }
-                    uint32_t a_smem = ring + rp.s * cfg.stage_bytes;
+                    uint32_t a_smem = ring + rp.s * a_slot;
                     const uint32_t bar = smem_u32(&s_full[rp.s]);
                     mbar_arrive_expect_tx(bar, tx);
                     rp.advance(NS);
@@ -295,7 +300,7 @@ k_conv_expand(const ConvParams p, const ExpandCfg cfg, const __grid_constant__ C
                         else
                             tma_load_im2col_4d(a_smem, &tm_x, bar, ch, w0, h0, n0, static_cast<uint16_t>(off_w),
                                                static_cast<uint16_t>(off_h));
-                        a_smem += cfg.sub_bytes;
+                        a_smem += cfg.a_bytes;
                         ch += 32;
                         if (ch >= p.c_in) {
                             ch = 0;
@@ -323,27 +328,33 @@ k_conv_expand(const ConvParams p, const ExpandCfg cfg, const __grid_constant__ C
                     bulk_load_1d(wres + c * cfg.b_bytes, p.wx + static_cast<size_t>(c) * w_step + static_cast<size_t>(slice) * cfg.bn * 32,
                                  w_bytes, smem_u32(&s_wres));
             } else {
+                // Stage t joins the full barrier of its activation slot, t modulo the activation ring; its weight slot, t modulo
+                // the (shorter) weight ring, is free once the MMAs of stage t - w_stages are done, which is what the free
+                // barrier of THAT stage's activation slot says.
                 int issued = 0;
-                RingPos rp;
+                RingPos rp, rf;      // full barrier of this stage, free barrier of the stage that used the weight slot before
+                int ws = 0;
+                bool wrapped = false;
                 SegIter<BAL> it = make_iter<BAL>(cfg);
                 Seg seg;
                 bool ok = true, free_now = true;
                 while (ok && it.next(seg)) {
                     const ItemPos item = item_of(seg.work, cfg);
-                    const uint32_t slice = item.slice;
                     const int c0 = static_cast<int>(item.ks) * n_blk32 + seg.sb * KBLK;
-                    const float* wsrc = p.wx + static_cast<size_t>(slice) * cfg.bn * 32 + static_cast<size_t>(c0) * w_step;
+                    const float* wsrc = p.wx + static_cast<size_t>(item.slice) * cfg.bn * 32 + static_cast<size_t>(c0) * w_step;
                     for (int c = seg.sb; c < seg.se; ++c) {
-                        if (!free_now && !wait_stage(smem_u32(&s_free[rp.s]), rp.parity ^ 1u, abort_flag, 9)) { ok = false; break; }
-                        uint32_t b_smem = ring + rp.s * cfg.stage_bytes + SUB_BYTES;
+                        if (!free_now && !wait_stage(smem_u32(&s_free[rf.s]), rf.parity, abort_flag, 9)) { ok = false; break; }
+                        if (wrapped) rf.advance(NS);
+                        uint32_t b_smem = w_ring + ws * w_slot;
                         const uint32_t bar = smem_u32(&s_full[rp.s]);
                         mbar_arrive_expect_tx(bar, static_cast<uint32_t>(KBLK) * w_bytes);
                         rp.advance(NS);
-                        free_now = !rp.wrapped || mbar_test_wait(smem_u32(&s_free[rp.s]), rp.parity ^ 1u);
+                        if (++ws == cfg.w_stages) { ws = 0; wrapped = true; }
+                        free_now = !wrapped || mbar_test_wait(smem_u32(&s_free[rf.s]), rf.parity);
 #pragma unroll
                         for (int j = 0; j < KBLK; ++j) {
                             bulk_load_1d(b_smem, wsrc, w_bytes, bar);
-                            b_smem += cfg.sub_bytes;
+                            b_smem += cfg.b_bytes;
                             wsrc += w_step;
                         }
                         ++issued;
@@ -370,6 +381,7 @@ k_conv_expand(const ConvParams p, const ExpandCfg cfg, const __grid_constant__ C
             const bool shared_k = cfg.n_iss == 2;
             if (cfg.w_res && !mbar_wait(smem_u32(&s_wres), 0)) *abort_flag = 9;
             RingPos rp;
+            int ws = 0;
             uint32_t ab = 0, acc_par = 0;   // accumulator buffer of this item, parity of its current use
             bool acc_wrapped = false;
             SegIter<BAL> it = make_iter<BAL>(cfg);
@@ -385,27 +397,27 @@ k_conv_expand(const ConvParams p, const ExpandCfg cfg, const __grid_constant__ C
                 for (int c = seg.sb; c < seg.se; ++c) {
                     if (shared_k && (rp.s & 1) != iss) {   // the other thread's slot
                         rp.advance(NS);
+                        if (++ws == cfg.w_stages) ws = 0;
                         continue;
                     }
                     if (!mbar_wait_lone(smem_u32(&s_full[rp.s]), rp.parity)) { *abort_flag = 6; break; }
                     tc_fence_after();
-                    const uint32_t a_smem = ring + rp.s * cfg.stage_bytes;
-                    uint64_t adesc = umma_desc_k_sw128(a_smem, 1024);
-                    uint64_t bdesc = umma_desc_k_sw128(cfg.w_res ? wres + c * KBLK * cfg.b_bytes : a_smem + SUB_BYTES, 1024);
-                    const uint32_t b_step = KBLK > 1 ? static_cast<uint32_t>(cfg.w_res ? cfg.b_bytes : cfg.sub_bytes) >> 4 : 0u;
+                    uint64_t adesc = umma_desc_k_sw128(ring + rp.s * a_slot, 1024);
+                    uint64_t bdesc = umma_desc_k_sw128(cfg.w_res ? wres + c * KBLK * cfg.b_bytes : w_ring + ws * w_slot, 1024);
 #pragma unroll
                     for (int j = 0; j < KBLK; ++j) {
 #pragma unroll
                         for (int kq = 0; kq < 4; ++kq)
                             umma_tf32_ss(acc, adesc + 2 * kq, bdesc + 2 * kq, idesc, (j > 0 || kq > 0) ? 1u : started);
                         if (j + 1 < KBLK) {
-                            adesc += static_cast<uint32_t>(cfg.sub_bytes) >> 4;   // next 32-column block (start address field, 16-byte units)
-                            bdesc += b_step;
+                            adesc += static_cast<uint32_t>(cfg.a_bytes) >> 4;   // next 32-column block (start address field, 16-byte units)
+                            bdesc += static_cast<uint32_t>(cfg.b_bytes) >> 4;
                         }
                     }
                     started = 1u;
                     umma_commit(smem_u32(&s_free[rp.s]));
                     rp.advance(NS);
+                    if (++ws == cfg.w_stages) ws = 0;
                 }
                 if (aborted(abort_flag)) break;
                 umma_commit(smem_u32(&s_accfull[ab]));
@@ -767,30 +779,6 @@ bool make_cfg(const ConvParams& p, const nm_plan_t* plan, ExpandCfg* cfg)
         cfg->wres_bytes = blk32 * cfg->b_bytes;
         if (cfg->wres_bytes > 64 * 1024) cfg->boxes = 1;   // a large slice: give the output staging's room to the ring
     }
-    cfg->sub_bytes = SUB_BYTES + (cfg->w_res ? 0 : cfg->b_bytes);
-    cfg->stage_bytes = kblk * cfg->sub_bytes;
-    const int room = 227 * 1024 - 1024 - 1024 - cfg->wres_bytes;
-    if (p.residual && splits == 1) {
-        // as many boxes as leave the ring four (three boxes) or three (two) blocks of 32 columns, or the stages asked for
-        const int want = plan && plan->stages > 0 ? plan->stages * cfg->stage_bytes : 0;
-        cfg->boxes = 1;
-        for (int b = BOXES_MAX; b >= 2 && cfg->boxes == 1; --b) {
-            const int ring = room - 8 * b * BOX_BYTES;
-            if (ring >= (want ? want : (b + 1) * cfg->sub_bytes) && ring >= 2 * cfg->stage_bytes) cfg->boxes = b;
-        }
-    }
-    const int budget = room - 8 * cfg->boxes * BOX_BYTES;
-    int stages = plan && plan->stages > 0 ? plan->stages : NSTAGE_MAX;
-    if (stages > NSTAGE_MAX) return false;
-    if (plan && plan->stages > 0) {
-        if (stages * cfg->stage_bytes > budget) return false;
-        if (n_iss == 2 && stages % 2 != 0) return false;   // two issuers own alternate ring slots
-    } else {
-        while (stages > 2 && stages * cfg->stage_bytes > budget) --stages;
-        if (n_iss == 2) stages &= ~1;
-        if (stages * cfg->stage_bytes > budget) return false;
-    }
-    cfg->stages = stages;
     cfg->flat = pointwise && p.stride_h == 1 && p.stride_w == 1 && p.pad_h == 0 && p.pad_w == 0;
     cfg->rows = BM;
     long long tiles = (p.pixels + BM - 1) / BM;
@@ -804,6 +792,41 @@ bool make_cfg(const ConvParams& p, const nm_plan_t* plan, ExpandCfg* cfg)
         if (cfg->rows < 32) cfg->rows = 32;   // a whole box; below that the weights cost more than the pixels
         tiles = (p.pixels + cfg->rows - 1) / cfg->rows;
     }
+    // Rings.  Both operands are bound by bytes in flight: activations come from HBM, weights (the same for every CTA, twice the
+    // bytes) from L2.  A slot holds the item's pixels only, and the weight ring gets as many slots as leave the activation
+    // ring one more (at least three where that many of both fit).  1024 -> 256 at 14x14, batch 64 (88-pixel items): 20.2 us with
+    // four slots of 16 + 32 KB, 18.8 with 5 + 4, 20.8 with 8 + 3; 256 -> 512 / 2 at 56x56: 39.9 -> 36.0 with 4 + 3, 51 with 2 + 4.
+    cfg->a_bytes = (cfg->rows * 128 + 1023) / 1024 * 1024;
+    const int a_slot = kblk * cfg->a_bytes, w_slot = cfg->w_res ? 0 : kblk * cfg->b_bytes;
+    const int room = 227 * 1024 - 1024 - 2048 - cfg->wres_bytes;   // alignment slack, barriers
+    const int asked = plan && plan->stages > 0 ? plan->stages : 0;
+    if (p.residual && splits == 1) {
+        // as many boxes as leave the ring four (three boxes) or three (two) blocks of 32 columns, or the stages asked for
+        const int want = asked * (a_slot + w_slot), block = cfg->a_bytes + (cfg->w_res ? 0 : cfg->b_bytes);
+        cfg->boxes = 1;
+        for (int b = BOXES_MAX; b >= 2 && cfg->boxes == 1; --b) {
+            const int left = room - 8 * b * BOX_BYTES;
+            if (left >= (want ? want : (b + 1) * block) && left >= 2 * (a_slot + w_slot)) cfg->boxes = b;
+        }
+    }
+    const int budget = room - 8 * cfg->boxes * BOX_BYTES;
+    int na = asked, nw = cfg->w_res ? 0 : asked;
+    if (asked == 0) {
+        if (!cfg->w_res) {
+            auto slots = [&](int n) { return std::min((budget - n * w_slot) / a_slot, NSTAGE_MAX); };
+            nw = 2;
+            while (slots(nw + 1) >= nw + 2) ++nw;
+            if (nw == 2 && slots(3) >= 3) nw = 3;
+        }
+        na = (budget - nw * w_slot) / a_slot;
+        if (na > NSTAGE_MAX) na = NSTAGE_MAX;
+        if (n_iss == 2) na &= ~1;
+    }
+    if (na < 2 || na > NSTAGE_MAX || na * a_slot + nw * w_slot > budget) return false;
+    if (nw > na) nw = na;
+    if (n_iss == 2 && na % 2 != 0) return false;   // two issuers own alternate ring slots
+    cfg->stages = na;
+    cfg->w_stages = nw;
     cfg->n_work = tiles * cfg->n_slices * splits;
     if (cfg->n_work >= (1ll << 31)) return false;
     cfg->balanced = 0;
@@ -859,7 +882,8 @@ nm_status_t launch_conv_expand(const ConvParams& p, const nm_plan_t* plan, cudaS
     if (cfg.rows % 32 != 0 && !nmtm::encode_y_tiled(q, &tm_tail, cfg.rows % 32))
         return fail(NM_ERR_CUDA, "nm_conv2d: tensor-map encoding failed (variant 4)");
     q.pixels = p.pixels;
-    size_t smem = 1024 + cfg.wres_bytes + static_cast<size_t>(cfg.stages) * cfg.stage_bytes + 8 * cfg.boxes * BOX_BYTES;
+    size_t smem = 1024 + cfg.wres_bytes + static_cast<size_t>(cfg.stages) * cfg.kblk * cfg.a_bytes +
+                  static_cast<size_t>(cfg.w_stages) * cfg.kblk * cfg.b_bytes + 8 * cfg.boxes * BOX_BYTES;
     if (smem < NM_EXCLUSIVE_SMEM) smem = NM_EXCLUSIVE_SMEM;   // one CTA per SM: it owns all 512 TMEM columns
     using Kernel = void (*)(const ConvParams, const ExpandCfg, const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap);
     const Kernel kernel = cfg.balanced ? (cfg.kblk == 2 ? k_conv_expand<2, true> : k_conv_expand<1, true>)
