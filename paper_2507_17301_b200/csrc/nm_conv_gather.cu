@@ -1,18 +1,27 @@
 // Variant 1: direct-gather sparse implicit GEMM (any shape).
 //
-// One CTA owns 128 output pixels and ONE pruning tile (tile_t output channels, which share a kept
-// set).  For every chunk of 32 retained columns the four warps gather the activations
+// A CTA owns 128 output pixels and G pruning tiles (each with its own kept set).  For every chunk of 32 retained columns
+// and every tile, eight warps gather the activations
 //     a[p][j] = x[n][oh*s - pad + kh_j*dil][ow*s - pad + kw_j*dil][c_j]      (zero outside the image)
-// straight from NHWC global memory (lane = retained column j, so a warp reads one pixel's
-// retained channels: neighbouring addresses), round them to TF32 and store them in the
-// 128-byte-swizzled K-major layout tcgen05 reads; the matching [tile_t x 32] weight chunk is
-// staged the same way.  One thread then issues four 128 x N x 8 TF32 MMAs that accumulate in
-// tensor memory.  This is Algorithm 1 with the vector register replaced by a 128-pixel operand
-// tile and the T accumulators by T TMEM columns; the gather is the fused im2col + packing of
-// Sec. 3.2 without its buffer.  Epilogue: TMEM -> registers, + bias, ReLU, NHWC store.
+// straight from NHWC global memory (lane = retained column j, so a warp reads one pixel's retained channels:
+// neighbouring addresses; the tiles of a CTA follow one another on the same chunk and share its lines in L1), round them to
+// TF32 and store them in the 128-byte-swizzled K-major layout tcgen05 reads.  One thread fetches the tile's weight
+// chunk (stored as the shared-memory image) with a bulk copy, one issues four 128 x N x 8 TF32 MMAs per chunk and tile into the
+// tile's accumulator columns in tensor memory.  This is Algorithm 1 with the vector register replaced by a 128-pixel
+// operand tile and the T accumulators by T TMEM columns; the gather is the fused im2col + packing of Sec. 3.2 without its
+// buffer.
 //
-// It is the fallback for shapes the slab kernel does not take (c_in not a multiple of 4, groups
-// that straddle slabs) and the reference point the faster variant is measured against.
+// It is the library's choice for every shape the TMA-fed kernels do not take (channel counts that are no multiple of
+// 32, small or odd tile widths, small inputs), so it has to be good at all of them.  What bounds it is the
+// gather's instruction stream, about 6.5 per warp and pixel row: two chunks are kept in flight in registers, the ring of
+// operand slots decouples the gathering warps from the MMAs, two CTAs share an SM, and where there are fewer pixel blocks
+// and tiles than SMs the chunks are split over the CTAs of a thread-block cluster (partial sums move as bulk copies
+// between their shared memories and are added in the order of the ranges).  XXX
+//
+//   warps 0-7  gather, then epilogue: TMEM -> staging in shared memory -> bias, shortcut, ReLU, coalesced NHWC stores
+//   warp 8     MMA issuer, tensor memory      warp 9  weight producer
+#include <algorithm>
+
 #include "nm_internal.h"
 #include "nm_ptx.cuh"
 
@@ -20,160 +29,426 @@ namespace {
 
 using namespace nmk;
 
-constexpr int BM = 128;  // output pixels per CTA = MMA M
+constexpr int BM = 128;                       // output pixels per CTA = MMA M
 constexpr int A_BYTES = BM * NM_KCHUNK * 4;
+constexpr int THREADS = 320;
+constexpr int GATHER = 256;                   // threads of the gathering warps
+constexpr int RPW = 16;                       // pixel rows per gathering warp
+constexpr int NA = 2;                         // operand slots
+constexpr int TAPS_AHEAD = 4;
+constexpr int NW_MAX = 8;                     // weight slots
+constexpr int PASS = 64;                      // output channels staged at a time
 
-__global__ void __launch_bounds__(128) k_conv_gather(const ConvParams p, const int umma_n, const int tmem_cols)
+struct GatherCfg {
+    int n;            // MMA width = accumulator columns per tile
+    int te;           // channels of a tile that can exist (the tile width, or c_out if that is smaller)
+    int g, n_groups;  // tiles per CTA, CTAs along the tiles
+    int cs;           // CTAs per cluster = ranges of the chunks
+    int chunks;
+    int w_stages, w_bytes;
+    int rps;          // pixel rows a CTA of the cluster finishes
+    int tmem_cols;
+};
+
+__device__ __forceinline__ bool aborted(volatile int* flag) { return *flag != 0; }
+
+// Shared memory of this CTA to that of a CTA of the cluster; the barrier is one of the receiving CTA.
+__device__ __forceinline__ void bulk_copy_cluster(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar)
+{
+    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "r"(src),
+                 "r"(bytes), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ int pitch_of(int cols)
+{
+    // floats per staged row: whole 16-byte pieces, an odd number of them (rows of a quarter warp then start in different banks)
+    const int c4 = (cols + 3) / 4;
+    return (c4 | 1) * 4;
+}
+
+// WIDE: kernels of more than 64 taps, or pixel blocks whose input spans 4 GB or more: bounds by comparison and 64-bit
+// addresses instead of a tap mask per pixel and 32-bit offsets.
+template <bool WIDE>
+__global__ void __launch_bounds__(THREADS, 2) k_conv_gather(const ConvParams p, const GatherCfg cfg)
 {
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t s_bar;
+    __shared__ uint64_t s_full[NA], s_free[NA], s_wfull[NW_MAX], s_wfree[NW_MAX], s_acc, s_part;
     __shared__ uint32_t s_tmem;
-    __shared__ int s_row_n[BM], s_row_ih0[BM], s_row_iw0[BM];
+    __shared__ int s_abort;
+    // per pixel: WIDE image, first input row, first input column; else byte offset, tap mask
+    __shared__ __align__(16) uint32_t s_off[BM], s_mask[WIDE ? 1 : 2][BM + 4];   // (+ 4: the two words of a row in different banks)
+    __shared__ int s_col[BM];
 
     const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
-    const int r = blockIdx.y;  // pruning tile
-    const long long pix0 = static_cast<long long>(blockIdx.x) * BM;
+    const uint32_t rank = cluster_ctarank();
+    const uint32_t ring = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    const uint32_t w_ring = ring + NA * A_BYTES;
+    const uint32_t part = w_ring + cfg.w_stages * cfg.w_bytes;
+    volatile int* abort_flag = &s_abort;
 
-    const uint32_t a_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    const uint32_t b_base = a_base + A_BYTES;
-    const uint32_t bar = smem_u32(&s_bar);
+    // ---- this CTA's pixels, tiles and chunks ------------------------------------------------------
+    const uint32_t item = blockIdx.x / static_cast<uint32_t>(cfg.cs);
+    const uint32_t block = item / static_cast<uint32_t>(cfg.n_groups);
+    const int tile0 = static_cast<int>(item - block * static_cast<uint32_t>(cfg.n_groups)) * cfg.g;
+    const int g = min(cfg.g, p.n_tiles - tile0);
+    const long long pix0 = static_cast<long long>(block) * BM;
+    const int count = p.pixels - pix0 < BM ? static_cast<int>(p.pixels - pix0) : BM;
+    const int c_begin = static_cast<int>(rank) * cfg.chunks / cfg.cs, c_end = (static_cast<int>(rank) + 1) * cfg.chunks / cfg.cs;
+    const int units = (c_end - c_begin) * g;   // (chunk, tile) pairs, tiles innermost
+    const int hw = p.ho * p.wo;
+    const int n_first = static_cast<int>(pix0 / hw);
+    const int row0 = static_cast<int>(rank) * cfg.rps;   // first pixel row this CTA finishes
+    const int my_rows = max(0, min(cfg.rps, count - row0));
 
     // ---- set-up --------------------------------------------------------------------------------
-    if (warp == 0) tmem_alloc(smem_u32(&s_tmem), tmem_cols);
+    if (warp == 8) tmem_alloc(smem_u32(&s_tmem), cfg.tmem_cols);
     if (tid == 0) {
-        mbar_init(bar, 1);
-        mbar_fence_init();
-    }
-    {
-        const long long pix = pix0 + tid;
-        if (pix < p.pixels) {
-            const int hw = p.ho * p.wo;
-            const int n = static_cast<int>(pix / hw);
-            const int rem = static_cast<int>(pix - static_cast<long long>(n) * hw);
-            const int oh = rem / p.wo, ow = rem - oh * p.wo;
-            s_row_n[tid] = n;
-            s_row_ih0[tid] = oh * p.stride_h - p.pad_h;
-            s_row_iw0[tid] = ow * p.stride_w - p.pad_w;
-        } else {
-            s_row_n[tid] = -1;
-            s_row_ih0[tid] = 0;
-            s_row_iw0[tid] = 0;
+        for (int i = 0; i < NA; ++i) {
+            mbar_init(smem_u32(&s_full[i]), GATHER / 32);   // the gathering warps
+            mbar_init(smem_u32(&s_free[i]), 1);
         }
+        for (int i = 0; i < NW_MAX; ++i) {
+            mbar_init(smem_u32(&s_wfull[i]), 1);
+            mbar_init(smem_u32(&s_wfree[i]), 1);
+        }
+        mbar_init(smem_u32(&s_acc), 1);
+        mbar_init(smem_u32(&s_part), 1);
+        mbar_fence_init();
+        s_abort = 0;
+    }
+    if (tid < BM) {
+        uint32_t off = WIDE ? 0xFFFFFFFFu : 0u;
+        unsigned long long mask = 0;
+        int col = 0;
+        if (tid < count) {
+            const int rem0 = static_cast<int>(pix0 - static_cast<long long>(n_first) * hw) + tid;
+            const int dn = rem0 / hw, rem = rem0 - dn * hw;
+            const int oh = rem / p.wo, ow = rem - oh * p.wo;
+            const int ih0 = oh * p.stride_h - p.pad_h, iw0 = ow * p.stride_w - p.pad_w;
+            if (WIDE) {
+                off = static_cast<uint32_t>(n_first + dn);
+                mask = static_cast<uint32_t>(ih0);
+                col = iw0;
+            } else {
+                unsigned long long cols = 0;
+                for (int j = 0; j < p.kw; ++j) cols |= (static_cast<unsigned>(iw0 + j * p.dil_w) < static_cast<unsigned>(p.w) ? 1ull : 0ull) << j;
+                for (int i = 0; i < p.kh; ++i)
+                    if (static_cast<unsigned>(ih0 + i * p.dil_h) < static_cast<unsigned>(p.h)) mask |= cols << (i * p.kw);
+                // taps outside the image are never read: the offset may wrap as long as offset + tap does not
+                off = (static_cast<uint32_t>(dn * p.h + ih0) * static_cast<uint32_t>(p.w) + static_cast<uint32_t>(iw0)) *
+                                     static_cast<uint32_t>(p.c_in) * 4u;
+            }
+        }
+        s_off[tid] = off;
+        s_mask[0][tid] = static_cast<uint32_t>(mask);
+        if (!WIDE) s_mask[1][tid] = static_cast<uint32_t>(mask >> 32);
+        s_col[tid] = col;
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = s_tmem;
-    const uint32_t idesc = umma_idesc_tf32(BM, umma_n);
-    const uint64_t adesc0 = umma_desc_k_sw128(a_base, 1024);
-    const uint64_t bdesc0 = umma_desc_k_sw128(b_base, 1024);
-
-    const uint32_t* taps = p.taps + static_cast<size_t>(r) * p.kk_pad;
-    const int row_base = warp * 32;
-    uint32_t phase = 0;
-    bool failed = false;
-
-    // ---- main loop over chunks of 32 retained columns --------------------------------------------
-    for (int c0 = 0; c0 < p.kk_pad; c0 += NM_KCHUNK) {
-        // gather: lane = retained column c0 + lane
-        const uint32_t tap = taps[c0 + lane];
-        const bool tap_ok = tap != NM_TAP_PAD;
-        const int dh = static_cast<int>(tap >> 24) * p.dil_h;
-        const int dw = static_cast<int>((tap >> 16) & 0xFFu) * p.dil_w;
-        const int c = static_cast<int>(tap & 0xFFFFu);
-#pragma unroll 8
-        for (int i = 0; i < 32; ++i) {
-            const int row = row_base + i;
-            const int n = s_row_n[row];
-            const int ih = s_row_ih0[row] + dh, iw = s_row_iw0[row] + dw;
-            float v = 0.f;
-            if (tap_ok && n >= 0 && ih >= 0 && ih < p.h && iw >= 0 && iw < p.w)
-                // self-checking build: the tap table may only name taps and channels of this layer
-                NM_CHECKED(c < p.c_in && static_cast<int>(tap >> 24) < p.kh && static_cast<int>((tap >> 16) & 0xFFu) < p.kw && n < p.batch,
-                           p.status, 101, tap)
-                v = __ldg(p.x + ((static_cast<size_t>(n) * p.h + ih) * p.w + iw) * p.c_in + c);
-            const uint32_t dst = a_base + row * 128 + ((((lane >> 2) ^ (row & 7))) << 4) + ((lane & 3) << 2);
-            NM_CHECKED(dst >= a_base && dst + 4 <= a_base + A_BYTES, p.status, 102, dst - a_base)
-            asm volatile("st.shared.f32 [%0], %1;" ::"r"(dst), "f"(to_tf32(v)) : "memory");
+    const int nch = min(g * cfg.te, p.c_out - tile0 * p.tile_t);   // channels this CTA computes
+    const int passes = (cfg.te <= PASS) ? (g + PASS / cfg.te - 1) / (PASS / cfg.te) : g * ((cfg.te + PASS - 1) / PASS);
+    // channels of pass i: first one (relative to the CTA's), how many
+    auto pass_range = [&](int i, int& first, int& cols) {
+        if (cfg.te <= PASS) {
+            const int per = PASS / cfg.te * cfg.te;
+            first = i * per;
+            cols = min(per, nch - first);
+        } else {
+            const int pieces = (cfg.te + PASS - 1) / PASS, t = i / pieces, q = i - t * pieces;
+            first = t * cfg.te + q * PASS;
+            cols = min(min(PASS, cfg.te - q * PASS), nch - first);
         }
-        // weight chunk [umma_n rows x 32 columns]; rows past the tile or past c_out are zero
-        for (int idx = tid; idx < umma_n * 8; idx += 128) {
-            const int row = idx >> 3, ch = idx & 7;
-            const int o = r * p.tile_t + row;
-            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (row < p.tile_t && o < p.c_out)
-                v = __ldg(reinterpret_cast<const float4*>(p.wt + static_cast<size_t>(o) * p.kk_pad + c0) + ch);
-            const uint32_t dst = b_base + row * 128 + ((ch ^ (row & 7)) << 4);
-            asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
-                         : "memory");
-        }
-        fence_proxy_async();
-        __syncthreads();
-        if (warp == 0 && elect_one()) {
-            tc_fence_after();
-#pragma unroll
-            for (int kq = 0; kq < NM_KCHUNK / 8; ++kq)
-                umma_tf32_ss(tmem, adesc0 + 2 * kq, bdesc0 + 2 * kq, idesc, (c0 > 0 || kq > 0) ? 1u : 0u);
-            umma_commit(bar);
-        }
-        const bool ok = mbar_wait(bar, phase);
-        phase ^= 1;
-        if (__syncthreads_or(ok ? 0 : 1)) {
-            failed = true;
-            break;
-        }
+    };
+    // Partial sums of this CTA's rows in pass i, from every CTA of the cluster.  A CTA without rows neither expects nor waits: an
+    // expectation of nothing would complete its phase at once, and the next pass's the one after it, past a warp of this
+    // CTA that has yet to look at the first (a wait by parity would then never end).
+    auto expect_part = [&](int i) {
+        if (my_rows == 0) return;
+        int first, cols;
+        pass_range(i, first, cols);
+        mbar_arrive_expect_tx(smem_u32(&s_part), static_cast<uint32_t>(my_rows * pitch_of(cols) * 4 * cfg.cs));
+    };
+    if (cfg.cs > 1) {
+        // the barrier knows what to expect, and every CTA of the cluster has started, before any of them sends (waited for below)
+        if (tid == 0) expect_part(0);
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     }
+    pdl_launch_dependents();
 
-    // ---- epilogue ----------------------------------------------------------------------------------
-    if (!failed) {
-        tc_fence_after();
-        const long long pix = pix0 + row_base + lane;
-        float* yrow = p.y + static_cast<size_t>(pix < p.pixels ? pix : 0) * p.c_out;
-        const int o_base = r * p.tile_t;
-        const int n_valid = min(p.tile_t, p.c_out - o_base);
-        const bool vec_ok = (p.c_out % 4 == 0) && (p.tile_t % 4 == 0);
-        for (int col0 = 0; col0 < n_valid; col0 += 16) {
-            uint32_t v[16];
-            tmem_ld16(tmem + (static_cast<uint32_t>(row_base) << 16) + col0, v);
-            tmem_ld_wait();
-            if (pix < p.pixels) {
-                if (vec_ok && col0 + 16 <= n_valid) {
+    if (warp < 8) {
+        // =========================== gather ===========================
+        const int base_row = warp * RPW;
+        const uint4* offs = reinterpret_cast<const uint4*>(s_off + base_row);    // four rows per load, the same for all lanes
+        uint32_t all[2] = {0xFFFFFFFFu, 0xFFFFFFFFu};   // taps inside the image for every row of this warp
+        if (!WIDE)
+            for (int i = 0; i < RPW; ++i) {
+                all[0] &= s_mask[0][base_row + i];
+                all[1] &= s_mask[1][base_row + i];
+            }
+        const char* xb = reinterpret_cast<const char*>(p.x) + (WIDE ? 0 : static_cast<size_t>(n_first) * p.h * p.w * p.c_in * 4);
+        auto at = [xb](uint32_t bytes) { return __ldg(reinterpret_cast<const float*>(xb + bytes)); };
+        const uint32_t* taps = p.taps + static_cast<size_t>(tile0) * p.kk_pad + lane;
+        // taps of the next units to be read: a unit takes less time than its tap needs to arrive
+        int fc = c_begin, ft = 0;
+        auto fetch = [&]() {
+            const uint32_t t = fc < c_end ? __ldg(taps + static_cast<size_t>(ft) * p.kk_pad + fc * NM_KCHUNK) : NM_TAP_PAD;
+            if (++ft == g) { ft = 0; ++fc; }
+            return t;
+        };
+        uint32_t queue[TAPS_AHEAD];
 #pragma unroll
-                    for (int q = 0; q < 16; q += 4) {
-                        float4 o4;
-                        float* o = reinterpret_cast<float*>(&o4);
+        for (int i = 0; i < TAPS_AHEAD; ++i) queue[i] = fetch();
+        auto read = [&](float (&v)[RPW]) {
+            const uint32_t tap = queue[0];
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            float t = __uint_as_float(v[q + e]);
-                            if (p.bias) t += __ldg(p.bias + o_base + col0 + q + e);
-                            if (p.residual) t += __ldg(p.residual + (yrow - p.y) + o_base + col0 + q + e);
-                            o[e] = p.relu ? fmaxf(t, 0.f) : t;
-                        }
-                        *reinterpret_cast<float4*>(yrow + o_base + col0 + q) = o4;
+            for (int i = 0; i + 1 < TAPS_AHEAD; ++i) queue[i] = queue[i + 1];
+            queue[TAPS_AHEAD - 1] = fetch();
+            const bool ok = tap != NM_TAP_PAD;
+            const int ki = static_cast<int>(tap >> 24), kj = static_cast<int>((tap >> 16) & 0xFFu), c = static_cast<int>(tap & 0xFFFFu);
+            // self-checking build: the tap table may only name taps and channels of this layer
+            NM_CHECKED(!ok || (c < p.c_in && ki < p.kh && kj < p.kw), p.status, 101, tap) {}
+            if (WIDE) {
+                const int dh = ki * p.dil_h, dw = kj * p.dil_w;
+#pragma unroll
+                for (int i = 0; i < RPW; ++i) {
+                    const int n = static_cast<int>(s_off[base_row + i]);
+                    const int ih = static_cast<int>(s_mask[0][base_row + i]) + dh, iw = s_col[base_row + i] + dw;
+                    v[i] = 0.f;
+                    if (ok && n >= 0 && static_cast<unsigned>(ih) < static_cast<unsigned>(p.h) && static_cast<unsigned>(iw) < static_cast<unsigned>(p.w))
+                        v[i] = __ldg(p.x + ((static_cast<size_t>(n) * p.h + ih) * p.w + iw) * p.c_in + c);
+                }
+            } else {
+                const uint32_t delta = (static_cast<uint32_t>(ki * p.dil_h * p.w + kj * p.dil_w) * static_cast<uint32_t>(p.c_in) + static_cast<uint32_t>(c)) * 4u;
+                const int tap_no = ki * p.kw + kj, word = tap_no >> 5;
+                const uint32_t bit = ok ? 1u << (tap_no & 31) : 0u;
+                const uint4* masks = reinterpret_cast<const uint4*>(s_mask[0] + (ok ? word : 0) * (BM + 4) + base_row);
+                if (__all_sync(0xFFFFFFFFu, ((word ? all[1] : all[0]) & bit) != 0u)) {   // inside the image for all rows and columns of this warp
+#pragma unroll
+                    for (int i = 0; i < RPW; i += 4) {
+                        const uint4 o = offs[i / 4];
+                        v[i] = at(o.x + delta); v[i + 1] = at(o.y + delta); v[i + 2] = at(o.z + delta); v[i + 3] = at(o.w + delta);
                     }
                 } else {
 #pragma unroll
-                    for (int q = 0; q < 16; ++q) {
-                        if (col0 + q < n_valid) {
-                            float t = __uint_as_float(v[q]);
-                            if (p.bias) t += __ldg(p.bias + o_base + col0 + q);
-                            if (p.residual) t += __ldg(p.residual + (yrow - p.y) + o_base + col0 + q);
-                            yrow[o_base + col0 + q] = p.relu ? fmaxf(t, 0.f) : t;
+                    for (int i = 0; i < RPW; i += 4) {
+                        const uint4 o = offs[i / 4], m = masks[i / 4];
+                        v[i] = v[i + 1] = v[i + 2] = v[i + 3] = 0.f;
+                        if (m.x & bit) v[i] = at(o.x + delta);
+                        if (m.y & bit) v[i + 1] = at(o.y + delta);
+                        if (m.z & bit) v[i + 2] = at(o.z + delta);
+                        if (m.w & bit) v[i + 3] = at(o.w + delta);
+                    }
+                }
+            }
+        };
+        RingPos rp;
+        auto store = [&](const float (&v)[RPW]) {
+            const bool ready = !rp.wrapped || mbar_wait_lone(smem_u32(&s_free[rp.s]), rp.parity ^ 1u);
+            if (!__all_sync(0xFFFFFFFFu, ready)) { *abort_flag = 2; return false; }
+            const uint32_t dst = ring + rp.s * A_BYTES + base_row * 128 + ((lane & 3) << 2);
+#pragma unroll
+            for (int i = 0; i < RPW; ++i)
+                asm volatile("st.shared.f32 [%0], %1;" ::"r"(dst + i * 128 + (((lane >> 2) ^ (i & 7)) << 4)), "f"(to_tf32(v[i])) : "memory");
+            fence_proxy_async();
+            __syncwarp();
+            if (elect_one()) mbar_arrive(smem_u32(&s_full[rp.s]));
+            rp.advance(NA);
+            return true;
+        };
+        pdl_wait();
+        float va[RPW], vb[RPW];
+        if (units > 0) read(va);
+        if (units > 1) read(vb);
+        for (int u = 0; u < units; u += 2) {
+            if (aborted(abort_flag) || !store(va)) break;
+            if (u + 2 < units) read(va);
+            if (u + 1 >= units || !store(vb)) break;
+            if (u + 3 < units) read(vb);
+        }
+        __syncwarp();
+    } else if (warp == 8) {
+        // =========================== MMA issuer ===========================
+        if (elect_one()) {
+            const uint32_t idesc = umma_idesc_tf32(BM, cfg.n);
+            RingPos rp, rw;
+            bool ok = true;
+            for (int c = c_begin; c < c_end && ok; ++c) {
+                const int steps = min(NM_KCHUNK, p.kk - c * NM_KCHUNK) + 7 >> 3;   // K-steps of eight columns that hold any
+                for (int t = 0; t < g; ++t) {
+                    if (!mbar_wait_lone(smem_u32(&s_wfull[rw.s]), rw.parity) || !mbar_wait_lone(smem_u32(&s_full[rp.s]), rp.parity)) {
+                        *abort_flag = 3;
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    const uint64_t adesc = umma_desc_k_sw128(ring + rp.s * A_BYTES, 1024);
+                    const uint64_t bdesc = umma_desc_k_sw128(w_ring + rw.s * cfg.w_bytes, 1024);
+#pragma unroll
+                    for (int kq = 0; kq < 4; ++kq)
+                        if (kq < steps) umma_tf32_ss(tmem + t * cfg.n, adesc + 2 * kq, bdesc + 2 * kq, idesc, (c > c_begin || kq > 0) ? 1u : 0u);
+                    umma_commit(smem_u32(&s_free[rp.s]));
+                    umma_commit(smem_u32(&s_wfree[rw.s]));
+                    rp.advance(NA);
+                    rw.advance(cfg.w_stages);
+                }
+            }
+            umma_commit(smem_u32(&s_acc));
+        }
+        __syncwarp();
+    } else {
+        // =========================== weight producer ===========================
+        // The weights are no earlier kernel's output (a handle is complete when the call that built it returns): no pdl_wait.
+        if (elect_one()) {
+            const uint32_t bytes = static_cast<uint32_t>(cfg.n) * 128u;
+            RingPos rp;
+            int issued = 0;
+            bool ok = true;
+            for (int c = c_begin; c < c_end && ok; ++c)
+                for (int t = 0; t < g; ++t) {
+                    if (rp.wrapped && !mbar_wait_lone(smem_u32(&s_wfree[rp.s]), rp.parity ^ 1u)) { *abort_flag = 4; ok = false; break; }
+                    const uint32_t bar = smem_u32(&s_wfull[rp.s]);
+                    mbar_arrive_expect_tx(bar, bytes);
+                    bulk_load_1d(w_ring + rp.s * cfg.w_bytes, p.wt + (static_cast<size_t>(tile0 + t) * cfg.chunks + c) * cfg.n * NM_KCHUNK, bytes, bar);
+                    rp.advance(cfg.w_stages);
+                    ++issued;
+                }
+            if (aborted(abort_flag))   // loads already issued still target this CTA's shared memory: let them land (bounded)
+                for (int back = 0; back < cfg.w_stages && back < issued; ++back) {
+                    if (rp.s == 0) { rp.s = cfg.w_stages; rp.parity ^= 1u; }
+                    --rp.s;
+                    (void)mbar_wait_polls(smem_u32(&s_wfull[rp.s]), rp.parity, 1u << 16);
+                }
+        }
+        __syncwarp();
+    }
+
+    // ---- epilogue ----------------------------------------------------------------------------------
+    if (cfg.cs > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // every CTA of the cluster is running
+    if (warp < 8) {
+        const bool ok = aborted(abort_flag) || mbar_wait(smem_u32(&s_acc), 0);
+        if (!__all_sync(0xFFFFFFFFu, ok)) *abort_flag = 5;
+        tc_fence_after();
+    }
+    const int q = warp & 3, half = warp >> 2;
+    const int row = q * 32 + lane;
+    for (int i = 0; i < passes; ++i) {
+        int first, cols;
+        pass_range(i, first, cols);
+        const int pitch = pitch_of(cols);
+        if (warp < 8) {
+            // accumulators -> staging [row][channel of the pass] over the ring, which is idle now; sixteen columns at a time
+            const int t0 = first / cfg.te, j0 = first - t0 * cfg.te;
+            const int tiles = cfg.te <= PASS ? (cols + cfg.te - 1) / cfg.te : 1;
+            const int per = cfg.te <= PASS ? cfg.te : cols;   // channels of a tile in this pass
+            const int pieces = (per + 15) / 16;
+            for (int k = half; k < tiles * pieces; k += 2) {
+                const int t = k / pieces, jb = (k - t * pieces) * 16;
+                uint32_t v[16];
+                tmem_ld16(tmem + (static_cast<uint32_t>(q * 32) << 16) + (t0 + t) * cfg.n + j0 + jb, v);
+                tmem_ld_wait();
+                const uint32_t dst = ring + (row * pitch + t * cfg.te + jb) * 4;
+                const int valid = min(min(16, per - jb), cols - t * cfg.te - jb);   // the last tile may have fewer channels
+                if ((cfg.te & 3) == 0) {
+#pragma unroll
+                    for (int e = 0; e < 16; e += 4)
+                        if (e < valid)
+                            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst + e * 4), "r"(v[e]), "r"(v[e + 1]), "r"(v[e + 2]),
+                                         "r"(v[e + 3])
+                                         : "memory");
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 16; ++e)
+                        if (e < valid) asm volatile("st.shared.b32 [%0], %1;" ::"r"(dst + e * 4), "r"(v[e]) : "memory");
+                }
+            }
+            tc_fence_before();
+            if (cfg.cs > 1) fence_proxy_async();
+            asm volatile("bar.sync 1, %0;" ::"n"(GATHER) : "memory");
+            if (cfg.cs > 1) {
+                // a run of rows to every CTA of the cluster
+                if (warp < cfg.cs) {
+                    const int rows = min(cfg.rps, count - warp * cfg.rps);
+                    if (rows > 0 && elect_one())
+                        bulk_copy_cluster(mapa_shared(part + rank * cfg.rps * pitch * 4, static_cast<uint32_t>(warp)), ring + warp * cfg.rps * pitch * 4,
+                                          static_cast<uint32_t>(rows * pitch * 4), mapa_shared(smem_u32(&s_part), static_cast<uint32_t>(warp)));
+                }
+                // a multiple of the other waits' limit: a CTA that gave up on one of those has sent by then
+                const uint32_t bar = smem_u32(&s_part), par = static_cast<uint32_t>(i & 1);
+                const bool landed = my_rows == 0 || mbar_wait_cluster(bar, par) || mbar_wait_cluster(bar, par) || mbar_wait_cluster(bar, par);
+                if (!__all_sync(0xFFFFFFFFu, landed)) *abort_flag = 6;
+            }
+            if (!aborted(abort_flag)) {
+                const uint32_t src = cfg.cs > 1 ? part : ring;
+                const uint32_t src_step = static_cast<uint32_t>(cfg.rps * pitch * 4);
+                const int o0 = tile0 * p.tile_t + first;
+                const long long pix = pix0 + row0;
+                if (((p.c_out | o0 | cols) & 3) == 0) {
+                    const int c4 = cols >> 2;
+                    for (int f = tid; f < my_rows * c4; f += GATHER) {
+                        const int r = f / c4, c = f - r * c4;
+                        const size_t at = static_cast<size_t>(pix + r) * p.c_out + o0 + c * 4;
+                        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+                        for (int k = 0; k < cfg.cs; ++k) {
+                            float4 a;
+                            asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w)
+                                         : "r"(src + k * src_step + (r * pitch + c * 4) * 4) : "memory");
+                            nm_add4(s, a);
                         }
+                        if (p.bias) nm_add4(s, __ldg(reinterpret_cast<const float4*>(p.bias + o0) + c));
+                        if (p.residual) nm_add4(s, __ldg(reinterpret_cast<const float4*>(p.residual + at)));
+                        if (p.relu) { s.x = fmaxf(s.x, 0.f); s.y = fmaxf(s.y, 0.f); s.z = fmaxf(s.z, 0.f); s.w = fmaxf(s.w, 0.f); }
+                        *reinterpret_cast<float4*>(p.y + at) = s;
+                    }
+                } else {
+                    for (int f = tid; f < my_rows * cols; f += GATHER) {
+                        const int r = f / cols, c = f - r * cols;
+                        const size_t at = static_cast<size_t>(pix + r) * p.c_out + o0 + c;
+                        float s = 0.f;
+                        for (int k = 0; k < cfg.cs; ++k) {
+                            float a;
+                            asm volatile("ld.shared.f32 %0, [%1];" : "=f"(a) : "r"(src + k * src_step + (r * pitch + c) * 4) : "memory");
+                            s += a;
+                        }
+                        if (p.bias) s += __ldg(p.bias + o0 + c);
+                        if (p.residual) s += __ldg(p.residual + at);
+                        p.y[at] = p.relu ? fmaxf(s, 0.f) : s;
                     }
                 }
             }
         }
-    } else if (tid == 0) {
-        atomicExch(p.status + 0, static_cast<int>(NM_ERR_TIMEOUT));
-        atomicExch(p.status + 1, 1);  // where: variant 1 main loop
-        atomicExch(p.status + 2, static_cast<int>(blockIdx.x));
+        if (cfg.cs > 1) {
+            // nobody sends the next pass's sums (or leaves, its copies unread) before every CTA has used this one's
+            if (tid == 0 && i + 1 < passes) expect_part(i + 1);
+            asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+            asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        } else if (warp < 8 && i + 1 < passes) {
+            asm volatile("bar.sync 1, %0;" ::"n"(GATHER) : "memory");   // the staging rows are free again
+        }
     }
 
     // ---- teardown ------------------------------------------------------------------------------------
     tc_fence_before();
     __syncthreads();
-    if (warp == 0) tmem_dealloc(tmem, tmem_cols);
+    if (tid == 0 && s_abort != 0) {
+        atomicExch(p.status + 0, static_cast<int>(NM_ERR_TIMEOUT));
+        atomicExch(p.status + 1, s_abort);
+        atomicExch(p.status + 2, static_cast<int>(blockIdx.x));
+    }
+    if (warp == 8) tmem_dealloc(tmem, cfg.tmem_cols);
+}
+
+int sm_count()
+{
+    static const int n = [] {
+        int dev = 0, v = 0;
+        if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0)
+            return v;
+        return 148;
+    }();
+    return n;
 }
 
 }  // namespace
@@ -182,28 +457,67 @@ namespace nmhost {
 
 nm_status_t launch_conv_gather(const ConvParams& p, cudaStream_t st)
 {
-    const int umma_n = p.tile_t <= 16 ? 16 : ((p.tile_t + 15) / 16) * 16;
-    if (umma_n > 256) return fail(NM_ERR_UNSUPPORTED, "nm_conv2d: tile_t %d exceeds 256", p.tile_t);
-    int tmem_cols = 32;
-    while (tmem_cols < umma_n) tmem_cols <<= 1;
-    // shared memory: alignment slack + A tile + B tile; padded so that the CTAs resident on one
-    // SM never ask for more than the 512 TMEM columns it has
-    size_t smem = 1024 + A_BYTES + static_cast<size_t>(umma_n) * 128;
-    const int max_ctas = 512 / tmem_cols;
-    const size_t floor_bytes = (227 * 1024) / (max_ctas + 1) + 1;
-    if (max_ctas < 16 && smem < floor_bytes) smem = floor_bytes;
-
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_conv_gather, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             static_cast<int>(smem));
-        if (e != cudaSuccess) return fail(NM_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
+    GatherCfg cfg = {};
+    cfg.te = std::min(p.tile_t, p.c_out);
+    cfg.n = gather_width(p.tile_t, p.c_out);
+    if (cfg.n > 256) return fail(NM_ERR_UNSUPPORTED, "nm_conv2d: tile_t %d exceeds 256", p.tile_t);
+    cfg.chunks = p.kk_pad / NM_KCHUNK;
+    const long long blocks = (p.pixels + BM - 1) / BM;
+    // Tiles per CTA: as many as 256 accumulator columns hold (128 where the chunks are split): they share the activations' lines
+    // in L1, a chunk's 32 KB from L2 otherwise cost twice a tile's instructions.  Chunks are split over a cluster until there
+    // are two CTAs per SM, and only where that does not give every SM one are the tiles spread over more CTAs.
+    const long long sms = sm_count();
+    cfg.g = std::min(p.n_tiles, 256 / cfg.n);
+    auto groups = [&] { return (p.n_tiles + cfg.g - 1) / cfg.g; };
+    cfg.cs = 1;
+    if (blocks * groups() < 2 * sms && cfg.chunks >= 4) {
+        cfg.g = std::min(cfg.g, std::max(1, 128 / cfg.n));
+        while (cfg.cs < 8 && blocks * groups() * cfg.cs < 2 * sms && cfg.chunks >= 4 * cfg.cs) cfg.cs *= 2;
     }
-    const long long tiles_m = (p.pixels + BM - 1) / BM;
-    if (tiles_m > 0x7FFFFFFFll) return fail(NM_ERR_UNSUPPORTED, "nm_conv2d: too many output pixels");
-    const dim3 grid(static_cast<unsigned>(tiles_m), p.n_tiles);
-    k_conv_gather<<<grid, 128, smem, st>>>(p, umma_n, tmem_cols);
+    while (cfg.g > 1 && blocks * groups() * cfg.cs < sms) cfg.g = (cfg.g + 1) / 2;
+    cfg.n_groups = groups();
+    cfg.rps = BM / cfg.cs;
+    cfg.tmem_cols = 32;
+    while (cfg.tmem_cols < cfg.g * cfg.n) cfg.tmem_cols <<= 1;
+    const long long grid = blocks * cfg.n_groups * cfg.cs;
+    if (grid > 0x7FFFFFFFll) return fail(NM_ERR_UNSUPPORTED, "nm_conv2d: too many output pixels");
+    cfg.w_bytes = cfg.n * 128;   // a multiple of 2 KB
+    // A weight chunk takes about 1 us to arrive from L2, several (chunk, tile) units' time: its ring is deeper than the operands'.
+    // The staging of a pass (128 rows of at most PASS + 4 floats) lies over the rings, with a cluster the received sums take
+    // as much again.
+    const int stage_out = BM * (PASS + 4) * 4;
+    cfg.w_stages = cfg.n <= 32 ? 6 : cfg.n <= 64 ? 4 : cfg.n <= 128 && cfg.cs == 1 ? 3 : 2;
+    size_t smem = 1024 + static_cast<size_t>(NA) * A_BYTES + static_cast<size_t>(cfg.w_stages) * cfg.w_bytes + (cfg.cs > 1 ? stage_out : 0);
+    // No more CTAs on an SM than its tensor memory holds; a cluster's CTAs, which wait for one another, take at least their
+    // columns' share of the shared memory (see NM_EXCLUSIVE_SMEM).
+    const size_t share = cfg.cs > 1 ? static_cast<size_t>(cfg.tmem_cols) * (228 * 1024 / 512)
+                                    : std::min<size_t>(static_cast<size_t>(cfg.tmem_cols) * (222 * 1024 / 512), 111 * 1024);
+    smem = std::max(std::max(smem, share), NM_BESIDE_EXCLUSIVE);
+
+    const long long images = BM / (static_cast<long long>(p.ho) * p.wo) + 2;   // images a pixel block can touch
+    const bool wide = p.kh * p.kw > 64 || images * p.h * p.w * p.c_in * 4 >= (1ll << 32);
+    const auto kernel = wide ? k_conv_gather<true> : k_conv_gather<false>;
+    cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), smem);
+    if (e != cudaSuccess) return fail(NM_ERR_CUDA, "cudaFuncSetAttribute (variant 1): %s", cudaGetErrorString(e));
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(static_cast<unsigned>(grid));
+    lc.blockDim = dim3(THREADS);
+    lc.dynamicSmemBytes = smem;
+    lc.stream = st;
+    cudaLaunchAttribute attr[3];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = static_cast<unsigned>(cfg.cs);
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;   // the rest of two CTAs' SM is L1
+    attr[1].val.sharedMemCarveout = static_cast<unsigned>(std::min<size_t>(100, (2 * (smem + 3072) * 100 + 228 * 1024 - 1) / (228 * 1024)));
+    attr[2].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[2].val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = attr;
+    lc.numAttrs = pdl_enabled() ? 3 : 2;
+    e = cudaLaunchKernelEx(&lc, kernel, p, cfg);
     count_launch(1);
-    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return fail(NM_ERR_CUDA, "nm_conv2d launch (variant 1): %s", cudaGetErrorString(e));
     return NM_OK;
 }

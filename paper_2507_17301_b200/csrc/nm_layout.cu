@@ -91,7 +91,7 @@ struct LayoutArgs {
     int c_out, k, kk, kk_pad, tile_t, n_tiles, n_keep, m_group, c_in, kh, kw;
     float* values;
     uint16_t* indices;           // import: the handle's copy of idx
-    float* wt;
+    float* wt; int wt_rows;
     uint32_t* taps;
     float* wt2; uint8_t* rel2; int v2_s, v2_kc, v2_chunks;         // NULL: not built
     float* wx; int wx_rows;
@@ -108,9 +108,7 @@ __global__ void k_build_layouts(const LayoutArgs a)
     if (j >= a.kk_pad) return;
     const int r = o / a.tile_t;
     const bool first_row = o == r * a.tile_t;   // this thread also writes what the tile's rows share
-    const size_t wt_at = static_cast<size_t>(o) * a.kk_pad + j;
     if (j >= a.kk) {
-        a.wt[wt_at] = 0.f;
         if (first_row) a.taps[static_cast<size_t>(r) * a.kk_pad + j] = NM_TAP_PAD;
         return;
     }
@@ -127,7 +125,11 @@ __global__ void k_build_layouts(const LayoutArgs a)
     const float v = a.import ? a.src[static_cast<size_t>(o) * a.kk + j] : a.src[static_cast<size_t>(o) * a.k + col];
     const float t = nmk::to_tf32(v);
     a.values[static_cast<size_t>(o) * a.kk + j] = v;
-    a.wt[wt_at] = t;
+    {
+        // gather layout: per (tile, chunk of 32 retained columns) the shared-memory image of the tile's rows, swizzled like wx
+        const int rr = o - r * a.tile_t, jj = j & (NM_KCHUNK - 1);
+        a.wt[((static_cast<size_t>(r) * (a.kk_pad / NM_KCHUNK) + j / NM_KCHUNK) * a.wt_rows + rr) * NM_KCHUNK + ((((jj >> 2) ^ (rr & 7)) << 2) | (jj & 3))] = t;
+    }
     if (first_row) {
         const int c = col % a.c_in, tap = col / a.c_in;
         a.taps[static_cast<size_t>(r) * a.kk_pad + j] =
@@ -257,11 +259,11 @@ nm_status_t alloc_handle_memory(nm_weights* h, const char* who)
     const size_t chunks3 = h->sel_s ? static_cast<size_t>(h->k / h->sel_s) : 0;
     const size_t at_values = place(h->c_out * kk1 * sizeof(float));
     const size_t at_indices = place(h->n_tiles * kk1 * sizeof(uint16_t));
-    const size_t at_wt = place(static_cast<size_t>(h->c_out) * h->kk_pad * sizeof(float));
     const size_t at_taps = place(static_cast<size_t>(h->n_tiles) * h->kk_pad * sizeof(uint32_t));
     h->zero_from = total;   // from here on the creating call clears the block: status, sums, layouts with padding
     const size_t at_status = place(4 * sizeof(int));
     const size_t at_mass = place(sizeof(Readback));
+    const size_t at_wt = place(static_cast<size_t>(h->n_tiles) * gather_width(h->tile_t, h->c_out) * h->kk_pad * sizeof(float));
     const size_t at_wt2 = place(h->v2_ok ? h->c_out * pitch2 * sizeof(float) : 0);
     const size_t at_rel2 = place(h->v2_ok ? h->n_tiles * pitch2 : 0);
     const size_t at_wx = place(h->wx_rows ? static_cast<size_t>((h->k + 31) / 32) * h->wx_rows * 128 : 0);
@@ -303,6 +305,7 @@ nm_status_t build_layouts(nm_weights* h, const float* src, const uint16_t* idx, 
     a.c_out = h->c_out; a.k = h->k; a.kk = h->kk; a.kk_pad = h->kk_pad; a.tile_t = h->tile_t; a.n_tiles = h->n_tiles;
     a.n_keep = h->n_keep; a.m_group = h->m_group; a.c_in = h->c_in; a.kh = h->kh; a.kw = h->kw;
     a.values = h->values; a.indices = h->indices; a.wt = h->wt; a.taps = h->taps;
+    a.wt_rows = gather_width(h->tile_t, h->c_out);
     a.wt2 = h->wt2; a.rel2 = h->rel2; a.v2_s = h->v2_s; a.v2_kc = h->v2_kc; a.v2_chunks = h->v2_chunks;
     a.wx = h->wx; a.wx_rows = h->wx_rows;
     a.w3 = h->w3; a.sel3 = h->sel3; a.sel_s = h->sel_s; a.sel_kc = h->sel_kc; a.sel_mw = h->sel_mw;
