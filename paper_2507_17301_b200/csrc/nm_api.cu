@@ -126,10 +126,9 @@ nm_status_t run_plan(const ConvParams& p, const nm_plan_t* plan, cudaStream_t st
     const int variant = plan ? plan->variant : 0;
     switch (variant) {
         case 0:
-            if (nmhost::stream_plan_ok(p, nullptr)) return nmhost::launch_conv_stream(p, nullptr, st);
+            // (all of these round activations to nearest and never read a pruned column)
+            if (nmhost::stream_plan_ok(p, nullptr) && !nmhost::stream_leaves_sms_idle(p)) return nmhost::launch_conv_stream(p, nullptr, st);
             if (nmhost::planes_plan_ok(p, nullptr)) return nmhost::launch_conv_planes(p, nullptr, st);
-            if (p.c_in % 32 != 0 && nmhost::rowrun_plan_ok(p, nullptr)) return nmhost::launch_conv_rowrun(p, nullptr, st);
-            if (nmhost::slab_plan_ok(p, nullptr)) return nmhost::launch_conv_slab(p, nullptr, st);
             return nmhost::launch_conv_gather(p, st);
         case 1:
             return nmhost::launch_conv_gather(p, st);

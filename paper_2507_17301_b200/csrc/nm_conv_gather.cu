@@ -59,6 +59,21 @@ __device__ __forceinline__ void bulk_copy_cluster(uint32_t dst, uint32_t src, ui
                  "r"(bytes), "r"(bar)
                  : "memory");
 }
+// *p where `on` is non-zero, else 0; a predicated load (written as a conditional it becomes a branch per pixel row).
+__device__ __forceinline__ float load_if(const float* p, uint32_t on)
+{
+    float v;
+    asm volatile(
+        "{\n\t"
+        ".reg .pred q;\n\t"
+        "setp.ne.u32 q, %2, 0;\n\t"
+        "mov.f32 %0, 0f00000000;\n\t"
+        "@q ld.global.nc.f32 %0, [%1];\n\t"
+        "}\n"
+        : "=f"(v)
+        : "l"(p), "r"(on));
+    return v;
+}
 __device__ __forceinline__ int pitch_of(int cols)
 {
     // floats per staged row: whole 16-byte pieces, an odd number of them (rows of a quarter warp then start in different banks)
@@ -189,7 +204,7 @@ __global__ void __launch_bounds__(THREADS, 2) k_conv_gather(const ConvParams p, 
                 all[1] &= s_mask[1][base_row + i];
             }
         const char* xb = reinterpret_cast<const char*>(p.x) + (WIDE ? 0 : static_cast<size_t>(n_first) * p.h * p.w * p.c_in * 4);
-        auto at = [xb](uint32_t bytes) { return __ldg(reinterpret_cast<const float*>(xb + bytes)); };
+        auto at = [xb](uint32_t bytes) { return reinterpret_cast<const float*>(xb + bytes); };
         const uint32_t* taps = p.taps + static_cast<size_t>(tile0) * p.kk_pad + lane;
         // taps of the next units to be read: a unit takes less time than its tap needs to arrive
         int fc = c_begin, ft = 0;
@@ -216,9 +231,8 @@ __global__ void __launch_bounds__(THREADS, 2) k_conv_gather(const ConvParams p, 
                 for (int i = 0; i < RPW; ++i) {
                     const int n = static_cast<int>(s_off[base_row + i]);
                     const int ih = static_cast<int>(s_mask[0][base_row + i]) + dh, iw = s_col[base_row + i] + dw;
-                    v[i] = 0.f;
-                    if (ok && n >= 0 && static_cast<unsigned>(ih) < static_cast<unsigned>(p.h) && static_cast<unsigned>(iw) < static_cast<unsigned>(p.w))
-                        v[i] = __ldg(p.x + ((static_cast<size_t>(n) * p.h + ih) * p.w + iw) * p.c_in + c);
+                    const bool in = ok && n >= 0 && static_cast<unsigned>(ih) < static_cast<unsigned>(p.h) && static_cast<unsigned>(iw) < static_cast<unsigned>(p.w);
+                    v[i] = load_if(p.x + ((static_cast<size_t>(n) * p.h + ih) * p.w + iw) * p.c_in + c, in ? 1u : 0u);
                 }
             } else {
                 const uint32_t delta = (static_cast<uint32_t>(ki * p.dil_h * p.w + kj * p.dil_w) * static_cast<uint32_t>(p.c_in) + static_cast<uint32_t>(c)) * 4u;
@@ -229,17 +243,16 @@ __global__ void __launch_bounds__(THREADS, 2) k_conv_gather(const ConvParams p, 
 #pragma unroll
                     for (int i = 0; i < RPW; i += 4) {
                         const uint4 o = offs[i / 4];
-                        v[i] = at(o.x + delta); v[i + 1] = at(o.y + delta); v[i + 2] = at(o.z + delta); v[i + 3] = at(o.w + delta);
+                        v[i] = __ldg(at(o.x + delta)); v[i + 1] = __ldg(at(o.y + delta)); v[i + 2] = __ldg(at(o.z + delta)); v[i + 3] = __ldg(at(o.w + delta));
                     }
                 } else {
 #pragma unroll
                     for (int i = 0; i < RPW; i += 4) {
                         const uint4 o = offs[i / 4], m = masks[i / 4];
-                        v[i] = v[i + 1] = v[i + 2] = v[i + 3] = 0.f;
-                        if (m.x & bit) v[i] = at(o.x + delta);
-                        if (m.y & bit) v[i + 1] = at(o.y + delta);
-                        if (m.z & bit) v[i + 2] = at(o.z + delta);
-                        if (m.w & bit) v[i + 3] = at(o.w + delta);
+                        v[i] = load_if(at(o.x + delta), m.x & bit);
+                        v[i + 1] = load_if(at(o.y + delta), m.y & bit);
+                        v[i + 2] = load_if(at(o.z + delta), m.z & bit);
+                        v[i + 3] = load_if(at(o.w + delta), m.w & bit);
                     }
                 }
             }
@@ -248,10 +261,10 @@ __global__ void __launch_bounds__(THREADS, 2) k_conv_gather(const ConvParams p, 
         auto store = [&](const float (&v)[RPW]) {
             const bool ready = !rp.wrapped || mbar_wait_lone(smem_u32(&s_free[rp.s]), rp.parity ^ 1u);
             if (!__all_sync(0xFFFFFFFFu, ready)) { *abort_flag = 2; return false; }
-            const uint32_t dst = ring + rp.s * A_BYTES + base_row * 128 + ((lane & 3) << 2);
+            const uint32_t dst = ring + rp.s * A_BYTES + base_row * 128 + lane * 4;   // 16-byte pieces XOR-ed with the row: bits 4-6
 #pragma unroll
             for (int i = 0; i < RPW; ++i)
-                asm volatile("st.shared.f32 [%0], %1;" ::"r"(dst + i * 128 + (((lane >> 2) ^ (i & 7)) << 4)), "f"(to_tf32(v[i])) : "memory");
+                asm volatile("st.shared.f32 [%0], %1;" ::"r"((dst ^ ((i & 7) << 4)) + i * 128), "f"(to_tf32(v[i])) : "memory");
             fence_proxy_async();
             __syncwarp();
             if (elect_one()) mbar_arrive(smem_u32(&s_full[rp.s]));
@@ -463,19 +476,22 @@ nm_status_t launch_conv_gather(const ConvParams& p, cudaStream_t st)
     if (cfg.n > 256) return fail(NM_ERR_UNSUPPORTED, "nm_conv2d: tile_t %d exceeds 256", p.tile_t);
     cfg.chunks = p.kk_pad / NM_KCHUNK;
     const long long blocks = (p.pixels + BM - 1) / BM;
-    // Tiles per CTA: as many as 256 accumulator columns hold (128 where the chunks are split): they share the activations' lines
-    // in L1, a chunk's 32 KB from L2 otherwise cost twice a tile's instructions.  Chunks are split over a cluster until there
-    // are two CTAs per SM, and only where that does not give every SM one are the tiles spread over more CTAs.
+    // Tiles per CTA and ranges of the chunks, by an estimate of the time: a (chunk, tile) unit takes a CTA about 0.3 us plus its
+    // share of bringing the chunk's 32 KB in from L2, which the tiles of a CTA share through L1; two CTAs fit an SM (in
+    // clusters not on every last one), and one that has it to itself is nearly twice as fast; a launch has a few us of
+    // its own.  At most 256 accumulator columns per CTA, 128 where CTAs of a cluster wait for one another.
     const long long sms = sm_count();
-    cfg.g = std::min(p.n_tiles, 256 / cfg.n);
-    auto groups = [&] { return (p.n_tiles + cfg.g - 1) / cfg.g; };
-    cfg.cs = 1;
-    if (blocks * groups() < 2 * sms && cfg.chunks >= 4) {
-        cfg.g = std::min(cfg.g, std::max(1, 128 / cfg.n));
-        while (cfg.cs < 8 && blocks * groups() * cfg.cs < 2 * sms && cfg.chunks >= 4 * cfg.cs) cfg.cs *= 2;
-    }
-    while (cfg.g > 1 && blocks * groups() * cfg.cs < sms) cfg.g = (cfg.g + 1) / 2;
-    cfg.n_groups = groups();
+    double best = 1e30;
+    for (int cs = 1; cs <= 8 && (cs == 1 || cfg.chunks >= 2 * cs); cs *= 2)
+        for (int g = std::min(p.n_tiles, std::max(1, (cs > 1 ? 128 : 256) / cfg.n));; g = (g + 1) / 2) {
+            const long long ctas = blocks * ((p.n_tiles + g - 1) / g) * cs;
+            const long long waves = (ctas + 2 * sms - (cs > 1 ? 33 : 1)) / (2 * sms - (cs > 1 ? 32 : 0));
+            const double unit = (0.3 + 0.3 / g) * (ctas <= sms ? 0.6 : 1.0);
+            const double t = waves * (((cfg.chunks + cs - 1) / cs) * g * unit + (cs > 1 ? 4.0 : 3.0));
+            if (t < best * 0.98) { best = t; cfg.g = g; cfg.cs = cs; }
+            if (g == 1) break;
+        }
+    cfg.n_groups = (p.n_tiles + cfg.g - 1) / cfg.g;
     cfg.rps = BM / cfg.cs;
     cfg.tmem_cols = 32;
     while (cfg.tmem_cols < cfg.g * cfg.n) cfg.tmem_cols <<= 1;

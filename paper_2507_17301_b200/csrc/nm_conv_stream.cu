@@ -527,6 +527,14 @@ bool stream_plan_ok(const ConvParams& p, const nm_plan_t* plan)
     return make_cfg(p, plan, &cfg);
 }
 
+bool stream_leaves_sms_idle(const ConvParams& p)
+{
+    // Work items on less than half of the SMs, sixteen chunks or more each.  3x3 448 -> 160 at 8x14 (7 pixel blocks, 3:4):
+    // 52.7 us here, 29 us in the gather kernel, which splits the chunks over a cluster; 1x1 352 -> 704 at 34x7 (six chunks): 7.2, 7.7.
+    StreamCfg cfg;
+    return make_cfg(p, nullptr, &cfg) && 2 * cfg.n_work < sm_count() && p.v2_chunks >= 16;
+}
+
 nm_status_t launch_conv_stream(const ConvParams& p, const nm_plan_t* plan, cudaStream_t st)
 {
     StreamCfg cfg;

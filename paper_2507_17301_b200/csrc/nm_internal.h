@@ -194,6 +194,7 @@ nm_status_t launch_conv_pair(const ConvParams& p, const nm_plan_t* plan, cudaStr
 
 // nm_conv_stream.cu — variant 3
 bool stream_plan_ok(const ConvParams& p, const nm_plan_t* plan);
+bool stream_leaves_sms_idle(const ConvParams& p);   // few work items, each with a long reduction: the gather kernel splits it
 nm_status_t launch_conv_stream(const ConvParams& p, const nm_plan_t* plan, cudaStream_t st);
 
 // nm_conv_select.cu — variant 8
