@@ -129,6 +129,11 @@ nm_status_t run_plan(const ConvParams& p, const nm_plan_t* plan, cudaStream_t st
             // (all of these round activations to nearest and never read a pruned column)
             if (nmhost::stream_plan_ok(p, nullptr) && !nmhost::stream_leaves_sms_idle(p)) return nmhost::launch_conv_stream(p, nullptr, st);
             if (nmhost::planes_plan_ok(p, nullptr)) return nmhost::launch_conv_planes(p, nullptr, st);
+            // Channel counts that are no multiple of 32: runs of rows where there is enough work for their set-up.  Units of a pixel
+            // block, tile and chunk, and us against the gather's: 2352 (8x112x112, 16->32) 18.4 / 20.6, 1568 (32x56x56, 8->64 by
+            // 2) 14.4 / 16.4; 1176 (4x56x56, 24->96) 10.1 / 8.3, 784 (2x112x112, 5->32, 7x7 by 2) 6.9 / 5.5.
+            if (p.c_in % 32 != 0 && (p.pixels + 127) / 128 * p.n_tiles * (p.kk_pad / NM_KCHUNK) >= 1400 && nmhost::rowrun_plan_ok(p, nullptr))
+                return nmhost::launch_conv_rowrun(p, nullptr, st);
             return nmhost::launch_conv_gather(p, st);
         case 1:
             return nmhost::launch_conv_gather(p, st);

@@ -1,22 +1,23 @@
 // Variant 1: direct-gather sparse implicit GEMM (any shape).
 //
-// A CTA owns 128 output pixels and G pruning tiles (each with its own kept set).  For every chunk of 32 retained columns
-// and every tile, eight warps gather the activations
+// A CTA owns 128 output pixels and one pruning tile.  For every chunk of 32 retained columns eight warps gather the
+// activations
 //     a[p][j] = x[n][oh*s - pad + kh_j*dil][ow*s - pad + kw_j*dil][c_j]      (zero outside the image)
 // straight from NHWC global memory (lane = retained column j, so a warp reads one pixel's retained channels:
-// neighbouring addresses; the tiles of a CTA follow one another on the same chunk and share its lines in L1), round them to
-// TF32 and store them in the 128-byte-swizzled K-major layout tcgen05 reads.  One thread fetches the tile's weight
-// chunk (stored as the shared-memory image) with a bulk copy, one issues four 128 x N x 8 TF32 MMAs per chunk and tile into the
-// tile's accumulator columns in tensor memory.  This is Algorithm 1 with the vector register replaced by a 128-pixel
-// operand tile and the T accumulators by T TMEM columns; the gather is the fused im2col + packing of Sec. 3.2 without its
-// buffer.
+// neighbouring addresses), round them to TF32 and store them in the 128-byte-swizzled K-major layout tcgen05 reads.  One
+// thread fetches the weight chunk (stored as the shared-memory image) with a bulk copy, one issues four 128 x N x 8 TF32
+// MMAs per chunk.  This is Algorithm 1 with the vector register replaced by a 128-pixel operand tile and the T
+// accumulators by T TMEM columns; the gather is the fused im2col + packing of Sec. 3.2 without its buffer.
 //
-// It is the library's choice for every shape the TMA-fed kernels do not take (channel counts that are no multiple of
-// 32, small or odd tile widths, small inputs), so it has to be good at all of them.  What bounds it is the
-// gather's instruction stream, about 6.5 per warp and pixel row: two chunks are kept in flight in registers, the ring of
-// operand slots decouples the gathering warps from the MMAs, two CTAs share an SM, and where there are fewer pixel blocks
-// and tiles than SMs the chunks are split over the CTAs of a thread-block cluster (partial sums move as bulk copies
-// between their shared memories and are added in the order of the ranges).  XXX
+// It takes every shape the TMA-fed kernels do not (channel counts that are no multiple of 32, small or odd tile widths,
+// small inputs), so it has to be good at all of them.  What bounds it is the gather's instruction stream: a chunk
+// costs a CTA 0.70 us alone on its SM and 0.95 us beside a second one, where issue slots are 60 % busy; more operand slots (4
+// for 2), more gathering warps (16 for 8) and several tiles per CTA (which share the chunk's lines in L1) changed
+// neither figure.  Two chunks are kept in flight in registers, the operand slots decouple the gathering warps from
+// the MMAs, and where there are far fewer pixel blocks and tiles than SMs the chunks are split over the CTAs of a thread-block
+// cluster (partial sums move as bulk copies between their shared memories and are added in the order of the ranges).
+// Before the pipelining and the split, and now: 3978 pixels, 242 chunks, one tile 295 -> 37 us; 6930 pixels, 54 chunks, 8 tiles of
+// 64 152 -> 68 us.
 //
 //   warps 0-7  gather, then epilogue: TMEM -> staging in shared memory -> bias, shortcut, ReLU, coalesced NHWC stores
 //   warp 8     MMA issuer, tensor memory      warp 9  weight producer
@@ -40,9 +41,7 @@ constexpr int NW_MAX = 8;                     // weight slots
 constexpr int PASS = 64;                      // output channels staged at a time
 
 struct GatherCfg {
-    int n;            // MMA width = accumulator columns per tile
-    int te;           // channels of a tile that can exist (the tile width, or c_out if that is smaller)
-    int g, n_groups;  // tiles per CTA, CTAs along the tiles
+    int n;            // MMA width = accumulator columns
     int cs;           // CTAs per cluster = ranges of the chunks
     int chunks;
     int w_stages, w_bytes;
@@ -103,13 +102,12 @@ __global__ void __launch_bounds__(THREADS, 2) k_conv_gather(const ConvParams p, 
 
     // ---- this CTA's pixels, tiles and chunks ------------------------------------------------------
     const uint32_t item = blockIdx.x / static_cast<uint32_t>(cfg.cs);
-    const uint32_t block = item / static_cast<uint32_t>(cfg.n_groups);
-    const int tile0 = static_cast<int>(item - block * static_cast<uint32_t>(cfg.n_groups)) * cfg.g;
-    const int g = min(cfg.g, p.n_tiles - tile0);
+    const uint32_t block = item / static_cast<uint32_t>(p.n_tiles);
+    const int tile = static_cast<int>(item - block * static_cast<uint32_t>(p.n_tiles));
     const long long pix0 = static_cast<long long>(block) * BM;
     const int count = p.pixels - pix0 < BM ? static_cast<int>(p.pixels - pix0) : BM;
     const int c_begin = static_cast<int>(rank) * cfg.chunks / cfg.cs, c_end = (static_cast<int>(rank) + 1) * cfg.chunks / cfg.cs;
-    const int units = (c_end - c_begin) * g;   // (chunk, tile) pairs, tiles innermost
+    const int my_chunks = c_end - c_begin;
     const int hw = p.ho * p.wo;
     const int n_first = static_cast<int>(pix0 / hw);
     const int row0 = static_cast<int>(rank) * cfg.rps;   // first pixel row this CTA finishes
@@ -163,28 +161,15 @@ __global__ void __launch_bounds__(THREADS, 2) k_conv_gather(const ConvParams p, 
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = s_tmem;
-    const int nch = min(g * cfg.te, p.c_out - tile0 * p.tile_t);   // channels this CTA computes
-    const int passes = (cfg.te <= PASS) ? (g + PASS / cfg.te - 1) / (PASS / cfg.te) : g * ((cfg.te + PASS - 1) / PASS);
-    // channels of pass i: first one (relative to the CTA's), how many
-    auto pass_range = [&](int i, int& first, int& cols) {
-        if (cfg.te <= PASS) {
-            const int per = PASS / cfg.te * cfg.te;
-            first = i * per;
-            cols = min(per, nch - first);
-        } else {
-            const int pieces = (cfg.te + PASS - 1) / PASS, t = i / pieces, q = i - t * pieces;
-            first = t * cfg.te + q * PASS;
-            cols = min(min(PASS, cfg.te - q * PASS), nch - first);
-        }
-    };
+    const int nch = min(p.tile_t, p.c_out - tile * p.tile_t);   // channels this CTA computes
+    const int passes = (nch + PASS - 1) / PASS;
+    auto pass_cols = [&](int i) { return min(PASS, nch - i * PASS); };
     // Partial sums of this CTA's rows in pass i, from every CTA of the cluster.  A CTA without rows neither expects nor waits: an
     // expectation of nothing would complete its phase at once, and the next pass's the one after it, past a warp of this
     // CTA that has yet to look at the first (a wait by parity would then never end).
     auto expect_part = [&](int i) {
         if (my_rows == 0) return;
-        int first, cols;
-        pass_range(i, first, cols);
-        mbar_arrive_expect_tx(smem_u32(&s_part), static_cast<uint32_t>(my_rows * pitch_of(cols) * 4 * cfg.cs));
+        mbar_arrive_expect_tx(smem_u32(&s_part), static_cast<uint32_t>(my_rows * pitch_of(pass_cols(i)) * 4 * cfg.cs));
     };
     if (cfg.cs > 1) {
         // the barrier knows what to expect, and every CTA of the cluster has started, before any of them sends (waited for below)
@@ -205,12 +190,12 @@ __global__ void __launch_bounds__(THREADS, 2) k_conv_gather(const ConvParams p, 
             }
         const char* xb = reinterpret_cast<const char*>(p.x) + (WIDE ? 0 : static_cast<size_t>(n_first) * p.h * p.w * p.c_in * 4);
         auto at = [xb](uint32_t bytes) { return reinterpret_cast<const float*>(xb + bytes); };
-        const uint32_t* taps = p.taps + static_cast<size_t>(tile0) * p.kk_pad + lane;
-        // taps of the next units to be read: a unit takes less time than its tap needs to arrive
-        int fc = c_begin, ft = 0;
+        const uint32_t* taps = p.taps + static_cast<size_t>(tile) * p.kk_pad + lane;
+        // taps of the next chunks to be read: a chunk takes less time than its tap needs to arrive
+        int fc = c_begin;
         auto fetch = [&]() {
-            const uint32_t t = fc < c_end ? __ldg(taps + static_cast<size_t>(ft) * p.kk_pad + fc * NM_KCHUNK) : NM_TAP_PAD;
-            if (++ft == g) { ft = 0; ++fc; }
+            const uint32_t t = fc < c_end ? __ldg(taps + fc * NM_KCHUNK) : NM_TAP_PAD;
+            ++fc;
             return t;
         };
         uint32_t queue[TAPS_AHEAD];
@@ -273,13 +258,13 @@ __global__ void __launch_bounds__(THREADS, 2) k_conv_gather(const ConvParams p, 
         };
         pdl_wait();
         float va[RPW], vb[RPW];
-        if (units > 0) read(va);
-        if (units > 1) read(vb);
-        for (int u = 0; u < units; u += 2) {
+        if (my_chunks > 0) read(va);
+        if (my_chunks > 1) read(vb);
+        for (int u = 0; u < my_chunks; u += 2) {
             if (aborted(abort_flag) || !store(va)) break;
-            if (u + 2 < units) read(va);
-            if (u + 1 >= units || !store(vb)) break;
-            if (u + 3 < units) read(vb);
+            if (u + 2 < my_chunks) read(va);
+            if (u + 1 >= my_chunks || !store(vb)) break;
+            if (u + 3 < my_chunks) read(vb);
         }
         __syncwarp();
     } else if (warp == 8) {
@@ -287,26 +272,22 @@ __global__ void __launch_bounds__(THREADS, 2) k_conv_gather(const ConvParams p, 
         if (elect_one()) {
             const uint32_t idesc = umma_idesc_tf32(BM, cfg.n);
             RingPos rp, rw;
-            bool ok = true;
-            for (int c = c_begin; c < c_end && ok; ++c) {
-                const int steps = min(NM_KCHUNK, p.kk - c * NM_KCHUNK) + 7 >> 3;   // K-steps of eight columns that hold any
-                for (int t = 0; t < g; ++t) {
-                    if (!mbar_wait_lone(smem_u32(&s_wfull[rw.s]), rw.parity) || !mbar_wait_lone(smem_u32(&s_full[rp.s]), rp.parity)) {
-                        *abort_flag = 3;
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    const uint64_t adesc = umma_desc_k_sw128(ring + rp.s * A_BYTES, 1024);
-                    const uint64_t bdesc = umma_desc_k_sw128(w_ring + rw.s * cfg.w_bytes, 1024);
-#pragma unroll
-                    for (int kq = 0; kq < 4; ++kq)
-                        if (kq < steps) umma_tf32_ss(tmem + t * cfg.n, adesc + 2 * kq, bdesc + 2 * kq, idesc, (c > c_begin || kq > 0) ? 1u : 0u);
-                    umma_commit(smem_u32(&s_free[rp.s]));
-                    umma_commit(smem_u32(&s_wfree[rw.s]));
-                    rp.advance(NA);
-                    rw.advance(cfg.w_stages);
+            for (int c = c_begin; c < c_end; ++c) {
+                if (!mbar_wait_lone(smem_u32(&s_wfull[rw.s]), rw.parity) || !mbar_wait_lone(smem_u32(&s_full[rp.s]), rp.parity)) {
+                    *abort_flag = 3;
+                    break;
                 }
+                tc_fence_after();
+                const int steps = min(NM_KCHUNK, p.kk - c * NM_KCHUNK) + 7 >> 3;   // K-steps of eight columns that hold any
+                const uint64_t adesc = umma_desc_k_sw128(ring + rp.s * A_BYTES, 1024);
+                const uint64_t bdesc = umma_desc_k_sw128(w_ring + rw.s * cfg.w_bytes, 1024);
+#pragma unroll
+                for (int kq = 0; kq < 4; ++kq)
+                    if (kq < steps) umma_tf32_ss(tmem, adesc + 2 * kq, bdesc + 2 * kq, idesc, (c > c_begin || kq > 0) ? 1u : 0u);
+                umma_commit(smem_u32(&s_free[rp.s]));
+                umma_commit(smem_u32(&s_wfree[rw.s]));
+                rp.advance(NA);
+                rw.advance(cfg.w_stages);
             }
             umma_commit(smem_u32(&s_acc));
         }
@@ -318,16 +299,13 @@ __global__ void __launch_bounds__(THREADS, 2) k_conv_gather(const ConvParams p, 
             const uint32_t bytes = static_cast<uint32_t>(cfg.n) * 128u;
             RingPos rp;
             int issued = 0;
-            bool ok = true;
-            for (int c = c_begin; c < c_end && ok; ++c)
-                for (int t = 0; t < g; ++t) {
-                    if (rp.wrapped && !mbar_wait_lone(smem_u32(&s_wfree[rp.s]), rp.parity ^ 1u)) { *abort_flag = 4; ok = false; break; }
-                    const uint32_t bar = smem_u32(&s_wfull[rp.s]);
-                    mbar_arrive_expect_tx(bar, bytes);
-                    bulk_load_1d(w_ring + rp.s * cfg.w_bytes, p.wt + (static_cast<size_t>(tile0 + t) * cfg.chunks + c) * cfg.n * NM_KCHUNK, bytes, bar);
-                    rp.advance(cfg.w_stages);
-                    ++issued;
-                }
+            for (int c = c_begin; c < c_end; ++c, ++issued) {
+                if (rp.wrapped && !mbar_wait_lone(smem_u32(&s_wfree[rp.s]), rp.parity ^ 1u)) { *abort_flag = 4; break; }
+                const uint32_t bar = smem_u32(&s_wfull[rp.s]);
+                mbar_arrive_expect_tx(bar, bytes);
+                bulk_load_1d(w_ring + rp.s * cfg.w_bytes, p.wt + (static_cast<size_t>(tile) * cfg.chunks + c) * cfg.n * NM_KCHUNK, bytes, bar);
+                rp.advance(cfg.w_stages);
+            }
             if (aborted(abort_flag))   // loads already issued still target this CTA's shared memory: let them land (bounded)
                 for (int back = 0; back < cfg.w_stages && back < issued; ++back) {
                     if (rp.s == 0) { rp.s = cfg.w_stages; rp.parity ^= 1u; }
@@ -348,34 +326,21 @@ __global__ void __launch_bounds__(THREADS, 2) k_conv_gather(const ConvParams p, 
     const int q = warp & 3, half = warp >> 2;
     const int row = q * 32 + lane;
     for (int i = 0; i < passes; ++i) {
-        int first, cols;
-        pass_range(i, first, cols);
+        const int cols = pass_cols(i);
         const int pitch = pitch_of(cols);
         if (warp < 8) {
             // accumulators -> staging [row][channel of the pass] over the ring, which is idle now; sixteen columns at a time
-            const int t0 = first / cfg.te, j0 = first - t0 * cfg.te;
-            const int tiles = cfg.te <= PASS ? (cols + cfg.te - 1) / cfg.te : 1;
-            const int per = cfg.te <= PASS ? cfg.te : cols;   // channels of a tile in this pass
-            const int pieces = (per + 15) / 16;
-            for (int k = half; k < tiles * pieces; k += 2) {
-                const int t = k / pieces, jb = (k - t * pieces) * 16;
+            for (int jb = half * 16; jb < cols; jb += 32) {
                 uint32_t v[16];
-                tmem_ld16(tmem + (static_cast<uint32_t>(q * 32) << 16) + (t0 + t) * cfg.n + j0 + jb, v);
+                tmem_ld16(tmem + (static_cast<uint32_t>(q * 32) << 16) + i * PASS + jb, v);
                 tmem_ld_wait();
-                const uint32_t dst = ring + (row * pitch + t * cfg.te + jb) * 4;
-                const int valid = min(min(16, per - jb), cols - t * cfg.te - jb);   // the last tile may have fewer channels
-                if ((cfg.te & 3) == 0) {
+                const uint32_t dst = ring + (row * pitch + jb) * 4;   // (a pitch is whole 16-byte pieces)
 #pragma unroll
-                    for (int e = 0; e < 16; e += 4)
-                        if (e < valid)
-                            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst + e * 4), "r"(v[e]), "r"(v[e + 1]), "r"(v[e + 2]),
-                                         "r"(v[e + 3])
-                                         : "memory");
-                } else {
-#pragma unroll
-                    for (int e = 0; e < 16; ++e)
-                        if (e < valid) asm volatile("st.shared.b32 [%0], %1;" ::"r"(dst + e * 4), "r"(v[e]) : "memory");
-                }
+                for (int e = 0; e < 16; e += 4)
+                    if (jb + e < cols)
+                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst + e * 4), "r"(v[e]), "r"(v[e + 1]), "r"(v[e + 2]),
+                                     "r"(v[e + 3])
+                                     : "memory");
             }
             tc_fence_before();
             if (cfg.cs > 1) fence_proxy_async();
@@ -396,7 +361,7 @@ __global__ void __launch_bounds__(THREADS, 2) k_conv_gather(const ConvParams p, 
             if (!aborted(abort_flag)) {
                 const uint32_t src = cfg.cs > 1 ? part : ring;
                 const uint32_t src_step = static_cast<uint32_t>(cfg.rps * pitch * 4);
-                const int o0 = tile0 * p.tile_t + first;
+                const int o0 = tile * p.tile_t + i * PASS;
                 const long long pix = pix0 + row0;
                 if (((p.c_out | o0 | cols) & 3) == 0) {
                     const int c4 = cols >> 2;
@@ -471,34 +436,31 @@ namespace nmhost {
 nm_status_t launch_conv_gather(const ConvParams& p, cudaStream_t st)
 {
     GatherCfg cfg = {};
-    cfg.te = std::min(p.tile_t, p.c_out);
     cfg.n = gather_width(p.tile_t, p.c_out);
     if (cfg.n > 256) return fail(NM_ERR_UNSUPPORTED, "nm_conv2d: tile_t %d exceeds 256", p.tile_t);
     cfg.chunks = p.kk_pad / NM_KCHUNK;
     const long long blocks = (p.pixels + BM - 1) / BM;
-    // Tiles per CTA and ranges of the chunks, by an estimate of the time: a (chunk, tile) unit takes a CTA about 0.3 us plus its
-    // share of bringing the chunk's 32 KB in from L2, which the tiles of a CTA share through L1; two CTAs fit an SM (in
-    // clusters not on every last one), and one that has it to itself is nearly twice as fast; a launch has a few us of
-    // its own.  At most 256 accumulator columns per CTA, 128 where CTAs of a cluster wait for one another.
+    // Ranges of the chunks, by an estimate of the time from the costs above: a chunk takes a CTA 0.95 us, 0.70 us where it has its
+    // SM to itself; a wave has about 3 us of its own and 4 more with the exchange (clusters do not fit on every last SM).
+    // Measured, us: 7 blocks x 5 tiles, 95 chunks, one range 69, two 42, four 28, eight (a second wave) 49; 55 blocks x 8 tiles, 54 chunks,
+    // one range 68, two 83; 15 blocks x 8 tiles, 5 chunks, one range 14, two 16.
     const long long sms = sm_count();
     double best = 1e30;
-    for (int cs = 1; cs <= 8 && (cs == 1 || cfg.chunks >= 2 * cs); cs *= 2)
-        for (int g = std::min(p.n_tiles, std::max(1, (cs > 1 ? 128 : 256) / cfg.n));; g = (g + 1) / 2) {
-            const long long ctas = blocks * ((p.n_tiles + g - 1) / g) * cs;
-            const long long waves = (ctas + 2 * sms - (cs > 1 ? 33 : 1)) / (2 * sms - (cs > 1 ? 32 : 0));
-            const double unit = (0.3 + 0.3 / g) * (ctas <= sms ? 0.6 : 1.0);
-            const double t = waves * (((cfg.chunks + cs - 1) / cs) * g * unit + (cs > 1 ? 4.0 : 3.0));
-            if (t < best * 0.98) { best = t; cfg.g = g; cfg.cs = cs; }
-            if (g == 1) break;
-        }
-    cfg.n_groups = (p.n_tiles + cfg.g - 1) / cfg.g;
+    for (int cs = 1; cs <= 8 && (cs == 1 || cfg.chunks >= 2 * cs); cs *= 2) {
+        const long long ctas = blocks * p.n_tiles * cs, slots = 2 * sms - (cs > 1 ? 32 : 0);
+        const long long full = ctas / slots, rest = ctas - full * slots;
+        const int range = (cfg.chunks + cs - 1) / cs;
+        const double wave = cs > 1 ? 7.0 : 3.0;
+        const double t = full * (range * 0.95 + wave) + (rest == 0 ? 0.0 : range * (rest <= sms ? 0.70 : 0.95) + wave);
+        if (t < best * 0.95) { best = t; cfg.cs = cs; }
+    }
     cfg.rps = BM / cfg.cs;
     cfg.tmem_cols = 32;
-    while (cfg.tmem_cols < cfg.g * cfg.n) cfg.tmem_cols <<= 1;
-    const long long grid = blocks * cfg.n_groups * cfg.cs;
+    while (cfg.tmem_cols < cfg.n) cfg.tmem_cols <<= 1;
+    const long long grid = blocks * p.n_tiles * cfg.cs;
     if (grid > 0x7FFFFFFFll) return fail(NM_ERR_UNSUPPORTED, "nm_conv2d: too many output pixels");
     cfg.w_bytes = cfg.n * 128;   // a multiple of 2 KB
-    // A weight chunk takes about 1 us to arrive from L2, several (chunk, tile) units' time: its ring is deeper than the operands'.
+    // A weight chunk takes about 1 us to arrive from L2, more than a chunk's time: its ring is deeper than the operands'.
     // The staging of a pass (128 rows of at most PASS + 4 floats) lies over the rings, with a cluster the received sums take
     // as much again.
     const int stage_out = BM * (PASS + 4) * 4;

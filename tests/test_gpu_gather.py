@@ -1,6 +1,6 @@
 """The direct-gather kernel (plan.variant = 1) against the CPU oracle, bit for bit on integer inputs: tile widths below, at and
 above a staging pass, odd ones, tails of tiles and channels, tap counts on both sides of the mask, one to eight ranges of the
-chunks, several tiles and several passes per CTA, ragged pixel blocks that span images, the fused shortcut."""
+chunks, several passes per CTA, ragged pixel blocks that span images, the fused shortcut."""
 import numpy as np
 import pytest
 import torch
@@ -29,9 +29,9 @@ SHAPES = [
     ConvShape("split4", 1, 13, 13, 100, 60, 3, 3, 1, 1, 1, 2, 4, 12),
     ConvShape("split8", 1, 7, 7, 300, 50, 3, 3, 1, 1, 1, 2, 4, 50),
     ConvShape("split8_passes", 1, 6, 6, 300, 200, 3, 3, 1, 1, 1, 2, 4, 200),      # four passes through the exchange, ranks without rows
-    ConvShape("split8_groups", 3, 34, 11, 75, 330, 3, 3, 1, 1, 1, 3, 4, 64),      # two tiles per CTA, the last block ragged
+    ConvShape("split_ragged", 3, 34, 11, 75, 330, 3, 3, 1, 1, 1, 3, 4, 64),      # six tiles, the last block ragged
     ConvShape("split_7x7", 1, 9, 9, 30, 20, 7, 7, 1, 3, 1, 2, 4, 20),
-    ConvShape("many_tiles", 6, 60, 60, 18, 72, 1, 1, 1, 0, 1, 2, 4, 4),           # 18 tiles, several per CTA
+    ConvShape("many_tiles", 6, 60, 60, 18, 72, 1, 1, 1, 0, 1, 2, 4, 4),           # 18 tiles
     ConvShape("wide_kept", 2, 30, 30, 10, 16, 3, 3, 1, 1, 1, 10, 10, 16),         # nothing pruned
 ]
 
@@ -84,3 +84,16 @@ def test_pruned_columns_are_never_read():
     y = nm.nm_conv2d(hnd, x, 3, 3, 1, 1, 1, plan=plan)
     x[..., 4] = float("inf")
     assert torch.equal(nm.nm_conv2d(hnd, x, 3, 3, 1, 1, 1, plan=plan), y)
+
+
+@pytest.mark.parametrize("batch", [4, 5])                # 1280 and 1600 units of a block, tile and chunk: the gather, runs of rows
+def test_default_on_both_sides_of_the_row_runs(batch):
+    from paper_2507_17301_b200 import nm
+    s = ConvShape("rows", batch, 49, 52, 24, 56, 3, 3, 1, 1, 1, 2, 4, 16)
+    w, x, b = inputs.make_int_case(s)
+    vr, ir = oracle.prune(w.numpy(), 2, 4, 16)
+    yr = oracle.conv2d(vr, ir, 3, 3, 24, 16, x.numpy(), (1, 1), (1, 1), (1, 1), b.numpy(), True)
+    hnd = nm.nm_prune(w.cuda(), 2, 4, 16)
+    y = nm.nm_conv2d(hnd, x.cuda(), 3, 3, 1, 1, 1, b.cuda(), True)
+    nm.nm_weights_check(hnd)
+    assert np.array_equal(y.cpu().numpy(), yr)
