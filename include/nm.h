@@ -81,11 +81,11 @@ typedef struct nm_weights nm_weights_t;
  *                halves the shared-memory traffic per FLOP on reduction-heavy layers (needs the
  *                conditions of variant 4, bn 128 or 256, c_out % bn == 0).
  *            8 = select kernel (persistent; contracts over the retained columns only: the dense
- *                activations of a chunk are staged once per CTA, each thread reads its pixel's row with
- *                16-byte loads and picks every tile's retained columns with M - N bitwise selects per
- *                column under precomputed masks; up to four MMA issuer threads; needs N:M one of
- *                1:4 2:4 3:4 1:8 2:8 4:8, K % M == 0, c_in a multiple of the chunk's 64 (3:4: 32) source
- *                columns, tile_t % 16 == 0, c_out % tile_t == 0, an input of at least 128 KiB).  Activation
+ *                activations are staged once per CTA, sixteen warps load every tile's retained columns from
+ *                them, by tables built at pruning time, in the fragment that a tensor-memory store takes; an MMA
+ *                issuer thread per tile; needs an N:M whose M divides 32 with 8, 16 or 24 columns kept of 32,
+ *                or divides 64 with 8 kept (1:2 1:4 2:4 3:4 1:8 2:8 4:8 6:8 4:16 2:16 ...), K % M == 0, c_in a multiple of the
+ *                32 or 64, tile_t % 16 == 0, c_out % tile_t == 0, an input of at least 128 KiB).  Activation
  *                loads (`loads`): im2col-mode TMA loads (any stride / dilation), or, for stride-1 layers
  *                whose output has the input's size, "patch" loads that fetch a pixel block and its halo
  *                once for all kh * kw taps.  `stages` = activation ring depth; `ksplit` > 1 splits the
@@ -109,8 +109,8 @@ typedef struct nm_weights nm_weights_t;
  *            one equal contiguous range per SM, an item shared by several CTAs is completed by the CTA
  *            that holds its first stage from the others' partial sums (per-SM slots in the same
  *            scratch; for layers with too few work items to fill every SM evenly);
- *            variant 6: M-tiles per work item (1-4); variant 8: 1 = four epilogue warps, 2 = eight (0 = eight where a
- *            work item has at most four chunks); variant 9: output rows per work item (1-4, 0 = most);
+ *            variant 6: M-tiles per work item (1-4); variant 8: 0, 1 and 2 are the same;
+ *            variant 9: output rows per work item (1-4, 0 = most);
  *            otherwise 0
  *   kblk     variants 4 and 7: 32-column blocks of the reduction axis per pipeline stage, 1 or 2 (0 = 1);
  *            two blocks halve the barrier round trips per MMA, which pays where the MMAs are short
@@ -124,9 +124,8 @@ typedef struct {
     int split;
     int kblk;
     int loads;    /* variant 8: 0 = the library's choice, 1 = im2col loads, 2 = patch loads */
-    int issuers;  /* MMA issuer threads: variant 8: 1-4 (0 = 4); the work item's accumulator columns are cut into
-                     that many MMA units where the tile width allows (units of at least 16 columns, none across two
-                     tiles), so fewer issuers mean wider MMAs;
+    int issuers;  /* MMA issuer threads: variant 8: 1-4 (0 = one per tile of the work item, which is also the least); more of
+                     them cut the tiles into narrower MMAs (of at least 16 columns) where the tile width allows;
                      variant 4: 1 or 2 (0 = 1); two threads take alternate pipeline stages of a work item, each into an
                      accumulator of its own that the epilogue adds (the ring then has an even number of stages, and
                      work items of more than 128 channels have one accumulator buffer instead of two) */

@@ -116,7 +116,7 @@ nm_status_t make_params(const char* who, const nm_weights* w, const float* x, in
     p->splitk_bytes = w->splitk_bytes;
     p->w3 = w->w3;
     p->sel3 = w->sel3;
-    p->sel_s = w->sel_s; p->sel_kc = w->sel_kc; p->sel_mw = w->sel_mw;
+    p->sel_s = w->sel_s; p->sel_kc = w->sel_kc;
     p->ws = w->ws;
     return NM_OK;
 }
@@ -231,11 +231,9 @@ std::vector<nm_plan_t> candidate_plans(const nm_weights* /*w*/, const ConvParams
     // tile, with the activation loads it prefers for the shape, and with the reduction axis split where few work
     // items exist (the split plans need the handle's scratch)
     for (int ksplit : {1, 2, 3, 4}) {
-        for (int bn : {256, 128, 64}) {
-            for (int epi : {1, 2}) {        // four or eight epilogue warps (split plans: the library's choice)
-                a.variant = 8; a.bn = bn; a.ksplit = ksplit; a.split = ksplit == 1 ? epi : 0;
-                if ((ksplit == 1 || epi == 1) && bn % p.tile_t == 0 && nmhost::select_plan_ok(p, &a)) out.push_back(a);
-            }
+        for (int bn : {128, 256, 64, 32}) {
+            a.variant = 8; a.bn = bn; a.ksplit = ksplit;
+            if (bn % p.tile_t == 0 && nmhost::select_plan_ok(p, &a)) out.push_back(a);
         }
     }
     std::memset(&a, 0, sizeof(a));

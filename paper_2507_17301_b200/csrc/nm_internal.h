@@ -42,11 +42,11 @@ struct nm_weights {
     size_t splitk_bytes;
     float* wx;           // [ceil(k / 32)][wx_rows][32] TF32, rows swizzled (see k_build_layouts); NULL when the shape rules the variant out
     int wx_rows;         // c_out rounded up to a multiple of 32 (the rows past c_out are zero)
-    // Select layout (variant 8): chunks of sel_s source columns of which every tile keeps sel_kc; NULL when the
-    // pattern or the shape rules the variant out.
-    float* w3;           // [k / sel_s][c_out][32] TF32, rows swizzled (see k_build_layouts)
-    uint8_t* sel3;       // [k / sel_s][n_tiles][sel_mw bytes] select masks, 32-bit words (see k_build_layouts)
-    int sel_s, sel_kc, sel_mw;
+    // Select layout (variant 8): steps of sel_s source columns of which every tile keeps sel_kc, chunks of as many steps as fit 32
+    // retained columns; NULL when the pattern or the shape rules the variant out.
+    float* w3;           // [sel_chunks][c_out][32] TF32, rows swizzled (see k_build_layouts)
+    uint8_t* sel3;       // [sel_chunks][n_tiles][32 words] column tables (see k_build_layouts)
+    int sel_s, sel_kc, sel_chunks;
     // Plane layout (variant 9): per kernel row a [c_out][32] tile of (kw, c) slots; NULL when the shape rules it out.
     float* ws;           // [kh][c_out][32] TF32, rows swizzled (see k_build_layouts)
 };
@@ -80,7 +80,7 @@ struct ConvParams {
     // select layout (variant 8)
     const float* w3;
     const uint8_t* sel3;
-    int sel_s, sel_kc, sel_mw;
+    int sel_s, sel_kc;
     // plane layout (variant 9)
     const float* ws;
 };
@@ -198,7 +198,7 @@ bool stream_leaves_sms_idle(const ConvParams& p);   // few work items, each with
 nm_status_t launch_conv_stream(const ConvParams& p, const nm_plan_t* plan, cudaStream_t st);
 
 // nm_conv_select.cu — variant 8
-bool select_layout_dims(const nm_weights* h, int* s, int* kc, int* mw);   // false: the pattern or shape rules the kernel out
+bool select_layout_dims(const nm_weights* h, int* s, int* kc);   // false: the pattern or shape rules the kernel out
 bool select_plan_ok(const ConvParams& p, const nm_plan_t* plan);
 size_t select_splitk_bytes(const ConvParams& p, int splits);
 nm_status_t launch_conv_select(const ConvParams& p, const nm_plan_t* plan, cudaStream_t st);

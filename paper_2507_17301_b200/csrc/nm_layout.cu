@@ -9,7 +9,7 @@
 // mutex.
 //
 // All layouts are written by ONE kernel from the index array and the values (k_build_layouts), after one memset of the
-// arrays that have padding: a thread per (row, retained column) decodes its column once and stores the value to each of
+// arrays that have padding: a thread decodes a retained column once and stores the values of a few rows to each of
 // them.  It is bound by the writes (28 MB for 512 x 3 x 3 x 512 at 2:4).
 #include <algorithm>
 #include <mutex>
@@ -95,19 +95,45 @@ struct LayoutArgs {
     uint32_t* taps;
     float* wt2; uint8_t* rel2; int v2_s, v2_kc, v2_chunks;         // NULL: not built
     float* wx; int wx_rows;
-    float* w3; uint8_t* sel3; int sel_s, sel_kc, sel_mw;
+    float* w3; uint8_t* sel3; int sel_s, sel_kc;
     float* ws;
     int* bad;
 };
 
-// One thread per (output channel, retained column or padding column).
+// Place of retained column e of a select step among the step's `kc` columns, given by their indices `idx`: quads of columns
+// that differ modulo 4 as far as the columns allow (the kernel loads a quad at a time, and columns equal modulo 4 share
+// their banks).  The i-th column of a class (its index modulo 4) goes to quad i; what a class has beyond the number of quads fills
+// the places the others leave, from the last quad down.
+__device__ int select_place(const uint16_t* idx, int kc, int e)
+{
+    const int quads = kc / 4;
+    uint32_t count = 0;   // of the four classes, a byte each
+    int left_over = 0, place = -1;
+#pragma unroll 8
+    for (int i = 0; i < kc; ++i) {
+        const uint32_t cls = idx[i] & 3u;
+        const int rank = static_cast<int>(count >> (8 * cls) & 255u);
+        count += 1u << (8 * cls);
+        if (i == e && rank < quads) place = rank * 4 + static_cast<int>(cls);
+        left_over += rank >= quads && i < e ? 1 : 0;
+    }
+    if (place >= 0) return place;
+    for (int quad = quads - 1; quad >= 0; --quad)
+        for (int c = 0; c < 4; ++c)
+            if (static_cast<int>(count >> (8 * c) & 255u) <= quad && left_over-- == 0) return quad * 4 + c;
+    return 0;   // (not reached: as many free places as columns left over)
+}
+
+constexpr int ROWS = 8;   // output channels per thread: a column is decoded and placed once for all of them (512 x 3 x 3 x 512: 106 us with one, 85 with 4, 82)
+
+// One thread per (retained column or padding column, ROWS output channels of a tile).
 __global__ void k_build_layouts(const LayoutArgs a)
 {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    const int o = blockIdx.y;
+    const int parts = (a.tile_t + ROWS - 1) / ROWS;
+    const int r = blockIdx.y / parts, rr0 = (blockIdx.y - r * parts) * ROWS;
+    const bool first_row = rr0 == 0;   // this thread also writes what the tile's rows share
     if (j >= a.kk_pad) return;
-    const int r = o / a.tile_t;
-    const bool first_row = o == r * a.tile_t;   // this thread also writes what the tile's rows share
     if (j >= a.kk) {
         if (first_row) a.taps[static_cast<size_t>(r) * a.kk_pad + j] = NM_TAP_PAD;
         return;
@@ -122,54 +148,62 @@ __global__ void k_build_layouts(const LayoutArgs a)
         if (first_row) a.indices[static_cast<size_t>(r) * a.kk + j] = static_cast<uint16_t>(col);
         if (bad) return;
     }
-    const float v = a.import ? a.src[static_cast<size_t>(o) * a.kk + j] : a.src[static_cast<size_t>(o) * a.k + col];
-    const float t = nmk::to_tf32(v);
-    a.values[static_cast<size_t>(o) * a.kk + j] = v;
-    {
-        // gather layout: per (tile, chunk of 32 retained columns) the shared-memory image of the tile's rows, swizzled like wx
-        const int rr = o - r * a.tile_t, jj = j & (NM_KCHUNK - 1);
-        a.wt[((static_cast<size_t>(r) * (a.kk_pad / NM_KCHUNK) + j / NM_KCHUNK) * a.wt_rows + rr) * NM_KCHUNK + ((((jj >> 2) ^ (rr & 7)) << 2) | (jj & 3))] = t;
-    }
-    if (first_row) {
-        const int c = col % a.c_in, tap = col / a.c_in;
+    const int tap = col / a.c_in, c = col - tap * a.c_in;
+    if (first_row)
         a.taps[static_cast<size_t>(r) * a.kk_pad + j] =
             (static_cast<uint32_t>(tap / a.kw) << 24) | (static_cast<uint32_t>(tap % a.kw) << 16) | static_cast<uint32_t>(c);
-    }
+
+    // slab layout: kept column j lies in chunk col / S at position j - chunk * KC (every group before the last is
+    // full, so a chunk of whole groups holds exactly KC kept columns)
+    const size_t pitch2 = static_cast<size_t>(a.v2_chunks) * 32;
+    size_t at2 = 0;
     if (a.wt2) {
-        // slab layout: kept column j lies in chunk col / S at position j - chunk * KC (every group before the last is
-        // full, so a chunk of whole groups holds exactly KC kept columns)
         const int chunk = col / a.v2_s, jj = j - chunk * a.v2_kc;
-        const size_t pitch = static_cast<size_t>(a.v2_chunks) * 32;
-        a.wt2[static_cast<size_t>(o) * pitch + chunk * 32 + jj] = t;
-        if (first_row) a.rel2[static_cast<size_t>(r) * pitch + chunk * 32 + jj] = static_cast<uint8_t>(col - chunk * a.v2_s);
+        at2 = static_cast<size_t>(chunk) * 32 + jj;
+        if (first_row) a.rel2[static_cast<size_t>(r) * pitch2 + at2] = static_cast<uint8_t>(col - chunk * a.v2_s);
     }
-    if (a.wx) {
-        // expanded layout: the shared-memory image the tensor core reads: blocks of 32 columns, inside a block one
-        // 128-byte row per output channel whose 16-byte pieces are XOR-ed with (o % 8) (the 128-byte swizzle), so that
-        // any run of channels starting at a multiple of 8 is one contiguous bulk copy
-        const int blk = col >> 5, kc = col & 31;
-        a.wx[(static_cast<size_t>(blk) * a.wx_rows + o) * 32 + ((((kc >> 2) ^ (o & 7)) << 2) | (kc & 3))] = t;
-    }
+    // select layout: w3[chunk][o][32], a chunk being as many steps (one tap of S source columns, of which KC are kept) as fit,
+    // the steps ordered by block of S channels, then tap; swizzled like wx.  The
+    // column tables hold, per chunk and tile, the byte offset of each column in its 128-byte row (and its 32-channel block in
+    // bit 7 and up), in the order in which a thread reads them: [step][place in a quad][quad].
+    int chunk3 = 0, k3 = 0;
     if (a.w3) {
-        // select layout: w3[chunk][o][32], of a row's 32 slots the first KC used, swizzled like wx; and the select masks:
-        // for the jn-th retained column of its group, at position pos in the group, the D = M - N words
-        // m[i] = all ones iff pos == jn + i (all zero: the column is the last candidate, jn + D)
-        const int chunk = col / a.sel_s, jj = j - chunk * a.sel_kc;
-        a.w3[(static_cast<size_t>(chunk) * a.c_out + o) * 32 + ((((jj >> 2) ^ (o & 7)) << 2) | (jj & 3))] = t;
+        const int spc = 32 / a.sel_kc, cb = c / a.sel_s, cc = c - cb * a.sel_s, n_cb = a.c_in / a.sel_s;
+        const int step = cb * a.kh * a.kw + tap, sub = step % spc;
+        chunk3 = step / spc;
+        const int js = (tap * n_cb + cb) * a.sel_kc;   // the step's first retained column
+        const int place = select_place(idx + js, a.sel_kc, j - js);
+        k3 = sub * a.sel_kc + (place >> 3) * 8 + (place & 3) * 2 + (place >> 2 & 1);   // (a thread's columns of two quads are neighbours)
         if (first_row) {
-            const int d = a.m_group - a.n_keep, jn = jj % a.n_keep, pos = col % a.m_group;
-            uint32_t* m = reinterpret_cast<uint32_t*>(a.sel3 + (static_cast<size_t>(chunk) * a.n_tiles + r) * a.sel_mw) +
-                          static_cast<size_t>(jj) * d;
-            for (int i = 0; i < d; ++i) m[i] = (pos == jn + i) ? 0xFFFFFFFFu : 0u;
+            reinterpret_cast<uint32_t*>(a.sel3)[(static_cast<size_t>(chunk3) * a.n_tiles + r) * 32 + sub * a.sel_kc + (place & 3) * (a.sel_kc / 4) + (place >> 2)] =
+                static_cast<uint32_t>((cc & 31) * 4 | (cc >> 5) << 7);
         }
     }
-    if (a.ws) {
-        // plane layout: ws[kh][c_out][32]: a row holds the taps of one kernel row as (kw, c), c padded to 4 and kw to 8,
-        // its 16-byte pieces (one tap each) XOR-ed with (o % 8)
-        const int run = a.kw * a.c_in;
-        const int khi = col / run, rr = col - khi * run;
-        const int kwi = rr / a.c_in, c = rr - kwi * a.c_in;
-        a.ws[(static_cast<size_t>(khi) * a.c_out + o) * 32 + ((kwi ^ (o & 7)) << 2) + c] = t;
+    // plane layout: ws[kh][c_out][32]: a row holds the taps of one kernel row as (kw, c), c padded to 4 and kw to 8,
+    // its 16-byte pieces (one tap each) XOR-ed with (o % 8)
+    const int khi = tap / a.kw, kwi = tap - khi * a.kw;
+
+    for (int rr = rr0; rr < min(rr0 + ROWS, a.tile_t); ++rr) {
+        const int o = r * a.tile_t + rr;
+        if (o >= a.c_out) break;
+        const float v = a.import ? a.src[static_cast<size_t>(o) * a.kk + j] : a.src[static_cast<size_t>(o) * a.k + col];
+        const float t = nmk::to_tf32(v);
+        a.values[static_cast<size_t>(o) * a.kk + j] = v;
+        {
+            // gather layout: per (tile, chunk of 32 retained columns) the shared-memory image of the tile's rows, swizzled like wx
+            const int jj = j & (NM_KCHUNK - 1);
+            a.wt[((static_cast<size_t>(r) * (a.kk_pad / NM_KCHUNK) + j / NM_KCHUNK) * a.wt_rows + rr) * NM_KCHUNK + ((((jj >> 2) ^ (rr & 7)) << 2) | (jj & 3))] = t;
+        }
+        if (a.wt2) a.wt2[static_cast<size_t>(o) * pitch2 + at2] = t;
+        if (a.wx) {
+            // expanded layout: the shared-memory image the tensor core reads: blocks of 32 columns, inside a block one
+            // 128-byte row per output channel whose 16-byte pieces are XOR-ed with (o % 8) (the 128-byte swizzle), so that
+            // any run of channels starting at a multiple of 8 is one contiguous bulk copy
+            const int blk = col >> 5, kc = col & 31;
+            a.wx[(static_cast<size_t>(blk) * a.wx_rows + o) * 32 + ((((kc >> 2) ^ (o & 7)) << 2) | (kc & 3))] = t;
+        }
+        if (a.w3) a.w3[(static_cast<size_t>(chunk3) * a.c_out + o) * 32 + ((((k3 >> 2) ^ (o & 7)) << 2) | (k3 & 3))] = t;
+        if (a.ws) a.ws[(static_cast<size_t>(khi) * a.c_out + o) * 32 + ((kwi ^ (o & 7)) << 2) + c] = t;
     }
 }
 
@@ -239,8 +273,13 @@ static void plan_layouts(nm_weights* h)
     // with zeros to blocks of 32), and either whole 32-column slabs (expanded-operand kernel) or a short reduction axis
     // (row-run kernel, pointwise layers)
     if (h->c_out % 4 == 0 && h->kk > 0 && (h->c_in % 32 == 0 || h->k <= 512)) h->wx_rows = (h->c_out + 31) / 32 * 32;
-    int s = 0, kc = 0, mw = 0;
-    if (select_layout_dims(h, &s, &kc, &mw)) { h->sel_s = s; h->sel_kc = kc; h->sel_mw = mw; }
+    int s = 0, kc = 0;
+    if (select_layout_dims(h, &s, &kc)) {
+        const int spc = 32 / kc, steps = h->c_in / s * h->kh * h->kw;
+        h->sel_s = s;
+        h->sel_kc = kc;
+        h->sel_chunks = (steps + spc - 1) / spc;
+    }
 }
 
 nm_status_t alloc_handle_memory(nm_weights* h, const char* who)
@@ -256,7 +295,7 @@ nm_status_t alloc_handle_memory(nm_weights* h, const char* who)
     };
     const size_t kk1 = static_cast<size_t>(std::max(h->kk, 1));
     const size_t pitch2 = static_cast<size_t>(h->v2_chunks) * 32;
-    const size_t chunks3 = h->sel_s ? static_cast<size_t>(h->k / h->sel_s) : 0;
+    const size_t chunks3 = static_cast<size_t>(h->sel_chunks);
     const size_t at_values = place(h->c_out * kk1 * sizeof(float));
     const size_t at_indices = place(h->n_tiles * kk1 * sizeof(uint16_t));
     const size_t at_taps = place(static_cast<size_t>(h->n_tiles) * h->kk_pad * sizeof(uint32_t));
@@ -268,7 +307,7 @@ nm_status_t alloc_handle_memory(nm_weights* h, const char* who)
     const size_t at_rel2 = place(h->v2_ok ? h->n_tiles * pitch2 : 0);
     const size_t at_wx = place(h->wx_rows ? static_cast<size_t>((h->k + 31) / 32) * h->wx_rows * 128 : 0);
     const size_t at_w3 = place(chunks3 * h->c_out * 128);
-    const size_t at_sel3 = place(chunks3 * h->n_tiles * h->sel_mw);
+    const size_t at_sel3 = place(chunks3 * h->n_tiles * 128);
     const size_t at_ws = place(planes ? static_cast<size_t>(h->kh) * h->c_out * 128 : 0);
     h->block_used = total;
     h->block = static_cast<uint8_t*>(device_block_alloc(total, h->device, &h->block_bytes));
@@ -308,12 +347,12 @@ nm_status_t build_layouts(nm_weights* h, const float* src, const uint16_t* idx, 
     a.wt_rows = gather_width(h->tile_t, h->c_out);
     a.wt2 = h->wt2; a.rel2 = h->rel2; a.v2_s = h->v2_s; a.v2_kc = h->v2_kc; a.v2_chunks = h->v2_chunks;
     a.wx = h->wx; a.wx_rows = h->wx_rows;
-    a.w3 = h->w3; a.sel3 = h->sel3; a.sel_s = h->sel_s; a.sel_kc = h->sel_kc; a.sel_mw = h->sel_mw;
+    a.w3 = h->w3; a.sel3 = h->sel3; a.sel_s = h->sel_s; a.sel_kc = h->sel_kc;
     a.ws = h->ws;
     a.bad = &reinterpret_cast<Readback*>(h->mass)->bad;
-    if (h->c_out > 65535) return fail(NM_ERR_CUDA, "weight layout kernel: more than 65535 output channels");   // grid.y
+    if (h->c_out > 65535) return fail(NM_ERR_CUDA, "weight layout kernel: more than 65535 output channels");   // bounds grid.y
     if (h->kk_pad > 0) {
-        const dim3 grid((h->kk_pad + 127) / 128, h->c_out);
+        const dim3 grid((h->kk_pad + 127) / 128, h->n_tiles * ((h->tile_t + ROWS - 1) / ROWS));
         k_build_layouts<<<grid, 128, 0, st>>>(a);
         count_launch(1);
     }

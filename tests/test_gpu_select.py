@@ -141,3 +141,39 @@ def test_select_kernel_with_shortcut(nm):
         nm.nm_weights_check(hnd)
         torch.cuda.synchronize()
         assert np.array_equal(y.cpu().numpy(), yr), plan.as_dict()
+
+
+# Chunks that cross channel blocks (9 taps of 8 or 16 columns), a last chunk with fewer steps, three tiles per item, several items
+# per CTA with the shortcut requested ahead, a ragged last block; patterns whose groups divide a step.
+MORE = [
+    ConvShape("sel_res_items", 13, 56, 56, 64, 96, 3, 3, 1, 1, 1, 2, 8, 32),          # 319 blocks, 18 steps in 5 chunks
+    ConvShape("sel_res_three", 2, 30, 31, 32, 192, 3, 3, 1, 1, 1, 1, 4, 64),           # 9 steps in 3 chunks
+    ConvShape("sel_1of2", 2, 15, 15, 96, 64, 3, 3, 1, 1, 1, 1, 2, 16),
+    ConvShape("sel_4of16", 3, 15, 15, 64, 128, 3, 3, 1, 1, 1, 4, 16, 64),
+    ConvShape("sel_2of16", 2, 15, 15, 128, 64, 3, 3, 1, 1, 1, 2, 16, 32),             # steps of 64 source columns
+    ConvShape("sel_6of8", 2, 16, 16, 64, 64, 3, 3, 2, 1, 1, 6, 8, 32),                # im2col, 24 of 32 columns
+]
+
+
+@pytest.mark.parametrize("s", MORE, ids=lambda s: s.name)
+def test_select_kernel_shortcut_integer_exact(nm, s):
+    import oracle
+    from paper_2507_17301_b200 import inputs
+    w, x, b = inputs.make_int_case(s)
+    vr, ir = oracle.prune(w.numpy(), s.n_keep, s.m_group, s.tile_t)
+    geom = ((s.stride,) * 2, (s.pad,) * 2, (s.dil,) * 2)
+    hnd = nm.nm_prune(w.cuda(), s.n_keep, s.m_group, s.tile_t)
+    ho, wo = nm.out_shape(x.shape, s.kh, s.kw, s.c_out, *geom)[1:3]
+    res = torch.randint(-9, 10, (s.batch, ho, wo, s.c_out), generator=torch.Generator().manual_seed(1)).float()
+    yr = oracle.conv2d_res(vr, ir, s.kh, s.kw, s.c_in, s.tile_t, x.numpy(), *geom, b.numpy(), res.numpy(), True)
+    ran = 0
+    for plan in (_plan(nm), _plan(nm, bn=s.tile_t), _plan(nm, bn=2 * s.tile_t), _plan(nm, loads=1), _plan(nm, issuers=4)):
+        try:
+            y = nm.nm_conv2d(hnd, x.cuda(), s.kh, s.kw, s.stride, s.pad, s.dil, b.cuda(), True, plan=plan, residual=res.cuda())
+        except nm.NmError as e:
+            assert e.status == nm.NM_ERR_UNSUPPORTED
+            continue
+        nm.nm_weights_check(hnd)
+        assert np.array_equal(y.cpu().numpy(), yr), plan.as_dict()
+        ran += 1
+    assert ran >= 2
