@@ -326,9 +326,9 @@ nm_status_t nm_maxpool2d(const float* x, int batch, int h, int w, int c, int kh,
  * several), writes the fastest to *best and its time to *best_ms (may be NULL).  x and y_scratch
  * are caller buffers of the sizes nm_conv2d expects; y_scratch is overwritten.  Synchronises the
  * stream.  A candidate that fails to launch is skipped; NM_ERR_UNSUPPORTED if none runs.
- * Every timed launch starts with a cold L2: the call allocates a 288 MiB buffer for its own
- * duration and overwrites it before each launch (if that allocation fails the launches run warm), so
- * layers that would fit the cache are tuned for operands that come from HBM.  Candidates are tried
+ * Layers whose input and output together stay well inside the L2 (64 MB) are compared in bursts of launches, as a network
+ * runs them; larger ones one launch at a time with a cold L2, and so is the time reported: the call allocates a 288 MiB
+ * buffer for its own duration and overwrites it before each such launch (if that allocation fails the launches run warm).  Candidates are tried
  * most promising first and a later one replaces the best so far only if it is at least 1 % faster.
  * This call allocates (the buffer above, and the split-K scratch described at nm_weights_reserve).
  * The environment variable NM_AUTOTUNE_VARIANTS (a list of variant digits such as "1,2,3,8") restricts the

@@ -572,16 +572,21 @@ nm_status_t nm_autotune(nm_weights_t* w, const float* x, int batch, int h, int w
         if (e0) cudaEventDestroy(e0);
         return nmhost::fail(NM_ERR_CUDA, "nm_autotune: cannot create events");
     }
-    // Every timed launch starts cold: a buffer larger than the L2 is overwritten first, so that a
-    // layer whose tensors fit the cache is tuned for the case the roofline assumes (operands in HBM)
-    // and candidates are compared under one condition.  Without the buffer the launches run warm.
+    // A layer is timed as a network meets it.  Where its input and output together stay well inside the L2, they are still there from
+    // the layer before, and a launch overlaps its neighbours' ends: bursts of launches.  Larger layers are timed one launch at a time
+    // and cold: a buffer larger than the L2 is overwritten first (without the buffer the launches run warm).  With cold launches
+    // for all, whole networks came to 226 us instead of 207 (ResNet-18 1:4, batch 8) and 312 instead of 300 (ResNet-50, batch 1); with bursts for
+    // all, ResNet-101 at batch 128 sometimes got plans 9 % slower.  The time reported is the best plan's, cold.
+    constexpr double kNearBytes = 64e6;
+    constexpr int kBurst = 10;
+    const bool near = 4.0 * (static_cast<double>(batch) * h * wd * w->c_in + static_cast<double>(p.pixels) * w->c_out) <= kNearBytes;
     constexpr size_t kFlushBytes = size_t(288) << 20;
     void* flush = nullptr;
     if (cudaMalloc(&flush, kFlushBytes) != cudaSuccess) {
         (void)cudaGetLastError();
         flush = nullptr;
     }
-    constexpr int kWarm = 2, kReps = 9;
+    constexpr int kWarm = 2, kReps = 9, kBurstReps = 5;
     float best_t = -1.f;
     // plan cache: a cached plan that still runs on this layer is returned with its time over three launches
     char key[384] = "";
@@ -616,21 +621,27 @@ nm_status_t nm_autotune(nm_weights_t* w, const float* x, int batch, int h, int w
             (void)cudaGetLastError();
         }
     }
+    // One launch, cold, or the mean of a burst; false when a launch fails.
+    auto measure = [&](const nm_plan_t& plan, int launches, std::vector<float>* t) {
+        if (launches == 1 && flush) cudaMemsetAsync(flush, static_cast<int>(t->size()), kFlushBytes, st);
+        cudaEventRecord(e0, st);
+        bool ok = true;
+        for (int k = 0; k < launches && ok; ++k) ok = run_plan(p, &plan, st) == NM_OK;
+        cudaEventRecord(e1, st);
+        if (cudaEventSynchronize(e1) != cudaSuccess) ok = false;
+        float ms = 0.f;
+        if (ok && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess) t->push_back(ms / static_cast<float>(launches));
+        return ok;
+    };
     for (const nm_plan_t& cand : candidate_plans(w, p)) {
         bool ok = true;
         for (int i = 0; i < kWarm && ok; ++i) ok = run_plan(p, &cand, st) == NM_OK;
         if (!ok || cudaStreamSynchronize(st) != cudaSuccess) continue;
         std::vector<float> t;
-        for (int i = 0; i < kReps && ok; ++i) {
-            // three launches tell a candidate that is out of reach (tuning a layer takes half the time this way)
+        for (int i = 0; i < (near ? kBurstReps : kReps) && ok; ++i) {
+            // three measurements tell a candidate that is out of reach (tuning a layer takes half the time this way)
             if (t.size() == 3 && best_t > 0.f && *std::min_element(t.begin(), t.end()) > 1.25f * best_t) break;
-            if (flush) cudaMemsetAsync(flush, i, kFlushBytes, st);
-            cudaEventRecord(e0, st);
-            ok = run_plan(p, &cand, st) == NM_OK;
-            cudaEventRecord(e1, st);
-            if (cudaEventSynchronize(e1) != cudaSuccess) ok = false;
-            float ms = 0.f;
-            if (ok && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess) t.push_back(ms);
+            ok = measure(cand, near ? kBurst : 1, &t);
         }
         if (!ok || t.empty()) continue;
         std::sort(t.begin(), t.end());
@@ -639,6 +650,15 @@ nm_status_t nm_autotune(nm_weights_t* w, const float* x, int batch, int h, int w
         if (best_t < 0.f || med < best_t * 0.99f) {
             best_t = med;
             *best = cand;
+        }
+    }
+    if (near && best_t >= 0.f) {
+        std::vector<float> t;
+        for (int i = 0; i < kReps; ++i)
+            if (!measure(*best, 1, &t)) break;
+        if (!t.empty()) {
+            std::sort(t.begin(), t.end());
+            best_t = t[t.size() / 2];
         }
     }
     if (flush) cudaFree(flush);
