@@ -251,7 +251,7 @@ k_conv_expand(const ConvParams p, const ExpandCfg cfg, const __grid_constant__ C
     tc_fence_after();
     const uint32_t tmem = s_tmem;
     pdl_launch_dependents();   // the next kernel may start its own set-up as SMs become free
-    pdl_wait();                // from here on global memory written by the previous kernel is read
+    if (warp != 2) pdl_wait(); // from here on global memory written by the previous kernel is read (weights are no kernel's output)
 
     if (warp == 0) {
         // =========================== activation producer ===========================

@@ -112,7 +112,7 @@ k_conv_window(const ConvParams p, const WinCfg cfg, const __grid_constant__ CUte
     tc_fence_after();
     const uint32_t tmem = s_tmem;
     pdl_launch_dependents();
-    pdl_wait();
+    if (warp != 1) pdl_wait();   // (the weights are no kernel's output)
 
     if (warp == 0) {
         // =========================== patch producer ===========================
