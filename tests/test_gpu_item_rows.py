@@ -49,3 +49,24 @@ def test_items_of_any_size(s, residual):
                 assert np.array_equal(y.cpu().numpy(), yr), plan.as_dict()
                 ran += 1
     assert ran >= 2
+
+
+@pytest.mark.parametrize("c_out,bn", [(96, 96), (160, 160), (320, 160), (32, 32)])
+def test_odd_numbers_of_channel_blocks(c_out, bn):
+    """Warps that take every other block change places from item to item: several items per CTA, with and without a shortcut."""
+    from paper_2507_17301_b200 import nm
+    s = ConvShape("odd_blocks", 9, 57, 59, 32, c_out, 1, 1, 1, 0, 1, 2, 4, 32)      # 237 blocks of 128 pixels
+    w, x, b = inputs.make_int_case(s)
+    vr, ir = oracle.prune(w.numpy(), s.n_keep, s.m_group, s.tile_t)
+    geom = ((1, 1), (0, 0), (1, 1))
+    res = torch.randint(-9, 10, (s.batch, s.h, s.w, c_out), generator=torch.Generator().manual_seed(1)).float()
+    hnd = nm.nm_prune(w.cuda(), s.n_keep, s.m_group, s.tile_t)
+    yr = oracle.conv2d(vr, ir, 1, 1, s.c_in, s.tile_t, x.numpy(), *geom, b.numpy(), True)
+    yres = oracle.conv2d_res(vr, ir, 1, 1, s.c_in, s.tile_t, x.numpy(), *geom, b.numpy(), res.numpy(), True)
+    for split in (0, 1):
+        plan = nm.nm_plan_t()
+        plan.variant, plan.bn, plan.split = 4, bn, split
+        for r, want in ((None, yr), (res.cuda(), yres)):
+            y = nm.nm_conv2d(hnd, x.cuda(), 1, 1, 1, 0, 1, b.cuda(), True, plan=plan, residual=r)
+            nm.nm_weights_check(hnd)
+            assert np.array_equal(y.cpu().numpy(), want), (split, r is not None)
