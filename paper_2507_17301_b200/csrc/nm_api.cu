@@ -639,8 +639,8 @@ nm_status_t nm_autotune(nm_weights_t* w, const float* x, int batch, int h, int w
         if (!ok || cudaStreamSynchronize(st) != cudaSuccess) continue;
         std::vector<float> t;
         for (int i = 0; i < (near ? kBurstReps : kReps) && ok; ++i) {
-            // three measurements tell a candidate that is out of reach (tuning a layer takes half the time this way)
-            if (t.size() == 3 && best_t > 0.f && *std::min_element(t.begin(), t.end()) > 1.25f * best_t) break;
+            // three launches, or one burst, tell a candidate that is out of reach (tuning a layer takes half the time this way)
+            if (t.size() == (near ? 1u : 3u) && best_t > 0.f && *std::min_element(t.begin(), t.end()) > 1.25f * best_t) break;
             ok = measure(cand, near ? kBurst : 1, &t);
         }
         if (!ok || t.empty()) continue;
