@@ -56,8 +56,10 @@ typedef struct nm_weights nm_weights_t;
 
 /*
  * Launch plan for nm_conv2d (the analogue of the paper's per-layer template parameters, Sec. 3.3).
- *   variant  0 = let the library choose;
- *            1 = direct-gather kernel (any shape);
+ *   variant  0 = let the library choose (variants 3, 9, 5 and 1: activations rounded to nearest, pruned columns never
+ *                read);
+ *            1 = direct-gather kernel (any shape; kept columns gathered from global memory, the reduction axis split over
+ *                clusters of CTAs where there are few);
  *            2 = slab kernel (dense activation slab staged once per CTA, kept columns picked by
  *                4-byte loads; needs c_in % 4 == 0 and whole N:M groups per slab);
  *            3 = stream kernel (persistent; slab read once with 16-byte loads, kept columns of
@@ -97,6 +99,10 @@ typedef struct nm_weights nm_weights_t;
  *                patch matrix is built (needs c_in <= 4, kw <= 8, dil_w = 1, stride_w 1 or 2, output rows of at
  *                most 128 pixels, c_out % 32 == 0 and <= 256; any tile_t, any N:M).  `split` = output rows per
  *                work item (1-4, 0 = as many as tensor memory holds), `stages` = row-band buffers (2 or 3).
+ *            10 = cluster kernel for small batches: an item of up to 128 pixels x `bn` (32, 64, 128; 0 = 32) channels is computed
+ *                by a cluster of `ksplit` (1, 2, 4, 8; 0 = 1) CTAs, each over a range of the reduction axis of variant 4's expanded
+ *                weights; the partial sums move between the CTAs' shared memories (conditions of variant 4, no
+ *                scratch; the tuner tries it unless NM_AUTOTUNE_VARIANTS restricts the search).
  *   bn       output channels per CTA / work item (variants 2, 3, 8: a multiple of tile_t; variant 4: a
  *            multiple of 32 up to 256 that divides c_out rounded up to a multiple of 32; variant 6: a multiple
  *            of 32 up to 256 that divides c_out; variant 7: 128 or 256), 0 = default
@@ -129,7 +135,8 @@ typedef struct {
                      variant 4: 1 or 2 (0 = 1); two threads take alternate pipeline stages of a work item, each into an
                      accumulator of its own that the epilogue adds (the ring then has an even number of stages, and
                      work items of more than 128 channels have one accumulator buffer instead of two) */
-    int ksplit;   /* variant 8: ranges the reduction axis is split into, 1-8 (0 = 1); more than one needs scratch */
+    int ksplit;   /* variant 8: ranges the reduction axis is split into, 1-8 (0 = 1); more than one needs scratch;
+                     variant 10: CTAs per cluster */
     int reserved[8];
 } nm_plan_t;
 
