@@ -8,8 +8,8 @@
 // after its device has been synchronised, so whoever takes it next may use it on any stream; the list is guarded by a
 // mutex.
 //
-// All layouts are written by ONE kernel from the index array and the values (k_build_layouts), after one memset of the
-// arrays that have padding: a thread decodes a retained column once and stores the values of a few rows to each of
+// All layouts are written by ONE kernel from the index array and the values (k_build_layouts), after one memset of those
+// that have padding or pruned columns: a thread decodes a retained column once and stores the values of a few rows to each of
 // them.  It is bound by the writes (28 MB for 512 x 3 x 3 x 512 at 2:4).
 #include <algorithm>
 #include <mutex>
@@ -299,16 +299,31 @@ nm_status_t alloc_handle_memory(nm_weights* h, const char* who)
     const size_t at_values = place(h->c_out * kk1 * sizeof(float));
     const size_t at_indices = place(h->n_tiles * kk1 * sizeof(uint16_t));
     const size_t at_taps = place(static_cast<size_t>(h->n_tiles) * h->kk_pad * sizeof(uint32_t));
-    h->zero_from = total;   // from here on the creating call clears the block: status, sums, layouts with padding
-    const size_t at_status = place(4 * sizeof(int));
-    const size_t at_mass = place(sizeof(Readback));
-    const size_t at_wt = place(static_cast<size_t>(h->n_tiles) * gather_width(h->tile_t, h->c_out) * h->kk_pad * sizeof(float));
-    const size_t at_wt2 = place(h->v2_ok ? h->c_out * pitch2 * sizeof(float) : 0);
-    const size_t at_rel2 = place(h->v2_ok ? h->n_tiles * pitch2 : 0);
-    const size_t at_wx = place(h->wx_rows ? static_cast<size_t>((h->k + 31) / 32) * h->wx_rows * 128 : 0);
-    const size_t at_w3 = place(chunks3 * h->c_out * 128);
-    const size_t at_sel3 = place(chunks3 * h->n_tiles * 128);
-    const size_t at_ws = place(planes ? static_cast<size_t>(h->kh) * h->c_out * 128 : 0);
+    // Layouts that every word of is written come before the part of the block that the creating call clears (status, sums and layouts with
+    // padding or zeros in the pruned columns): 512 x 3 x 3 x 512 at 2:4 has 9 of 24 MB to clear, 58 -> 51 us.
+    const int gather_rows = gather_width(h->tile_t, h->c_out), spc = h->sel_s ? 32 / h->sel_kc : 1;
+    const bool full_wt = h->kk % NM_KCHUNK == 0 && gather_rows == h->tile_t && h->c_out % h->tile_t == 0;
+    const bool full_wt2 = h->v2_kc == 32 && h->k % std::max(h->v2_s, 1) == 0;
+    const bool full_w3 = h->sel_s && h->sel_kc * spc == 32 && h->k / h->sel_s % spc == 0;
+    size_t at_status = 0, at_mass = 0, at_wt = 0, at_wt2 = 0, at_rel2 = 0, at_wx = 0, at_w3 = 0, at_sel3 = 0, at_ws = 0;
+    for (const bool full : {true, false}) {
+        if (!full) {
+            h->zero_from = total;
+            at_status = place(4 * sizeof(int));
+            at_mass = place(sizeof(Readback));
+        }
+        if (full_wt == full) at_wt = place(static_cast<size_t>(h->n_tiles) * gather_rows * h->kk_pad * sizeof(float));
+        if (full_wt2 == full) {
+            at_wt2 = place(h->v2_ok ? h->c_out * pitch2 * sizeof(float) : 0);
+            at_rel2 = place(h->v2_ok ? h->n_tiles * pitch2 : 0);
+        }
+        if (full_w3 == full) {
+            at_w3 = place(chunks3 * h->c_out * 128);
+            at_sel3 = place(chunks3 * h->n_tiles * 128);
+        }
+    }
+    at_wx = place(h->wx_rows ? static_cast<size_t>((h->k + 31) / 32) * h->wx_rows * 128 : 0);
+    at_ws = place(planes ? static_cast<size_t>(h->kh) * h->c_out * 128 : 0);
     h->block_used = total;
     h->block = static_cast<uint8_t*>(device_block_alloc(total, h->device, &h->block_bytes));
     if (!h->block) return fail(NM_ERR_ALLOC, "%s: cannot allocate %zu bytes on the device", who, total);
