@@ -273,8 +273,8 @@ nm_status_t nm_weights_free(nm_weights_t* w);
  * multiply it by a zero weight, so an Inf or NaN in a PRUNED column turns the outputs of that pixel into NaN there
  * while the definition above (and variants 1, 2, 3, 8) keep them finite.  Finite inputs give the same results in all.
  * Arithmetic: operands rounded to TF32 (weights once at prune time, round-to-nearest; activations
- * round-to-nearest where they pass through registers (variants 1-3), truncated where the staged
- * slab feeds the tensor core directly (variants 4, 5, 6)), products accumulated in fp32.
+ * round-to-nearest, with ties away from zero where they pass through registers (variants 1-3) and to even where the TMA unit
+ * rounds them (variants 4, 6, 7, 8, 10), truncated in variants 5 and 9), products accumulated in fp32.
  *
  *   x      device fp32 [batch][h][wd][c_in]      bias  device fp32 [c_out] or NULL
  *   y      device fp32 [batch][ho][wo][c_out]    relu  0 = identity, 1 = ReLU

@@ -418,7 +418,7 @@ bool encode_x(const ConvParams& p, const ClusterCfg& cfg, CUtensorMap* tm)
     const cuuint32_t box2[2] = {32, static_cast<cuuint32_t>(cfg.rows)};
     const cuuint32_t box4[4] = {32, static_cast<cuuint32_t>(p.wo), static_cast<cuuint32_t>(cfg.r_rows), 1};
     const cuuint32_t es[4] = {1, 1, 1, 1};
-    return nmtm::encoders().tiled(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, rows ? 2 : 4, const_cast<float*>(p.x), rows ? dims2 : dims4, strides,
+    return nmtm::encoders().tiled(tm, nmtm::kOperandType, rows ? 2 : 4, const_cast<float*>(p.x), rows ? dims2 : dims4, strides,
                                   rows ? box2 : box4, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }

@@ -40,8 +40,7 @@
 // bitwise selects per element, 93 us; the dense kernel 46.  The gain over the dense kernel grows with M / N: at 2:8
 // 55 -> 38 us (128 -> 128 at 28x28), 74 -> 62 (64 -> 64 at 56x56), at 2:4, batch 64, 30 -> 29 and 45 -> 41, but 28.5 -> 31.5 at 14x14.
 //
-// Activations are fed to the tensor core as they are (it reads the upper 19 bits: truncation to
-// TF32); weights were rounded to nearest at pruning time.
+// Activations are rounded to TF32 by the TMA unit (nm_tmap.cuh), weights were at pruning time, both to nearest.
 #include <algorithm>
 
 #include "nm_internal.h"
@@ -884,7 +883,7 @@ bool encode_x_rows(const ConvParams& p, int rows, CUtensorMap* tm)
     const cuuint64_t strides[1] = {static_cast<cuuint64_t>(p.c_in) * 4};
     const cuuint32_t box[2] = {32, static_cast<cuuint32_t>(rows)};
     const cuuint32_t es[2] = {1, 1};
-    return nmtm::encoders().tiled(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(p.x), dims, strides, box, es,
+    return nmtm::encoders().tiled(tm, nmtm::kOperandType, 2, const_cast<float*>(p.x), dims, strides, box, es,
                                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
