@@ -166,7 +166,14 @@ PyObject* maxpool2d(PyObject*, PyObject* const* a, Py_ssize_t n)
     return a[4];
 }
 
-PyObject* stream_ptr(PyObject*, PyObject*) { return PyLong_FromVoidPtr(current_stream()); }
+PyObject* stream_ptr(PyObject*, PyObject* const*, Py_ssize_t n)
+{
+    if (n != 0) {
+        PyErr_SetString(PyExc_TypeError, "stream_ptr takes no arguments");
+        return nullptr;
+    }
+    return PyLong_FromVoidPtr(current_stream());
+}
 
 PyObject* bind(PyObject*, PyObject* const* a, Py_ssize_t n)
 {
@@ -181,7 +188,7 @@ PyObject* bind(PyObject*, PyObject* const* a, Py_ssize_t n)
     Py_RETURN_NONE;
 }
 
-// C++ exceptions of torch (an allocation that fails) become Python exceptions.
+// C++ exceptions of torch (an allocation that fails, a process without a usable device) become Python exceptions.
 template <PyObject* (*F)(PyObject*, PyObject* const*, Py_ssize_t)>
 PyObject* guarded(PyObject* self, PyObject* const* a, Py_ssize_t n)
 {
@@ -195,6 +202,8 @@ PyObject* guarded(PyObject* self, PyObject* const* a, Py_ssize_t n)
         Py_XDECREF(torch);
     } catch (const std::exception& e) {
         PyErr_SetString(PyExc_RuntimeError, e.what());
+    } catch (...) {
+        PyErr_SetString(PyExc_RuntimeError, "unknown C++ exception");
     }
     return nullptr;
 }
@@ -203,7 +212,7 @@ PyMethodDef methods[] = {
     {"conv2d", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(guarded<conv2d>)), METH_FASTCALL, nullptr},
     {"maxpool2d", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(guarded<maxpool2d>)), METH_FASTCALL, nullptr},
     {"bind", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(bind)), METH_FASTCALL, nullptr},
-    {"stream_ptr", stream_ptr, METH_NOARGS, nullptr},
+    {"stream_ptr", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(guarded<stream_ptr>)), METH_FASTCALL, nullptr},
     {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module_def = {PyModuleDef_HEAD_INIT, "_nm_binding", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 

@@ -1,8 +1,14 @@
 """The per-call extension: argument checks (no GPU) and the output it allocates."""
+import os
+import subprocess
+import sys
+
 import pytest
 import torch
 
 from paper_2507_17301_b200 import build
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 build.build()
 from paper_2507_17301_b200 import nm  # noqa: E402
@@ -19,6 +25,15 @@ def test_host_tensors_and_wrong_types_are_refused():
             nm.nm_maxpool2d(bad)
     with pytest.raises((TypeError, IndexError)):
         nm.nm_conv2d(w, x, 1, 1, stride=(1,))
+
+
+def test_no_usable_device_is_a_python_exception():
+    """In a process of its own: a C++ exception that leaves the extension ends the process."""
+    code = ("from paper_2507_17301_b200 import nm\n"
+            "try:\n    nm._stream()\nexcept RuntimeError:\n    print('refused')\n")
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, env=dict(os.environ, CUDA_VISIBLE_DEVICES=""), capture_output=True,
+                       text=True, timeout=300)
+    assert r.returncode == 0 and r.stdout.strip() == "refused", r.stderr[-1000:]
 
 
 @pytest.mark.gpu

@@ -14,7 +14,7 @@ C1 = ConvShape("1x1", 2, 28, 28, 128, 256, 1, 1, 1, 0, 1, 2, 4, 64)
 S2 = ConvShape("3x3_s2", 2, 28, 28, 64, 64, 3, 3, 2, 1, 1, 1, 4, 16)
 BOX = ConvShape("7x7_map", 1, 7, 7, 128, 64, 3, 3, 1, 1, 1, 2, 4, 32)        # below 128 KiB
 ROWS = ConvShape("7x7_rows", 1, 7, 7, 512, 96, 1, 1, 1, 0, 1, 2, 8, 8)      # below 128 KiB
-ODD = ConvShape("odd", 2, 17, 15, 20, 48, 3, 3, 1, 1, 1, 2, 4, 8)
+ODD = ConvShape("odd", 2, 17, 15, 20, 64, 3, 3, 1, 1, 1, 2, 4, 8)
 
 CASES = [
     (1, {}, C3, "away"), (1, {}, ODD, "away"), (2, {}, C3, "away"), (2, {"split": 1}, ODD, "away"), (3, {}, C1, "away"), (3, {}, S2, "away"),
