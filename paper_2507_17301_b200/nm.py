@@ -294,13 +294,19 @@ def out_shape(x_shape, kh, kw, c_out, stride, pad, dil):
     return (b, ho, wo, c_out)
 
 
+def _plan_addr(plan: nm_plan_t) -> int:
+    addr = ctypes.addressof(plan)   # (a TypeError for what is no ctypes object)
+    if not isinstance(plan, nm_plan_t):
+        raise ctypes.ArgumentError(f"plan must be an nm_plan_t, not {type(plan).__name__}")
+    return addr
+
+
 def nm_conv2d(w: Weights, x: torch.Tensor, kh: int, kw: int, stride=1, pad=0, dil=1, bias=None, relu=False,
               y: torch.Tensor | None = None, plan: nm_plan_t | None = None,
               residual: torch.Tensor | None = None) -> torch.Tensor:
     """``x``: CUDA fp32 NHWC.  Allocates ``y`` (NHWC) unless given.  Asynchronous on the current stream.
     With ``residual`` (NHWC, the output's shape) it calls ``nm_conv2d_res``: act(conv + bias + residual)."""
-    y = _nm_binding.conv2d(w._addr, w.c_out, x, kh, kw, stride, pad, dil, bias, relu, y,
-                           0 if plan is None else ctypes.addressof(plan), residual)
+    y = _nm_binding.conv2d(w._addr, w.c_out, x, kh, kw, stride, pad, dil, bias, relu, y, 0 if plan is None else _plan_addr(plan), residual)
     if y.__class__ is int:
         _check(y)
     return y

@@ -1,4 +1,5 @@
 """The per-call extension: argument checks (no GPU) and the output it allocates."""
+import ctypes
 import os
 import subprocess
 import sys
@@ -25,6 +26,25 @@ def test_host_tensors_and_wrong_types_are_refused():
             nm.nm_maxpool2d(bad)
     with pytest.raises((TypeError, IndexError)):
         nm.nm_conv2d(w, x, 1, 1, stride=(1,))
+
+
+def test_a_plan_of_another_type_is_refused():
+    w = nm.Weights.__new__(nm.Weights)
+    w._h, w._addr, w.c_out = None, 0, 8
+    x = torch.zeros(1, 4, 4, 8)
+    for bad in (ctypes.c_int(4), (ctypes.c_int * 16)(), nm.nm_plan_t):
+        with pytest.raises((ctypes.ArgumentError, TypeError), match="plan|ctypes|invalid type"):
+            nm.nm_conv2d(w, x, 1, 1, plan=bad)
+    with pytest.raises(TypeError, match="x must be"):       # the plan is looked at first and is in order
+        nm.nm_conv2d(w, x, 1, 1, plan=nm.nm_plan_t())
+
+
+@pytest.mark.gpu
+def test_the_window_is_not_needed_beside_an_output():
+    x = torch.randn(1, 5, 5, 8, device="cuda")
+    hnd = nm.nm_prune(torch.randn(12, 3, 3, 8, device="cuda"), 2, 4, 4)
+    y = nm.nm_conv2d(hnd, x, 3, 3, 1, 1)
+    assert torch.equal(nm.nm_conv2d(hnd, x, None, None, 1, 1, y=torch.empty_like(y)), y)
 
 
 def test_no_usable_device_is_a_python_exception():
