@@ -74,7 +74,7 @@ PyObject* conv2d(PyObject*, PyObject* const* a, Py_ssize_t n)
         return nullptr;
     }
     const auto* w = static_cast<const nm_weights_t*>(PyLong_AsVoidPtr(a[0]));
-    const long c_out = PyLong_AsLong(a[1]), kh = PyLong_AsLong(a[3]), kw = PyLong_AsLong(a[4]);
+    const long c_out = PyLong_AsLong(a[1]);
     const auto* plan = static_cast<const nm_plan_t*>(PyLong_AsVoidPtr(a[11]));
     if (PyErr_Occurred()) return nullptr;
     int stride[2], pad[2], dil[2];
@@ -84,7 +84,9 @@ PyObject* conv2d(PyObject*, PyObject* const* a, Py_ssize_t n)
     const int64_t b = x->size(0), h = x->size(1), wd = x->size(2);
     at::Tensor made;
     const at::Tensor* y;
-    if (a[10] == Py_None) {
+    if (a[10] == Py_None) {   // (the window's extent is looked at for the output's shape only: the handle knows it)
+        const long kh = PyLong_AsLong(a[3]), kw = PyLong_AsLong(a[4]);
+        if (PyErr_Occurred()) return nullptr;
         if (stride[0] < 1 || stride[1] < 1 || dil[0] < 1 || dil[1] < 1) {   // the library reports it
             made = at::empty({4}, x->options());
         } else {
