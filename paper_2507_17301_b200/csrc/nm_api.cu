@@ -374,7 +374,8 @@ nm_status_t nm_weights_export(const nm_weights_t* w, float* values, uint16_t* in
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     cudaError_t e = cudaSuccess;
     const size_t vb = static_cast<size_t>(w->c_out) * w->kk * sizeof(float), ib = static_cast<size_t>(w->n_tiles) * w->kk * sizeof(uint16_t);
-    if (values && indices && w->kk > 0 && aligned16(values) && aligned16(indices)) {
+    if (values && indices && w->kk > 0 && aligned16(values) && aligned16(indices) &&
+        nmhost::kernel_may_touch(values, indices, w->device)) {
         // both arrays in one launch (512 x 2304 values: 33 us as two copies, 20)
         k_export<<<static_cast<unsigned>(std::min<size_t>((vb + ib) / 4096 + 1, 1184)), 256, 0, st>>>(
             reinterpret_cast<const char*>(w->values), reinterpret_cast<char*>(values), vb, reinterpret_cast<const char*>(w->indices),

@@ -148,6 +148,14 @@ cudaError_t ensure_dynamic_smem(const void* kernel, size_t bytes);
 nm_status_t fail(nm_status_t s, const char* fmt, ...);
 void count_launch(int n = 1);
 
+// Whether a kernel of device `current` may read or write memory of this kind and owner.  Everything else (another device's
+// memory without a peer mapping, pageable host memory) is left to cudaMemcpyAsync, which copies it or refuses it.
+constexpr bool kernel_may_touch(cudaMemoryType type, int owner, int current)
+{
+    return type == cudaMemoryTypeManaged || (type == cudaMemoryTypeDevice && owner == current);
+}
+bool kernel_may_touch(const void* a, const void* b, int device);   // both of them; false unless `device` is the current one
+
 // nm_layout.cu: the handles' device memory, and the kernel-side copies of the compressed form
 void* device_block_alloc(size_t bytes, int device, size_t* got);   // NULL when there is no memory; reuses blocks of freed handles
 void device_block_free(void* ptr, size_t bytes, int device, bool idle);   // idle: nothing on the device uses it any more

@@ -211,6 +211,21 @@ __global__ void k_build_layouts(const LayoutArgs a)
 
 namespace nmhost {
 
+bool kernel_may_touch(const void* a, const void* b, int device)
+{
+    int current = -1;
+    if (cudaGetDevice(&current) != cudaSuccess || current != device) return false;
+    for (const void* ptr : {a, b}) {
+        cudaPointerAttributes at;
+        if (cudaPointerGetAttributes(&at, ptr) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return false;
+        }
+        if (!kernel_may_touch(at.type, at.device, current)) return false;
+    }
+    return true;
+}
+
 void* device_block_alloc(size_t bytes, int device, size_t* got)
 {
     const size_t want = rounded(bytes);

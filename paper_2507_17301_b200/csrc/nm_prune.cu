@@ -208,6 +208,15 @@ nm_status_t build_from_compressed(const float* values, const uint16_t* indices, 
 {
     int bad = 0;
     nm_status_t s = clear_handle_memory(h, st);
+    if (s == NM_OK && !kernel_may_touch(values, indices, h->device)) {
+        // through the handle's own arrays, which the layout kernel then reads and writes back unchanged
+        cudaError_t e = cudaMemcpyAsync(h->values, values, static_cast<size_t>(h->c_out) * h->kk * sizeof(float), cudaMemcpyDeviceToDevice, st);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(h->indices, indices, static_cast<size_t>(h->n_tiles) * h->kk * sizeof(uint16_t), cudaMemcpyDeviceToDevice, st);
+        if (e != cudaSuccess) return fail(NM_ERR_CUDA, "nm_weights_import: %s", cudaGetErrorString(e));
+        values = h->values;
+        indices = h->indices;
+    }
     if (s == NM_OK) s = build_layouts(h, values, indices, true, st);
     if (s == NM_OK) s = finish_handle(h, st, nullptr, &bad);
     if (s == NM_OK && bad)
