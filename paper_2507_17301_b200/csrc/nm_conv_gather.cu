@@ -296,14 +296,16 @@ __global__ void __launch_bounds__(THREADS, 2) k_conv_gather(const ConvParams p, 
         // =========================== weight producer ===========================
         // The weights are no earlier kernel's output (a handle is complete when the call that built it returns): no pdl_wait.
         if (elect_one()) {
-            const uint32_t bytes = static_cast<uint32_t>(cfg.n) * 128u;
+            // the tile's own rows; what the MMA reads behind them ends in accumulator columns nobody reads
+            const uint32_t bytes = static_cast<uint32_t>(nch) * 128u;
+            const float* src = p.wt + static_cast<size_t>(tile) * p.tile_t * p.kk_pad;
             RingPos rp;
             int issued = 0;
             for (int c = c_begin; c < c_end; ++c, ++issued) {
                 if (rp.wrapped && !mbar_wait_lone(smem_u32(&s_wfree[rp.s]), rp.parity ^ 1u)) { *abort_flag = 4; break; }
                 const uint32_t bar = smem_u32(&s_wfull[rp.s]);
                 mbar_arrive_expect_tx(bar, bytes);
-                bulk_load_1d(w_ring + rp.s * cfg.w_bytes, p.wt + (static_cast<size_t>(tile) * cfg.chunks + c) * cfg.n * NM_KCHUNK, bytes, bar);
+                bulk_load_1d(w_ring + rp.s * cfg.w_bytes, src + static_cast<size_t>(c) * nch * NM_KCHUNK, bytes, bar);
                 rp.advance(cfg.w_stages);
             }
             if (aborted(abort_flag))   // loads already issued still target this CTA's shared memory: let them land (bounded)

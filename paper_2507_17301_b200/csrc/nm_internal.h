@@ -28,7 +28,7 @@ struct nm_weights {
     double l1_total, l1_kept;   // L1 mass of the dense weights / of the retained ones (l1_total < 0: not known)
     float* values;       // [c_out][kk]     exact fp32 copies of the retained weights
     uint16_t* indices;   // [n_tiles][kk]   retained column positions, ascending
-    float* wt;           // [n_tiles][kk_pad / 32][gather_width][32] retained weights rounded to TF32 (nearest), rows swizzled, zero padded
+    float* wt;           // [n_tiles][kk_pad / 32][rows of the tile][32] retained weights rounded to TF32 (nearest), rows swizzled, zero padded
     uint32_t* taps;      // [n_tiles][kk_pad] kh << 24 | kw << 16 | c per retained column, NM_TAP_PAD in the padding
     int* status;         // device int[4]: [0] error code, [1] where, [2] block, [3] spare
     // Slab layout (variant 2); v2_ok = 0 when the N:M pattern does not fit it.
@@ -170,7 +170,7 @@ nm_status_t prune_on_device(const float* w_dense, nm_weights* h, cudaStream_t st
 nm_status_t build_from_compressed(const float* values, const uint16_t* indices, nm_weights* h, cudaStream_t st);
 
 // nm_conv_gather.cu — variant 1
-// rows of a tile's weight chunk = its MMA width: the channels a tile can have, in sixteens
+// MMA width of a tile: the channels it can have, in sixteens
 inline int gather_width(int tile_t, int c_out) { return ((tile_t < c_out ? tile_t : c_out) + 15) / 16 * 16; }
 nm_status_t launch_conv_gather(const ConvParams& p, cudaStream_t st);
 

@@ -91,7 +91,7 @@ struct LayoutArgs {
     int c_out, k, kk, kk_pad, tile_t, n_tiles, n_keep, m_group, c_in, kh, kw;
     float* values;
     uint16_t* indices;           // import: the handle's copy of idx
-    float* wt; int wt_rows;
+    float* wt;
     uint32_t* taps;
     float* wt2; uint8_t* rel2; int v2_s, v2_kc, v2_chunks;         // NULL: not built
     float* wx; int wx_rows;
@@ -190,9 +190,11 @@ __global__ void k_build_layouts(const LayoutArgs a)
         const float t = nmk::to_tf32(v);
         a.values[static_cast<size_t>(o) * a.kk + j] = v;
         {
-            // gather layout: per (tile, chunk of 32 retained columns) the shared-memory image of the tile's rows, swizzled like wx
-            const int jj = j & (NM_KCHUNK - 1);
-            a.wt[((static_cast<size_t>(r) * (a.kk_pad / NM_KCHUNK) + j / NM_KCHUNK) * a.wt_rows + rr) * NM_KCHUNK + ((((jj >> 2) ^ (rr & 7)) << 2) | (jj & 3))] = t;
+            // gather layout: per (tile, chunk of 32 retained columns) the shared-memory image of the tile's rows, swizzled like wx;
+            // as many rows as the tile has, so it is as large as the values whatever the tile width (padded to the MMA's 16 rows,
+            // 512 x 3 x 3 x 512 at 2:4 and T = 1 took 75 MB here instead of 4.7)
+            const int jj = j & (NM_KCHUNK - 1), rows = min(a.tile_t, a.c_out - r * a.tile_t);
+            a.wt[static_cast<size_t>(r) * a.tile_t * a.kk_pad + (static_cast<size_t>(j / NM_KCHUNK) * rows + rr) * NM_KCHUNK + ((((jj >> 2) ^ (rr & 7)) << 2) | (jj & 3))] = t;
         }
         if (a.wt2) a.wt2[static_cast<size_t>(o) * pitch2 + at2] = t;
         if (a.wx) {
@@ -316,8 +318,8 @@ nm_status_t alloc_handle_memory(nm_weights* h, const char* who)
     const size_t at_taps = place(static_cast<size_t>(h->n_tiles) * h->kk_pad * sizeof(uint32_t));
     // Layouts that every word of is written come before the part of the block that the creating call clears (status, sums and layouts with
     // padding or zeros in the pruned columns): 512 x 3 x 3 x 512 at 2:4 has 9 of 24 MB to clear, 58 -> 51 us.
-    const int gather_rows = gather_width(h->tile_t, h->c_out), spc = h->sel_s ? 32 / h->sel_kc : 1;
-    const bool full_wt = h->kk % NM_KCHUNK == 0 && gather_rows == h->tile_t && h->c_out % h->tile_t == 0;
+    const int spc = h->sel_s ? 32 / h->sel_kc : 1;
+    const bool full_wt = h->kk % NM_KCHUNK == 0;
     const bool full_wt2 = h->v2_kc == 32 && h->k % std::max(h->v2_s, 1) == 0;
     const bool full_w3 = h->sel_s && h->sel_kc * spc == 32 && h->k / h->sel_s % spc == 0;
     size_t at_status = 0, at_mass = 0, at_wt = 0, at_wt2 = 0, at_rel2 = 0, at_wx = 0, at_w3 = 0, at_sel3 = 0, at_ws = 0;
@@ -327,7 +329,7 @@ nm_status_t alloc_handle_memory(nm_weights* h, const char* who)
             at_status = place(4 * sizeof(int));
             at_mass = place(sizeof(Readback));
         }
-        if (full_wt == full) at_wt = place(static_cast<size_t>(h->n_tiles) * gather_rows * h->kk_pad * sizeof(float));
+        if (full_wt == full) at_wt = place(static_cast<size_t>(h->c_out) * h->kk_pad * sizeof(float));
         if (full_wt2 == full) {
             at_wt2 = place(h->v2_ok ? h->c_out * pitch2 * sizeof(float) : 0);
             at_rel2 = place(h->v2_ok ? h->n_tiles * pitch2 : 0);
@@ -374,7 +376,6 @@ nm_status_t build_layouts(nm_weights* h, const float* src, const uint16_t* idx, 
     a.c_out = h->c_out; a.k = h->k; a.kk = h->kk; a.kk_pad = h->kk_pad; a.tile_t = h->tile_t; a.n_tiles = h->n_tiles;
     a.n_keep = h->n_keep; a.m_group = h->m_group; a.c_in = h->c_in; a.kh = h->kh; a.kw = h->kw;
     a.values = h->values; a.indices = h->indices; a.wt = h->wt; a.taps = h->taps;
-    a.wt_rows = gather_width(h->tile_t, h->c_out);
     a.wt2 = h->wt2; a.rel2 = h->rel2; a.v2_s = h->v2_s; a.v2_kc = h->v2_kc; a.v2_chunks = h->v2_chunks;
     a.wx = h->wx; a.wx_rows = h->wx_rows;
     a.w3 = h->w3; a.sel3 = h->sel3; a.sel_s = h->sel_s; a.sel_kc = h->sel_kc;

@@ -47,3 +47,33 @@ def test_layouts_on_used_memory(n, m):
             y = nm.nm_conv2d(hnd, x.cuda(), 3, 3, 1, 1, 1, None, False, plan=plan)
             nm.nm_weights_check(hnd)
             assert np.array_equal(y.cpu().numpy(), yr), variant
+
+
+@pytest.mark.parametrize("t", [1, 3, 8, 24])
+def test_gather_layout_of_narrow_tiles_on_used_memory(t):
+    """Rows of a tile only, a ragged last tile, retained columns that end inside a chunk; on memory of an earlier handle."""
+    from paper_2507_17301_b200 import nm
+    g = torch.Generator().manual_seed(6)
+    x = torch.randint(-3, 4, (2, 9, 11, 20), generator=g).float()
+    w = torch.randint(-3, 4, (50, 3, 3, 20), generator=g).float()
+    vr, ir = oracle.prune(w.numpy(), 2, 4, t)
+    yr = oracle.conv2d(vr, ir, 3, 3, 20, t, x.numpy(), (1, 1), (1, 1), (1, 1), None, False)
+    plan = nm.nm_plan_t()
+    plan.variant = 1
+    for _ in range(2):
+        nm.nm_prune(torch.full((50, 3, 3, 20), float("inf"), device="cuda"), 2, 4, t).free()
+        hnd = nm.nm_prune(w.cuda(), 2, 4, t)
+        y = nm.nm_conv2d(hnd, x.cuda(), 3, 3, 1, 1, 1, plan=plan)
+        nm.nm_weights_check(hnd)
+        assert np.array_equal(y.cpu().numpy(), yr)
+
+
+def test_a_handle_of_one_channel_tiles_is_not_padded():
+    """512 x 3 x 3 x 512 at 2:4, T = 1: values, gather and slab layouts 4.7 MB each, taps 4.7, expanded 9.4, indices 3.5: 32 MB."""
+    from paper_2507_17301_b200 import nm
+    w = torch.randn((512, 3, 3, 512), device="cuda")
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    hnd = nm.nm_prune(w, 2, 4, 1)
+    assert before - torch.cuda.mem_get_info()[0] <= 36 << 20
+    hnd.free()
