@@ -190,6 +190,12 @@ __global__ void __launch_bounds__(THREADS, 2) k_conv_gather(const ConvParams p, 
             }
         const char* xb = reinterpret_cast<const char*>(p.x) + (WIDE ? 0 : static_cast<size_t>(n_first) * p.h * p.w * p.c_in * 4);
         auto at = [xb](uint32_t bytes) { return reinterpret_cast<const float*>(xb + bytes); };
+        auto on = [&](uint32_t bytes, uint32_t tap_inside) {   // self-checking build: the load lies in the input
+            if (NM_SELF_CHECKING && tap_inside != 0u &&
+                !NM_ALLOWED(nm_bytes_in_span(bytes, 4, 0, static_cast<uint64_t>(p.batch - n_first) * p.h * p.w * p.c_in * 4), p.status, 103, bytes))
+                return 0u;
+            return tap_inside;
+        };
         const uint32_t* taps = p.taps + static_cast<size_t>(tile) * p.kk_pad + lane;
         // taps of the next chunks to be read: a chunk takes less time than its tap needs to arrive
         int fc = c_begin;
@@ -206,17 +212,16 @@ __global__ void __launch_bounds__(THREADS, 2) k_conv_gather(const ConvParams p, 
 #pragma unroll
             for (int i = 0; i + 1 < TAPS_AHEAD; ++i) queue[i] = queue[i + 1];
             queue[TAPS_AHEAD - 1] = fetch();
-            const bool ok = tap != NM_TAP_PAD;
+            bool ok = tap != NM_TAP_PAD;
+            if (NM_SELF_CHECKING) ok = ok && NM_ALLOWED(nm_tap_in_layer(tap, p.kh, p.kw, p.c_in), p.status, 101, tap);
             const int ki = static_cast<int>(tap >> 24), kj = static_cast<int>((tap >> 16) & 0xFFu), c = static_cast<int>(tap & 0xFFFFu);
-            // self-checking build: the tap table may only name taps and channels of this layer
-            NM_CHECKED(!ok || (c < p.c_in && ki < p.kh && kj < p.kw), p.status, 101, tap) {}
             if (WIDE) {
                 const int dh = ki * p.dil_h, dw = kj * p.dil_w;
 #pragma unroll
                 for (int i = 0; i < RPW; ++i) {
                     const int n = static_cast<int>(s_off[base_row + i]);
                     const int ih = static_cast<int>(s_mask[0][base_row + i]) + dh, iw = s_col[base_row + i] + dw;
-                    const bool in = ok && n >= 0 && static_cast<unsigned>(ih) < static_cast<unsigned>(p.h) && static_cast<unsigned>(iw) < static_cast<unsigned>(p.w);
+                    const bool in = ok && n >= 0 && NM_ALLOWED(n < p.batch, p.status, 102, n) && static_cast<unsigned>(ih) < static_cast<unsigned>(p.h) && static_cast<unsigned>(iw) < static_cast<unsigned>(p.w);
                     v[i] = load_if(p.x + ((static_cast<size_t>(n) * p.h + ih) * p.w + iw) * p.c_in + c, in ? 1u : 0u);
                 }
             } else {
@@ -224,7 +229,7 @@ __global__ void __launch_bounds__(THREADS, 2) k_conv_gather(const ConvParams p, 
                 const int tap_no = ki * p.kw + kj, word = tap_no >> 5;
                 const uint32_t bit = ok ? 1u << (tap_no & 31) : 0u;
                 const uint4* masks = reinterpret_cast<const uint4*>(s_mask[0] + (ok ? word : 0) * (BM + 4) + base_row);
-                if (__all_sync(0xFFFFFFFFu, ((word ? all[1] : all[0]) & bit) != 0u)) {   // inside the image for all rows and columns of this warp
+                if (!NM_SELF_CHECKING && __all_sync(0xFFFFFFFFu, ((word ? all[1] : all[0]) & bit) != 0u)) {   // inside the image for all rows and columns of this warp
 #pragma unroll
                     for (int i = 0; i < RPW; i += 4) {
                         const uint4 o = offs[i / 4];
@@ -234,10 +239,10 @@ __global__ void __launch_bounds__(THREADS, 2) k_conv_gather(const ConvParams p, 
 #pragma unroll
                     for (int i = 0; i < RPW; i += 4) {
                         const uint4 o = offs[i / 4], m = masks[i / 4];
-                        v[i] = load_if(at(o.x + delta), m.x & bit);
-                        v[i + 1] = load_if(at(o.y + delta), m.y & bit);
-                        v[i + 2] = load_if(at(o.z + delta), m.z & bit);
-                        v[i + 3] = load_if(at(o.w + delta), m.w & bit);
+                        v[i] = load_if(at(o.x + delta), on(o.x + delta, m.x & bit));
+                        v[i + 1] = load_if(at(o.y + delta), on(o.y + delta, m.y & bit));
+                        v[i + 2] = load_if(at(o.z + delta), on(o.z + delta, m.z & bit));
+                        v[i + 3] = load_if(at(o.w + delta), on(o.w + delta, m.w & bit));
                     }
                 }
             }

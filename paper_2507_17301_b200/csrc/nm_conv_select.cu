@@ -201,10 +201,12 @@ __device__ __forceinline__ void load_table(uint32_t at, uint32_t (&table)[P::QUA
 template <class P, int G>
 struct Piece {
     uint32_t v[G][2][2 * P::QUADS];
-    // r: this lane's rows, with their swizzle phase folded in; WHOLE: all at their places (8 rows apart: the same phase)
+    // r: this lane's rows, with their swizzle phase folded in; WHOLE: all at their places (8 rows apart: the same phase);
+    // slot: where the activation slot begins (looked at by the self-checking build: a word outside it reads as zero)
     template <bool WHOLE>
-    __device__ __forceinline__ void load(const uint32_t* r, uint32_t table_at, uint32_t seg_bytes)
+    __device__ __forceinline__ void load(const uint32_t* r, uint32_t table_at, uint32_t seg_bytes, uint32_t slot, int* status)
     {
+        auto in_slot = [&](uint32_t a) { return NM_ALLOWED(nm_bytes_in_span(a, 4, slot, slot + P::SEGS * seg_bytes), status, 802, a - slot); };
         uint32_t table[G][P::QUADS];
 #pragma unroll
         for (int t = 0; t < G; ++t) load_table<P>(table_at + t * TABLE_BYTES, table[t]);
@@ -215,7 +217,12 @@ struct Piece {
                 const uint32_t at = P::SEGS == 1 ? table[t][i] : table[t][i] & 127u;
                 const uint32_t seg = P::SEGS == 1 ? 0u : (table[t][i] >> 7) * seg_bytes;
                 const int k = (i >> 1) * 4 + (i & 1);
-                if (WHOLE) {
+                if (NM_SELF_CHECKING) {
+                    for (int e = 0; e < 4; ++e) {
+                        const uint32_t a = ((WHOLE ? r[0] : r[e]) ^ at) + seg + (WHOLE ? e * 1024u : 0u);
+                        v[t][e >> 1][k + (e & 1) * 2] = in_slot(a) ? lds32<0>(a) : 0u;
+                    }
+                } else if (WHOLE) {
                     const uint32_t a = (r[0] ^ at) + seg;
                     v[t][0][k] = lds32<0>(a);
                     v[t][0][k + 2] = lds32<1024>(a);
@@ -670,17 +677,15 @@ k_conv_select(const ConvParams p, const SelCfg cfg, const __grid_constant__ CUte
                         const uint32_t phase = (row & 7u) << 4, bit = 1u << tap;
                         uint32_t rows[4] = {act + row * 128u + phase};
                         const uint32_t table_at = tab + s * (P::KC * 4);
-                        // self-checking build: the rows lie in the slot
-                        NM_CHECKED(rows[0] + 3072u <= act + static_cast<uint32_t>(cfg.seg_bytes) && rows[0] >= act, p.status, 802, row) {}
                         if (all & bit) {
-                            piece.template load<true>(rows, table_at, cfg.seg_bytes);
+                            piece.template load<true>(rows, table_at, cfg.seg_bytes, act, p.status);
                         } else {
                             const uint32_t zero = act + cfg.prow * 128u + (phase << 3) + phase;
                             rows[1] = v1 & bit ? rows[0] + 1024u : zero;
                             rows[2] = v2 & bit ? rows[0] + 2048u : zero;
                             rows[3] = v3 & bit ? rows[0] + 3072u : zero;
                             rows[0] = v0 & bit ? rows[0] : zero;
-                            piece.template load<false>(rows, table_at, cfg.seg_bytes);
+                            piece.template load<false>(rows, table_at, cfg.seg_bytes, act, p.status);
                         }
                         if (s == 0) set_free();
                         piece.store(dst + s * P::KC);
@@ -705,7 +710,7 @@ k_conv_select(const ConvParams p, const SelCfg cfg, const __grid_constant__ CUte
                         __syncwarp();
                         if (mine) {
                             const uint32_t row = act + first_row * 128u + ((lane >> 2) << 4);
-                            piece.template load<true>(&row, tab + s * (P::KC * 4), cfg.seg_bytes);
+                            piece.template load<true>(&row, tab + s * (P::KC * 4), cfg.seg_bytes, act, p.status);
                             if (s == 0) set_free();
                             piece.store(dst + s * P::KC);
                         }

@@ -98,6 +98,18 @@ __device__ __forceinline__ void nm_add4(float4& a, const float4& b)
 }
 #endif
 
+// What the self-checking build checks: a tap-table entry names a tap and a channel of the layer; `bytes` bytes at `at` lie in [lo, hi).
+#ifdef __CUDACC__
+#define NM_HOST_DEVICE __host__ __device__
+#else
+#define NM_HOST_DEVICE
+#endif
+NM_HOST_DEVICE constexpr bool nm_tap_in_layer(uint32_t tap, int kh, int kw, int c_in)
+{
+    return static_cast<int>(tap >> 24) < kh && static_cast<int>((tap >> 16) & 0xFFu) < kw && static_cast<int>(tap & 0xFFFFu) < c_in;
+}
+NM_HOST_DEVICE constexpr bool nm_bytes_in_span(uint64_t at, uint64_t bytes, uint64_t lo, uint64_t hi) { return at >= lo && at + bytes <= hi; }
+
 #ifdef __CUDACC__
 // Self-checking build (-DNM_DEBUG_BOUNDS): the kernels that compute addresses from index data range-check
 // every such address; a violation is recorded in the handle's status word (error code NM_ERR_INTERNAL, the
@@ -113,8 +125,13 @@ __device__ __forceinline__ void nm_debug_violation(int* status, int site, uint32
 }
 #define NM_CHECKED(cond, status, site, value) \
     if (!(cond)) nm_debug_violation((status), (site), static_cast<uint32_t>(value)); else
+// `cond` where it decides whether an access is made: false, and recorded, on a violation.
+#define NM_ALLOWED(cond, status, site, value) ((cond) || (nm_debug_violation((status), (site), static_cast<uint32_t>(value)), false))
+constexpr bool NM_SELF_CHECKING = true;
 #else
 #define NM_CHECKED(cond, status, site, value)
+#define NM_ALLOWED(cond, status, site, value) true
+constexpr bool NM_SELF_CHECKING = false;
 #endif
 #endif
 

@@ -1,19 +1,41 @@
-"""Which memory the handle-building kernels may touch: a rule of the host code, compiled here without a device."""
+"""Rules of the library's code that need no device, compiled here for the host: which memory the handle-building kernels may
+touch, and what the self-checking build lets an access pass by."""
 import os
+import re
 import subprocess
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CUDA = os.environ.get("CUDA_HOME", "/usr/local/cuda")
 
 
+def _run(tmp_path, body):
+    src, exe = tmp_path / "rule.cpp", tmp_path / "rule"
+    src.write_text('#include <cstdio>\n#include "nm_internal.h"\nint main()\n{\n' + body + "}\n")
+    subprocess.check_call(["g++", "-std=c++17", f"-I{ROOT}/paper_2507_17301_b200/csrc", f"-I{CUDA}/include", "-o", str(exe), str(src)])
+    return subprocess.check_output([str(exe)], text=True)
+
+
 def test_kernels_touch_memory_of_their_own_device_only(tmp_path):
     """Export from a handle of another GPU, and import of arrays that lie there, go through copies."""
-    src = tmp_path / "rule.cpp"
-    src.write_text('#include <cstdio>\n#include "nm_internal.h"\nint main()\n{\n'
-                   "    for (cudaMemoryType t : {cudaMemoryTypeUnregistered, cudaMemoryTypeHost, cudaMemoryTypeDevice, cudaMemoryTypeManaged})\n"
-                   "        for (int owner : {-2, 0, 1})\n"
-                   '            for (int current : {0, 1}) std::printf("%d", nmhost::kernel_may_touch(t, owner, current) ? 1 : 0);\n}\n')
-    exe = tmp_path / "rule"
-    subprocess.check_call(["g++", "-std=c++17", f"-I{ROOT}/paper_2507_17301_b200/csrc", f"-I{CUDA}/include", "-o", str(exe), str(src)])
-    out = subprocess.check_output([str(exe)], text=True)
+    out = _run(tmp_path,
+               "    for (cudaMemoryType t : {cudaMemoryTypeUnregistered, cudaMemoryTypeHost, cudaMemoryTypeDevice, cudaMemoryTypeManaged})\n"
+               "        for (int owner : {-2, 0, 1})\n"
+               '            for (int current : {0, 1}) std::printf("%d", nmhost::kernel_may_touch(t, owner, current) ? 1 : 0);\n')
     assert out == "000000" + "000000" + "001001" + "111111"     # unregistered, pinned, device (own device only), managed
+
+
+def test_what_the_self_checking_build_lets_pass(tmp_path):
+    out = _run(tmp_path,
+               "    for (uint32_t tap : {0u, (2u << 24) | (1u << 16) | 7u, 3u << 24, 2u << 16, 8u, 0xFFFFFFFFu})\n"
+               '        std::printf("%d", nm_tap_in_layer(tap, 3, 2, 8) ? 1 : 0);\n'
+               '    std::printf(" ");\n'
+               "    for (uint64_t at : {99ull, 100ull, 196ull, 197ull, 200ull, 0xFFFFFFFFull})\n"
+               '        std::printf("%d", nm_bytes_in_span(at, 4, 100, 200) ? 1 : 0);\n')
+    assert out == "110000 011000"
+
+
+def test_no_check_of_the_self_checking_build_guards_an_empty_statement():
+    """A check that is not part of the access's condition records a bad address and reads it all the same."""
+    for name in os.listdir(f"{ROOT}/paper_2507_17301_b200/csrc"):
+        with open(f"{ROOT}/paper_2507_17301_b200/csrc/{name}") as f:
+            assert not re.search(r"NM_CHECKED\([^;{]*\)\s*\{\s*\}", f.read()), name
