@@ -1,5 +1,5 @@
 """The direct-gather kernel (plan.variant = 1) against the CPU oracle, bit for bit on integer inputs: tile widths below, at and
-above a staging pass, odd ones, tails of tiles and channels, tap counts on both sides of the mask, one to eight ranges of the
+above a staging pass, odd ones, tails of tiles and channels, tap counts up to the mask's 64 and above (bounds by comparison), one to eight ranges of the
 chunks, several passes per CTA, ragged pixel blocks that span images, the fused shortcut."""
 import numpy as np
 import pytest
@@ -33,6 +33,13 @@ SHAPES = [
     ConvShape("split_7x7", 1, 9, 9, 30, 20, 7, 7, 1, 3, 1, 2, 4, 20),
     ConvShape("many_tiles", 6, 60, 60, 18, 72, 1, 1, 1, 0, 1, 2, 4, 4),           # 18 tiles
     ConvShape("wide_kept", 2, 30, 30, 10, 16, 3, 3, 1, 1, 1, 10, 10, 16),         # nothing pruned
+    ConvShape("k8x8", 2, 13, 12, 6, 20, 8, 8, 1, 4, 1, 2, 4, 8),                  # 64 taps: the mask's last bit
+    ConvShape("k9x9_s2", 2, 21, 19, 4, 24, 9, 9, 2, 4, 1, 2, 4, 8),               # 81 taps from here on: no mask
+    ConvShape("k5x13_dil", 1, 24, 40, 7, 12, 5, 13, 1, 6, 2, 2, 7, 5),
+    ConvShape("k1x65", 1, 3, 70, 3, 8, 1, 65, 1, 0, 1, 1, 3, 8),
+    ConvShape("k9x9_images", 30, 5, 5, 6, 36, 9, 9, 1, 4, 1, 1, 4, 12),           # a block of 128 pixels spans six images, the last block ragged
+    ConvShape("k9x9_split8", 1, 9, 9, 40, 72, 9, 9, 1, 4, 1, 2, 4, 72),           # 51 chunks over a cluster, two passes
+    ConvShape("k11x11_split", 3, 14, 15, 16, 30, 11, 11, 2, 5, 1, 1, 8, 30),
 ]
 
 
