@@ -254,8 +254,13 @@ nm_status_t nm_weights_reserve(nm_weights_t* w, size_t bytes);
  * cleared, the context stays usable). */
 nm_status_t nm_weights_check(const nm_weights_t* w, void* cuda_stream);
 
-/* Releases the handle and its device memory (synchronises the device first). NULL is accepted. */
+/* Releases the handle (synchronises its device first). NULL is accepted.  Its device memory may serve the next handle: the
+ * process keeps at most 256 MB of freed handles' memory, none that the last 64 frees have not wanted, and gives all of it
+ * back before an allocation of the library fails. */
 nm_status_t nm_weights_free(nm_weights_t* w);
+
+/* Gives the memory kept from freed handles back to the driver (for the process's other allocators). */
+nm_status_t nm_memory_trim(void);
 
 /* ---------------------------------------------------------------------------------------------
  * Convolution

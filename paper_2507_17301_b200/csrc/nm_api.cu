@@ -90,6 +90,22 @@ nm_status_t make_handle(const char* who, int c_out, int kh, int kw, int c_in, in
     return NM_OK;
 }
 
+// Makes a handle's device the current one, where it is not, for as long as the object lives.
+struct OnDevice {
+    int before = -1;
+    explicit OnDevice(int device)
+    {
+        int dev = device;
+        if (cudaGetDevice(&dev) == cudaSuccess && dev != device && cudaSetDevice(device) == cudaSuccess) before = dev;
+    }
+    ~OnDevice()
+    {
+        if (before >= 0) cudaSetDevice(before);
+    }
+    OnDevice(const OnDevice&) = delete;
+    OnDevice& operator=(const OnDevice&) = delete;
+};
+
 bool valid(const nm_weights* w) { return w && w->magic == NM_MAGIC; }
 
 // Checks a conv call and fills the kernel parameters.
@@ -410,16 +426,15 @@ nm_status_t nm_weights_reserve(nm_weights_t* w, size_t bytes)
 {
     if (!valid(w)) return nmhost::fail(NM_ERR_INVALID_ARG, "nm_weights_reserve: bad weights handle");
     if (bytes <= w->splitk_bytes) return NM_OK;
+    const OnDevice on(w->device);
     cudaDeviceSynchronize();
     cudaFree(w->splitk);
     w->splitk = nullptr;
     w->splitk_bytes = 0;
-    if (cudaMalloc(&w->splitk, bytes) != cudaSuccess) {
-        (void)cudaGetLastError();
+    if (nmhost::device_malloc(reinterpret_cast<void**>(&w->splitk), bytes) != cudaSuccess)
         return nmhost::fail(NM_ERR_ALLOC, "nm_weights_reserve: cannot allocate %zu bytes", bytes);
-    }
-    // balanced plans keep flag words in the scratch: they start cleared
-    if (cudaMemset(w->splitk, 0, bytes) != cudaSuccess) {
+    // balanced plans keep flag words in the scratch: they start cleared, before a launch on any stream can read them
+    if (cudaMemset(w->splitk, 0, bytes) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) {
         (void)cudaGetLastError();
         cudaFree(w->splitk);
         w->splitk = nullptr;
@@ -452,12 +467,15 @@ nm_status_t nm_weights_free(nm_weights_t* w)
 {
     if (!w) return NM_OK;
     if (!valid(w)) return nmhost::fail(NM_ERR_INVALID_ARG, "nm_weights_free: bad weights handle");
-    // the device the handle lives on, which need not be the current one
-    int dev = w->device;
-    const bool moved = cudaGetDevice(&dev) == cudaSuccess && dev != w->device && cudaSetDevice(w->device) == cudaSuccess;
+    const OnDevice on(w->device);
     const bool idle = cudaDeviceSynchronize() == cudaSuccess;
     free_handle_memory(w, idle);
-    if (moved) cudaSetDevice(dev);
+    return NM_OK;
+}
+
+nm_status_t nm_memory_trim(void)
+{
+    nmhost::device_blocks_trim();
     return NM_OK;
 }
 
@@ -602,10 +620,7 @@ nm_status_t nm_autotune(nm_weights_t* w, const float* x, int batch, int h, int w
     const bool near = 4.0 * (static_cast<double>(batch) * h * wd * w->c_in + static_cast<double>(p.pixels) * w->c_out) <= kNearBytes;
     constexpr size_t kFlushBytes = size_t(288) << 20;
     void* flush = nullptr;
-    if (cudaMalloc(&flush, kFlushBytes) != cudaSuccess) {
-        (void)cudaGetLastError();
-        flush = nullptr;
-    }
+    (void)nmhost::device_malloc(&flush, kFlushBytes);   // (NULL where there is no room)
     constexpr int kWarm = 2, kReps = 9, kBurstReps = 5;
     float best_t = -1.f;
     // plan cache: a cached plan that still runs on this layer is returned with its time over three launches

@@ -176,6 +176,8 @@ bool kernel_may_touch(const void* a, const void* b, int device);   // both of th
 // nm_layout.cu: the handles' device memory, and the kernel-side copies of the compressed form
 void* device_block_alloc(size_t bytes, int device, size_t* got);   // NULL when there is no memory; reuses blocks of freed handles
 void device_block_free(void* ptr, size_t bytes, int device, bool idle);   // idle: nothing on the device uses it any more
+void device_blocks_trim();                                 // gives back every block kept for later handles
+cudaError_t device_malloc(void** ptr, size_t bytes);       // cudaMalloc, tried again after a trim
 nm_status_t alloc_handle_memory(nm_weights* h, const char* who);
 nm_status_t clear_handle_memory(nm_weights* h, cudaStream_t st);   // the part of the block that is not written in full
 // Values and layouts from the index array `idx` and the dense weights (import = false) or the retained values (true).

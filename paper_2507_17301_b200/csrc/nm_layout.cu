@@ -4,7 +4,8 @@
 // convolution kernels read are carved out of it.  (Fourteen cudaMalloc / cudaFree calls per handle used to be nearly all of
 // nm_prune's time: 3.1 ms for a 512 x 3 x 3 x 512 layer whose kernels take about 0.1 ms.)  Blocks of freed handles
 // are kept for the next one, within bounds: at most kCacheBytes per process, none that kCacheAge later frees did not
-// want, all of them returned to the driver before an allocation is reported as failed.  A block enters the cache only
+// want, all of them returned to the driver before an allocation of the library is reported as failed and when
+// nm_memory_trim asks for it.  A block enters the cache only
 // after its device has been synchronised, so whoever takes it next may use it on any stream; the list is guarded by a
 // mutex.
 //
@@ -46,6 +47,11 @@ void drop(size_t i)
     cudaFree(g_cache[i].ptr);
     g_cached -= g_cache[i].bytes;
     g_cache.erase(g_cache.begin() + static_cast<long>(i));
+}
+
+void drop_all()
+{
+    while (!g_cache.empty()) drop(g_cache.size() - 1);
 }
 
 // Pinned words for the few bytes a creating call reads back (L1 masses, validity): pageable memory would make the
@@ -247,7 +253,7 @@ void* device_block_alloc(size_t bytes, int device, size_t* got)
     void* p = nullptr;
     if (cudaMalloc(&p, want) != cudaSuccess) {
         (void)cudaGetLastError();
-        while (!g_cache.empty()) drop(g_cache.size() - 1);   // everything kept goes back before giving up
+        drop_all();   // before giving up
         if (cudaMalloc(&p, want) != cudaSuccess) {
             (void)cudaGetLastError();
             return nullptr;
@@ -255,6 +261,27 @@ void* device_block_alloc(size_t bytes, int device, size_t* got)
     }
     *got = want;
     return p;
+}
+
+void device_blocks_trim()
+{
+    std::lock_guard<std::mutex> lock(g_mu);
+    drop_all();
+}
+
+cudaError_t device_malloc(void** ptr, size_t bytes)
+{
+    cudaError_t e = cudaMalloc(ptr, bytes);
+    if (e != cudaSuccess) {
+        (void)cudaGetLastError();
+        device_blocks_trim();
+        e = cudaMalloc(ptr, bytes);
+        if (e != cudaSuccess) {
+            (void)cudaGetLastError();
+            *ptr = nullptr;
+        }
+    }
+    return e;
 }
 
 void device_block_free(void* ptr, size_t bytes, int device, bool idle)

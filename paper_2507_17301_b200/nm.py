@@ -85,6 +85,8 @@ def _load():
     lib.nm_plan_cache_store.restype = ctypes.c_int
     lib.nm_plan_cache_lookup.argtypes = [ctypes.c_char_p, ctypes.c_char_p, pp]
     lib.nm_plan_cache_lookup.restype = ctypes.c_int
+    lib.nm_memory_trim.argtypes = []
+    lib.nm_memory_trim.restype = ctypes.c_int
     lib.nm_status_string.argtypes = [ctypes.c_int]
     lib.nm_status_string.restype = ctypes.c_char_p
     lib.nm_last_error.argtypes = []
@@ -103,7 +105,7 @@ except ImportError as e:
                       f"(there is no fallback path without it): {e}") from e
 _nm_binding.bind(*(ctypes.cast(f, ctypes.c_void_p).value for f in (_lib.nm_conv2d, _lib.nm_conv2d_res, _lib.nm_maxpool2d)))
 
-EXPORTS = ("nm_plan_key", "nm_plan_cache_store", "nm_plan_cache_lookup", "nm_selftest_wait_expiry", "nm_maxpool2d", "nm_weights_retained_l1", "nm_conv2d_res", "nm_plan_scratch_bytes", "nm_weights_reserve", "nm_prune", "nm_prune_noalloc", "nm_weights_dims", "nm_weights_export", "nm_weights_import", "nm_weights_check",
+EXPORTS = ("nm_memory_trim", "nm_plan_key", "nm_plan_cache_store", "nm_plan_cache_lookup", "nm_selftest_wait_expiry", "nm_maxpool2d", "nm_weights_retained_l1", "nm_conv2d_res", "nm_plan_scratch_bytes", "nm_weights_reserve", "nm_prune", "nm_prune_noalloc", "nm_weights_dims", "nm_weights_export", "nm_weights_import", "nm_weights_check",
            "nm_weights_free", "nm_conv2d", "nm_conv2d_host", "nm_autotune", "nm_autotune_tile",
            "nm_status_string", "nm_last_error", "nm_launch_count")
 
@@ -236,6 +238,11 @@ def nm_plan_scratch_bytes(w: Weights, x_shape, stride, pad, dil, plan: nm_plan_t
 def nm_weights_reserve(w: Weights, nbytes: int):
     """Reserves handle-owned scratch memory (allocates; call outside the timed / captured region)."""
     _check(_lib.nm_weights_reserve(w.handle, nbytes))
+
+
+def nm_memory_trim():
+    """Gives the device memory kept from freed handles back to the driver."""
+    _check(_lib.nm_memory_trim())
 
 
 def nm_maxpool2d(x: torch.Tensor, kernel=3, stride=2, pad=1, y: torch.Tensor | None = None) -> torch.Tensor:
