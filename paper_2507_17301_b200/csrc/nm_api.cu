@@ -578,9 +578,14 @@ nm_status_t nm_plan_cache_lookup(const char* path, const char* key, nm_plan_t* p
     return NM_OK;
 }
 
-nm_status_t nm_autotune(nm_weights_t* w, const float* x, int batch, int h, int wd, int stride_h, int stride_w,
-                        int pad_h, int pad_w, int dil_h, int dil_w, const float* bias, int relu, float* y_scratch,
-                        void* cuda_stream, nm_plan_t* best, float* best_ms)
+}  // extern "C"
+
+namespace {
+
+// nm_autotune; *rank_ms (may be NULL): the time by which the candidates were compared, for a cached plan measured in the same way.
+nm_status_t tune(nm_weights_t* w, const float* x, int batch, int h, int wd, int stride_h, int stride_w, int pad_h, int pad_w,
+                 int dil_h, int dil_w, const float* bias, int relu, float* y_scratch, void* cuda_stream, nm_plan_t* best,
+                 float* best_ms, float* rank_ms)
 {
     if (!best) return nmhost::fail(NM_ERR_INVALID_ARG, "nm_autotune: best is NULL");
     ConvParams p;
@@ -623,6 +628,33 @@ nm_status_t nm_autotune(nm_weights_t* w, const float* x, int batch, int h, int w
     (void)nmhost::device_malloc(&flush, kFlushBytes);   // (NULL where there is no room)
     constexpr int kWarm = 2, kReps = 9, kBurstReps = 5;
     float best_t = -1.f;
+    // One launch, cold, or the mean of a burst; false when a launch fails.
+    auto measure = [&](const nm_plan_t& plan, int launches, std::vector<float>* t) {
+        if (launches == 1 && flush) cudaMemsetAsync(flush, static_cast<int>(t->size()), kFlushBytes, st);
+        cudaEventRecord(e0, st);
+        bool ok = true;
+        for (int k = 0; k < launches && ok; ++k) ok = run_plan(p, &plan, st) == NM_OK;
+        cudaEventRecord(e1, st);
+        if (cudaEventSynchronize(e1) != cudaSuccess) ok = false;
+        float ms = 0.f;
+        if (ok && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess) t->push_back(ms / static_cast<float>(launches));
+        return ok;
+    };
+    // Median over a plan's launches or bursts, by which candidates are compared; negative when it does not run.  `reach`: three
+    // launches, or one burst, tell a candidate that is slower than this (tuning a layer takes half the time this way).
+    auto rank = [&](const nm_plan_t& plan, float reach) {
+        bool ok = true;
+        for (int i = 0; i < kWarm && ok; ++i) ok = run_plan(p, &plan, st) == NM_OK;
+        if (!ok || cudaStreamSynchronize(st) != cudaSuccess) return -1.f;
+        std::vector<float> t;
+        for (int i = 0; i < (near ? kBurstReps : kReps) && ok; ++i) {
+            if (t.size() == (near ? 1u : 3u) && reach > 0.f && *std::min_element(t.begin(), t.end()) > reach) break;
+            ok = measure(plan, near ? kBurst : 1, &t);
+        }
+        if (!ok || t.empty()) return -1.f;
+        std::sort(t.begin(), t.end());
+        return t[t.size() / 2];
+    };
     // plan cache: a cached plan that still runs on this layer is returned with its time over three launches
     char key[384] = "";
     const char* cache = std::getenv("NM_PLAN_CACHE");
@@ -647,6 +679,7 @@ nm_status_t nm_autotune(nm_weights_t* w, const float* x, int batch, int h, int w
                 if (ok) {
                     *best = cached;
                     if (best_ms) *best_ms = ms / 3.f;
+                    if (rank_ms) *rank_ms = rank(cached, -1.f);
                     if (flush) cudaFree(flush);
                     cudaEventDestroy(e0);
                     cudaEventDestroy(e1);
@@ -656,37 +689,16 @@ nm_status_t nm_autotune(nm_weights_t* w, const float* x, int batch, int h, int w
             (void)cudaGetLastError();
         }
     }
-    // One launch, cold, or the mean of a burst; false when a launch fails.
-    auto measure = [&](const nm_plan_t& plan, int launches, std::vector<float>* t) {
-        if (launches == 1 && flush) cudaMemsetAsync(flush, static_cast<int>(t->size()), kFlushBytes, st);
-        cudaEventRecord(e0, st);
-        bool ok = true;
-        for (int k = 0; k < launches && ok; ++k) ok = run_plan(p, &plan, st) == NM_OK;
-        cudaEventRecord(e1, st);
-        if (cudaEventSynchronize(e1) != cudaSuccess) ok = false;
-        float ms = 0.f;
-        if (ok && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess) t->push_back(ms / static_cast<float>(launches));
-        return ok;
-    };
     for (const nm_plan_t& cand : candidate_plans(w, p)) {
-        bool ok = true;
-        for (int i = 0; i < kWarm && ok; ++i) ok = run_plan(p, &cand, st) == NM_OK;
-        if (!ok || cudaStreamSynchronize(st) != cudaSuccess) continue;
-        std::vector<float> t;
-        for (int i = 0; i < (near ? kBurstReps : kReps) && ok; ++i) {
-            // three launches, or one burst, tell a candidate that is out of reach (tuning a layer takes half the time this way)
-            if (t.size() == (near ? 1u : 3u) && best_t > 0.f && *std::min_element(t.begin(), t.end()) > 1.25f * best_t) break;
-            ok = measure(cand, near ? kBurst : 1, &t);
-        }
-        if (!ok || t.empty()) continue;
-        std::sort(t.begin(), t.end());
-        const float med = t[t.size() / 2];
+        const float med = rank(cand, best_t > 0.f ? 1.25f * best_t : -1.f);
+        if (med < 0.f) continue;
         // candidates come most promising first: a later one must win by more than the timing noise
         if (best_t < 0.f || med < best_t * 0.99f) {
             best_t = med;
             *best = cand;
         }
     }
+    if (rank_ms) *rank_ms = best_t;
     if (near && best_t >= 0.f) {
         std::vector<float> t;
         for (int i = 0; i < kReps; ++i)
@@ -705,6 +717,18 @@ nm_status_t nm_autotune(nm_weights_t* w, const float* x, int batch, int h, int w
     return nm_weights_check(w, cuda_stream);
 }
 
+}  // namespace
+
+extern "C" {
+
+nm_status_t nm_autotune(nm_weights_t* w, const float* x, int batch, int h, int wd, int stride_h, int stride_w,
+                        int pad_h, int pad_w, int dil_h, int dil_w, const float* bias, int relu, float* y_scratch,
+                        void* cuda_stream, nm_plan_t* best, float* best_ms)
+{
+    return tune(w, x, batch, h, wd, stride_h, stride_w, pad_h, pad_w, dil_h, dil_w, bias, relu, y_scratch, cuda_stream, best, best_ms,
+                nullptr);
+}
+
 nm_status_t nm_autotune_tile(const float* w_dense, int c_out, int kh, int kw, int c_in, int n_keep, int m_group,
                              const int* tile_candidates, int n_candidates, const float* x, int batch, int h, int wd,
                              int stride_h, int stride_w, int pad_h, int pad_w, int dil_h, int dil_w, const float* bias,
@@ -713,26 +737,28 @@ nm_status_t nm_autotune_tile(const float* w_dense, int c_out, int kh, int kw, in
 {
     if (!tile_candidates || n_candidates < 1 || !best_tile || !best)
         return nmhost::fail(NM_ERR_INVALID_ARG, "nm_autotune_tile: candidates / outputs missing");
-    float best_t = -1.f;
+    float best_t = -1.f, reported = 0.f;
     nm_status_t last = NM_ERR_UNSUPPORTED;
     for (int i = 0; i < n_candidates; ++i) {
         nm_weights_t* hnd = nullptr;
         last = nm_prune(w_dense, c_out, kh, kw, c_in, n_keep, m_group, tile_candidates[i], cuda_stream, &hnd);
         if (last != NM_OK) continue;
         nm_plan_t plan;
-        float ms = 0.f;
-        last = nm_autotune(hnd, x, batch, h, wd, stride_h, stride_w, pad_h, pad_w, dil_h, dil_w, bias, relu, y_scratch,
-                           cuda_stream, &plan, &ms);
+        float ms = 0.f, rank_ms = -1.f;
+        last = tune(hnd, x, batch, h, wd, stride_h, stride_w, pad_h, pad_w, dil_h, dil_w, bias, relu, y_scratch, cuda_stream, &plan, &ms,
+                    &rank_ms);
         nm_weights_free(hnd);
-        if (last != NM_OK) continue;
-        if (best_t < 0.f || ms < best_t) {
-            best_t = ms;
+        if (last != NM_OK || rank_ms < 0.f) continue;
+        // widths are compared by what their plans were compared by, not by the reported time (cold, or a cached plan's few launches)
+        if (best_t < 0.f || rank_ms < best_t) {
+            best_t = rank_ms;
+            reported = ms;
             *best_tile = tile_candidates[i];
             *best = plan;
         }
     }
     if (best_t < 0.f) return last == NM_OK ? nmhost::fail(NM_ERR_UNSUPPORTED, "nm_autotune_tile: nothing ran") : last;
-    if (best_ms) *best_ms = best_t;
+    if (best_ms) *best_ms = reported;
     return NM_OK;
 }
 
