@@ -155,7 +155,7 @@ nm_status_t run_plan(const ConvParams& p, const nm_plan_t* plan, cudaStream_t st
     const int variant = plan ? plan->variant : 0;
     switch (variant) {
         case 0:
-            // (all of these round activations to nearest and never read a pruned column)
+            // (the row-run and plane kernels truncate activations and multiply zeros for pruned columns, the others do neither)
             if (nmhost::stream_plan_ok(p, nullptr) && !nmhost::stream_leaves_sms_idle(p)) return nmhost::launch_conv_stream(p, nullptr, st);
             if (nmhost::planes_plan_ok(p, nullptr)) return nmhost::launch_conv_planes(p, nullptr, st);
             // Channel counts that are no multiple of 32: runs of rows where there is enough work for their set-up.  Units of a pixel
@@ -163,6 +163,7 @@ nm_status_t run_plan(const ConvParams& p, const nm_plan_t* plan, cudaStream_t st
             // 2) 14.4 / 16.4; 1176 (4x56x56, 24->96) 10.1 / 8.3, 784 (2x112x112, 5->32, 7x7 by 2) 6.9 / 5.5.
             if (p.c_in % 32 != 0 && (p.pixels + 127) / 128 * p.n_tiles * (p.kk_pad / NM_KCHUNK) >= 1400 && nmhost::rowrun_plan_ok(p, nullptr))
                 return nmhost::launch_conv_rowrun(p, nullptr, st);
+            if (nmhost::slab_beats_gather(p)) return nmhost::launch_conv_slab(p, nullptr, st);
             return nmhost::launch_conv_gather(p, st);
         case 1:
             return nmhost::launch_conv_gather(p, st);
@@ -301,6 +302,16 @@ nm_status_t fail(nm_status_t s, const char* fmt, ...)
     vsnprintf(g_err, sizeof(g_err), fmt, ap);
     va_end(ap);
     return s;
+}
+int sm_count()
+{
+    static const int n = [] {
+        int dev = 0, v = 0;
+        if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0)
+            return v;
+        return 148;
+    }();
+    return n;
 }
 bool pdl_enabled()
 {

@@ -331,17 +331,6 @@ k_conv_cluster(const ConvParams p, const ClusterCfg cfg, const __grid_constant__
     if (warp == 1) tmem_dealloc(tmem, tmem_cols);
 }
 
-int sm_count()
-{
-    static const int n = [] {
-        int dev = 0, v = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0)
-            return v;
-        return 148;
-    }();
-    return n;
-}
-
 bool make_cfg(const ConvParams& p, const nm_plan_t* plan, ClusterCfg* cfg, size_t* smem)
 {
     if (!p.wx || !nmtm::available()) return false;
@@ -404,7 +393,7 @@ bool make_cfg(const ConvParams& p, const nm_plan_t* plan, ClusterCfg* cfg, size_
     if (*smem < share) *smem = share;
     if (*smem < NM_BESIDE_EXCLUSIVE) *smem = NM_BESIDE_EXCLUSIVE;
     // Short launches only: with many rounds of CTAs the persistent kernels keep the tensor core busier.
-    return static_cast<long long>(cfg->tiles) * cfg->n_slices * cfg->cs <= 12ll * sm_count();
+    return static_cast<long long>(cfg->tiles) * cfg->n_slices * cfg->cs <= 12ll * nmhost::sm_count();
 }
 
 bool encode_x(const ConvParams& p, const ClusterCfg& cfg, CUtensorMap* tm)

@@ -718,20 +718,6 @@ __global__ void k_splitk_reduce(const float4* __restrict__ part, int splits, siz
     }
 }
 
-int sm_count()
-{
-    static int n = 0;
-    if (n == 0) {
-        int dev = 0, v = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess &&
-            cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0)
-            n = v;
-        else
-            n = 148;
-    }
-    return n;
-}
-
 bool make_cfg(const ConvParams& p, const nm_plan_t* plan, ExpandCfg* cfg)
 {
     if (!p.wx || !nmtm::available()) return false;
@@ -781,7 +767,7 @@ bool make_cfg(const ConvParams& p, const nm_plan_t* plan, ExpandCfg* cfg)
     // multiple of the slice count.
     cfg->wres_bytes = 0;
     cfg->w_res = 0;
-    if (splits == 1 && !balanced && !(plan && plan->split == 1) && blk32 * cfg->b_bytes <= WRES_MAX && cfg->n_slices <= sm_count()) {
+    if (splits == 1 && !balanced && !(plan && plan->split == 1) && blk32 * cfg->b_bytes <= WRES_MAX && cfg->n_slices <= nmhost::sm_count()) {
         cfg->w_res = 1;
         cfg->wres_bytes = blk32 * cfg->b_bytes;
         if (cfg->wres_bytes > 64 * 1024) cfg->boxes = 1;   // a large slice: give the output staging's room to the ring
@@ -791,7 +777,7 @@ bool make_cfg(const ConvParams& p, const nm_plan_t* plan, ExpandCfg* cfg)
     long long tiles = (p.pixels + BM - 1) / BM;
     if (splits == 1 && !balanced) {
         // fewest pixels per item (in steps of 8) that the same number of rounds covers
-        const long long ctas = cfg->w_res ? sm_count() / cfg->n_slices * cfg->n_slices : sm_count();
+        const long long ctas = cfg->w_res ? nmhost::sm_count() / cfg->n_slices * cfg->n_slices : nmhost::sm_count();
         const long long rounds = (tiles * cfg->n_slices + ctas - 1) / ctas;
         const long long most = rounds * ctas / cfg->n_slices;   // pixel tiles that fit into them
         cfg->rows = static_cast<int>(((p.pixels + most - 1) / most + 7) / 8 * 8);
@@ -840,7 +826,7 @@ bool make_cfg(const ConvParams& p, const nm_plan_t* plan, ExpandCfg* cfg)
     if (balanced) {
         // one range per SM; needs at least one (item, stage) unit per CTA and the per-CTA slots + flags in the scratch
         const long long units = cfg->n_work * cfg->n_sub;
-        if (units < sm_count() || units >= (1ll << 31)) return false;
+        if (units < nmhost::sm_count() || units >= (1ll << 31)) return false;
         if (!p.splitk || p.splitk_bytes < nmhost::expand_balanced_bytes(bn)) return false;
         cfg->balanced = 1;
     }
@@ -854,7 +840,7 @@ namespace nmhost {
 size_t expand_balanced_bytes(int bn)
 {
     // per SM: a slot of 128 rows x bn partial sums, and eight flag words (one per epilogue warp)
-    return static_cast<size_t>(sm_count()) * (static_cast<size_t>(BM) * bn * sizeof(float) + 8 * sizeof(uint32_t));
+    return static_cast<size_t>(nmhost::sm_count()) * (static_cast<size_t>(BM) * bn * sizeof(float) + 8 * sizeof(uint32_t));
 }
 
 bool expand_plan_ok(const ConvParams& p, const nm_plan_t* plan)
@@ -897,8 +883,8 @@ nm_status_t launch_conv_expand(const ConvParams& p, const nm_plan_t* plan, cudaS
                                        : (cfg.kblk == 2 ? k_conv_expand<2, false> : k_conv_expand<1, false>);
     cudaError_t e = nmhost::ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), smem);
     if (e != cudaSuccess) return fail(NM_ERR_CUDA, "cudaFuncSetAttribute (variant 4): %s", cudaGetErrorString(e));
-    long long grid = cfg.n_work < sm_count() ? cfg.n_work : sm_count();
-    if (cfg.balanced) grid = sm_count();
+    long long grid = cfg.n_work < nmhost::sm_count() ? cfg.n_work : nmhost::sm_count();
+    if (cfg.balanced) grid = nmhost::sm_count();
     if (cfg.w_res) grid = (grid / cfg.n_slices) * cfg.n_slices;   // n_work is a multiple of n_slices, so grid >= n_slices
     e = nmhost::launch_pdl(kernel, static_cast<unsigned>(grid), THREADS, smem, st, q, cfg, tm_x, tm_y, tm_tail, tm_res);
     nmhost::count_launch(1);
@@ -913,7 +899,7 @@ nm_status_t launch_splitk_reduce(const ConvParams& p, int splits, int p_pad, cud
     const size_t n4 = static_cast<size_t>(p.pixels) * p.c_out / 4;
     const size_t stride4 = static_cast<size_t>(p_pad) * p.c_out / 4;
     size_t blocks = (n4 + 255) / 256;
-    if (blocks > static_cast<size_t>(sm_count()) * 8) blocks = static_cast<size_t>(sm_count()) * 8;
+    if (blocks > static_cast<size_t>(nmhost::sm_count()) * 8) blocks = static_cast<size_t>(nmhost::sm_count()) * 8;
     cudaError_t e = nmhost::launch_pdl(k_splitk_reduce, static_cast<unsigned>(blocks), 256u, 0, st,
                                        reinterpret_cast<const float4*>(p.splitk), splits, stride4, n4, p.c_out / 4,
                                        reinterpret_cast<const float4*>(p.bias), reinterpret_cast<const float4*>(p.residual),

@@ -425,20 +425,15 @@ __global__ void __launch_bounds__(THREADS, 2) k_conv_gather(const ConvParams p, 
     if (warp == 8) tmem_dealloc(tmem, cfg.tmem_cols);
 }
 
-int sm_count()
-{
-    static const int n = [] {
-        int dev = 0, v = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0)
-            return v;
-        return 148;
-    }();
-    return n;
-}
-
 }  // namespace
 
 namespace nmhost {
+
+double gather_time_us(const ConvParams& p)
+{
+    const double chunks = p.kk_pad / NM_KCHUNK, channels = std::min(p.tile_t, p.c_out);
+    return cta_rounds((p.pixels + BM - 1) / BM * p.n_tiles, nmhost::sm_count()) * (3.0 + 0.80 * chunks + 0.040 * channels) + 0.7 + 0.19 * chunks;
+}
 
 nm_status_t launch_conv_gather(const ConvParams& p, cudaStream_t st)
 {
@@ -451,7 +446,7 @@ nm_status_t launch_conv_gather(const ConvParams& p, cudaStream_t st)
     // SM to itself; a wave has about 3 us of its own and 4 more with the exchange (clusters do not fit on every last SM).
     // Measured, us: 7 blocks x 5 tiles, 95 chunks, one range 69, two 42, four 28, eight (a second wave) 49; 55 blocks x 8 tiles, 54 chunks,
     // one range 68, two 83; 15 blocks x 8 tiles, 5 chunks, one range 14, two 16.
-    const long long sms = sm_count();
+    const long long sms = nmhost::sm_count();
     double best = 1e30;
     for (int cs = 1; cs <= 8 && (cs == 1 || cfg.chunks >= 2 * cs); cs *= 2) {
         const long long ctas = blocks * p.n_tiles * cs, slots = 2 * sms - (cs > 1 ? 32 : 0);

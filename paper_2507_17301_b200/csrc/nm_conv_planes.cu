@@ -275,20 +275,6 @@ k_conv_planes(const ConvParams p, const PlaneCfg cfg, const __grid_constant__ CU
     if (warp == 4) tmem_dealloc(tmem, 512);
 }
 
-int sm_count()
-{
-    static int n = 0;
-    if (n == 0) {
-        int dev = 0, v = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess &&
-            cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0)
-            n = v;
-        else
-            n = 148;
-    }
-    return n;
-}
-
 bool make_cfg(const ConvParams& p, const nm_plan_t* plan, PlaneCfg* cfg, size_t* smem_out)
 {
     if (!p.ws || !nmtm::available()) return false;
@@ -368,7 +354,7 @@ nm_status_t launch_conv_planes(const ConvParams& p, const nm_plan_t* plan, cudaS
     auto kernel = p.stride_w == 2 ? k_conv_planes<2> : k_conv_planes<1>;
     cudaError_t e = nmhost::ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), smem);
     if (e != cudaSuccess) return fail(NM_ERR_CUDA, "cudaFuncSetAttribute (variant 9): %s", cudaGetErrorString(e));
-    const long long grid = cfg.n_work < sm_count() ? cfg.n_work : sm_count();
+    const long long grid = cfg.n_work < nmhost::sm_count() ? cfg.n_work : nmhost::sm_count();
     e = nmhost::launch_pdl(kernel, static_cast<unsigned>(grid), THREADS, smem, st, p, cfg, tm_y);
     nmhost::count_launch(1);
     if (e == cudaSuccess) e = cudaGetLastError();

@@ -736,17 +736,6 @@ k_conv_select(const ConvParams p, const SelCfg cfg, const __grid_constant__ CUte
 
 // ---- launch configuration --------------------------------------------------------------------------
 
-int sm_count()
-{
-    static const int n = [] {
-        int dev = 0, v = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0)
-            return v;
-        return 148;
-    }();
-    return n;
-}
-
 // Source and retained columns of a step: 32 source columns, or 64 where those keep too few for an MMA's depth of 8.  Groups
 // may not cross steps.  False: the kernel does not cover the pattern.
 bool pattern_dims(int n_keep, int m_group, int* s, int* kc)
@@ -838,7 +827,7 @@ bool make_cfg(const ConvParams& p, const nm_plan_t* plan, SelCfg* cfg)
     cfg->by_taps = divisor(taps);
     cfg->by_hw = divisor(p.ho * p.wo);
     cfg->by_wo = divisor(p.wo);
-    cfg->alias_staging = cfg->n_work <= sm_count();
+    cfg->alias_staging = cfg->n_work <= nmhost::sm_count();
     // Staging boxes per warp: three with a shortcut (it is requested two blocks ahead; fewer where a plan's rings need the room), one
     // where the epilogue has a long main loop beside it and the rings need it (256 -> 256, 3x3 at 14x14, 2:8: 37 -> 34 us),
     // else two.
@@ -919,7 +908,7 @@ nm_status_t launch(const ConvParams& p, const SelCfg& cfg, cudaStream_t st)
     const auto kernel = cfg.halo ? (pairs ? k_conv_select<P, 1, 2> : k_conv_select<P, 1, 1>) : (pairs ? k_conv_select<P, 0, 2> : k_conv_select<P, 0, 1>);
     cudaError_t e = nmhost::ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), smem);
     if (e != cudaSuccess) return nmhost::fail(NM_ERR_CUDA, "cudaFuncSetAttribute (variant 8): %s", cudaGetErrorString(e));
-    const long long grid = cfg.n_work < sm_count() ? cfg.n_work : sm_count();
+    const long long grid = cfg.n_work < nmhost::sm_count() ? cfg.n_work : nmhost::sm_count();
     e = nmhost::launch_pdl(kernel, static_cast<unsigned>(grid), THREADS, smem, st, q, cfg, tm_x, tm_y, tm_res);
     nmhost::count_launch(1);
     if (e == cudaSuccess) e = cudaGetLastError();

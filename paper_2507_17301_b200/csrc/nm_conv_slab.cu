@@ -21,6 +21,8 @@
 // Epilogue (the compactor warps): TMEM -> registers, + bias, ReLU, NHWC store.
 // Every mbarrier wait is bounded; on expiry the CTA raises an abort flag, reports through the
 // status word and drains to the common exit where TMEM is released.
+#include <algorithm>
+
 #include "nm_internal.h"
 #include "nm_ptx.cuh"
 #include "nm_tmap.cuh"
@@ -453,6 +455,27 @@ bool slab_plan_ok(const ConvParams& p, const nm_plan_t* plan)
 {
     SlabCfg cfg;
     return make_cfg(p, plan, &cfg);
+}
+
+bool slab_beats_gather(const ConvParams& p)
+{
+    // This kernel brings a pixel block's slab once for a CTA's tiles, the gather kernel gathers it once per tile; but a chunk is a longer
+    // chain here, and only the gather kernel splits the chunks of a launch that leaves SMs idle.  Both times by estimates fitted to
+    // 537 random layers that the stream kernel does not take (c_in 20-512, c_out 32-512, T 1-128, 1:16 to 3:4, 1x1 and 3x3).
+    // Measured, us, gather / this: 64 -> 256 1x1 at 56x56, batch 64, 2:4, T = 8 676 / 402, T = 40 199 / 181; 32 -> 128
+    // at 80x80, batch 16, T = 8 167 / 96; but 256 -> 256 3x3 at 14x14, batch 32, T = 8 193 / 252, 56x56, batch 8 708 / 725.
+    // On 331 others the choice is 0.4 % behind the better of the two in the middle, 12 % for 3 in 100, 34 % at worst (on the 537
+    // the gather kernel alone was up to 159 % behind, this one alone 647 %).
+    SlabCfg cfg;
+    const long long blocks = (p.pixels + BM - 1) / BM;
+    const int sms = nmhost::sm_count();
+    if (blocks * p.n_tiles < 4ll * sms || !make_cfg(p, nullptr, &cfg)) return false;   // (below two rounds the gather kernel may split)
+    const double g = cfg.g_tiles, chunks = p.v2_chunks, channels = std::min(cfg.g_tiles * p.tile_t, p.c_out);
+    const double rounds = cta_rounds(blocks * cfg.n_slices, sms);
+    const double us = cfg.use_tma ? rounds * (3.6 + chunks * (0.26 * cfg.segs + g * (0.11 + 0.013 * p.v2_kc)) + 0.010 * channels + 1.0 * g) +
+                                        1.9 + 0.007 * chunks * g * p.v2_kc
+                                  : rounds * (chunks * (3.6 * cfg.segs + 0.019 * g * p.v2_kc) + 0.046 * channels + 0.8 * g) + 2.5 + 0.13 * g;
+    return us < gather_time_us(p);
 }
 
 nm_status_t launch_conv_slab(const ConvParams& p, const nm_plan_t* plan, cudaStream_t st)

@@ -414,20 +414,6 @@ k_conv_stream(const ConvParams p, const StreamCfg cfg, const __grid_constant__ C
 
 // ---- launch configuration --------------------------------------------------------------------------
 
-int sm_count()
-{
-    static int n = 0;
-    if (n == 0) {
-        int dev = 0, v = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess &&
-            cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0)
-            n = v;
-        else
-            n = 148;
-    }
-    return n;
-}
-
 // 0 = pattern not covered, otherwise NK * 16 + MG of the kernel instance.
 int pattern_code(const ConvParams& p)
 {
@@ -509,7 +495,7 @@ nm_status_t launch(const ConvParams& p, const StreamCfg& cfg, cudaStream_t st)
     if (smem < NM_EXCLUSIVE_SMEM) smem = NM_EXCLUSIVE_SMEM;   // one CTA per SM: it owns all 512 TMEM columns
     cudaError_t e = nmhost::ensure_dynamic_smem(reinterpret_cast<const void*>(k_conv_stream<NK, MG>), smem);
     if (e != cudaSuccess) return nmhost::fail(NM_ERR_CUDA, "cudaFuncSetAttribute (variant 3): %s", cudaGetErrorString(e));
-    const long long grid = cfg.n_work < sm_count() ? cfg.n_work : sm_count();
+    const long long grid = cfg.n_work < nmhost::sm_count() ? cfg.n_work : nmhost::sm_count();
     e = nmhost::launch_pdl(k_conv_stream<NK, MG>, static_cast<unsigned>(grid), THREADS, smem, st, p, cfg, tm_x, tm_w, tm_y);
     nmhost::count_launch(1);
     if (e == cudaSuccess) e = cudaGetLastError();
@@ -532,7 +518,7 @@ bool stream_leaves_sms_idle(const ConvParams& p)
     // Work items on less than half of the SMs, sixteen chunks or more each.  3x3 448 -> 160 at 8x14 (7 pixel blocks, 3:4):
     // 52.7 us here, 29 us in the gather kernel, which splits the chunks over a cluster; 1x1 352 -> 704 at 34x7 (six chunks): 7.2, 7.7.
     StreamCfg cfg;
-    return make_cfg(p, nullptr, &cfg) && 2 * cfg.n_work < sm_count() && p.v2_chunks >= 16;
+    return make_cfg(p, nullptr, &cfg) && 2 * cfg.n_work < nmhost::sm_count() && p.v2_chunks >= 16;
 }
 
 nm_status_t launch_conv_stream(const ConvParams& p, const nm_plan_t* plan, cudaStream_t st)

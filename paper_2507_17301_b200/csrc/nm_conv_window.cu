@@ -288,20 +288,6 @@ k_conv_window(const ConvParams p, const WinCfg cfg, const __grid_constant__ CUte
     if (warp == 6) tmem_dealloc(tmem, 512);
 }
 
-int sm_count()
-{
-    static int n = 0;
-    if (n == 0) {
-        int dev = 0, v = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess &&
-            cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0)
-            n = v;
-        else
-            n = 148;
-    }
-    return n;
-}
-
 bool make_cfg(const ConvParams& p, const nm_plan_t* plan, WinCfg* cfg, size_t* smem_out)
 {
     if (!p.wx || !nmtm::available()) return false;
@@ -393,7 +379,7 @@ nm_status_t launch_conv_window(const ConvParams& p, const nm_plan_t* plan, cudaS
         return fail(NM_ERR_CUDA, "nm_conv2d: tensor-map encoding failed (variant 6)");
     cudaError_t e = nmhost::ensure_dynamic_smem(reinterpret_cast<const void*>(k_conv_window), smem);
     if (e != cudaSuccess) return fail(NM_ERR_CUDA, "cudaFuncSetAttribute (variant 6): %s", cudaGetErrorString(e));
-    const long long grid = cfg.n_work < sm_count() ? cfg.n_work : sm_count();
+    const long long grid = cfg.n_work < nmhost::sm_count() ? cfg.n_work : nmhost::sm_count();
     e = launch_pdl(k_conv_window, static_cast<unsigned>(grid), THREADS, smem, st, p, cfg, tm_x);
     count_launch(1);
     if (e == cudaSuccess) e = cudaGetLastError();

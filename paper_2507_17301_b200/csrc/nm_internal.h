@@ -136,6 +136,15 @@ constexpr bool NM_SELF_CHECKING = false;
 #endif
 
 namespace nmhost {
+int sm_count();   // of the device that is current at the first call
+
+// Rounds of `ctas` CTAs, two per SM: the last one counts in full while there are few, half where they drift apart.
+inline double cta_rounds(long long ctas, int sms)
+{
+    const double x = static_cast<double>(ctas) / (2.0 * sms);
+    return x < 4.0 ? static_cast<double>((ctas + 2 * sms - 1) / (2 * sms)) : x + 0.5;
+}
+
 // Launches `kernel` so that it may begin while the previous kernel of the stream drains
 // (programmatic dependent launch); the kernel orders itself with griddepcontrol.wait.
 // NM_NO_PDL=1 in the environment falls back to a plain launch.
@@ -192,10 +201,14 @@ nm_status_t build_from_compressed(const float* values, const uint16_t* indices, 
 // MMA width of a tile: the channels it can have, in sixteens
 inline int gather_width(int tile_t, int c_out) { return ((tile_t < c_out ? tile_t : c_out) + 15) / 16 * 16; }
 nm_status_t launch_conv_gather(const ConvParams& p, cudaStream_t st);
+double gather_time_us(const ConvParams& p);   // estimate, one range of the chunks
 
 // nm_conv_slab.cu — variant 2
 bool slab_plan_ok(const ConvParams& p, const nm_plan_t* plan);
 nm_status_t launch_conv_slab(const ConvParams& p, const nm_plan_t* plan, cudaStream_t st);
+// Whether the library default takes this kernel rather than the gather kernel: many CTAs of few chunks, tiles narrow enough that
+// several share a pixel block (see the estimates).
+bool slab_beats_gather(const ConvParams& p);
 
 // nm_conv_expand.cu — variant 4
 bool expand_plan_ok(const ConvParams& p, const nm_plan_t* plan);

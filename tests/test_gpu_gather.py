@@ -104,3 +104,20 @@ def test_default_on_both_sides_of_the_row_runs(batch):
     y = nm.nm_conv2d(hnd, x.cuda(), 3, 3, 1, 1, 1, b.cuda(), True)
     nm.nm_weights_check(hnd)
     assert np.array_equal(y.cpu().numpy(), yr)
+
+
+@pytest.mark.parametrize("s", [
+    ConvShape("tma", 4, 56, 56, 64, 64, 1, 1, 1, 0, 1, 2, 4, 8),            # the slab kernel: 98 blocks of 8 tiles, one chunk
+    ConvShape("tma_tail", 3, 57, 55, 32, 76, 3, 3, 1, 1, 1, 1, 8, 8),       # last tile of four channels, last block ragged
+    ConvShape("no_tma", 2, 40, 40, 36, 60, 1, 1, 1, 0, 1, 2, 4, 2),         # channels and tile width that no tensor map takes
+    ConvShape("many_chunks", 1, 56, 56, 96, 200, 3, 3, 1, 1, 1, 2, 4, 8),   # the gather kernel: 14 chunks
+], ids=lambda s: s.name)
+def test_default_for_many_narrow_tiles(s):
+    from paper_2507_17301_b200 import nm
+    w, x, b = inputs.make_int_case(s)
+    vr, ir = oracle.prune(w.numpy(), s.n_keep, s.m_group, s.tile_t)
+    yr = oracle.conv2d(vr, ir, s.kh, s.kw, s.c_in, s.tile_t, x.numpy(), (1, 1), (s.pad,) * 2, (1, 1), b.numpy(), True)
+    hnd = nm.nm_prune(w.cuda(), s.n_keep, s.m_group, s.tile_t)
+    y = nm.nm_conv2d(hnd, x.cuda(), s.kh, s.kw, 1, s.pad, 1, b.cuda(), True)
+    nm.nm_weights_check(hnd)
+    assert np.array_equal(y.cpu().numpy(), yr)
