@@ -63,13 +63,6 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const void* tmap, uint
         ::"r"(dst), "l"(tmap), "r"(bar), "r"(c), "r"(w), "r"(h), "r"(n)
         : "memory");
 }
-// Shared memory of this CTA to that of a CTA of the cluster; the barrier is one of the receiving CTA.
-__device__ __forceinline__ void bulk_copy_cluster(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar)
-{
-    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "r"(src),
-                 "r"(bytes), "r"(bar)
-                 : "memory");
-}
 __device__ __forceinline__ float4 ld_shared_f4(uint32_t addr)
 {
     float4 v;

@@ -51,13 +51,6 @@ struct GatherCfg {
 
 __device__ __forceinline__ bool aborted(volatile int* flag) { return *flag != 0; }
 
-// Shared memory of this CTA to that of a CTA of the cluster; the barrier is one of the receiving CTA.
-__device__ __forceinline__ void bulk_copy_cluster(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar)
-{
-    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "r"(src),
-                 "r"(bytes), "r"(bar)
-                 : "memory");
-}
 // *p where `on` is non-zero, else 0; a predicated load (written as a conditional it becomes a branch per pixel row).
 __device__ __forceinline__ float load_if(const float* p, uint32_t on)
 {

@@ -870,18 +870,6 @@ bool make_cfg(const ConvParams& p, const nm_plan_t* plan, SelCfg* cfg)
     return true;
 }
 
-// The input as a plain 2-D tensor [batch * h * w pixels][c_in] with a box of 32 channels x `rows` pixels.
-bool encode_x_rows(const ConvParams& p, int rows, CUtensorMap* tm)
-{
-    const cuuint64_t dims[2] = {static_cast<cuuint64_t>(p.c_in), static_cast<cuuint64_t>(p.batch) * p.h * p.w};
-    const cuuint64_t strides[1] = {static_cast<cuuint64_t>(p.c_in) * 4};
-    const cuuint32_t box[2] = {32, static_cast<cuuint32_t>(rows)};
-    const cuuint32_t es[2] = {1, 1};
-    return nmtm::encoders().tiled(tm, nmtm::kOperandType, 2, const_cast<float*>(p.x), dims, strides, box, es,
-                                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 template <class P>
 nm_status_t launch(const ConvParams& p, const SelCfg& cfg, cudaStream_t st)
 {
@@ -894,7 +882,7 @@ nm_status_t launch(const ConvParams& p, const SelCfg& cfg, cudaStream_t st)
         q.relu = 0;
     }
     alignas(64) CUtensorMap tm_x, tm_y, tm_res;
-    const bool ok_x = cfg.rows2d ? encode_x_rows(p, cfg.prow, &tm_x) : nmtm::encode_x_im2col(p, BM, &tm_x);
+    const bool ok_x = cfg.rows2d ? nmtm::encode_x_rows(p, cfg.prow, &tm_x) : nmtm::encode_x_im2col(p, BM, &tm_x);
     if (!ok_x || !nmtm::encode_y_tiled(q, &tm_y))
         return nmhost::fail(NM_ERR_CUDA, "nm_conv2d: tensor-map encoding failed (variant 8)");
     tm_res = tm_y;

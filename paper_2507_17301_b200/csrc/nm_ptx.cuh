@@ -142,6 +142,13 @@ __device__ __forceinline__ uint32_t cluster_ctarank()
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
     return r;
 }
+// Shared memory of this CTA to that of a CTA of the cluster; the barrier is one of the receiving CTA.
+__device__ __forceinline__ void bulk_copy_cluster(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar)
+{
+    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "r"(src),
+                 "r"(bytes), "r"(bar)
+                 : "memory");
+}
 // Barrier over every thread of the cluster; orders the shared-memory writes before it (barrier
 // initialisation included) against the reads after it in the other CTA.
 __device__ __forceinline__ void cluster_sync_all()
