@@ -1,9 +1,12 @@
 """A CPU model of the barrier protocol of the expanded-operand kernel's main loop with TWO MMA issuer threads (host logic,
-no GPU): a producer fills ring slots in order, each issuer waits on a slot's "full" barrier by phase parity, releases it
-with a commit that lands some time later, and both hand the accumulators to the epilogue.  The model counts barrier
+no GPU): two producers fill the activation ring and the (shorter) weight ring in order, both arriving on the "full" barrier
+of a stage's activation slot; each issuer waits on that barrier by phase parity, releases the slot with a commit that lands
+some time later, and both hand the accumulators to the epilogue.  There is no barrier per weight slot: the weight producer
+waits for the commit of the stage that used its slot before, on the "free" barrier of THAT stage's activation slot.  The model counts barrier
 phases in full but lets a waiter see only the phase's parity, as the hardware does, and fails on
 
-  * a wait that passes on a slot that does not hold the stage the waiter expects (a stale phase of the same parity),
+  * a wait that passes on a slot of either ring that does not hold the stage the waiter expects (a stale phase of the same parity),
+  * a load into a weight slot whose last reader has not been committed,
   * more arrivals on a barrier than its phase expects,
   * a state in which nobody can move.
 
@@ -41,13 +44,16 @@ class Ring:
             self.s, self.par, self.wrapped = 0, self.par ^ 1, True
 
 
-def simulate(pieces, n_slots, n_acc, by_slot, seed):
+def simulate(pieces, n_slots, n_w, n_acc, by_slot, seed, wait_stage=lambda g, n_w: g - n_w):
     rnd = random.Random(seed)
-    full = [Bar(f"full{i}", 1) for i in range(n_slots)]
+    full = [Bar(f"full{i}", 2) for i in range(n_slots)]
     free = [Bar(f"free{i}", 1) for i in range(n_slots)]
     accfull = [Bar(f"accfull{i}", 2) for i in range(2)]
     accfree = [Bar(f"accfree{i}", 1) for i in range(2)]
-    holds = [None] * n_slots         # the stage whose load landed in the slot last
+    holds = [None] * n_slots         # the stage whose activations landed in the slot last
+    w_holds = [None] * n_w           # the same for weights
+    done = set()                     # stages whose MMAs have been committed
+    landing = []                     # (slot's full barrier, what lands): loads still under way, in any order
     commits = []                     # (issuer, barrier): tcgen05.commit arrivals still in flight, in order per issuer
 
     def producer():
@@ -57,10 +63,28 @@ def simulate(pieces, n_slots, n_acc, by_slot, seed):
                 if rp.wrapped:
                     while not free[rp.s].passed(rp.par ^ 1):
                         yield
-                holds[rp.s] = g
-                full[rp.s].arrive("producer")
+                landing.append((full[rp.s], holds, rp.s, g))
                 g += 1
                 rp.adv(n_slots)
+                yield
+
+    def weight_producer():
+        # the kernel's walk: `rf` is the place of the stage that used the weight slot before (n_w stages back)
+        rp, rf, g, ws, wrapped = Ring(), Ring(), 0, 0, False
+        for length in pieces:
+            for _ in range(length):
+                if wrapped:
+                    while not free[rf.s].passed(rf.par):
+                        yield
+                    if wait_stage(g, n_w) not in done:
+                        raise RuntimeError(f"weights of stage {g} overwrite stage {wait_stage(g, n_w)}, which is still read")
+                    rf.adv(n_slots)
+                landing.append((full[rp.s], w_holds, ws, g))
+                g += 1
+                rp.adv(n_slots)
+                ws += 1
+                if ws == n_w:
+                    ws, wrapped = 0, True
                 yield
 
     def issuer(i):
@@ -75,13 +99,13 @@ def simulate(pieces, n_slots, n_acc, by_slot, seed):
                 if mine:
                     while not full[rp.s].passed(rp.par):
                         yield
-                    if holds[rp.s] != g:
-                        raise RuntimeError(f"issuer {i} passed a stale phase: slot {rp.s} holds stage {holds[rp.s]}, not {g}")
-                    commits.append((i, free[rp.s]))
+                    if holds[rp.s] != g or w_holds[g % n_w] != g:
+                        raise RuntimeError(f"issuer {i} passed a stale phase: slots hold stages {holds[rp.s]} and {w_holds[g % n_w]}, not {g}")
+                    commits.append((i, free[rp.s], g))
                 g += 1
                 rp.adv(n_slots)
                 yield
-            commits.append((i, accfull[ab]))
+            commits.append((i, accfull[ab], None))
             if n_acc == 2:
                 if ab == 1:
                     par ^= 1
@@ -101,18 +125,24 @@ def simulate(pieces, n_slots, n_acc, by_slot, seed):
             yield
             accfree[ab].arrive("epilogue")
 
-    agents = {"producer": producer(), "epilogue": epilogue(), "issuer0": issuer(0), "issuer1": issuer(1)}
+    agents = {"producer": producer(), "weights": weight_producer(), "epilogue": epilogue(), "issuer0": issuer(0), "issuer1": issuer(1)}
     bars = full + free + accfull + accfree
     idle = 0
     while agents:
         before = tuple((b.phase, b.pending) for b in bars)
         moved = False
-        for who in {a for a, _ in commits}:
+        for who in {c[0] for c in commits}:
             if rnd.random() < 0.5:
-                k = next(j for j, (a, _) in enumerate(commits) if a == who)
-                a, bar = commits.pop(k)
+                k = next(j for j, c in enumerate(commits) if c[0] == who)
+                a, bar, stage = commits.pop(k)
+                done.add(stage)
                 bar.arrive(f"issuer{a}")
                 moved = True
+        while landing and rnd.random() < 0.5:
+            bar, ring, slot, stage = landing.pop(rnd.randrange(len(landing)))
+            ring[slot] = stage
+            bar.arrive("a load")
+            moved = True
         names = list(agents)
         rnd.shuffle(names)
         for n in names:
@@ -122,7 +152,7 @@ def simulate(pieces, n_slots, n_acc, by_slot, seed):
                 del agents[n]
                 moved = True
         moved = moved or tuple((b.phase, b.pending) for b in bars) != before
-        idle = 0 if moved or commits else idle + 1
+        idle = 0 if moved or commits or landing else idle + 1
         if idle > 200:
             raise RuntimeError(f"deadlock: {sorted(agents)} cannot move")
 
@@ -134,18 +164,25 @@ def _cases():
 
 
 @pytest.mark.parametrize("n_acc", [1, 2])
-@pytest.mark.parametrize("n_slots", [2, 4, 6, 10])
-def test_slot_ownership_is_safe(n_slots, n_acc):
+@pytest.mark.parametrize("n_slots,n_w", [(2, 2), (4, 4), (4, 3), (4, 2), (6, 4), (10, 3), (10, 2)])
+def test_slot_ownership_is_safe(n_slots, n_w, n_acc):
     for seed, pieces in _cases():
-        simulate(pieces, n_slots, n_acc, True, seed)
+        simulate(pieces, n_slots, n_w, n_acc, True, seed)
 
 
 def test_ownership_by_position_in_the_item_is_not():
     failures = 0
     for seed, pieces in _cases():
         try:
-            simulate(pieces, 2, 2, False, seed)
+            simulate(pieces, 2, 2, 2, False, seed)
         except RuntimeError as e:
-            assert "stale phase" in str(e) or "over-arrival" in str(e) or "deadlock" in str(e)
+            assert "stale phase" in str(e) or "over-arrival" in str(e) or "deadlock" in str(e) or "still read" in str(e)
             failures += 1
     assert failures > 0
+
+
+def test_the_model_notices_a_weight_slot_taken_too_early():
+    """A producer that looked one stage too far back would overwrite weights under their readers: the check is not vacuous."""
+    with pytest.raises(RuntimeError, match="still read"):
+        for seed, pieces in _cases():
+            simulate(pieces, 6, 3, 2, True, seed, wait_stage=lambda g, n_w: g - n_w + 1)
