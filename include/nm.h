@@ -56,8 +56,10 @@ typedef struct nm_weights nm_weights_t;
 
 /*
  * Launch plan for nm_conv2d (the analogue of the paper's per-layer template parameters, Sec. 3.3).
- *   variant  0 = let the library choose (variants 3, 9, 5 and 1: activations rounded to nearest, pruned columns never
- *                read);
+ *   variant  0 = let the library choose: variants 3, 2 and 1, which round activations to nearest and never read a pruned
+ *                column, and for channel counts that are no multiple of 32 also 9 and 5, which do neither (see
+ *                nm_conv2d).  The choice depends on the amount of work, so a layer of such a channel count may change
+ *                between 1 and 5 with the batch;
  *            1 = direct-gather kernel (any shape; kept columns gathered from global memory, the reduction axis split over
  *                clusters of CTAs where there are few);
  *            2 = slab kernel (dense activation slab staged once per CTA, kept columns picked by
@@ -274,9 +276,10 @@ nm_status_t nm_memory_trim(void);
  *                          x[n][oh*stride_h - pad_h + kh_j*dil_h][ow*stride_w - pad_w + kw_j*dil_w][c_j] )
  * with (kh_j, kw_j, c_j) decoded from indices[o / tile_t][j] and reads outside the image = 0.
  * Non-finite activations: the kernels that contract over the retained columns only (variants 1, 2, 3, 8) never
- * read a pruned column's activation, as Algorithm 1 does not; the expanded-operand kernels (variants 4-7)
+ * read a pruned column's activation, as Algorithm 1 does not; the kernels that multiply expanded weights (variants 4-7, 9, 10)
  * multiply it by a zero weight, so an Inf or NaN in a PRUNED column turns the outputs of that pixel into NaN there
- * while the definition above (and variants 1, 2, 3, 8) keep them finite.  Finite inputs give the same results in all.
+ * while the definition above (and variants 1, 2, 3, 8) keep them finite.  Finite inputs give the same results in all, up to
+ * rounding; a finite activation whose nearest TF32 value is out of range (above 3.4026e38) counts as infinite where it is rounded.
  * Arithmetic: operands rounded to TF32 (weights once at prune time, round-to-nearest; activations
  * round-to-nearest, with ties away from zero where they pass through registers (variants 1-3) and to even where the TMA unit
  * rounds them (variants 4, 6, 7, 8, 10), truncated in variants 5 and 9), products accumulated in fp32.
