@@ -263,7 +263,7 @@ std::vector<nm_plan_t> candidate_plans(const nm_weights* /*w*/, const ConvParams
     for (int ksplit : {1, 2, 3, 4}) {
         for (int bn : {128, 256, 64, 32}) {
             a.variant = 8; a.bn = bn; a.ksplit = ksplit;
-            if (bn % p.tile_t == 0 && nmhost::select_plan_ok(p, &a)) out.push_back(a);
+            if (bn % p.tile_t == 0 && nmhost::select_ranges(p, &a) == ksplit) out.push_back(a);
         }
     }
     std::memset(&a, 0, sizeof(a));

@@ -815,7 +815,8 @@ bool make_cfg(const ConvParams& p, const nm_plan_t* plan, ExpandCfg* cfg)
         if (na > NSTAGE_MAX) na = NSTAGE_MAX;
         if (n_iss == 2) na &= ~1;
     }
-    if (na < 2 || na > NSTAGE_MAX || na * a_slot + nw * w_slot > budget) return false;
+    // (a plan may ask for a single slot; the default is at least two)
+    if (na < (asked ? 1 : 2) || na > NSTAGE_MAX || na * a_slot + nw * w_slot > budget) return false;
     if (nw > na) nw = na;
     if (n_iss == 2 && na % 2 != 0) return false;   // two issuers own alternate ring slots
     cfg->stages = na;

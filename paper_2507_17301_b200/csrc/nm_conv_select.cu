@@ -811,13 +811,13 @@ bool make_cfg(const ConvParams& p, const nm_plan_t* plan, SelCfg* cfg)
     cfg->m_bytes = g * TABLE_BYTES;
     cfg->wstage_bytes = ((cfg->w_bytes + cfg->m_bytes + 1023) / 1024) * 1024;
     // split of the reduction axis: whole chunks per range
-    const int ksplit = plan && plan->ksplit > 1 ? plan->ksplit : 1;
-    if (ksplit > 8 || cfg->chunks < ksplit || (plan && (plan->split < 0 || plan->split > 2))) return false;
+    if (plan && (plan->ksplit > 8 || plan->split < 0 || plan->split > 2)) return false;
+    const int asked = plan && plan->ksplit > 1 ? plan->ksplit : 1, ksplit = std::min(asked, cfg->chunks);   // (no more ranges than chunks)
     cfg->ksplit = ksplit;
     cfg->p_pad = static_cast<int>(((p.pixels + BM - 1) / BM) * BM);
-    if (ksplit > 1 && (!p.splitk || p.c_out % 4 != 0 ||
-                       p.splitk_bytes < static_cast<size_t>(ksplit) * cfg->p_pad * p.c_out * sizeof(float) ||
-                       static_cast<long long>(ksplit) * cfg->p_pad >= (1ll << 31)))
+    if (asked > 1 && (!p.splitk || p.c_out % 4 != 0 ||
+                      p.splitk_bytes < static_cast<size_t>(asked) * cfg->p_pad * p.c_out * sizeof(float) ||
+                      static_cast<long long>(asked) * cfg->p_pad >= (1ll << 31)))
         return false;   // the partial-sum scratch is reserved by nm_autotune / nm_weights_reserve
     const long long pix_blocks = (p.pixels + BM - 1) / BM;
     cfg->n_work = pix_blocks * cfg->n_slices * ksplit;
@@ -843,6 +843,9 @@ bool make_cfg(const ConvParams& p, const nm_plan_t* plan, SelCfg* cfg)
     if (plan && plan->stages > 0) {
         n_p = plan->stages;
         if (n_p > MAX_P) return false;
+        // (one slot fewer where only the zero rows behind the blocks are too much)
+        const int zeros = cfg->halo ? S / 32 * 1024 : 0;
+        if (n_p > 1 && n_p * cfg->p_bytes + 2 * cfg->wstage_bytes > budget && n_p * (cfg->p_bytes - zeros) + 2 * cfg->wstage_bytes <= budget) --n_p;
     } else {
         auto fits = [&](int a, int w) { return a * cfg->p_bytes + w * cfg->wstage_bytes <= budget; };
         // (where a team gets less than a chunk from a slot, a third slot is worth more than its second weight slot)
@@ -852,6 +855,8 @@ bool make_cfg(const ConvParams& p, const nm_plan_t* plan, SelCfg* cfg)
     }
     int n_w = (budget - n_p * cfg->p_bytes) / cfg->wstage_bytes;
     if (n_w > MAX_W) n_w = MAX_W;
+    // A plan's activation slots may leave room for two weight slots only: two teams then take the chunks in turn, the others idle.
+    while (cfg->cycle > 2 && n_w < cfg->cycle) cfg->cycle /= 2;
     n_w -= n_w % cfg->cycle;
     if (n_w < 2) return false;
     cfg->n_p = n_p;
@@ -919,6 +924,12 @@ bool select_plan_ok(const ConvParams& p, const nm_plan_t* plan)
 {
     SelCfg cfg;
     return make_cfg(p, plan, &cfg);
+}
+
+int select_ranges(const ConvParams& p, const nm_plan_t* plan)
+{
+    SelCfg cfg;
+    return make_cfg(p, plan, &cfg) ? cfg.ksplit : 0;
 }
 
 size_t select_splitk_bytes(const ConvParams& p, int splits)

@@ -240,6 +240,7 @@ nm_status_t launch_conv_stream(const ConvParams& p, const nm_plan_t* plan, cudaS
 // nm_conv_select.cu — variant 8
 bool select_layout_dims(const nm_weights* h, int* s, int* kc);   // false: the pattern or shape rules the kernel out
 bool select_plan_ok(const ConvParams& p, const nm_plan_t* plan);
+int select_ranges(const ConvParams& p, const nm_plan_t* plan);   // of the reduction axis, 0: the plan does not fit
 size_t select_splitk_bytes(const ConvParams& p, int splits);
 nm_status_t launch_conv_select(const ConvParams& p, const nm_plan_t* plan, cudaStream_t st);
 
