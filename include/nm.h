@@ -281,8 +281,9 @@ nm_status_t nm_memory_trim(void);
  * while the definition above (and variants 1, 2, 3, 8) keep them finite.  Finite inputs give the same results in all, up to
  * rounding; a finite activation whose nearest TF32 value is out of range (above 3.4026e38) counts as infinite where it is rounded.
  * Arithmetic: operands rounded to TF32 (weights once at prune time, round-to-nearest; activations
- * round-to-nearest, with ties away from zero where they pass through registers (variants 1-3) and to even where the TMA unit
- * rounds them (variants 4, 6, 7, 8, 10), truncated in variants 5 and 9), products accumulated in fp32.
+ * round-to-nearest where they pass through registers (variants 1-3, ties away from zero) and in variant 10 for inputs of
+ * less than 128 KiB (ties to even), truncated where the staged data feeds the tensor core directly (variants 4-9, variant 10
+ * for larger inputs)), products accumulated in fp32.
  *
  *   x      device fp32 [batch][h][wd][c_in]      bias  device fp32 [c_out] or NULL
  *   y      device fp32 [batch][ho][wo][c_out]    relu  0 = identity, 1 = ReLU

@@ -52,6 +52,7 @@ struct ClusterCfg {
     int b_off;        // offset of the weight tile inside a stage
     int stage_bytes;
     int rps;          // rows a CTA finishes
+    int round;        // 1: activations rounded to nearest (inputs that have no im2col form, of less than 128 KiB for instance)
 };
 
 __device__ __forceinline__ bool aborted(volatile int* flag) { return *flag != 0; }
@@ -336,6 +337,7 @@ bool make_cfg(const ConvParams& p, const nm_plan_t* plan, ClusterCfg* cfg, size_
     else if (!small && nmtm::im2col_geometry_ok(p)) cfg->form = IM2COL;
     else if (unit && p.wo <= 128) cfg->form = BOX_4D;
     else return false;
+    cfg->round = small || cfg->form == BOX_4D ? 1 : 0;
     cfg->n_blk = (p.k + 31) / 32;
     cfg->cs = plan && plan->ksplit > 0 ? plan->ksplit : 1;
     if ((cfg->cs != 1 && cfg->cs != 2 && cfg->cs != 4 && cfg->cs != 8) || cfg->n_blk < cfg->cs) return false;
@@ -393,6 +395,11 @@ bool encode_x(const ConvParams& p, const ClusterCfg& cfg, CUtensorMap* tm)
 {
     if (cfg.form == IM2COL) return nmtm::encode_x_im2col(p, cfg.rows, tm);
     const bool rows = cfg.form == ROWS_2D;
+    // Inputs that have no im2col form (below 128 KiB) are otherwise taken by kernels that round activations to nearest (variants 1 and
+    // 2): for them the TMA unit rounds on the way into shared memory (to nearest, ties to even, in no extra time), where the tensor core would truncate.
+    // Last map of ResNet-50 at 96 x 96, batch 1, against 64 bits: 3.1e-3 truncated, 1.8e-3 rounded
+    // (248 us either way); ResNet-101 at 100 x 100, batch 2, 3:4: 1.5e-2 and 7.7e-3.
+    const CUtensorMapDataType type = cfg.round ? CU_TENSOR_MAP_DATA_TYPE_TFLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
     const cuuint64_t c = static_cast<cuuint64_t>(p.c_in), w = static_cast<cuuint64_t>(p.w), h = static_cast<cuuint64_t>(p.h),
                      n = static_cast<cuuint64_t>(p.batch);
     const cuuint64_t dims2[2] = {c, n * h * w}, dims4[4] = {c, w, h, n};
@@ -400,7 +407,7 @@ bool encode_x(const ConvParams& p, const ClusterCfg& cfg, CUtensorMap* tm)
     const cuuint32_t box2[2] = {32, static_cast<cuuint32_t>(cfg.rows)};
     const cuuint32_t box4[4] = {32, static_cast<cuuint32_t>(p.wo), static_cast<cuuint32_t>(cfg.r_rows), 1};
     const cuuint32_t es[4] = {1, 1, 1, 1};
-    return nmtm::encoders().tiled(tm, nmtm::kOperandType, rows ? 2 : 4, const_cast<float*>(p.x), rows ? dims2 : dims4, strides,
+    return nmtm::encoders().tiled(tm, type, rows ? 2 : 4, const_cast<float*>(p.x), rows ? dims2 : dims4, strides,
                                   rows ? box2 : box4, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }

@@ -40,7 +40,8 @@
 // bitwise selects per element, 93 us; the dense kernel 46.  The gain over the dense kernel grows with M / N: at 2:8
 // 55 -> 38 us (128 -> 128 at 28x28), 74 -> 62 (64 -> 64 at 56x56), at 2:4, batch 64, 30 -> 29 and 45 -> 41, but 28.5 -> 31.5 at 14x14.
 //
-// Activations are rounded to TF32 by the TMA unit (nm_tmap.cuh), weights were at pruning time, both to nearest.
+// Activations are fed to the tensor core as they are (it reads the upper 19 bits: truncation to
+// TF32); weights were rounded to nearest at pruning time.
 #include <algorithm>
 
 #include "nm_internal.h"

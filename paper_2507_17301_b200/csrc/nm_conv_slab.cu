@@ -423,7 +423,7 @@ nm_status_t launch(const ConvParams& p, const SlabCfg& cfg, cudaStream_t st)
     memset(&tm_x, 0, sizeof(tm_x));
     memset(&tm_w, 0, sizeof(tm_w));
     memset(&tm_y, 0, sizeof(tm_y));
-    if (TMA && (!nmtm::encode_x_im2col(p, BM, &tm_x, CU_TENSOR_MAP_DATA_TYPE_FLOAT32) || !nmtm::encode_w_tiled(p, cfg.b_rows, &tm_w)))
+    if (TMA && (!nmtm::encode_x_im2col(p, BM, &tm_x) || !nmtm::encode_w_tiled(p, cfg.b_rows, &tm_w)))
         return nmhost::fail(NM_ERR_CUDA, "nm_conv2d: tensor-map encoding failed");
     if (cfg.tma_store && !nmtm::encode_y_tiled(p, &tm_y))
         return nmhost::fail(NM_ERR_CUDA, "nm_conv2d: output tensor-map encoding failed");

@@ -488,7 +488,7 @@ template <int NK, int MG>
 nm_status_t launch(const ConvParams& p, const StreamCfg& cfg, cudaStream_t st)
 {
     alignas(64) CUtensorMap tm_x, tm_w, tm_y;
-    if (!nmtm::encode_x_im2col(p, BM, &tm_x, CU_TENSOR_MAP_DATA_TYPE_FLOAT32) || !nmtm::encode_w_tiled(p, cfg.bn, &tm_w) ||
+    if (!nmtm::encode_x_im2col(p, BM, &tm_x) || !nmtm::encode_w_tiled(p, cfg.bn, &tm_w) ||
         !nmtm::encode_y_tiled(p, &tm_y))
         return nmhost::fail(NM_ERR_CUDA, "nm_conv2d: tensor-map encoding failed (variant 3)");
     size_t smem = 1024 + static_cast<size_t>(cfg.stages) * cfg.stage_bytes + STAGING_BYTES;

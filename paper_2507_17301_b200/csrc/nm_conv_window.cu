@@ -352,7 +352,7 @@ bool encode_x_patch(const ConvParams& p, const WinCfg& cfg, CUtensorMap* tm)
                                    static_cast<cuuint64_t>(p.h) * p.w * p.c_in * 4};
     const cuuint32_t box[4] = {32, static_cast<cuuint32_t>(cfg.wp), static_cast<cuuint32_t>(cfg.pr), 1};
     const cuuint32_t es[4] = {1, 1, 1, 1};
-    return nmtm::encoders().tiled(tm, nmtm::kOperandType, 4, const_cast<float*>(p.x), dims, strides, box, es,
+    return nmtm::encoders().tiled(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<float*>(p.x), dims, strides, box, es,
                                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }

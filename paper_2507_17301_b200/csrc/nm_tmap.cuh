@@ -44,16 +44,10 @@ inline const Encoders& encoders()
 
 inline bool available() { return encoders().tiled && encoders().im2col; }
 
-// Element type of the activation maps whose boxes the tensor core reads as they are: the TMA unit rounds to TF32 on the way into shared
-// memory (to nearest, ties to even: the bits of an identity layer's output, all finite values and ties), where an fp32 map would leave
-// the tensor core to truncate, with twice the error and all of it towards zero.  Last feature map of ResNet-50 at batch 1 /
-// 64 against 64 bits: 3.4e-3 / 3.7e-3 truncated, 6.5e-4 / 6.5e-4 rounded, in the same 295 / 1890 us.  Kernels that round in registers load fp32.
-constexpr CUtensorMapDataType kOperandType = CU_TENSOR_MAP_DATA_TYPE_TFLOAT32;
-
 // Activations as an im2col tensor map: NHWC seen as (C, W, H, N); the box is 32 channels x
 // `pixels` output pixels; the base-pixel window runs from -pad to pad - (K - 1) * dil in each
 // direction and is walked with the convolution stride.  128-byte swizzle.
-inline bool encode_x_im2col(const ConvParams& p, int pixels, CUtensorMap* tm, CUtensorMapDataType type = kOperandType)
+inline bool encode_x_im2col(const ConvParams& p, int pixels, CUtensorMap* tm)
 {
     const cuuint64_t dims[4] = {static_cast<cuuint64_t>(p.c_in), static_cast<cuuint64_t>(p.w),
                                 static_cast<cuuint64_t>(p.h), static_cast<cuuint64_t>(p.batch)};
@@ -62,7 +56,7 @@ inline bool encode_x_im2col(const ConvParams& p, int pixels, CUtensorMap* tm, CU
     const int lower[2] = {-p.pad_w, -p.pad_h};
     const int upper[2] = {p.pad_w - (p.kw - 1) * p.dil_w, p.pad_h - (p.kh - 1) * p.dil_h};
     const cuuint32_t trav[4] = {1, static_cast<cuuint32_t>(p.stride_w), static_cast<cuuint32_t>(p.stride_h), 1};
-    return encoders().im2col(tm, type, 4, const_cast<float*>(p.x), dims, strides, lower,
+    return encoders().im2col(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<float*>(p.x), dims, strides, lower,
                              upper, 32, static_cast<cuuint32_t>(pixels), trav, CU_TENSOR_MAP_INTERLEAVE_NONE,
                              CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
@@ -97,7 +91,7 @@ inline bool encode_x_rows(const ConvParams& p, int rows, CUtensorMap* tm)
     const cuuint64_t strides[1] = {static_cast<cuuint64_t>(p.c_in) * 4};
     const cuuint32_t box[2] = {32, static_cast<cuuint32_t>(rows)};
     const cuuint32_t es[2] = {1, 1};
-    return encoders().tiled(tm, kOperandType, 2, const_cast<float*>(p.x), dims, strides, box, es,
+    return encoders().tiled(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(p.x), dims, strides, box, es,
                             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
