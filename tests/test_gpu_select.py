@@ -1,5 +1,5 @@
-"""The select kernel (plan.variant = 8: contraction over the retained columns only, kept columns picked in
-registers under precomputed masks) against the CPU oracle, element by element: both forms of its activation
+"""The select kernel (plan.variant = 8: contraction over the retained columns only, kept columns loaded by
+tables built at pruning time) against the CPU oracle, element by element: both forms of its activation
 loads, every N:M pattern it covers, one to four tiles per work item, one to four MMA issuer threads, short
 rings, several work items per CTA, blocks that span several images, split reduction axis."""
 import numpy as np
@@ -31,7 +31,7 @@ def _plans(nm, s):
     return [_plan(nm), _plan(nm, loads=1), _plan(nm, loads=2), _plan(nm, bn=t), _plan(nm, bn=t, loads=1, stages=2),
             _plan(nm, bn=2 * t, issuers=1), _plan(nm, bn=4 * t, issuers=2, loads=1), _plan(nm, bn=4 * t, loads=2, stages=1), _plan(nm, loads=1, stages=4),
             _plan(nm, bn=256), _plan(nm, bn=128, loads=2),
-            # four and eight epilogue warps (split = 1, 2; the default picks by the item's chunk count)
+            # (split = 0, 1 and 2 are the same)
             _plan(nm, split=1), _plan(nm, split=2), _plan(nm, bn=t, split=2, loads=1), _plan(nm, bn=256, split=2), _plan(nm, bn=2 * t, split=1, issuers=2)]
 
 
