@@ -11,9 +11,9 @@ tensor of the right shape.  One step = one pass over all 53 layers through the C
 Prints ONE JSON line on stdout, short enough to survive where only the end of the output is kept: images/s over all GPUs
 (inputs resident in HBM), the same through the host-buffer entry point (`e2e`), a roofline object (algorithmic bytes /
 measured time against the measured HBM copy peak) and clocks sampled during the timed region.  Everything measured beside it
-goes to stderr as one JSON line (and to `--json-out`): the CPU checker timed on a bounded sample (`cpu_baseline`), the chained network, a
+goes to stderr as one JSON line (and to `--json-out`): the CPU oracle timed on a bounded sample (`cpu_baseline`), the chained network, a
 per-layer table (time, useful TFLOP/s, fraction of max(kept FLOPs / TF32 peak, bytes / HBM peak)).  `--impl reference` times
-the CPU checker instead.
+the CPU oracle instead.
 """
 from __future__ import annotations
 
