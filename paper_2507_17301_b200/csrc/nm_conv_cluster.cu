@@ -34,7 +34,6 @@ using namespace nmk;
 constexpr int THREADS = 192;      // warps: 0 producer, 1 MMA issuer and tensor memory, 2-5 reduction and store
 constexpr int NSTAGE_MAX = 12;
 constexpr int EPI = 128;          // threads of the reduction
-constexpr int AHEAD = 4;          // float4s per thread whose bias and shortcut are fetched before the accumulator is ready
 
 enum LoadForm { ROWS_2D = 0, IM2COL = 1, BOX_4D = 2 };
 
@@ -130,7 +129,6 @@ k_conv_cluster(const ConvParams p, const ClusterCfg cfg, const __grid_constant__
     int my_rows = count - row0;                          // how many of its rows exist
     if (my_rows > cfg.rps) my_rows = cfg.rps;
     if (my_rows < 0) my_rows = 0;
-    const int n_f4 = my_rows << Q4;
     if (CS > 1) {
         // the barrier knows how many bytes to expect, and every CTA of the cluster has started, before any of them sends
         // (waited for below)
@@ -231,32 +229,55 @@ k_conv_cluster(const ConvParams p, const ClusterCfg cfg, const __grid_constant__
     if (CS > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // every CTA of the cluster is running
     if (warp >= 2) {
         // =========================== reduction and store ===========================
+        // Everything that does not depend on the sums is worked out, and the bias and the first shortcut pieces are loaded, before the
+        // accumulator is ready.  A thread's output pieces (16 bytes) lie STEP rows apart in the same channels, so it needs one piece
+        // of the bias.  (Fetched piece by piece between the stores, bias and shortcut cost a CTA without a cluster 1.1 us at its end:
+        // 192 -> 32 at 28x28, batch 32, 4.9 us.)
         const int e = tid - 64;
-        const int o0 = slice * BN;
-        float4 extra[AHEAD];               // bias + shortcut of this thread's first float4s
-        auto fetch = [&](int f) {
-            const int r = f >> Q4, o = o0 + (f & ((1 << Q4) - 1)) * 4;
-            float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (o < p.c_out) {
-                if (p.bias) a = __ldg(reinterpret_cast<const float4*>(p.bias + o));
-                if (p.residual) nm_add4(a, __ldg(reinterpret_cast<const float4*>(p.residual + (pix0 + row0 + r) * p.c_out + o)));
-            }
-            return a;
-        };
-        pdl_wait();   // the shortcut is read, and y written, only after the previous kernel
+        constexpr int STEP = EPI >> Q4;
+        // output pieces whose shortcut is fetched together: all of a thread's, up to eight
+        constexpr int AHEAD = (1 << Q4) / CS > 8 ? 8 : (1 << Q4) / CS;
+        const int c = e & ((1 << Q4) - 1), r0 = e >> Q4, o = slice * BN + c * 4;
+        const bool mine = o < p.c_out;
+        const size_t at_out = static_cast<size_t>(pix0 + row0 + r0) * p.c_out + o, out_step = static_cast<size_t>(STEP) * p.c_out;
+        const float* res = p.residual && mine ? p.residual + at_out : nullptr;
+        float* out = p.y + at_out;
+        const int q = warp & 3;        // tensor-memory lane quadrant this warp may read
+        const int row = q * 32 + lane;
+        const int lrow = CS > 1 ? row % cfg.rps : row;
+        const uint32_t dst = (CS > 1 ? ring : part) + row * (BN * 4), dst_swz = static_cast<uint32_t>(lrow & 7) << 4;
+        const uint32_t src_step = static_cast<uint32_t>(cfg.rps) * (BN * 4);
+        // the copies this warp sends: source, destination, barrier there, bytes
+        constexpr int SENDS = CS > 4 ? 2 : 1;
+        uint32_t send_src[SENDS], send_dst[SENDS], send_bar[SENDS], send_bytes[SENDS];
+        if (CS > 1) {
 #pragma unroll
-        for (int k = 0; k < AHEAD; ++k)
-            if (e + k * EPI < n_f4) extra[k] = fetch(e + k * EPI);
+            for (int k = 0; k < SENDS; ++k) {
+                const int owner = q + 4 * k;
+                int rows = owner < CS ? count - owner * cfg.rps : 0;
+                if (rows > cfg.rps) rows = cfg.rps;
+                send_bytes[k] = rows > 0 ? static_cast<uint32_t>(rows) * (BN * 4) : 0u;
+                send_src[k] = ring + owner * src_step;
+                send_dst[k] = send_bytes[k] ? mapa_shared(part + rank * src_step, static_cast<uint32_t>(owner)) : 0u;
+                send_bar[k] = send_bytes[k] ? mapa_shared(smem_u32(&s_part), static_cast<uint32_t>(owner)) : 0u;
+            }
+        }
+        pdl_wait();   // bias and shortcut are read, and y written, only after the previous kernel
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 bias = p.bias && mine ? __ldg(reinterpret_cast<const float4*>(p.bias + o)) : zero;
+        float4 ahead[AHEAD];               // shortcut pieces
+        auto fetch = [&](int r) {
+#pragma unroll
+            for (int k = 0; k < AHEAD; ++k)
+                ahead[k] = res && r + k * STEP < my_rows ? __ldg(reinterpret_cast<const float4*>(res + k * out_step)) : zero;
+        };
+        fetch(r0);
         const bool ok = aborted(abort_flag) || mbar_wait(smem_u32(&s_acc), 0);
         if (!__all_sync(0xFFFFFFFFu, ok)) *abort_flag = 4;
         tc_fence_after();
         // A row of partial sums per thread, into this CTA's own shared memory: over the ring, which is idle now (with one CTA
         // per item straight to where they are added up).  16-byte pieces are XOR-ed with the row inside its run, so that the
         // 32 rows of a warp do not meet in one bank.
-        const int q = warp & 3;        // tensor-memory lane quadrant this warp may read
-        const int row = q * 32 + lane;
-        const int lrow = CS > 1 ? row % cfg.rps : row;
-        const uint32_t dst = (CS > 1 ? ring : part) + row * (BN * 4);
 #pragma unroll
         for (int blk = 0; blk < BN / 32; ++blk) {
             uint32_t v[32];
@@ -265,7 +286,7 @@ k_conv_cluster(const ConvParams p, const ClusterCfg cfg, const __grid_constant__
             if (row < count) {
 #pragma unroll
                 for (int k = 0; k < 8; ++k)
-                    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst + blk * 128 + ((k ^ (lrow & 7)) << 4)), "r"(v[4 * k]),
+                    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst + blk * 128 + ((k << 4) ^ dst_swz)), "r"(v[4 * k]),
                                  "r"(v[4 * k + 1]), "r"(v[4 * k + 2]), "r"(v[4 * k + 3])
                                  : "memory");
             }
@@ -274,13 +295,12 @@ k_conv_cluster(const ConvParams p, const ClusterCfg cfg, const __grid_constant__
         if (CS > 1) fence_proxy_async();
         asm volatile("bar.sync 1, %0;" ::"n"(EPI) : "memory");
         if (CS > 1) {
-            for (int owner = q; owner < CS; owner += 4) {
-                const int rows = count - owner * cfg.rps < cfg.rps ? count - owner * cfg.rps : cfg.rps;
-                if (rows > 0 && elect_one())
-                    bulk_copy_cluster(mapa_shared(part + rank * cfg.rps * (BN * 4), static_cast<uint32_t>(owner)),
-                                      ring + owner * cfg.rps * (BN * 4), static_cast<uint32_t>(rows) * (BN * 4),
-                                      mapa_shared(smem_u32(&s_part), static_cast<uint32_t>(owner)));
+            if (elect_one()) {
+#pragma unroll
+                for (int k = 0; k < SENDS; ++k)
+                    if (send_bytes[k]) bulk_copy_cluster(send_dst[k], send_src[k], send_bytes[k], send_bar[k]);
             }
+            __syncwarp();
             // every partial sum of this CTA's rows has landed; the limit is a multiple of the other waits', so that a CTA of the
             // cluster that gave up on one of those has sent by then
             const uint32_t bar_own = smem_u32(&s_part);
@@ -289,24 +309,27 @@ k_conv_cluster(const ConvParams p, const ClusterCfg cfg, const __grid_constant__
             asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
         }
         if (!aborted(abort_flag)) {
-            const uint32_t src_step = static_cast<uint32_t>(cfg.rps) * (BN * 4);
-            auto finish = [&](int f, float4 a) {
-                const int r = f >> Q4, c = f & ((1 << Q4) - 1);
-                const uint32_t at = part + ((r << Q4) + ((c & ~7) | ((c ^ r) & 7))) * 16;
-                float4 s[CS];
+            for (int r = r0; r < my_rows; r += AHEAD * STEP) {
+                if (r != r0) fetch(r);
 #pragma unroll
-                for (int k = 0; k < CS; ++k) s[k] = ld_shared_f4(at + k * src_step);
+                for (int k = 0; k < AHEAD; ++k) {
+                    const int rk = r + k * STEP;
+                    if (rk < my_rows) {
+                        const uint32_t at = part + ((rk << Q4) + ((c & ~7) | ((c ^ rk) & 7))) * 16;
+                        float4 s[CS];
 #pragma unroll
-                for (int k = 1; k < CS; ++k) nm_add4(s[0], s[k]);
-                nm_add4(s[0], a);
-                if (p.relu) { s[0].x = fmaxf(s[0].x, 0.f); s[0].y = fmaxf(s[0].y, 0.f); s[0].z = fmaxf(s[0].z, 0.f); s[0].w = fmaxf(s[0].w, 0.f); }
-                const int o = o0 + c * 4;
-                if (o < p.c_out) *reinterpret_cast<float4*>(p.y + (pix0 + row0 + r) * p.c_out + o) = s[0];
-            };
+                        for (int i = 0; i < CS; ++i) s[i] = ld_shared_f4(at + i * src_step);
 #pragma unroll
-            for (int k = 0; k < AHEAD; ++k)
-                if (e + k * EPI < n_f4) finish(e + k * EPI, extra[k]);
-            for (int f = e + AHEAD * EPI; f < n_f4; f += EPI) finish(f, fetch(f));
+                        for (int i = 1; i < CS; ++i) nm_add4(s[0], s[i]);
+                        nm_add4(ahead[k], bias);
+                        nm_add4(s[0], ahead[k]);
+                        if (p.relu) { s[0].x = fmaxf(s[0].x, 0.f); s[0].y = fmaxf(s[0].y, 0.f); s[0].z = fmaxf(s[0].z, 0.f); s[0].w = fmaxf(s[0].w, 0.f); }
+                        if (mine) *reinterpret_cast<float4*>(out + k * out_step) = s[0];
+                    }
+                }
+                out += AHEAD * out_step;
+                if (res) res += AHEAD * out_step;
+            }
         }
     }
 
