@@ -67,24 +67,6 @@ constexpr int BOX_BYTES = 4096;    // staging box: 32 pixels x 32 channels
 constexpr int RING_BUDGET = 227 * 1024 - 1024 - 1024;   // alignment slack, static shared
 constexpr int TABLE_BYTES = 128;   // column table of a unit: [step][place in a quad][quad] 32-bit words
 
-// Division of n < 2^31 by a divisor known to the host, without the hardware's long sequence (Granlund and Montgomery, "Division by
-// invariant integers using multiplication", 1994): an item's eight divisions took 2000 cycles of every warp, as long as
-// three chunks.
-struct Divisor {
-    uint32_t mul, shift;
-};
-__device__ __forceinline__ int div_by(int n, const Divisor& d)
-{
-    return static_cast<int>((__umulhi(static_cast<uint32_t>(n), d.mul) + static_cast<uint32_t>(n)) >> d.shift);
-}
-Divisor divisor(int d)
-{
-    Divisor r = {0u, 0u};
-    while ((1ll << r.shift) < d) ++r.shift;
-    r.mul = static_cast<uint32_t>(((1ull << 32) * ((1ull << r.shift) - static_cast<uint64_t>(d))) / static_cast<uint64_t>(d) + 1);
-    return r;
-}
-
 struct SelCfg {
     int g, bn, n_slices, n_acc, n_iss;
     int mma_n, sub;     // accumulator columns per MMA; MMAs (issuers) side by side in a tile: T = sub * mma_n

@@ -22,6 +22,7 @@ struct nm_weights {
     int device;
     uint8_t* block;      // the handle's device memory: one allocation that every array below except `splitk` lies in
     size_t block_bytes, block_used, zero_from;   // size of the block, bytes of it in use, first byte of the part that is cleared
+    bool clear_layouts;  // there are layouts in that part
     double* mass;        // device double[2] + int: L1 sums of the pruning pass, validity of imported indices
     int c_out, kh, kw, c_in, k, kk, n_keep, m_group, tile_t, n_tiles;
     int kk_pad;          // kk rounded up to a multiple of NM_KCHUNK
@@ -40,16 +41,36 @@ struct nm_weights {
     // Expanded layout (variant 4): the pruned matrix back in dense shape, zeros in the pruned columns.
     float* splitk;       // scratch for split-K partial sums (variant 4), allocated by nm_autotune; may be NULL
     size_t splitk_bytes;
-    float* wx;           // [ceil(k / 32)][wx_rows][32] TF32, rows swizzled (see k_build_layouts); NULL when the shape rules the variant out
+    float* wx;           // [ceil(k / 32)][wx_rows][32] TF32, rows swizzled (see k_compress); NULL when the shape rules the variant out
     int wx_rows;         // c_out rounded up to a multiple of 32 (the rows past c_out are zero)
     // Select layout (variant 8): steps of sel_s source columns of which every tile keeps sel_kc, chunks of as many steps as fit 32
     // retained columns; NULL when the pattern or the shape rules the variant out.
-    float* w3;           // [sel_chunks][c_out][32] TF32, rows swizzled (see k_build_layouts)
-    uint8_t* sel3;       // [sel_chunks][n_tiles][32 words] column tables (see k_build_layouts)
+    float* w3;           // [sel_chunks][c_out][32] TF32, rows swizzled (see k_compress)
+    uint8_t* sel3;       // [sel_chunks][n_tiles][32 words] column tables (see k_compress)
     int sel_s, sel_kc, sel_chunks;
     // Plane layout (variant 9): per kernel row a [c_out][32] tile of (kw, c) slots; NULL when the shape rules it out.
-    float* ws;           // [kh][c_out][32] TF32, rows swizzled (see k_build_layouts)
+    float* ws;           // [kh][c_out][32] TF32, rows swizzled (see k_compress)
 };
+
+// Division of n < 2^31 by a divisor known to the host, without the hardware's long sequence (Granlund and Montgomery, "Division by
+// invariant integers using multiplication", 1994): the eight
+// divisions of an item of the select kernel took 2000 cycles of every warp, as long as three chunks.
+struct Divisor {
+    uint32_t mul, shift;
+};
+#ifdef __CUDACC__
+__device__ __forceinline__ int div_by(int n, const Divisor& d)
+{
+    return static_cast<int>((__umulhi(static_cast<uint32_t>(n), d.mul) + static_cast<uint32_t>(n)) >> d.shift);
+}
+#endif
+inline Divisor divisor(int d)
+{
+    Divisor r = {0u, 0u};
+    while ((1ll << r.shift) < d) ++r.shift;
+    r.mul = static_cast<uint32_t>(((1ull << 32) * ((1ull << r.shift) - static_cast<uint64_t>(d))) / static_cast<uint64_t>(d) + 1);
+    return r;
+}
 
 // Geometry handed to the convolution kernels.
 struct ConvParams {
@@ -192,6 +213,10 @@ nm_status_t clear_handle_memory(nm_weights* h, cudaStream_t st);   // the part o
 // Values and layouts from the index array `idx` and the dense weights (import = false) or the retained values (true).
 nm_status_t build_layouts(nm_weights* h, const float* src, const uint16_t* idx, bool import, cudaStream_t st);
 nm_status_t finish_handle(nm_weights* h, cudaStream_t st, double* mass2, int* bad);   // synchronises `st`
+// Groups that fit a block: selection (`idx` NULL, `src` dense) or check of given indices (`src`: retained values) and all layouts in one
+// kernel; synchronises `st`.
+bool compressed_in_one(const nm_weights* h);
+nm_status_t compress_in_one(nm_weights* h, const float* src, const uint16_t* idx, cudaStream_t st, double* mass2, int* bad);
 
 // nm_prune.cu
 nm_status_t prune_on_device(const float* w_dense, nm_weights* h, cudaStream_t st);

@@ -9,9 +9,11 @@
 // after its device has been synchronised, so whoever takes it next may use it on any stream; the list is guarded by a
 // mutex.
 //
-// All layouts are written by ONE kernel from the index array and the values (k_build_layouts), after one memset of those
-// that have padding or pruned columns: a thread decodes a retained column once and stores the values of a few rows to each of
-// them.  It is bound by the writes (28 MB for 512 x 3 x 3 x 512 at 2:4).
+// With groups of at most 128 columns a handle is built by ONE kernel (k_compress): a block owns a span of whole groups of one tile
+// (up to 64 of its rows), reads that piece of the dense weights (import: of the retained values) once into shared memory, selects
+// the columns there, and writes the piece's part of every layout, zeros of the expanded one included.  Wider groups are
+// selected by the kernels of nm_prune.cu, and k_build_layouts writes the layouts from the index array after a memset.
+// Both are bound by the writes (28 MB for 512 x 3 x 3 x 512 at 2:4).
 #include <algorithm>
 #include <mutex>
 #include <vector>
@@ -61,6 +63,13 @@ struct Readback {
     double mass[2];
     int bad;
 };
+// What the blocks of a creating call add up, one per pinned slot: zero before and after every call (its last block hands the sums over
+// and clears them), so that no call has to.
+struct Accum {
+    Readback sum;
+    unsigned done;
+};
+__device__ Accum g_accum[kSlots];
 std::mutex g_slot_mu;
 Readback* g_slots = nullptr;
 bool g_slots_tried = false;
@@ -104,6 +113,8 @@ struct LayoutArgs {
     float* w3; uint8_t* sel3; int sel_s, sel_kc;
     float* ws;
     int* bad;
+    int* status;
+    Divisor by_c_in, by_kw, by_v2_s;
 };
 
 // Place of retained column e of a select step among the step's `kc` columns, given by their indices `idx`: quads of columns
@@ -215,6 +226,237 @@ __global__ void k_build_layouts(const LayoutArgs a)
     }
 }
 
+constexpr int SPAN = 128;   // columns of a k_compress block, at most
+constexpr int PART = 64;    // rows of a tile that a block writes, at most
+
+// Selection (import: check) and every layout of a span of whole groups, PART rows of one tile.  The selection is the one described at the
+// head of nm_prune.cu.  Threads: a column each while scores are summed (the tile's rows in order, PART at a time through shared memory).
+// Then 128 threads work out where the retained columns go in every layout, while the others write the expanded layout, whose 128-byte rows
+// a warp writes whole; then all write the other layouts, a retained column and every threads >> log_j-th row each.  The last warp
+// adds the block's sums to the call's meanwhile (2 us with its fence, when it was part of the others' way).
+// 512 x 3 x 3 x 512 at 2:4, T = 64 (28 MB written): 12 us; a memset, a kernel for the selection and one for the layouts took 18 and the
+// gaps between them.  nm_prune and export of that layer 66 -> 46 us, import and export of 1024 -> 2048, 1x1 54 -> 45.
+template <bool IMPORT>
+__global__ void __launch_bounds__(544) k_compress(const LayoutArgs a, int span, int log_j, Readback* sums, int slot, Readback* host)
+{
+    __shared__ __align__(16) float s_tile[PART][SPAN];
+    __shared__ double s_score[SPAN];
+    __shared__ uint16_t s_idx[SPAN];   // retained columns of the span, 0xFFFF: a bad one (import)
+    __shared__ short s_pos[SPAN];      // place of a column of the span among them, -1: pruned
+    __shared__ uint32_t s_at2[SPAN], s_at3[SPAN], s_ats[SPAN];   // places of a retained column in wt2, w3 (chunk, position), ws
+    const int tid = threadIdx.x, threads = blockDim.x - 32, r = blockIdx.y, row0 = r * a.tile_t;   // (without the last warp)
+    const int c0 = blockIdx.x * span, cols = min(span, a.k - c0);
+    const int tile_rows = min(a.tile_t, a.c_out - row0);
+    const int p0 = blockIdx.z * PART, rows = max(0, min(PART, tile_rows - p0));   // (none in a short last tile: the block is only counted)
+    const int groups = span / a.m_group, j0 = static_cast<int>(blockIdx.x) * groups * a.n_keep;
+    const int nk = min(a.kk, j0 + groups * a.n_keep) - j0;
+    const bool first = blockIdx.z == 0;   // this block also writes what the tile's rows share
+    const int j = tid & ((1 << log_j) - 1);
+    if (blockIdx.x == 0 && r == 0 && first && tid < 4) a.status[tid] = 0;
+
+    if (!IMPORT) {
+        double score = 0.0;
+        const bool quads = ((a.k | span) & 3) == 0 && (reinterpret_cast<uintptr_t>(a.src) & 15) == 0;
+        auto load = [&](int from) {   // rows [from, from + PART) of the tile
+            const int n = min(PART, tile_rows - from);
+            const float* src = a.src + static_cast<size_t>(row0 + from) * a.k + c0;
+            if (tid >= threads) return;
+            if (quads) {
+                const int t = (tid & (SPAN / 4 - 1)) * 4;
+                if (t < cols)
+#pragma unroll 8
+                    for (int rr = tid / (SPAN / 4); rr < n; rr += threads / (SPAN / 4))
+                        *reinterpret_cast<float4*>(&s_tile[rr][t]) = __ldg(reinterpret_cast<const float4*>(src + static_cast<size_t>(rr) * a.k + t));
+            } else {
+                const int t = tid & (SPAN - 1);
+                if (t < cols)
+#pragma unroll 8
+                    for (int rr = tid / SPAN; rr < n; rr += threads / SPAN) s_tile[rr][t] = __ldg(src + static_cast<size_t>(rr) * a.k + t);
+            }
+        };
+        int from = 0;
+        for (;; from += PART) {
+            load(from);
+            __syncthreads();
+            if (tid < cols) {
+                const int n = min(PART, tile_rows - from);
+#pragma unroll 8
+                for (int rr = 0; rr < n; ++rr) score += fabs(static_cast<double>(s_tile[rr][tid]));
+            }
+            if (from + PART >= tile_rows) break;
+            __syncthreads();
+        }
+        if (from != p0 && rows > 0) {
+            __syncthreads();
+            load(p0);
+        }
+        if (tid < cols) {
+            if (!(score == score)) score = static_cast<double>(INFINITY);
+            s_score[tid] = score;
+        }
+        __syncthreads();
+        const int g_first = tid / a.m_group * a.m_group;
+        bool keep = false;
+        if (tid < cols) {
+            const int g_end = min(g_first + a.m_group, cols);
+            int beaten_by = 0;
+            for (int i = g_first; i < g_end; ++i) {
+                const double si = s_score[i];
+                beaten_by += (si > score) || (si == score && i < tid);
+            }
+            keep = beaten_by < a.n_keep;
+            s_pos[tid] = keep ? 1 : 0;
+        }
+        __syncthreads();
+        int pos = -1;
+        if (keep) {
+            const int g = tid / a.m_group;
+            pos = g * a.n_keep;   // every earlier group is a full one and kept exactly n_keep
+            for (int i = g_first; i < tid; ++i) pos += s_pos[i];
+            // the order of the scores is total, so a group keeps at most N columns; the bound makes sure that no input
+            // whatsoever can place a column outside its group's slots
+            if (pos >= min(nk, (g + 1) * a.n_keep)) pos = -1;
+        }
+        __syncthreads();
+        if (tid < cols) s_pos[tid] = static_cast<short>(pos);
+        if (pos >= 0) s_idx[pos] = static_cast<uint16_t>(c0 + tid);
+    } else {
+        if (tid < SPAN) s_pos[tid] = -1;
+        __syncthreads();
+        if (tid < nk) {
+            // strictly ascending below K, and retained column j in group j / N of M consecutive columns (a tail group of
+            // m' < M columns keeps min(N, m'), which the same quotient covers); nothing is stored for a bad column
+            const uint16_t* idx = a.idx + static_cast<size_t>(r) * a.kk;
+            const int jj = j0 + tid, col = idx[jj];
+            const bool bad = col >= a.k || col / a.m_group != jj / a.n_keep;
+            if (first && (bad || (jj > 0 && idx[jj - 1] >= col))) {
+                atomicExch(slot >= 0 ? &g_accum[slot].sum.bad : &sums->bad, 1);
+                __threadfence();
+            }
+            s_idx[tid] = bad ? 0xFFFFu : static_cast<uint16_t>(col);
+            if (!bad) s_pos[col - c0] = static_cast<short>(tid);
+        }
+        const float* src = a.src + static_cast<size_t>(row0 + p0) * a.kk + j0;
+        if (tid < threads && j < nk)
+#pragma unroll 8
+            for (int rr = tid >> log_j; rr < rows; rr += threads >> log_j) s_tile[rr][j] = src[static_cast<size_t>(rr) * a.kk + j];
+    }
+    __syncthreads();
+
+    if (tid >= threads) {
+        // L1 mass of all columns and of the retained ones
+        const int lane = tid & 31;
+        Readback* const acc = slot >= 0 ? &g_accum[slot].sum : sums;
+        if (!IMPORT && first) {
+            double all = 0.0, kept = 0.0;
+            for (int i = lane; i < cols; i += 32) {
+                all += s_score[i];
+                if (s_pos[i] >= 0) kept += s_score[i];
+            }
+            for (int d = 16; d > 0; d >>= 1) {
+                all += __shfl_down_sync(0xFFFFFFFFu, all, d);
+                kept += __shfl_down_sync(0xFFFFFFFFu, kept, d);
+            }
+            if (lane == 0) {
+                atomicAdd(acc->mass, all);
+                atomicAdd(acc->mass + 1, kept);
+            }
+        }
+        if (slot >= 0 && lane == 0) {
+            __threadfence();
+            if (atomicAdd(&g_accum[slot].done, 1u) + 1 == gridDim.x * gridDim.y * gridDim.z) {
+                // the last block to add its sums hands them over (the host reads them once the stream is done)
+                __threadfence();
+                volatile Accum* const total = &g_accum[slot];
+                volatile Readback* const out = host;
+                out->mass[0] = total->sum.mass[0];
+                out->mass[1] = total->sum.mass[1];
+                out->bad = total->sum.bad;
+                total->sum.mass[0] = total->sum.mass[1] = 0.0;
+                total->sum.bad = 0;
+                total->done = 0u;
+            }
+        }
+        return;
+    }
+    const size_t pitch2 = static_cast<size_t>(a.v2_chunks) * 32;
+    if (tid < SPAN) {
+        const int jj = j0 + tid, col = tid < nk ? s_idx[tid] : 0xFFFF;
+        if (col != 0xFFFF) {
+            const int tap = div_by(col, a.by_c_in), c = col - tap * a.c_in, khi = div_by(tap, a.by_kw), kwi = tap - khi * a.kw;
+            if (first) {
+                a.indices[static_cast<size_t>(r) * a.kk + jj] = static_cast<uint16_t>(col);
+                a.taps[static_cast<size_t>(r) * a.kk_pad + jj] = (static_cast<uint32_t>(khi) << 24) | (static_cast<uint32_t>(kwi) << 16) | static_cast<uint32_t>(c);
+            }
+            // slab layout: kept column jj lies in chunk col / S at position jj - chunk * KC (every group before the last is
+            // full, so a chunk of whole groups holds exactly KC kept columns)
+            if (a.wt2) {
+                const int chunk = div_by(col, a.by_v2_s), at = chunk * 32 + (jj - chunk * a.v2_kc);
+                s_at2[tid] = static_cast<uint32_t>(at);
+                if (first) a.rel2[static_cast<size_t>(r) * pitch2 + at] = static_cast<uint8_t>(col - chunk * a.v2_s);
+            }
+            // select layout: w3[chunk][o][32], a chunk being as many steps (one tap of S source columns, of which KC are kept) as fit,
+            // the steps ordered by block of S channels, then tap; swizzled like wx.  The
+            // column tables hold, per chunk and tile, the byte offset of each column in its 128-byte row (and its 32-channel block in
+            // bit 7 and up), in the order in which a thread reads them: [step][place in a quad][quad].  (A span is whole steps.)
+            if (a.w3) {
+                // (steps of 32 or 64 columns; four, two or one of them in a chunk as 8, 16 or 24 columns stay; a step's columns begin at its column's)
+                const int shift_s = a.sel_s == 64 ? 6 : 5, shift_c = a.sel_kc == 8 ? 2 : a.sel_kc == 16 ? 1 : 0, cb = c >> shift_s, cc = c - (cb << shift_s);
+                const int step = cb * a.kh * a.kw + tap, chunk = step >> shift_c, sub = step - (chunk << shift_c), js = ((col - c0) >> shift_s) * a.sel_kc;
+                const int place = select_place(s_idx + js, a.sel_kc, tid - js);
+                // (a thread's columns of two quads are neighbours)
+                s_at3[tid] = static_cast<uint32_t>(chunk * 32 + sub * a.sel_kc + (place >> 3) * 8 + (place & 3) * 2 + (place >> 2 & 1));
+                if (first)
+                    reinterpret_cast<uint32_t*>(a.sel3)[(static_cast<size_t>(chunk) * a.n_tiles + r) * 32 + sub * a.sel_kc + (place & 3) * (a.sel_kc / 4) + (place >> 2)] =
+                        static_cast<uint32_t>((cc & 31) * 4 | (cc >> 5) << 7);
+            }
+            if (a.ws) s_ats[tid] = static_cast<uint32_t>(khi << 5 | kwi << 2 | c);
+        }
+        if (first && blockIdx.x + 1 == gridDim.x)
+            for (int i = a.kk + tid; i < a.kk_pad; i += SPAN) a.taps[static_cast<size_t>(r) * a.kk_pad + i] = NM_TAP_PAD;
+    } else if (a.wx) {
+        // expanded layout: the shared-memory image the tensor core reads: blocks of 32 columns, inside a block one
+        // 128-byte row per output channel whose 16-byte pieces are XOR-ed with (o % 8) (the 128-byte swizzle), so that
+        // any run of channels starting at a multiple of 8 is one contiguous bulk copy
+        auto cell = [&](int o, int col) {
+            const int kc = col & 31;
+            return a.wx + (static_cast<size_t>(col >> 5) * a.wx_rows + o) * 32 + ((((kc >> 2) ^ (o & 7)) << 2) | (kc & 3));
+        };
+        const int at = tid - SPAN, n = threads - SPAN, t = at & (SPAN - 1);
+        if (t < cols) {
+            const int pos = s_pos[t], from = IMPORT ? pos : t;
+            for (int rr = at / SPAN; rr < rows; rr += n / SPAN) *cell(row0 + p0 + rr, c0 + t) = pos >= 0 ? nmk::to_tf32(s_tile[rr][from]) : 0.f;
+        }
+        // zeros: columns up to the last block's 32nd, rows up to the last 32nd
+        const int pad_cols = blockIdx.x + 1 == gridDim.x ? (32 - (a.k & 31)) & 31 : 0;
+        for (int i = at; i < rows * pad_cols; i += n) *cell(row0 + p0 + i / pad_cols, a.k + i % pad_cols) = 0.f;
+        if (r + 1 == static_cast<int>(gridDim.y) && first)
+            for (int i = at; i < (a.wx_rows - a.c_out) * (cols + pad_cols); i += n) *cell(a.c_out + i / (cols + pad_cols), c0 + i % (cols + pad_cols)) = 0.f;
+    }
+    asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory");
+
+    const int col = j < nk ? s_idx[j] : 0xFFFF;
+    if (col == 0xFFFF) return;
+    // gather layout: per (tile, chunk of 32 retained columns) the shared-memory image of the tile's rows, swizzled like wx; as many
+    // rows as the tile has, so it is as large as the values whatever the tile width
+    const int jj = j0 + j, w = jj & (NM_KCHUNK - 1), from = IMPORT ? j : col - c0;
+    float* const wt = a.wt + static_cast<size_t>(row0) * a.kk_pad + static_cast<size_t>(jj / NM_KCHUNK) * tile_rows * NM_KCHUNK;
+    float* const wt2 = a.wt2 ? a.wt2 + s_at2[j] : nullptr;
+    const int k3 = a.w3 ? s_at3[j] & 31 : 0;
+    float* const w3 = a.w3 ? a.w3 + static_cast<size_t>(s_at3[j] >> 5) * a.c_out * 32 : nullptr;
+    for (int rr = tid >> log_j; rr < rows; rr += threads >> log_j) {
+        const int tr = p0 + rr, o = row0 + tr;
+        const float v = s_tile[rr][from], t = nmk::to_tf32(v);
+        a.values[static_cast<size_t>(o) * a.kk + jj] = v;
+        wt[tr * NM_KCHUNK + ((((w >> 2) ^ (tr & 7)) << 2) | (w & 3))] = t;
+        if (wt2) wt2[static_cast<size_t>(o) * pitch2] = t;
+        if (w3) w3[static_cast<size_t>(o) * 32 + ((((k3 >> 2) ^ (o & 7)) << 2) | (k3 & 3))] = t;
+        // plane layout: ws[kh][c_out][32]: a row holds the taps of one kernel row as (kw, c), c padded to 4 and kw to 8,
+        // its 16-byte pieces (one tap each) XOR-ed with (o % 8)
+        if (a.ws) a.ws[(static_cast<size_t>(s_ats[j] >> 5) * a.c_out + o) * 32 + (((s_ats[j] >> 2 & 7) ^ (o & 7)) << 2) + (s_ats[j] & 3)] = t;
+    }
+}
+
 }  // namespace
 
 namespace nmhost {
@@ -299,6 +541,8 @@ void device_block_free(void* ptr, size_t bytes, int device, bool idle)
     while (!g_cache.empty() && (g_cached > kCacheBytes || g_cache.front().stamp + kCacheAge < g_frees)) drop(0);
 }
 
+bool compressed_in_one(const nm_weights* h) { return h->m_group <= SPAN && h->kk > 0; }
+
 // Which layouts this layer's kernels can read, and their dimensions (no device work).
 static void plan_layouts(nm_weights* h)
 {
@@ -346,29 +590,30 @@ nm_status_t alloc_handle_memory(nm_weights* h, const char* who)
     // Layouts that every word of is written come before the part of the block that the creating call clears (status, sums and layouts with
     // padding or zeros in the pruned columns): 512 x 3 x 3 x 512 at 2:4 has 9 of 24 MB to clear, 58 -> 51 us.
     const int spc = h->sel_s ? 32 / h->sel_kc : 1;
+    const bool full_wx = compressed_in_one(h);
     const bool full_wt = h->kk % NM_KCHUNK == 0;
     const bool full_wt2 = h->v2_kc == 32 && h->k % std::max(h->v2_s, 1) == 0;
     const bool full_w3 = h->sel_s && h->sel_kc * spc == 32 && h->k / h->sel_s % spc == 0;
-    size_t at_status = 0, at_mass = 0, at_wt = 0, at_wt2 = 0, at_rel2 = 0, at_wx = 0, at_w3 = 0, at_sel3 = 0, at_ws = 0;
+    size_t sums_end = 0, at_status = 0, at_mass = 0, at_wt = 0, at_wt2 = 0, at_rel2 = 0, at_wx = 0, at_w3 = 0, at_sel3 = 0, at_ws = 0;
     for (const bool full : {true, false}) {
         if (!full) {
             h->zero_from = total;
             at_status = place(4 * sizeof(int));
             at_mass = place(sizeof(Readback));
+            sums_end = total;
         }
+        if (h->wx_rows && full_wx == full) at_wx = place(static_cast<size_t>((h->k + 31) / 32) * h->wx_rows * 128);
         if (full_wt == full) at_wt = place(static_cast<size_t>(h->c_out) * h->kk_pad * sizeof(float));
         if (full_wt2 == full) {
-            at_wt2 = place(h->v2_ok ? h->c_out * pitch2 * sizeof(float) : 0);
-            at_rel2 = place(h->v2_ok ? h->n_tiles * pitch2 : 0);
+            if (h->v2_ok) at_wt2 = place(h->c_out * pitch2 * sizeof(float)), at_rel2 = place(h->n_tiles * pitch2);
         }
         if (full_w3 == full) {
-            at_w3 = place(chunks3 * h->c_out * 128);
-            at_sel3 = place(chunks3 * h->n_tiles * 128);
+            if (h->sel_s) at_w3 = place(chunks3 * h->c_out * 128), at_sel3 = place(chunks3 * h->n_tiles * 128);
         }
     }
-    at_wx = place(h->wx_rows ? static_cast<size_t>((h->k + 31) / 32) * h->wx_rows * 128 : 0);
-    at_ws = place(planes ? static_cast<size_t>(h->kh) * h->c_out * 128 : 0);
+    if (planes) at_ws = place(static_cast<size_t>(h->kh) * h->c_out * 128);
     h->block_used = total;
+    h->clear_layouts = total > sums_end;
     h->block = static_cast<uint8_t*>(device_block_alloc(total, h->device, &h->block_bytes));
     if (!h->block) return fail(NM_ERR_ALLOC, "%s: cannot allocate %zu bytes on the device", who, total);
     h->values = reinterpret_cast<float*>(h->block + at_values);
@@ -396,7 +641,7 @@ nm_status_t clear_handle_memory(nm_weights* h, cudaStream_t st)
     return e == cudaSuccess ? NM_OK : fail(NM_ERR_CUDA, "clearing the handle's memory: %s", cudaGetErrorString(e));
 }
 
-nm_status_t build_layouts(nm_weights* h, const float* src, const uint16_t* idx, bool import, cudaStream_t st)
+static LayoutArgs layout_args(nm_weights* h, const float* src, const uint16_t* idx, bool import)
 {
     LayoutArgs a = {};
     a.src = src; a.idx = idx; a.import = import ? 1 : 0;
@@ -408,6 +653,14 @@ nm_status_t build_layouts(nm_weights* h, const float* src, const uint16_t* idx, 
     a.w3 = h->w3; a.sel3 = h->sel3; a.sel_s = h->sel_s; a.sel_kc = h->sel_kc;
     a.ws = h->ws;
     a.bad = &reinterpret_cast<Readback*>(h->mass)->bad;
+    a.status = h->status;
+    a.by_c_in = divisor(h->c_in); a.by_kw = divisor(h->kw); a.by_v2_s = divisor(std::max(h->v2_s, 1));
+    return a;
+}
+
+nm_status_t build_layouts(nm_weights* h, const float* src, const uint16_t* idx, bool import, cudaStream_t st)
+{
+    const LayoutArgs a = layout_args(h, src, idx, import);
     if (h->c_out > 65535) return fail(NM_ERR_CUDA, "weight layout kernel: more than 65535 output channels");   // bounds grid.y
     if (h->kk_pad > 0) {
         const dim3 grid((h->kk_pad + 127) / 128, h->n_tiles * ((h->tile_t + ROWS - 1) / ROWS));
@@ -416,6 +669,39 @@ nm_status_t build_layouts(nm_weights* h, const float* src, const uint16_t* idx, 
     }
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? NM_OK : fail(NM_ERR_CUDA, "weight layout kernel: %s", cudaGetErrorString(e));
+}
+
+nm_status_t compress_in_one(nm_weights* h, const float* src, const uint16_t* idx, cudaStream_t st, double* mass2, int* bad)
+{
+    if (h->c_out > 65535) return fail(NM_ERR_CUDA, "weight layout kernel: more than 65535 output channels");   // bounds grid.y
+    Readback* slot = take_slot();
+    // without a slot the sums lie in the handle, and are cleared and copied
+    if (h->clear_layouts || !slot) {
+        const nm_status_t s = clear_handle_memory(h, st);
+        if (s != NM_OK) {
+            if (slot) give_slot(slot);
+            return s;
+        }
+    }
+    const LayoutArgs a = layout_args(h, src, idx, idx != nullptr);
+    const int span = SPAN / h->m_group * h->m_group, rows = std::min(h->tile_t, h->c_out);
+    int log_j = 0;
+    while ((1 << log_j) < span / h->m_group * h->n_keep) ++log_j;
+    const dim3 grid((h->k + span - 1) / span, h->n_tiles, (rows + PART - 1) / PART);
+    const unsigned threads = (rows > 16 ? 512u : 256u) + 32u;
+    const int number = slot ? static_cast<int>(slot - g_slots) : -1;
+    if (idx) k_compress<true><<<grid, threads, 0, st>>>(a, span, log_j, reinterpret_cast<Readback*>(h->mass), number, slot);
+    else k_compress<false><<<grid, threads, 0, st>>>(a, span, log_j, reinterpret_cast<Readback*>(h->mass), number, slot);
+    count_launch(1);
+    cudaError_t e = cudaGetLastError();
+    if (!slot && e == cudaSuccess) return finish_handle(h, st, mass2, bad);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    const Readback got = slot ? *slot : Readback{};
+    if (slot) give_slot(slot);
+    if (e != cudaSuccess) return fail(NM_ERR_CUDA, "building the weight handle: %s", cudaGetErrorString(e));
+    if (mass2) { mass2[0] = got.mass[0]; mass2[1] = got.mass[1]; }
+    if (bad) *bad = got.bad;
+    return NM_OK;
 }
 
 nm_status_t finish_handle(nm_weights* h, cudaStream_t st, double* mass2, int* bad)

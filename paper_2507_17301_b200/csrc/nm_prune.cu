@@ -1,17 +1,16 @@
 // Column-wise N:M pruning at tile level (Sec. 3.1) on the device, and construction of the
 // kernel-side copies of the compressed form (Sec. 2.1; inputs W and Idx of Algorithm 1).
 //
-// k_prune_tile does the whole selection in one launch wherever a group fits a block (M <= 128): a block owns a span of
-// whole groups of one tile, a thread one column:
+// The selection:
 //   score    s[k]    = sum over the tile's rows of |w[o][k]|, fp64, ascending row order (bit-reproducible); a sum that
 //            is NaN (a NaN weight) counts as +infinity, so that the order below is total
 //   select   kept iff fewer than N columns of k's group beat it, where column i beats column k when s[i] > s[k], or
 //            s[i] == s[k] and i < k (lower column wins ties)
 //   place    position of a kept column = N * group + number of kept columns before it in its group
-// Scores and flags stay in shared memory (fp64 scores in global memory and four launches before).  Wider groups (the
-// adaptive form, M up to K) take the same steps as three kernels with the scores in scratch memory.
-// The selection rule is the closed form of "pick the largest N times": both orderings are the sort by (score
-// descending, column ascending), so the result is unique.  nm_layout.cu then writes values and kernel layouts.
+// It is the closed form of "pick the largest N times": both orderings are the sort by (score
+// descending, column ascending), so the result is unique.  Where a group fits a block (M <= 128) one kernel of nm_layout.cu selects and
+// writes values and kernel layouts.  Wider groups (the adaptive form, M up to K) take the steps as the kernels below with the scores in
+// scratch memory; nm_layout.cu then writes the rest.
 #include <algorithm>
 
 #include "nm_internal.h"
@@ -89,78 +88,31 @@ __global__ void k_compact(const uint8_t* __restrict__ keep, int k, int kk, int n
     indices[static_cast<size_t>(r) * kk + pos] = static_cast<uint16_t>(col);
 }
 
-constexpr int SPAN = 128;   // columns (threads) of a k_prune_tile block
-
-__global__ void __launch_bounds__(SPAN) k_prune_tile(const float* __restrict__ w, int c_out, int k, int kk, int tile_t, int n_keep,
-                                                     int m_group, int span, uint16_t* __restrict__ indices,
-                                                     double* __restrict__ mass)
+// Groups wider than a block of k_compress.
+nm_status_t prune_wide(const float* w_dense, nm_weights* h, cudaStream_t st, double* mass)
 {
-    __shared__ double s_score[SPAN], s_sum[2][SPAN / 32];
-    __shared__ uint8_t s_keep[SPAN];
-    const int t = threadIdx.x, r = blockIdx.y;
-    const int col = blockIdx.x * span + t;
-    const bool mine = t < span && col < k;
-    double s = 0.0;
-    if (mine) {
-        const int row0 = r * tile_t, rows = min(tile_t, c_out - row0);
-        const float* src = w + static_cast<size_t>(row0) * k + col;
-        int o = 0;
-        for (; o + 16 <= rows; o += 16) {   // the loads of sixteen rows in flight, the additions in row order
-            float v[16];
-#pragma unroll
-            for (int i = 0; i < 16; ++i) v[i] = __ldg(src + static_cast<size_t>(o + i) * k);
-#pragma unroll
-            for (int i = 0; i < 16; ++i) s += fabs(static_cast<double>(v[i]));
-        }
-        for (; o < rows; ++o) s += fabs(static_cast<double>(__ldg(src + static_cast<size_t>(o) * k)));
-        if (!(s == s)) s = static_cast<double>(INFINITY);
-        s_score[t] = s;
-    }
-    __syncthreads();
-    const int g0 = t / m_group * m_group;
-    bool keep = false;
-    if (mine) {
-        const int g1 = min(min(g0 + m_group, span), k - static_cast<int>(blockIdx.x) * span);
-        int beaten_by = 0;
-        for (int i = g0; i < g1; ++i) {
-            const double si = s_score[i];
-            beaten_by += (si > s) || (si == s && i < t);
-        }
-        keep = beaten_by < n_keep;
-        s_keep[t] = keep ? 1 : 0;
-    }
-    __syncthreads();
-    if (keep) {
-        const int g = col / m_group;
-        int pos = g * n_keep;   // every earlier group is a full one and kept exactly n_keep
-        for (int i = g0; i < t; ++i) pos += s_keep[i];
-        // the order of the scores is total, so a group keeps at most N columns; the bound makes sure that no input
-        // whatsoever can place a column outside its group's slots
-        if (pos < min(kk, (g + 1) * n_keep)) indices[static_cast<size_t>(r) * kk + pos] = static_cast<uint16_t>(col);
-    }
-    // L1 mass of all columns and of the retained ones
-    double all = mine ? s : 0.0, kept = keep ? s : 0.0;
-    for (int d = 16; d > 0; d >>= 1) {
-        all += __shfl_down_sync(0xFFFFFFFFu, all, d);
-        kept += __shfl_down_sync(0xFFFFFFFFu, kept, d);
-    }
-    if ((t & 31) == 0) { s_sum[0][t >> 5] = all; s_sum[1][t >> 5] = kept; }
-    __syncthreads();
-    if (t < 2) {
-        double sum = 0.0;
-        for (int i = 0; i < SPAN / 32; ++i) sum += s_sum[t][i];
-        atomicAdd(mass + t, sum);
-    }
+    using namespace nmhost;
+    nm_status_t st_out = clear_handle_memory(h, st);
+    if (st_out != NM_OK) return st_out;
+    size_t scratch_bytes = 0;
+    const size_t cells = static_cast<size_t>(h->n_tiles) * h->k;
+    uint8_t* scratch = static_cast<uint8_t*>(device_block_alloc(cells * 9, h->device, &scratch_bytes));
+    if (!scratch) return fail(NM_ERR_ALLOC, "nm_prune: cannot allocate %zu bytes of scratch", cells * 9);
+    double* score = reinterpret_cast<double*>(scratch);
+    uint8_t* keep = scratch + cells * sizeof(double);
+    const dim3 blk(128), grid((h->k + 127) / 128, h->n_tiles);
+    k_score<<<grid, blk, 0, st>>>(w_dense, h->c_out, h->k, h->tile_t, score);
+    k_select<<<grid, blk, 0, st>>>(score, h->k, h->n_keep, h->m_group, keep);
+    k_compact<<<grid, blk, 0, st>>>(keep, h->k, h->kk, h->n_keep, h->m_group, h->indices);
+    k_mass<<<static_cast<unsigned>(std::min<size_t>((cells + 255) / 256, 1024)), 256, 0, st>>>(score, keep, cells, h->mass);
+    count_launch(4);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) st_out = fail(NM_ERR_CUDA, "pruning kernels: %s", cudaGetErrorString(e));
+    if (st_out == NM_OK) st_out = build_layouts(h, w_dense, h->indices, false, st);
+    if (st_out == NM_OK) st_out = finish_handle(h, st, mass, nullptr);
+    device_block_free(scratch, scratch_bytes, h->device, st_out == NM_OK);
+    return st_out;
 }
-
-#define NM_CUDA_TRY(call)                                                                                   \
-    do {                                                                                                    \
-        cudaError_t e__ = (call);                                                                           \
-        if (e__ != cudaSuccess) {                                                                           \
-            st_out = nmhost::fail(NM_ERR_CUDA, "%s failed: %s", #call, cudaGetErrorString(e__));            \
-            goto done;                                                                                      \
-        }                                                                                                   \
-    } while (0)
 
 }  // namespace
 
@@ -168,46 +120,20 @@ namespace nmhost {
 
 nm_status_t prune_on_device(const float* w_dense, nm_weights* h, cudaStream_t st)
 {
-    nm_status_t st_out = clear_handle_memory(h, st);
-    if (st_out != NM_OK) return st_out;
-    uint8_t* scratch = nullptr;
-    size_t scratch_bytes = 0;
     double mass[2] = {0.0, 0.0};
-    if (h->m_group <= SPAN) {
-        const int span = SPAN / h->m_group * h->m_group;
-        k_prune_tile<<<dim3((h->k + span - 1) / span, h->n_tiles), SPAN, 0, st>>>(w_dense, h->c_out, h->k, h->kk, h->tile_t, h->n_keep,
-                                                                                 h->m_group, span, h->indices, h->mass);
-        count_launch(1);
-    } else {
-        const size_t cells = static_cast<size_t>(h->n_tiles) * h->k;
-        scratch = static_cast<uint8_t*>(device_block_alloc(cells * 9, h->device, &scratch_bytes));
-        if (!scratch) return fail(NM_ERR_ALLOC, "nm_prune: cannot allocate %zu bytes of scratch", cells * 9);
-        double* score = reinterpret_cast<double*>(scratch);
-        uint8_t* keep = scratch + cells * sizeof(double);
-        const dim3 blk(128), grid((h->k + 127) / 128, h->n_tiles);
-        k_score<<<grid, blk, 0, st>>>(w_dense, h->c_out, h->k, h->tile_t, score);
-        k_select<<<grid, blk, 0, st>>>(score, h->k, h->n_keep, h->m_group, keep);
-        k_compact<<<grid, blk, 0, st>>>(keep, h->k, h->kk, h->n_keep, h->m_group, h->indices);
-        k_mass<<<static_cast<unsigned>(std::min<size_t>((cells + 255) / 256, 1024)), 256, 0, st>>>(score, keep, cells, h->mass);
-        count_launch(4);
-    }
-    NM_CUDA_TRY(cudaGetLastError());
-    st_out = build_layouts(h, w_dense, h->indices, false, st);
-    // the one synchronisation: the handle is complete when the call returns, whatever stream uses it next
-    if (st_out == NM_OK) st_out = finish_handle(h, st, mass, nullptr);
+    // (either way the one synchronisation: the handle is complete when the call returns, whatever stream uses it next)
+    nm_status_t st_out = compressed_in_one(h) ? compress_in_one(h, w_dense, nullptr, st, mass, nullptr) : prune_wide(w_dense, h, st, mass);
     if (st_out == NM_OK) {
         h->l1_total = mass[0];
         h->l1_kept = mass[1];
     }
-done:
-    if (scratch) device_block_free(scratch, scratch_bytes, h->device, st_out == NM_OK);
     return st_out;
 }
 
 nm_status_t build_from_compressed(const float* values, const uint16_t* indices, nm_weights* h, cudaStream_t st)
 {
     int bad = 0;
-    nm_status_t s = clear_handle_memory(h, st);
+    nm_status_t s = compressed_in_one(h) ? NM_OK : clear_handle_memory(h, st);
     if (s == NM_OK && !kernel_may_touch(values, indices, h->device)) {
         // through the handle's own arrays, which the layout kernel then reads and writes back unchanged
         cudaError_t e = cudaMemcpyAsync(h->values, values, static_cast<size_t>(h->c_out) * h->kk * sizeof(float), cudaMemcpyDeviceToDevice, st);
@@ -217,8 +143,12 @@ nm_status_t build_from_compressed(const float* values, const uint16_t* indices, 
         values = h->values;
         indices = h->indices;
     }
-    if (s == NM_OK) s = build_layouts(h, values, indices, true, st);
-    if (s == NM_OK) s = finish_handle(h, st, nullptr, &bad);
+    if (s == NM_OK && compressed_in_one(h)) {
+        s = compress_in_one(h, values, indices, st, nullptr, &bad);
+    } else {
+        if (s == NM_OK) s = build_layouts(h, values, indices, true, st);
+        if (s == NM_OK) s = finish_handle(h, st, nullptr, &bad);
+    }
     if (s == NM_OK && bad)
         s = fail(NM_ERR_INVALID_ARG, "nm_weights_import: an index row is not strictly ascending below K, or does not hold N columns per group of M");
     return s;
