@@ -9,8 +9,8 @@
 //                           padding done by the hardware), a tiled load brings the weight chunk
 //                           [BN x KC] (K-major, 128-byte swizzle), a bulk copy brings each tile's
 //                           kept-column offsets.  Ring of 3-6 stages keeps HBM requests in flight.
-//   compactors (8 warps)    thread = pixel row = TMEM lane, two warps per lane quadrant (one per
-//                           half of the chunk).  Each reads its row's share of the slab ONCE with
+//   compactors (two teams   The teams take the chunks in turn.  Thread = pixel row = TMEM lane, two warps of a team per lane
+//   of 8 warps)             quadrant (one per half of the chunk).  Each reads its row's share of the slab ONCE with
 //                           conflict-free 16-byte loads (one load = one group of 4 source columns)
 //                           and, for every tile of the CTA, selects that tile's kept columns
 //                           in registers (warp-uniform selectors), rounds them to TF32 and writes
@@ -22,9 +22,17 @@
 //                           swizzled layout and written to NHWC with TMA stores.  With two
 //                           accumulator buffers it overlaps the next item's main loop.
 //
+// A chunk's chain (barrier, loads, selection, TMEM store, barrier) takes a team 0.5 us and more whatever it moves, so two teams
+// take chunks in turn, with operand sets of their own: one team and two, us: 256 -> 256, 3x3 at 14x14, batch 32, 2:4 31.1, 25.9; 64 -> 64 at 56x56, batch 16
+// 24.0, 20.6; 96 -> 96 at 31x38, batch 5, 3x3, 3:4, T = 16 18.5, 16.0.
+// The tiles of a layer are dealt to the CTAs in groups of G; the last group may be smaller (its missing tiles are neither fetched nor
+// multiplied, and the store clips their channels).
+//
 // Every wait is bounded; on expiry the CTA raises an abort flag, every role drains to the common
 // exit, the producer waits (bounded) for loads still in flight, TMEM is released, and the host
 // learns of it through the status word.
+#include <algorithm>
+
 #include "nm_internal.h"
 #include "nm_ptx.cuh"
 #include "nm_tmap.cuh"
@@ -37,8 +45,9 @@ constexpr int BM = 128;
 constexpr int SUB_BYTES = BM * 128;   // one 32-column slab sub-tile
 constexpr int NSTAGE_MAX = 6;
 constexpr int A_COL0 = 256;           // TMEM: accumulators in columns [0, 256), operand sets above
-constexpr int THREADS = 512;
-constexpr int STAGING_BYTES = 4 * 2 * 4096;  // per epilogue warp two 32 x 32 output boxes
+constexpr int THREADS = 768;          // warps: 0 producer, 1 MMA issuer, 2 tensor memory, 4-7 epilogue, 8-23 compactors
+constexpr int MAX_SETS = 4;
+constexpr int BOX_BYTES = 4096;       // 32 x 32 output box of an epilogue warp
 
 struct StreamCfg {
     int g;            // pruning tiles per CTA
@@ -48,7 +57,9 @@ struct StreamCfg {
     int stages;
     int b_bytes;      // weight bytes per stage
     int stage_bytes;
+    int boxes;        // staging boxes per epilogue warp: two, or one where the ring gains two stages by it
     int set_cols;     // TMEM columns of one operand set = g * 32
+    int n_sets;       // operand sets: two per team where 256 columns hold them, else one
     long long n_work;
 };
 
@@ -123,7 +134,7 @@ k_conv_stream(const ConvParams p, const StreamCfg cfg, const __grid_constant__ C
 {
     using P = Pattern<NK, MG>;
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t s_full[NSTAGE_MAX], s_free[NSTAGE_MAX], s_aready[2], s_afree[2], s_accfull[2], s_accfree[2];
+    __shared__ uint64_t s_full[NSTAGE_MAX], s_free[NSTAGE_MAX], s_aready[MAX_SETS], s_afree[MAX_SETS], s_accfull[2], s_accfree[2];
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
 
@@ -132,6 +143,7 @@ k_conv_stream(const ConvParams p, const StreamCfg cfg, const __grid_constant__ C
     const int NS = cfg.stages, n_chunks = p.v2_chunks, g = cfg.g, T = p.tile_t;
     const uint32_t ring = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t staging = ring + NS * cfg.stage_bytes;
+    auto live_tiles = [&](int slice) { return min(g, p.n_tiles - slice * g); };
     volatile int* abort_flag = &s_abort;
 
     // ---- set-up ----------------------------------------------------------------------------------
@@ -139,11 +151,13 @@ k_conv_stream(const ConvParams p, const StreamCfg cfg, const __grid_constant__ C
     if (tid == 0) {
         for (int i = 0; i < NSTAGE_MAX; ++i) {
             mbar_init(smem_u32(&s_full[i]), 1);       // producer's expect-tx arrival
-            mbar_init(smem_u32(&s_free[i]), 8 + 1);   // compactor warps + MMA commit
+            mbar_init(smem_u32(&s_free[i]), 8 + 1);   // a team's warps + MMA commit
+        }
+        for (int i = 0; i < MAX_SETS; ++i) {
+            mbar_init(smem_u32(&s_aready[i]), 8);     // a team's warps
+            mbar_init(smem_u32(&s_afree[i]), 1);      // MMA commit
         }
         for (int i = 0; i < 2; ++i) {
-            mbar_init(smem_u32(&s_aready[i]), 8);     // compactor warps
-            mbar_init(smem_u32(&s_afree[i]), 1);      // MMA commit
             mbar_init(smem_u32(&s_accfull[i]), 1);    // MMA commit
             mbar_init(smem_u32(&s_accfree[i]), 4);    // epilogue warps
         }
@@ -165,7 +179,6 @@ k_conv_stream(const ConvParams p, const StreamCfg cfg, const __grid_constant__ C
         if (elect_one()) {
             const int hw = p.ho * p.wo;
             const size_t rpitch = static_cast<size_t>(n_chunks) * 32;
-            const uint32_t tx_fixed = static_cast<uint32_t>(cfg.bn) * 128u + static_cast<uint32_t>(g) * 32u;
             RingPos rp;
             int issued = 0;
             for (uint32_t work = blockIdx.x; work < n_work && !aborted(abort_flag); work += gridDim.x) {
@@ -176,6 +189,8 @@ k_conv_stream(const ConvParams p, const StreamCfg cfg, const __grid_constant__ C
                 const int oh0 = rem / p.wo, ow0 = rem - oh0 * p.wo;
                 const int w0 = ow0 * p.stride_w - p.pad_w, h0 = oh0 * p.stride_h - p.pad_h;
                 const uint8_t* rsrc = p.rel2 + static_cast<size_t>(slice * g) * rpitch;
+                const int tiles = live_tiles(slice);
+                const uint32_t tx_fixed = static_cast<uint32_t>(cfg.bn) * 128u + static_cast<uint32_t>(tiles) * 32u;   // (rows past the last channel arrive as zeros)
                 int ch = 0, off_w = 0, off_h = 0, tw = 0, k0 = 0;   // position of the next 32-column sub-tile
                 for (int c = 0; c < n_chunks; ++c) {
                     if (rp.wrapped && !mbar_wait_lone(smem_u32(&s_free[rp.s]), rp.parity ^ 1u)) *abort_flag = 2;
@@ -199,7 +214,7 @@ k_conv_stream(const ConvParams p, const StreamCfg cfg, const __grid_constant__ C
                         }
                     }
                     tma_load_2d(b_smem, &tm_w, bar, c * 32, slice * cfg.bn);
-                    for (int t = 0; t < g; ++t) bulk_load_1d(relbuf + t * 32, rsrc + t * rpitch + c * 32, 32u, bar);
+                    for (int t = 0; t < tiles; ++t) bulk_load_1d(relbuf + t * 32, rsrc + t * rpitch + c * 32, 32u, bar);
                     rp.advance(NS);
                     ++issued;
                 }
@@ -218,7 +233,7 @@ k_conv_stream(const ConvParams p, const StreamCfg cfg, const __grid_constant__ C
         if (elect_one()) {
             const uint32_t idesc = umma_idesc_tf32(BM, T);
             RingPos rp;
-            uint32_t set = 0, set_par = 0;          // operand set of this chunk, parity of its current use
+            RingPos rs;                             // operand set of this chunk
             uint32_t ab = 0, acc_par = 0;           // accumulator buffer of this item, parity of its current use
             bool acc_wrapped = false;
             for (uint32_t work = blockIdx.x; work < n_work && !aborted(abort_flag); work += gridDim.x) {
@@ -228,25 +243,25 @@ k_conv_stream(const ConvParams p, const StreamCfg cfg, const __grid_constant__ C
                 }
                 tc_fence_after();
                 const uint32_t acc = tmem + ab * cfg.bn;
+                const int tiles = live_tiles(static_cast<int>(work % static_cast<uint32_t>(cfg.n_slices)));
                 for (int c = 0; c < n_chunks; ++c) {
                     if (!mbar_wait_lone(smem_u32(&s_full[rp.s]), rp.parity)) { *abort_flag = 6; break; }
-                    if (!mbar_wait_lone(smem_u32(&s_aready[set]), set_par)) { *abort_flag = 7; break; }
+                    if (!mbar_wait_lone(smem_u32(&s_aready[rs.s]), rs.parity)) { *abort_flag = 7; break; }
                     if (aborted(abort_flag)) break;
                     tc_fence_after();
                     const uint32_t b_smem = ring + rp.s * cfg.stage_bytes;
-                    const uint32_t a_set = tmem + A_COL0 + set * cfg.set_cols;
-                    for (int t = 0; t < g; ++t) {
+                    const uint32_t a_set = tmem + A_COL0 + rs.s * cfg.set_cols;
+                    for (int t = 0; t < tiles; ++t) {
                         const uint64_t bdesc = umma_desc_k_sw128(b_smem + t * T * 128, 1024);
 #pragma unroll
                         for (int kq = 0; kq < P::KC / 8; ++kq)
                             umma_tf32_ts(acc + t * T, a_set + t * 32 + kq * 8, bdesc + 2 * kq, idesc,
                                          (c > 0 || kq > 0) ? 1u : 0u);
                     }
-                    umma_commit(smem_u32(&s_afree[set]));
+                    umma_commit(smem_u32(&s_afree[rs.s]));
                     umma_commit(smem_u32(&s_free[rp.s]));
                     rp.advance(NS);
-                    if (set == 1) set_par ^= 1u;
-                    set ^= 1u;
+                    rs.advance(cfg.n_sets);
                 }
                 if (aborted(abort_flag)) break;
                 umma_commit(smem_u32(&s_accfull[ab]));
@@ -263,44 +278,55 @@ k_conv_stream(const ConvParams p, const StreamCfg cfg, const __grid_constant__ C
         // =========================== epilogue ===========================
         const int q = warp & 3;
         const uint32_t lane_addr = static_cast<uint32_t>(q * 32) << 16;
-        const uint32_t my_staging = staging + q * 2 * 4096;
+        const uint32_t my_staging = staging + q * cfg.boxes * BOX_BYTES;
         const uint32_t rx = static_cast<uint32_t>(lane & 7);
-        const int n_blk = cfg.bn / 32;
         uint32_t ti = 0;
         uint32_t nb = 0;  // staging boxes this warp has filled so far
         for (uint32_t work = blockIdx.x; work < n_work; work += gridDim.x, ++ti) {
             const int slice = static_cast<int>(work % static_cast<uint32_t>(cfg.n_slices));
             const uint32_t pix0 = (work / static_cast<uint32_t>(cfg.n_slices)) * BM;
             const int ab = cfg.n_acc == 2 ? static_cast<int>(ti & 1u) : 0;
+            const int o0 = slice * cfg.bn;
+            const int n_blk = (min(cfg.bn, p.c_out - o0) + 31) / 32;   // (the last one may end in the middle of a block)
+            float bias_of[8];   // of the item's blocks, a channel per lane, fetched while the main loop runs
+#pragma unroll
+            for (int i = 0; i < 8; ++i) bias_of[i] = i < n_blk ? bias_lane_load(p.bias, o0 + i * 32, p.c_out, lane) : 0.f;
             const bool ok = aborted(abort_flag) ||
                             mbar_wait(smem_u32(&s_accfull[ab]), (cfg.n_acc == 2 ? (ti >> 1) : ti) & 1u);
             if (!__all_sync(0xFFFFFFFFu, ok)) *abort_flag = 8;
             if (__any_sync(0xFFFFFFFFu, aborted(abort_flag))) break;
             tc_fence_after();
-            const int o0 = slice * cfg.bn;
             for (int blk = 0; blk < n_blk; ++blk, ++nb) {
                 uint32_t v[32];
                 tmem_ld32(tmem + lane_addr + ab * cfg.bn + blk * 32, v);
-                tmem_ld_wait();
+                tmem_ld_wait(v);
                 if (blk == n_blk - 1) {
                     // the accumulator buffer may be overwritten from here on
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(smem_u32(&s_accfree[ab]));
                 }
-                const uint32_t box = my_staging + (nb & 1u) * 4096;
-                if (nb >= 2 && elect_one()) tma_store_wait_read_n<1>();  // the box's previous store has read it
+                const uint32_t box = my_staging + (cfg.boxes == 2 ? nb & 1u : 0u) * BOX_BYTES;
+                if (elect_one()) {   // the box's previous store has read it
+                    if (cfg.boxes == 2) tma_store_wait_read_n<1>();
+                    else tma_store_wait_read_n<0>();
+                }
                 __syncwarp();
                 const uint32_t stage_row = box + lane * 128;
                 // with a shortcut input the activation waits for the second pass below
                 const long long box_pix = static_cast<long long>(pix0) + q * 32;
                 const bool res_pass = p.residual != nullptr && box_pix < p.pixels;
                 const int relu_now = res_pass ? 0 : p.relu;
+                // (all shuffles before the first store: both are ordered statements)
+                float4 bias4[8];
+#pragma unroll
+                for (int qq = 0; qq < 8; ++qq) bias4[qq] = bias_quad(bias_of[0], qq);
+#pragma unroll
+                for (int i = 0; i < 7; ++i) bias_of[i] = bias_of[i + 1];
 #pragma unroll
                 for (int qq = 0; qq < 8; ++qq) {
                     float o[4];
-                    float4 bv = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (p.bias) bv = __ldg(reinterpret_cast<const float4*>(p.bias + o0 + blk * 32) + qq);
+                    const float4 bv = bias4[qq];
                     o[0] = __uint_as_float(v[qq * 4 + 0]) + bv.x;
                     o[1] = __uint_as_float(v[qq * 4 + 1]) + bv.y;
                     o[2] = __uint_as_float(v[qq * 4 + 2]) + bv.z;
@@ -317,7 +343,7 @@ k_conv_stream(const ConvParams p, const StreamCfg cfg, const __grid_constant__ C
                     __syncwarp();
                     const long long left = p.pixels - box_pix;
                     add_residual_box(box, p.residual + box_pix * p.c_out + o0 + blk * 32, p.c_out,
-                                     left < 32 ? static_cast<int>(left) : 32, p.relu, lane);
+                                     left < 32 ? static_cast<int>(left) : 32, p.relu, lane, p.c_out - (o0 + blk * 32));
                 }
                 fence_proxy_async();
                 __syncwarp();
@@ -331,21 +357,29 @@ k_conv_stream(const ConvParams p, const StreamCfg cfg, const __grid_constant__ C
         if (elect_one()) tma_store_wait_read();   // shared memory must outlive the stores' reads; the writes complete with the grid
     } else if (warp >= 8) {
         // =========================== compactors ===========================
-        const int wg = (warp - 8) >> 2;   // which half of the chunk
+        const int wg = (warp - 8) >> 2 & 1;   // which half of the chunk
+        const int team = (warp - 8) >> 3;
         const int q = warp & 3;           // TMEM lane quadrant
         const int row = q * 32 + lane;
         const uint32_t lane_addr = static_cast<uint32_t>(q * 32) << 16;
         const uint32_t rx = static_cast<uint32_t>(row & 7);
         constexpr int CI0_STEP = P::LW;   // first 16-byte piece of half `wg`
-        RingPos rp;
-        uint32_t set = 0, set_par = 0;
-        bool set_wrapped = false;
+        // The chunks of all of this CTA's items are numbered through; a team has those of its parity.  Stages and sets are even in number, so a
+        // stage or set always belongs to the same team, which so sees each of its uses.
+        RingPos rp, rs;
+        rp.s = rs.s = team;
+        int turn = 0;
         for (uint32_t work = blockIdx.x; work < n_work && !aborted(abort_flag); work += gridDim.x) {
+            const int tiles = live_tiles(static_cast<int>(work % static_cast<uint32_t>(cfg.n_slices)));
             for (int c = 0; c < n_chunks; ++c) {
+                const bool mine = turn == team;
+                turn ^= 1;
+                if (!mine) continue;
                 const int s = rp.s;
+                const uint32_t set = static_cast<uint32_t>(rs.s);
                 bool ok = mbar_wait_lone(smem_u32(&s_full[s]), rp.parity);
                 if (!__all_sync(0xFFFFFFFFu, ok)) *abort_flag = 3;
-                ok = !set_wrapped || mbar_wait_lone(smem_u32(&s_afree[set]), set_par ^ 1u);
+                ok = !rs.wrapped || mbar_wait_lone(smem_u32(&s_afree[set]), rs.parity ^ 1u);
                 if (!__all_sync(0xFFFFFFFFu, ok)) *abort_flag = 4;
                 if (__any_sync(0xFFFFFFFFu, aborted(abort_flag))) break;
                 tc_fence_after();
@@ -363,7 +397,7 @@ k_conv_stream(const ConvParams p, const StreamCfg cfg, const __grid_constant__ C
                     if (live) L[i] = lds128(slab + (ci >> 3) * SUB_BYTES + row * 128 + ((static_cast<uint32_t>(ci & 7) ^ rx) << 4));
                 }
                 const uint32_t a_set = tmem + lane_addr + A_COL0 + set * cfg.set_cols + wg * P::KW;
-                for (int t = 0; t < g; ++t) {
+                for (int t = 0; t < tiles; ++t) {
                     uint32_t sel[P::KW / 4];
                     if constexpr (!P::DENSE) {
 #pragma unroll
@@ -395,8 +429,9 @@ k_conv_stream(const ConvParams p, const StreamCfg cfg, const __grid_constant__ C
                     mbar_arrive(smem_u32(&s_free[s]));
                 }
                 rp.advance(NS);
-                if (set == 1) { set_par ^= 1u; set_wrapped = true; }
-                set ^= 1u;
+                rp.advance(NS);
+                rs.advance(cfg.n_sets);
+                rs.advance(cfg.n_sets);
             }
         }
     }
@@ -429,6 +464,13 @@ bool layout_matches(const ConvParams& p)
     return p.v2_s == Pattern<NK, MG>::S && p.v2_kc == Pattern<NK, MG>::KC;
 }
 
+// Rounds of the SMs that the work items of `slices` slices take.
+double item_rounds(const ConvParams& p, int slices)
+{
+    const long long items = (p.pixels + BM - 1) / BM * slices, sms = nmhost::sm_count();
+    return static_cast<double>((items + sms - 1) / sms);
+}
+
 bool make_cfg(const ConvParams& p, const nm_plan_t* plan, StreamCfg* cfg)
 {
     if (!p.wt2 || !p.rel2 || !nmtm::available()) return false;
@@ -456,27 +498,40 @@ bool make_cfg(const ConvParams& p, const nm_plan_t* plan, StreamCfg* cfg)
         if (plan->bn % T != 0) return false;
         g = plan->bn / T;
     } else {
+        // largest group of up to 128 channels that divides the tiles
         g = 1;
         for (int cand = 4; cand >= 1; --cand)
             if (cand * T <= 128 && p.n_tiles % cand == 0 && (cand * T) % 32 == 0) { g = cand; break; }
+        // The library default deals tiles out in groups that need not divide them, by an estimate of the time (a
+        // chunk takes 0.24 us and 0.12-0.17 per tile): 128 -> 128, 3x3 at 28x28, batch 4, T = 32 19.1 us in the gather kernel, 12.0 with
+        // a tile per CTA, 21.9 with four; 96 -> 80, T = 16 (five tiles) at 31x38, batch 5 21.6 in the gather kernel, 15.9 with two.
+        if (!plan) {
+            double best = 0.0;
+            for (int cand = 4; cand >= 1; --cand) {
+                if (cand * T > 128 || (cand * T) % 32 != 0) continue;
+                const double t = item_rounds(p, (p.n_tiles + cand - 1) / cand) * (0.25 + 0.15 * cand);
+                if (best == 0.0 || t < best) { best = t; g = cand; }
+            }
+        }
     }
-    if (g < 1 || g > 4 || g * T > 256 || p.n_tiles % g != 0 || (g * T) % 32 != 0) return false;
+    if (g < 1 || g > 4 || g * T > 256 || (plan && p.n_tiles % g != 0) || (g * T) % 32 != 0) return false;
     cfg->g = g;
     cfg->bn = g * T;
-    cfg->n_slices = p.n_tiles / g;
+    cfg->n_slices = (p.n_tiles + g - 1) / g;
     cfg->n_acc = cfg->bn <= 128 ? 2 : 1;
     cfg->set_cols = g * 32;
+    cfg->n_sets = 4 * cfg->set_cols <= 512 - A_COL0 ? 4 : 2;
     cfg->b_bytes = ((cfg->bn * 128 + 1023) / 1024) * 1024;   // whole swizzle atoms
     cfg->stage_bytes = cfg->b_bytes + (p.v2_s / 32) * SUB_BYTES + 1024;  // offsets area padded to keep stages aligned
-    const int budget = 227 * 1024 - 1024 - STAGING_BYTES - 1024;         // alignment slack, staging, static shared
-    int stages = plan && plan->stages > 0 ? plan->stages : NSTAGE_MAX;
-    if (stages > NSTAGE_MAX) return false;
-    if (plan && plan->stages > 0) {
-        if (stages * cfg->stage_bytes > budget) return false;
-    } else {
-        while (stages > 2 && stages * cfg->stage_bytes > budget) --stages;
-        if (stages * cfg->stage_bytes > budget) return false;
-    }
+    // The teams own alternate stages, so their number is even; an odd number asked for is taken down, two always fit.
+    const int budget = 227 * 1024 - 1024 - 1024;         // alignment slack, static shared
+    const int asked = plan && plan->stages > 0 ? plan->stages : 0;
+    if (asked > NSTAGE_MAX || (asked && asked * cfg->stage_bytes > budget - 8 * BOX_BYTES)) return false;
+    auto most = [&](int boxes) { return std::min((budget - 4 * boxes * BOX_BYTES) / cfg->stage_bytes, NSTAGE_MAX) & ~1; };
+    // (64 -> 256, one chunk of 64 columns, at 56x56, batch 4: 7.2 us with two boxes, 8.5 with one; 256 -> 256, 3x3 at 14x14, batch 32: 35.1, 25.9)
+    cfg->boxes = p.v2_chunks > 4 && most(1) > most(2) ? 1 : 2;
+    int stages = asked ? std::max(asked & ~1, 2) : most(cfg->boxes);
+    if (stages < 2 || stages > most(cfg->boxes)) return false;
     cfg->stages = stages;
     const long long pix_blocks = (p.pixels + BM - 1) / BM;
     cfg->n_work = pix_blocks * cfg->n_slices;
@@ -491,7 +546,7 @@ nm_status_t launch(const ConvParams& p, const StreamCfg& cfg, cudaStream_t st)
     if (!nmtm::encode_x_im2col(p, BM, &tm_x) || !nmtm::encode_w_tiled(p, cfg.bn, &tm_w) ||
         !nmtm::encode_y_tiled(p, &tm_y))
         return nmhost::fail(NM_ERR_CUDA, "nm_conv2d: tensor-map encoding failed (variant 3)");
-    size_t smem = 1024 + static_cast<size_t>(cfg.stages) * cfg.stage_bytes + STAGING_BYTES;
+    size_t smem = 1024 + static_cast<size_t>(cfg.stages) * cfg.stage_bytes + 4 * cfg.boxes * BOX_BYTES;
     if (smem < NM_EXCLUSIVE_SMEM) smem = NM_EXCLUSIVE_SMEM;   // one CTA per SM: it owns all 512 TMEM columns
     cudaError_t e = nmhost::ensure_dynamic_smem(reinterpret_cast<const void*>(k_conv_stream<NK, MG>), smem);
     if (e != cudaSuccess) return nmhost::fail(NM_ERR_CUDA, "cudaFuncSetAttribute (variant 3): %s", cudaGetErrorString(e));
@@ -515,10 +570,13 @@ bool stream_plan_ok(const ConvParams& p, const nm_plan_t* plan)
 
 bool stream_leaves_sms_idle(const ConvParams& p)
 {
-    // Work items on less than half of the SMs, sixteen chunks or more each.  3x3 448 -> 160 at 8x14 (7 pixel blocks, 3:4):
-    // 52.7 us here, 29 us in the gather kernel, which splits the chunks over a cluster; 1x1 352 -> 704 at 34x7 (six chunks): 7.2, 7.7.
+    // Work items on less than half of the SMs and sixteen chunks or more each, or on less than a quarter and twelve, us here and in the gather
+    // kernel, which splits the chunks over a cluster: 3x3 256 -> 256 at 14x14, batch 4 (28 items, 36 chunks) 20.3, 10.9; 128 -> 128 at 28x28, batch
+    // 4 (50, 18) 12.1, 10.5; 96 -> 96 at 20x20, batch 2 (21, 14) 9.9, 7.1; 1x1 512 -> 64 at 14x14, batch 4 (7, 8) 7.4, 9.2.
     StreamCfg cfg;
-    return make_cfg(p, nullptr, &cfg) && 2 * cfg.n_work < nmhost::sm_count() && p.v2_chunks >= 16;
+    if (!make_cfg(p, nullptr, &cfg)) return false;
+    const long long sms = nmhost::sm_count();
+    return (2 * cfg.n_work < sms && p.v2_chunks >= 16) || (4 * cfg.n_work < sms && p.v2_chunks >= 12);
 }
 
 nm_status_t launch_conv_stream(const ConvParams& p, const nm_plan_t* plan, cudaStream_t st)

@@ -352,10 +352,10 @@ __device__ __forceinline__ void apply_residual_box(uint32_t box, const float4 (&
 // Both steps at once (the loads first: the shared-memory accesses are ordered asm statements and would
 // otherwise serialise them).  Kernels that can afford the registers call the two halves apart, with
 // the loads issued a box ahead.
-__device__ __forceinline__ void add_residual_box(uint32_t box, const float* res, int c_out, int rows, int relu, int lane)
+__device__ __forceinline__ void add_residual_box(uint32_t box, const float* res, int c_out, int rows, int relu, int lane, int cols = 32)
 {
     float4 rv[8];
-    load_residual_box(rv, res, c_out, rows, lane);
+    load_residual_box(rv, res, c_out, rows, lane, cols);
     apply_residual_box(box, rv, relu, lane);
 }
 
