@@ -1,5 +1,5 @@
-// CPython extension behind nm.py: the per-call work of the convolution and pooling entry points (type checks, output
-// allocation, pointers, current stream) in native code.  A layer of a batch-1 network runs for a few microseconds; the
+// CPython extension behind nm.py: the per-call work of the convolution and pooling entry points and of those that make and export a handle (type
+// checks, output allocation, pointers, current stream) in native code.  A layer of a batch-1 network runs for a few microseconds; the
 // same steps in Python with ctypes cost more than that: 12.8 us per nm_conv2d call before, 3.2 of them for
 // torch.cuda.current_stream() alone.
 //
@@ -17,6 +17,10 @@ namespace {
 decltype(&nm_conv2d) p_conv2d = nullptr;
 decltype(&nm_conv2d_res) p_conv2d_res = nullptr;
 decltype(&nm_maxpool2d) p_maxpool2d = nullptr;
+decltype(&nm_prune) p_prune = nullptr;
+decltype(&nm_weights_import) p_import = nullptr;
+decltype(&nm_weights_export) p_export = nullptr;
+decltype(&nm_weights_dims) p_dims = nullptr;
 
 void* current_stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
 
@@ -168,6 +172,109 @@ PyObject* maxpool2d(PyObject*, PyObject* const* a, Py_ssize_t n)
     return a[4];
 }
 
+// `n` ints from `a` on; false with an exception set
+bool ints_of(PyObject* const* a, int n, int* out)
+{
+    for (int i = 0; i < n; ++i) out[i] = static_cast<int>(PyLong_AsLong(a[i]));
+    return !PyErr_Occurred();
+}
+
+// (handle, c_out, k, kk, n_tiles, tile_t) of a new handle, or the status as an int
+PyObject* made_handle(nm_status_t s, nm_weights_t* w)
+{
+    int dims[5] = {0, 0, 0, 0, 0};
+    if (s == NM_OK) s = p_dims(w, dims, dims + 1, dims + 2, dims + 3, dims + 4);
+    if (s != NM_OK) return PyLong_FromLong(s);
+    return Py_BuildValue("(Niiiii)", PyLong_FromVoidPtr(w), dims[0], dims[1], dims[2], dims[3], dims[4]);
+}
+
+// prune(w_dense, n_keep, m_group, tile_t)
+PyObject* prune(PyObject*, PyObject* const* a, Py_ssize_t n)
+{
+    if (n != 4) {
+        PyErr_SetString(PyExc_TypeError, "prune takes 4 arguments");
+        return nullptr;
+    }
+    const at::Tensor* w = dev_f32(a[0], "w_dense");
+    if (!w) return nullptr;
+    if (w->dim() != 4) {
+        PyErr_SetString(PyExc_TypeError, "w_dense must be [c_out, kh, kw, c_in]");
+        return nullptr;
+    }
+    int v[3];
+    if (!ints_of(a + 1, 3, v)) return nullptr;
+    const float* ptr = w->const_data_ptr<float>();
+    const int c_out = static_cast<int>(w->size(0)), kh = static_cast<int>(w->size(1)), kw = static_cast<int>(w->size(2)), c_in = static_cast<int>(w->size(3));
+    void* st = current_stream();
+    nm_weights_t* out = nullptr;
+    nm_status_t s;
+    Py_BEGIN_ALLOW_THREADS
+    s = p_prune(ptr, c_out, kh, kw, c_in, v[0], v[1], v[2], st, &out);
+    Py_END_ALLOW_THREADS
+    return made_handle(s, out);
+}
+
+// weights_import(values, indices, kh, kw, c_in, n_keep, m_group, tile_t)
+PyObject* weights_import(PyObject*, PyObject* const* a, Py_ssize_t n)
+{
+    if (n != 8) {
+        PyErr_SetString(PyExc_TypeError, "weights_import takes 8 arguments");
+        return nullptr;
+    }
+    const at::Tensor* values = dev_f32(a[0], "values");
+    if (!values) return nullptr;
+    const at::Tensor* indices = THPVariable_Check(a[1]) ? &THPVariable_Unpack(a[1]) : nullptr;
+    if (!indices || !indices->is_cuda() || indices->scalar_type() != at::kUInt16 || !indices->is_contiguous()) {
+        PyErr_SetString(PyExc_TypeError, "indices must be a contiguous uint16 CUDA tensor");
+        return nullptr;
+    }
+    if (values->dim() < 1) {
+        PyErr_SetString(PyExc_IndexError, "values has no rows");
+        return nullptr;
+    }
+    int v[6];
+    if (!ints_of(a + 2, 6, v)) return nullptr;
+    const float* vp = values->const_data_ptr<float>();
+    const auto* ip = static_cast<const uint16_t*>(indices->const_data_ptr());
+    const int c_out = static_cast<int>(values->size(0));
+    void* st = current_stream();
+    nm_weights_t* out = nullptr;
+    nm_status_t s;
+    Py_BEGIN_ALLOW_THREADS
+    s = p_import(vp, ip, c_out, v[0], v[1], v[2], v[3], v[4], v[5], st, &out);
+    Py_END_ALLOW_THREADS
+    return made_handle(s, out);
+}
+
+// weights_export(handle, c_out, kk, n_tiles) -> (values, indices), or the status as an int
+PyObject* weights_export(PyObject*, PyObject* const* a, Py_ssize_t n)
+{
+    if (n != 4) {
+        PyErr_SetString(PyExc_TypeError, "weights_export takes 4 arguments");
+        return nullptr;
+    }
+    const auto* w = static_cast<const nm_weights_t*>(PyLong_AsVoidPtr(a[0]));
+    int v[3];
+    if (PyErr_Occurred() || !ints_of(a + 1, 3, v)) return nullptr;
+    at::Tensor values = at::empty({v[0], v[1]}, at::TensorOptions().dtype(at::kFloat).device(at::kCUDA));
+    at::Tensor indices = at::empty({v[2], v[1]}, at::TensorOptions().dtype(at::kUInt16).device(at::kCUDA));
+    float* vp = values.mutable_data_ptr<float>();
+    auto* ip = static_cast<uint16_t*>(indices.mutable_data_ptr());
+    void* st = current_stream();
+    nm_status_t s;
+    Py_BEGIN_ALLOW_THREADS
+    s = p_export(w, vp, ip, st);
+    Py_END_ALLOW_THREADS
+    if (s != NM_OK) return PyLong_FromLong(s);
+    PyObject* vo = THPVariable_Wrap(std::move(values));
+    PyObject* io = vo ? THPVariable_Wrap(std::move(indices)) : nullptr;
+    if (!io) {
+        Py_XDECREF(vo);
+        return nullptr;
+    }
+    return Py_BuildValue("(NN)", vo, io);
+}
+
 PyObject* stream_ptr(PyObject*, PyObject* const*, Py_ssize_t n)
 {
     if (n != 0) {
@@ -179,13 +286,17 @@ PyObject* stream_ptr(PyObject*, PyObject* const*, Py_ssize_t n)
 
 PyObject* bind(PyObject*, PyObject* const* a, Py_ssize_t n)
 {
-    if (n != 3) {
-        PyErr_SetString(PyExc_TypeError, "bind takes 3 addresses");
+    if (n != 7) {
+        PyErr_SetString(PyExc_TypeError, "bind takes 7 addresses");
         return nullptr;
     }
     p_conv2d = reinterpret_cast<decltype(p_conv2d)>(PyLong_AsVoidPtr(a[0]));
     p_conv2d_res = reinterpret_cast<decltype(p_conv2d_res)>(PyLong_AsVoidPtr(a[1]));
     p_maxpool2d = reinterpret_cast<decltype(p_maxpool2d)>(PyLong_AsVoidPtr(a[2]));
+    p_prune = reinterpret_cast<decltype(p_prune)>(PyLong_AsVoidPtr(a[3]));
+    p_import = reinterpret_cast<decltype(p_import)>(PyLong_AsVoidPtr(a[4]));
+    p_export = reinterpret_cast<decltype(p_export)>(PyLong_AsVoidPtr(a[5]));
+    p_dims = reinterpret_cast<decltype(p_dims)>(PyLong_AsVoidPtr(a[6]));
     if (PyErr_Occurred()) return nullptr;
     Py_RETURN_NONE;
 }
@@ -213,6 +324,9 @@ PyObject* guarded(PyObject* self, PyObject* const* a, Py_ssize_t n)
 PyMethodDef methods[] = {
     {"conv2d", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(guarded<conv2d>)), METH_FASTCALL, nullptr},
     {"maxpool2d", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(guarded<maxpool2d>)), METH_FASTCALL, nullptr},
+    {"prune", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(guarded<prune>)), METH_FASTCALL, nullptr},
+    {"weights_import", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(guarded<weights_import>)), METH_FASTCALL, nullptr},
+    {"weights_export", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(guarded<weights_export>)), METH_FASTCALL, nullptr},
     {"bind", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(bind)), METH_FASTCALL, nullptr},
     {"stream_ptr", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(guarded<stream_ptr>)), METH_FASTCALL, nullptr},
     {nullptr, nullptr, 0, nullptr}};

@@ -103,7 +103,8 @@ try:
 except ImportError as e:
     raise ImportError("the CPython extension _nm_binding is not built; run `python -m paper_2507_17301_b200.build` "
                       f"(there is no fallback path without it): {e}") from e
-_nm_binding.bind(*(ctypes.cast(f, ctypes.c_void_p).value for f in (_lib.nm_conv2d, _lib.nm_conv2d_res, _lib.nm_maxpool2d)))
+_nm_binding.bind(*(ctypes.cast(f, ctypes.c_void_p).value for f in (
+    _lib.nm_conv2d, _lib.nm_conv2d_res, _lib.nm_maxpool2d, _lib.nm_prune, _lib.nm_weights_import, _lib.nm_weights_export, _lib.nm_weights_dims)))
 
 EXPORTS = ("nm_memory_trim", "nm_plan_key", "nm_plan_cache_store", "nm_plan_cache_lookup", "nm_selftest_wait_expiry", "nm_maxpool2d", "nm_weights_retained_l1", "nm_conv2d_res", "nm_plan_scratch_bytes", "nm_weights_reserve", "nm_prune", "nm_prune_noalloc", "nm_weights_dims", "nm_weights_export", "nm_weights_import", "nm_weights_check",
            "nm_weights_free", "nm_conv2d", "nm_conv2d_host", "nm_autotune", "nm_autotune_tile",
@@ -143,12 +144,14 @@ def _pair(v):
 class Weights:
     """Owner of one ``nm_weights_t*`` handle (freed with the object)."""
 
-    def __init__(self, handle: int):
+    def __init__(self, handle: int, dims=None):
         self._h = ctypes.c_void_p(handle)
         self._addr = handle or 0
-        dims = [ctypes.c_int() for _ in range(5)]
-        _check(_lib.nm_weights_dims(self._h, *[ctypes.byref(d) for d in dims]))
-        self.c_out, self.k, self.kk, self.n_tiles, self.tile_t = (d.value for d in dims)
+        if dims is None:
+            out = [ctypes.c_int() for _ in range(5)]
+            _check(_lib.nm_weights_dims(self._h, *[ctypes.byref(d) for d in out]))
+            dims = [d.value for d in out]
+        self.c_out, self.k, self.kk, self.n_tiles, self.tile_t = dims
 
     @property
     def handle(self):
@@ -167,15 +170,15 @@ class Weights:
             pass
 
 
+def _made(made) -> Weights:
+    if made.__class__ is int:
+        _check(made)
+    return Weights(made[0], made[1:])
+
+
 def nm_prune(w_dense: torch.Tensor, n_keep: int, m_group: int, tile_t: int) -> Weights:
     """``w_dense``: CUDA fp32 OHWI ``[c_out, kh, kw, c_in]``.  Returns the compressed-weight handle."""
-    ptr = _dev_f32(w_dense, "w_dense")
-    if w_dense.dim() != 4:
-        raise TypeError("w_dense must be [c_out, kh, kw, c_in]")
-    c_out, kh, kw, c_in = w_dense.shape
-    out = ctypes.c_void_p()
-    _check(_lib.nm_prune(ptr, c_out, kh, kw, c_in, n_keep, m_group, tile_t, _stream(), ctypes.byref(out)))
-    return Weights(out.value)
+    return _made(_nm_binding.prune(w_dense, n_keep, m_group, tile_t))
 
 
 NM_NOALLOC_MAX_CELLS = 1 << 19
@@ -208,21 +211,15 @@ def nm_prune_noalloc(w_dense: torch.Tensor, n_keep: int, m_group: int, tile_t: i
 
 def nm_weights_export(w: Weights):
     """Returns ``(values [c_out, kk] fp32, indices [n_tiles, kk] uint16)`` as CUDA tensors."""
-    values = torch.empty((w.c_out, w.kk), dtype=torch.float32, device="cuda")
-    indices = torch.empty((w.n_tiles, w.kk), dtype=torch.uint16, device="cuda")
-    _check(_lib.nm_weights_export(w.handle, values.data_ptr(), indices.data_ptr(), _stream()))
-    return values, indices
+    out = _nm_binding.weights_export(w._addr, w.c_out, w.kk, w.n_tiles)
+    if out.__class__ is int:
+        _check(out)
+    return out
 
 
 def nm_weights_import(values: torch.Tensor, indices: torch.Tensor, kh: int, kw: int, c_in: int, n_keep: int,
                       m_group: int, tile_t: int) -> Weights:
-    vptr = _dev_f32(values, "values")
-    if not (indices.is_cuda and indices.dtype == torch.uint16 and indices.is_contiguous()):
-        raise TypeError("indices must be a contiguous uint16 CUDA tensor")
-    out = ctypes.c_void_p()
-    _check(_lib.nm_weights_import(vptr, indices.data_ptr(), values.shape[0], kh, kw, c_in, n_keep, m_group, tile_t,
-                                  _stream(), ctypes.byref(out)))
-    return Weights(out.value)
+    return _made(_nm_binding.weights_import(values, indices, kh, kw, c_in, n_keep, m_group, tile_t))
 
 
 def nm_plan_scratch_bytes(w: Weights, x_shape, stride, pad, dil, plan: nm_plan_t) -> int:
