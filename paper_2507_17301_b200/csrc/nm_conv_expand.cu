@@ -556,9 +556,9 @@ k_conv_expand(const ConvParams p, const ExpandCfg cfg, const __grid_constant__ C
                 s_bias[warp - 4][lane] = bias_of[0];   // (the block before it has been read: see its __syncwarp)
                 bias_of[0] = bias_of[1]; bias_of[1] = bias_of[2]; bias_of[2] = bias_of[3];
                 __syncwarp();
-                float4 extra[8];   // bias, then bias + shortcut
+                float4 bias[8];
 #pragma unroll
-                for (int qq = 0; qq < 8; ++qq) extra[qq] = reinterpret_cast<const float4*>(s_bias[warp - 4])[qq];
+                for (int qq = 0; qq < 8; ++qq) bias[qq] = reinterpret_cast<const float4*>(s_bias[warp - 4])[qq];
                 uint32_t v[32];
                 if (BAL) tmem_ld32(acc_addr + blk * 32, vn);
                 if (two_acc) {
@@ -643,21 +643,27 @@ k_conv_expand(const ConvParams p, const ExpandCfg cfg, const __grid_constant__ C
                     __syncwarp();
                 }
                 const uint32_t stage_row = box + lane * 128;
-                // (all loads before the first store: the stores are ordered statements, which no later load is moved ahead of)
+                // Sum, then bias, then shortcut, as in the split-K form's second pass: a plan's schedule does not show in the order of the
+                // additions.  (All loads before the first store: the stores are ordered statements, which no later load is moved ahead of.)
+                float4 o8[8];
+#pragma unroll
+                for (int qq = 0; qq < 8; ++qq) {
+                    o8[qq] = make_float4(__uint_as_float(v[qq * 4 + 0]), __uint_as_float(v[qq * 4 + 1]), __uint_as_float(v[qq * 4 + 2]),
+                                         __uint_as_float(v[qq * 4 + 3]));
+                    nm_add4(o8[qq], bias[qq]);
+                }
                 if (res) {
 #pragma unroll
                     for (int qq = 0; qq < 8; ++qq) {
                         float4 x;
                         asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(stage_row + ((qq ^ rx) << 4)));
-                        nm_add4(extra[qq], x);
+                        nm_add4(o8[qq], x);
                     }
                 }
 #pragma unroll
                 for (int qq = 0; qq < 8; ++qq) {
                     const uint32_t at = stage_row + ((qq ^ rx) << 4);
-                    float4 o = make_float4(__uint_as_float(v[qq * 4 + 0]), __uint_as_float(v[qq * 4 + 1]), __uint_as_float(v[qq * 4 + 2]),
-                                           __uint_as_float(v[qq * 4 + 3]));
-                    nm_add4(o, extra[qq]);
+                    float4 o = o8[qq];
                     if (p.relu) { o.x = fmaxf(o.x, 0.f); o.y = fmaxf(o.y, 0.f); o.z = fmaxf(o.z, 0.f); o.w = fmaxf(o.w, 0.f); }
                     asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(at), "f"(o.x), "f"(o.y), "f"(o.z), "f"(o.w) : "memory");
                 }
