@@ -219,7 +219,7 @@ k_conv_expand(const ConvParams p, const ExpandCfg cfg, const __grid_constant__ C
     __shared__ uint64_t s_full[NSTAGE_MAX], s_free[NSTAGE_MAX], s_accfull[2], s_accfree[2], s_wres, s_res[8][BOXES_MAX];
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
-    __shared__ float s_bias[8][32];   // bias of the block an epilogue warp works on
+    __shared__ __align__(16) float s_bias[8][32];   // bias of the block an epilogue warp works on
 
     const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
     const int NS = cfg.stages, n_sub = cfg.n_sub;

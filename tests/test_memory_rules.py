@@ -39,3 +39,19 @@ def test_no_check_of_the_self_checking_build_guards_an_empty_statement():
     for name in os.listdir(f"{ROOT}/paper_2507_17301_b200/csrc"):
         with open(f"{ROOT}/paper_2507_17301_b200/csrc/{name}") as f:
             assert not re.search(r"NM_CHECKED\([^;{]*\)\s*\{\s*\}", f.read()), name
+
+
+def test_shared_arrays_read_as_vectors_are_aligned_for_them():
+    """A float array may start at any multiple of four bytes; read as float4 it has to say that it does not."""
+    vectors = {"float4": 16, "uint4": 16, "int4": 16, "double2": 16, "float2": 8, "uint2": 8, "int2": 8}
+    found = 0
+    for name in os.listdir(f"{ROOT}/paper_2507_17301_b200/csrc"):
+        with open(f"{ROOT}/paper_2507_17301_b200/csrc/{name}") as f:
+            text = f.read()
+        for align, arrays in re.findall(r"__shared__\s+(?:__align__\((\d+)\)\s+)?(?:float|int|uint32_t|uint16_t|uint8_t|short)\s+([^;]*);", text):
+            for array in re.findall(r"(\w+)\[", arrays):
+                for vector in re.findall(rf"reinterpret_cast<(?:const )?(\w+)\s*\*>\(&?{array}\b", text):
+                    if vector in vectors:
+                        found += 1
+                        assert int(align or 4) >= vectors[vector], (name, array, vector)
+    assert found >= 2
