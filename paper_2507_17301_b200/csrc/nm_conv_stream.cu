@@ -8,9 +8,9 @@
 //                           [128 pixels x S columns] (stride, dilation, tap offset and zero
 //                           padding done by the hardware), a tiled load brings the weight chunk
 //                           [BN x KC] (K-major, 128-byte swizzle), a bulk copy brings each tile's
-//                           kept-column offsets.  Ring of 3-6 stages keeps HBM requests in flight.
-//   compactors (two teams   The teams take the chunks in turn.  Thread = pixel row = TMEM lane, two warps of a team per lane
-//   of 8 warps)             quadrant (one per half of the chunk).  Each reads its row's share of the slab ONCE with
+//                           kept-column offsets.  Ring of 2-6 stages keeps HBM requests in flight.
+//   compactors (one or two  Two teams take the chunks in turn.  Thread = pixel row = TMEM lane, two warps of a team per lane
+//   teams of 8 warps)       quadrant (one per half of the chunk).  Each reads its row's share of the slab ONCE with
 //                           conflict-free 16-byte loads (one load = one group of 4 source columns)
 //                           and, for every tile of the CTA, selects that tile's kept columns
 //                           in registers (warp-uniform selectors), rounds them to TF32 and writes
@@ -22,9 +22,11 @@
 //                           swizzled layout and written to NHWC with TMA stores.  With two
 //                           accumulator buffers it overlaps the next item's main loop.
 //
-// A chunk's chain (barrier, loads, selection, TMEM store, barrier) takes a team 0.5 us and more whatever it moves, so two teams
-// take chunks in turn, with operand sets of their own: one team and two, us: 256 -> 256, 3x3 at 14x14, batch 32, 2:4 31.1, 25.9; 64 -> 64 at 56x56, batch 16
-// 24.0, 20.6; 96 -> 96 at 31x38, batch 5, 3x3, 3:4, T = 16 18.5, 16.0.
+// A chunk's chain (barrier, loads, selection, TMEM store, barrier) takes a team 0.4 us and more whatever it moves, so where much is selected two teams
+// take chunks in turn, with operand sets of their own; where little is, the second one only takes registers and a stage (see make_cfg).  One team and
+// two, us: 256 -> 256, 3x3 at 14x14, batch 32, 2:4 29.1, 26.2; 96 -> 96 at 31x38, batch 5, 3x3, 3:4, T = 16 18.5, 15.9; but 96 -> 192, 1x1 at 67x43, batch
+// 32, 1:4, T = 16 43.1, 46.0; 64 -> 384, 1x1 at 77x43, batch 24, 2:4, T = 96 26.5, 28.9.  The epilogue's bias goes through shared memory: by shuffles
+// (32 a block) the last of these took 32.5 us.
 // The tiles of a layer are dealt to the CTAs in groups of G; the last group may be smaller (its missing tiles are neither fetched nor
 // multiplied, and the store clips their channels).
 //
@@ -45,7 +47,8 @@ constexpr int BM = 128;
 constexpr int SUB_BYTES = BM * 128;   // one 32-column slab sub-tile
 constexpr int NSTAGE_MAX = 6;
 constexpr int A_COL0 = 256;           // TMEM: accumulators in columns [0, 256), operand sets above
-constexpr int THREADS = 768;          // warps: 0 producer, 1 MMA issuer, 2 tensor memory, 4-7 epilogue, 8-23 compactors
+// warps: 0 producer, 1 MMA issuer, 2 tensor memory, 4-7 epilogue, from 8 on compactors
+constexpr int threads_of(int teams) { return 256 + teams * 256; }
 constexpr int MAX_SETS = 4;
 constexpr int BOX_BYTES = 4096;       // 32 x 32 output box of an epilogue warp
 
@@ -59,6 +62,7 @@ struct StreamCfg {
     int stage_bytes;
     int boxes;        // staging boxes per epilogue warp: two, or one where the ring gains two stages by it
     int set_cols;     // TMEM columns of one operand set = g * 32
+    int teams;        // compactor teams that take chunks: 1 or 2
     int n_sets;       // operand sets: two per team where 256 columns hold them, else one
     long long n_work;
 };
@@ -127,32 +131,36 @@ struct Pattern {
     static constexpr int LW = S / 8;         // 16-byte loads per compactor thread and chunk
 };
 
-template <int NK, int MG>
-__global__ void __launch_bounds__(THREADS, 1)
+template <int NK, int MG, int TEAMS>
+__global__ void __launch_bounds__(threads_of(TEAMS), 1)
 k_conv_stream(const ConvParams p, const StreamCfg cfg, const __grid_constant__ CUtensorMap tm_x,
               const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_y)
 {
     using P = Pattern<NK, MG>;
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t s_full[NSTAGE_MAX], s_free[NSTAGE_MAX], s_aready[MAX_SETS], s_afree[MAX_SETS], s_accfull[2], s_accfree[2];
+    __shared__ uint64_t s_full[2 * NSTAGE_MAX], s_free[NSTAGE_MAX], s_aready[MAX_SETS], s_afree[MAX_SETS], s_accfull[2], s_accfree[2];
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
+    __shared__ __align__(16) float s_bias[4][32];   // bias of the block an epilogue warp works on
 
     const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
     const uint32_t n_work = static_cast<uint32_t>(cfg.n_work);   // below 2^31: per-item arithmetic stays 32-bit
     const int NS = cfg.stages, n_chunks = p.v2_chunks, g = cfg.g, T = p.tile_t;
+    // A stage of an odd ring goes to two teams in turn, and a team that passes by every second phase of a barrier cannot tell an earlier
+    // phase from its own: such a ring has a full barrier per stage and team, used in turn, so that whoever waits on one sees all its phases.
+    const int NF = TEAMS == 2 && (NS & 1) ? 2 * NS : NS;
     const uint32_t ring = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t staging = ring + NS * cfg.stage_bytes;
-    auto live_tiles = [&](int slice) { return min(g, p.n_tiles - slice * g); };
+    // tiles of an item: g, or what is left of them in the last group (the division only where the tiles do not fill it)
+    const bool ragged = cfg.n_slices * g != p.n_tiles;
+    auto live_tiles = [&](uint32_t work) { return ragged ? min(g, p.n_tiles - static_cast<int>(work % static_cast<uint32_t>(cfg.n_slices)) * g) : g; };
     volatile int* abort_flag = &s_abort;
 
     // ---- set-up ----------------------------------------------------------------------------------
     if (warp == 2) tmem_alloc(smem_u32(&s_tmem), 512);
     if (tid == 0) {
-        for (int i = 0; i < NSTAGE_MAX; ++i) {
-            mbar_init(smem_u32(&s_full[i]), 1);       // producer's expect-tx arrival
-            mbar_init(smem_u32(&s_free[i]), 8 + 1);   // a team's warps + MMA commit
-        }
+        for (int i = 0; i < 2 * NSTAGE_MAX; ++i) mbar_init(smem_u32(&s_full[i]), 1);   // producer's expect-tx arrival
+        for (int i = 0; i < NSTAGE_MAX; ++i) mbar_init(smem_u32(&s_free[i]), 8 + 1);   // a team's warps + MMA commit
         for (int i = 0; i < MAX_SETS; ++i) {
             mbar_init(smem_u32(&s_aready[i]), 8);     // a team's warps
             mbar_init(smem_u32(&s_afree[i]), 1);      // MMA commit
@@ -179,7 +187,7 @@ k_conv_stream(const ConvParams p, const StreamCfg cfg, const __grid_constant__ C
         if (elect_one()) {
             const int hw = p.ho * p.wo;
             const size_t rpitch = static_cast<size_t>(n_chunks) * 32;
-            RingPos rp;
+            RingPos rp, rf;
             int issued = 0;
             for (uint32_t work = blockIdx.x; work < n_work && !aborted(abort_flag); work += gridDim.x) {
                 const int slice = static_cast<int>(work % static_cast<uint32_t>(cfg.n_slices));
@@ -189,7 +197,7 @@ k_conv_stream(const ConvParams p, const StreamCfg cfg, const __grid_constant__ C
                 const int oh0 = rem / p.wo, ow0 = rem - oh0 * p.wo;
                 const int w0 = ow0 * p.stride_w - p.pad_w, h0 = oh0 * p.stride_h - p.pad_h;
                 const uint8_t* rsrc = p.rel2 + static_cast<size_t>(slice * g) * rpitch;
-                const int tiles = live_tiles(slice);
+                const int tiles = live_tiles(work);
                 const uint32_t tx_fixed = static_cast<uint32_t>(cfg.bn) * 128u + static_cast<uint32_t>(tiles) * 32u;   // (rows past the last channel arrive as zeros)
                 int ch = 0, off_w = 0, off_h = 0, tw = 0, k0 = 0;   // position of the next 32-column sub-tile
                 for (int c = 0; c < n_chunks; ++c) {
@@ -198,7 +206,7 @@ k_conv_stream(const ConvParams p, const StreamCfg cfg, const __grid_constant__ C
                     const uint32_t b_smem = ring + rp.s * cfg.stage_bytes;
                     const uint32_t slab = b_smem + cfg.b_bytes;
                     const uint32_t relbuf = slab + P::SEGS * SUB_BYTES;
-                    const uint32_t bar = smem_u32(&s_full[rp.s]);
+                    const uint32_t bar = smem_u32(&s_full[rf.s]);
                     const int live = (P::SEGS == 2 && k0 + 32 >= p.k) ? 1 : P::SEGS;
                     mbar_arrive_expect_tx(bar, static_cast<uint32_t>(live) * SUB_BYTES + tx_fixed);
                     for (int seg = 0; seg < P::SEGS; ++seg) {
@@ -216,15 +224,16 @@ k_conv_stream(const ConvParams p, const StreamCfg cfg, const __grid_constant__ C
                     tma_load_2d(b_smem, &tm_w, bar, c * 32, slice * cfg.bn);
                     for (int t = 0; t < tiles; ++t) bulk_load_1d(relbuf + t * 32, rsrc + t * rpitch + c * 32, 32u, bar);
                     rp.advance(NS);
+                    rf.advance(NF);
                     ++issued;
                 }
             }
             if (aborted(abort_flag)) {
                 // loads already issued still target this CTA's shared memory: let them land
                 for (int back = 0; back < NS && back < issued; ++back) {
-                    if (rp.s == 0) { rp.s = NS; rp.parity ^= 1u; }
-                    --rp.s;
-                    (void)mbar_wait(smem_u32(&s_full[rp.s]), rp.parity);
+                    if (rf.s == 0) { rf.s = NF; rf.parity ^= 1u; }
+                    --rf.s;
+                    (void)mbar_wait(smem_u32(&s_full[rf.s]), rf.parity);
                 }
             }
         }
@@ -232,7 +241,7 @@ k_conv_stream(const ConvParams p, const StreamCfg cfg, const __grid_constant__ C
         // =========================== MMA issuer ===========================
         if (elect_one()) {
             const uint32_t idesc = umma_idesc_tf32(BM, T);
-            RingPos rp;
+            RingPos rf;                             // full barrier, stage and
             RingPos rs;                             // operand set of this chunk
             uint32_t ab = 0, acc_par = 0;           // accumulator buffer of this item, parity of its current use
             bool acc_wrapped = false;
@@ -243,13 +252,14 @@ k_conv_stream(const ConvParams p, const StreamCfg cfg, const __grid_constant__ C
                 }
                 tc_fence_after();
                 const uint32_t acc = tmem + ab * cfg.bn;
-                const int tiles = live_tiles(static_cast<int>(work % static_cast<uint32_t>(cfg.n_slices)));
+                const int tiles = live_tiles(work);
                 for (int c = 0; c < n_chunks; ++c) {
-                    if (!mbar_wait_lone(smem_u32(&s_full[rp.s]), rp.parity)) { *abort_flag = 6; break; }
+                    if (!mbar_wait_lone(smem_u32(&s_full[rf.s]), rf.parity)) { *abort_flag = 6; break; }
                     if (!mbar_wait_lone(smem_u32(&s_aready[rs.s]), rs.parity)) { *abort_flag = 7; break; }
                     if (aborted(abort_flag)) break;
                     tc_fence_after();
-                    const uint32_t b_smem = ring + rp.s * cfg.stage_bytes;
+                    const int stage = TEAMS == 1 || rf.s < NS ? rf.s : rf.s - NS;
+                    const uint32_t b_smem = ring + stage * cfg.stage_bytes;
                     const uint32_t a_set = tmem + A_COL0 + rs.s * cfg.set_cols;
                     for (int t = 0; t < tiles; ++t) {
                         const uint64_t bdesc = umma_desc_k_sw128(b_smem + t * T * 128, 1024);
@@ -259,8 +269,8 @@ k_conv_stream(const ConvParams p, const StreamCfg cfg, const __grid_constant__ C
                                          (c > 0 || kq > 0) ? 1u : 0u);
                     }
                     umma_commit(smem_u32(&s_afree[rs.s]));
-                    umma_commit(smem_u32(&s_free[rp.s]));
-                    rp.advance(NS);
+                    umma_commit(smem_u32(&s_free[stage]));
+                    rf.advance(NF);
                     rs.advance(cfg.n_sets);
                 }
                 if (aborted(abort_flag)) break;
@@ -299,6 +309,13 @@ k_conv_stream(const ConvParams p, const StreamCfg cfg, const __grid_constant__ C
             for (int blk = 0; blk < n_blk; ++blk, ++nb) {
                 uint32_t v[32];
                 tmem_ld32(tmem + lane_addr + ab * cfg.bn + blk * 32, v);
+                s_bias[q][lane] = bias_of[0];   // (the block before it has been read: see its __syncwarp)
+#pragma unroll
+                for (int i = 0; i < 7; ++i) bias_of[i] = bias_of[i + 1];
+                __syncwarp();
+                float4 bias[8];
+#pragma unroll
+                for (int qq = 0; qq < 8; ++qq) bias[qq] = reinterpret_cast<const float4*>(s_bias[q])[qq];
                 tmem_ld_wait(v);
                 if (blk == n_blk - 1) {
                     // the accumulator buffer may be overwritten from here on
@@ -317,16 +334,10 @@ k_conv_stream(const ConvParams p, const StreamCfg cfg, const __grid_constant__ C
                 const long long box_pix = static_cast<long long>(pix0) + q * 32;
                 const bool res_pass = p.residual != nullptr && box_pix < p.pixels;
                 const int relu_now = res_pass ? 0 : p.relu;
-                // (all shuffles before the first store: both are ordered statements)
-                float4 bias4[8];
-#pragma unroll
-                for (int qq = 0; qq < 8; ++qq) bias4[qq] = bias_quad(bias_of[0], qq);
-#pragma unroll
-                for (int i = 0; i < 7; ++i) bias_of[i] = bias_of[i + 1];
 #pragma unroll
                 for (int qq = 0; qq < 8; ++qq) {
                     float o[4];
-                    const float4 bv = bias4[qq];
+                    const float4 bv = bias[qq];
                     o[0] = __uint_as_float(v[qq * 4 + 0]) + bv.x;
                     o[1] = __uint_as_float(v[qq * 4 + 1]) + bv.y;
                     o[2] = __uint_as_float(v[qq * 4 + 2]) + bv.z;
@@ -358,26 +369,28 @@ k_conv_stream(const ConvParams p, const StreamCfg cfg, const __grid_constant__ C
     } else if (warp >= 8) {
         // =========================== compactors ===========================
         const int wg = (warp - 8) >> 2 & 1;   // which half of the chunk
-        const int team = (warp - 8) >> 3;
+        const int team = TEAMS == 1 ? 0 : (warp - 8) >> 3;
         const int q = warp & 3;           // TMEM lane quadrant
         const int row = q * 32 + lane;
         const uint32_t lane_addr = static_cast<uint32_t>(q * 32) << 16;
         const uint32_t rx = static_cast<uint32_t>(row & 7);
         constexpr int CI0_STEP = P::LW;   // first 16-byte piece of half `wg`
-        // The chunks of all of this CTA's items are numbered through; a team has those of its parity.  Stages and sets are even in number, so a
-        // stage or set always belongs to the same team, which so sees each of its uses.
-        RingPos rp, rs;
-        rp.s = rs.s = team;
+        // The chunks of all of this CTA's items are numbered through; of two teams one has the even, one the odd ones.  Full barriers and sets
+        // are then even in number, so one always belongs to the same team, which so sees each of its uses.
+        RingPos rf, rs;
+        rf.s = rs.s = team;
         int turn = 0;
         for (uint32_t work = blockIdx.x; work < n_work && !aborted(abort_flag); work += gridDim.x) {
-            const int tiles = live_tiles(static_cast<int>(work % static_cast<uint32_t>(cfg.n_slices)));
+            const int tiles = live_tiles(work);
             for (int c = 0; c < n_chunks; ++c) {
-                const bool mine = turn == team;
-                turn ^= 1;
-                if (!mine) continue;
-                const int s = rp.s;
+                if (TEAMS == 2) {
+                    const bool mine = turn == team;
+                    turn ^= 1;
+                    if (!mine) continue;
+                }
+                const int s = TEAMS == 1 || rf.s < NS ? rf.s : rf.s - NS;
                 const uint32_t set = static_cast<uint32_t>(rs.s);
-                bool ok = mbar_wait_lone(smem_u32(&s_full[s]), rp.parity);
+                bool ok = mbar_wait_lone(smem_u32(&s_full[rf.s]), rf.parity);
                 if (!__all_sync(0xFFFFFFFFu, ok)) *abort_flag = 3;
                 ok = !rs.wrapped || mbar_wait_lone(smem_u32(&s_afree[set]), rs.parity ^ 1u);
                 if (!__all_sync(0xFFFFFFFFu, ok)) *abort_flag = 4;
@@ -428,10 +441,8 @@ k_conv_stream(const ConvParams p, const StreamCfg cfg, const __grid_constant__ C
                     mbar_arrive(smem_u32(&s_aready[set]));
                     mbar_arrive(smem_u32(&s_free[s]));
                 }
-                rp.advance(NS);
-                rp.advance(NS);
-                rs.advance(cfg.n_sets);
-                rs.advance(cfg.n_sets);
+                rf.advance_by(TEAMS, NF);
+                rs.advance_by(TEAMS, cfg.n_sets);
             }
         }
     }
@@ -520,18 +531,20 @@ bool make_cfg(const ConvParams& p, const nm_plan_t* plan, StreamCfg* cfg)
     cfg->n_slices = (p.n_tiles + g - 1) / g;
     cfg->n_acc = cfg->bn <= 128 ? 2 : 1;
     cfg->set_cols = g * 32;
-    cfg->n_sets = 4 * cfg->set_cols <= 512 - A_COL0 ? 4 : 2;
+    // Two teams from four chunks and 24 kept columns of a CTA's tiles per chunk on; below that the selection is short beside the loads, and what
+    // a second team costs (80 registers a thread instead of 128, another stage held) shows.  Of 900 layer and width pairs the choice is 0.2 % behind
+    // the better of the two in the middle, more than 2 % for 41, 8 % at worst; always two is behind by more than 2 % for 272, always one for 407.
+    cfg->teams = p.v2_chunks >= 4 && g * p.v2_kc >= 24 ? 2 : 1;
+    cfg->n_sets = cfg->teams == 2 && 4 * cfg->set_cols <= 512 - A_COL0 ? 4 : 2;
     cfg->b_bytes = ((cfg->bn * 128 + 1023) / 1024) * 1024;   // whole swizzle atoms
     cfg->stage_bytes = cfg->b_bytes + (p.v2_s / 32) * SUB_BYTES + 1024;  // offsets area padded to keep stages aligned
-    // The teams own alternate stages, so their number is even; an odd number asked for is taken down, two always fit.
     const int budget = 227 * 1024 - 1024 - 1024;         // alignment slack, static shared
     const int asked = plan && plan->stages > 0 ? plan->stages : 0;
-    if (asked > NSTAGE_MAX || (asked && asked * cfg->stage_bytes > budget - 8 * BOX_BYTES)) return false;
-    auto most = [&](int boxes) { return std::min((budget - 4 * boxes * BOX_BYTES) / cfg->stage_bytes, NSTAGE_MAX) & ~1; };
+    auto most = [&](int boxes) { return std::min((budget - 4 * boxes * BOX_BYTES) / cfg->stage_bytes, NSTAGE_MAX); };
     // (64 -> 256, one chunk of 64 columns, at 56x56, batch 4: 7.2 us with two boxes, 8.5 with one; 256 -> 256, 3x3 at 14x14, batch 32: 35.1, 25.9)
-    cfg->boxes = p.v2_chunks > 4 && most(1) > most(2) ? 1 : 2;
-    int stages = asked ? std::max(asked & ~1, 2) : most(cfg->boxes);
-    if (stages < 2 || stages > most(cfg->boxes)) return false;
+    cfg->boxes = asked ? (asked > most(2) ? 1 : 2) : p.v2_chunks > 4 && most(1) > most(2) ? 1 : 2;
+    const int stages = asked ? asked : most(cfg->boxes);
+    if (stages < (asked ? 1 : 2) || stages > most(cfg->boxes)) return false;
     cfg->stages = stages;
     const long long pix_blocks = (p.pixels + BM - 1) / BM;
     cfg->n_work = pix_blocks * cfg->n_slices;
@@ -539,8 +552,8 @@ bool make_cfg(const ConvParams& p, const nm_plan_t* plan, StreamCfg* cfg)
     return true;
 }
 
-template <int NK, int MG>
-nm_status_t launch(const ConvParams& p, const StreamCfg& cfg, cudaStream_t st)
+template <int NK, int MG, int TEAMS>
+nm_status_t launch_teams(const ConvParams& p, const StreamCfg& cfg, cudaStream_t st)
 {
     alignas(64) CUtensorMap tm_x, tm_w, tm_y;
     if (!nmtm::encode_x_im2col(p, BM, &tm_x) || !nmtm::encode_w_tiled(p, cfg.bn, &tm_w) ||
@@ -548,14 +561,20 @@ nm_status_t launch(const ConvParams& p, const StreamCfg& cfg, cudaStream_t st)
         return nmhost::fail(NM_ERR_CUDA, "nm_conv2d: tensor-map encoding failed (variant 3)");
     size_t smem = 1024 + static_cast<size_t>(cfg.stages) * cfg.stage_bytes + 4 * cfg.boxes * BOX_BYTES;
     if (smem < NM_EXCLUSIVE_SMEM) smem = NM_EXCLUSIVE_SMEM;   // one CTA per SM: it owns all 512 TMEM columns
-    cudaError_t e = nmhost::ensure_dynamic_smem(reinterpret_cast<const void*>(k_conv_stream<NK, MG>), smem);
+    cudaError_t e = nmhost::ensure_dynamic_smem(reinterpret_cast<const void*>(k_conv_stream<NK, MG, TEAMS>), smem);
     if (e != cudaSuccess) return nmhost::fail(NM_ERR_CUDA, "cudaFuncSetAttribute (variant 3): %s", cudaGetErrorString(e));
     const long long grid = cfg.n_work < nmhost::sm_count() ? cfg.n_work : nmhost::sm_count();
-    e = nmhost::launch_pdl(k_conv_stream<NK, MG>, static_cast<unsigned>(grid), THREADS, smem, st, p, cfg, tm_x, tm_w, tm_y);
+    e = nmhost::launch_pdl(k_conv_stream<NK, MG, TEAMS>, static_cast<unsigned>(grid), static_cast<unsigned>(threads_of(TEAMS)), smem, st, p, cfg, tm_x, tm_w, tm_y);
     nmhost::count_launch(1);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return nmhost::fail(NM_ERR_CUDA, "nm_conv2d launch (variant 3): %s", cudaGetErrorString(e));
     return NM_OK;
+}
+
+template <int NK, int MG>
+nm_status_t launch(const ConvParams& p, const StreamCfg& cfg, cudaStream_t st)
+{
+    return cfg.teams == 2 ? launch_teams<NK, MG, 2>(p, cfg, st) : launch_teams<NK, MG, 1>(p, cfg, st);
 }
 
 }  // namespace

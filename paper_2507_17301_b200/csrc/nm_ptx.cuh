@@ -116,6 +116,14 @@ struct RingPos {
             wrapped = true;
         }
     }
+    __device__ __forceinline__ void advance_by(int k, int n)   // k <= n
+    {
+        if ((s += k) >= n) {
+            s -= n;
+            parity ^= 1u;
+            wrapped = true;
+        }
+    }
 };
 
 // The same wait with an explicit poll budget (self-test of the expiry path).
