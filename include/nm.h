@@ -105,7 +105,8 @@ typedef struct nm_weights nm_weights_t;
  *                by a cluster of `ksplit` (1, 2, 4, 8; 0 = 1) CTAs, each over a range of the reduction axis of variant 4's expanded
  *                weights; the partial sums move between the CTAs' shared memories (conditions of variant 4, no
  *                scratch; the tuner tries it unless NM_AUTOTUNE_VARIANTS restricts the search).
- *   bn       output channels per CTA / work item (variants 2, 3, 8: a multiple of tile_t; variant 4: a
+ *   bn       output channels per CTA / work item (variants 2, 3, 8: a multiple of tile_t, for variant 3 one to four tiles that make
+ *            whole blocks of 32 channels and at most 256, and need not divide c_out; variant 4: a
  *            multiple of 32 up to 256 that divides c_out rounded up to a multiple of 32; variant 6: a multiple
  *            of 32 up to 256 that divides c_out; variant 7: 128 or 256), 0 = default
  *   stages   depth of the shared-memory ring, 0 = default

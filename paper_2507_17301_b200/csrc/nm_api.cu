@@ -267,9 +267,13 @@ std::vector<nm_plan_t> candidate_plans(const nm_weights* /*w*/, const ConvParams
         }
     }
     std::memset(&a, 0, sizeof(a));
-    for (int bn : {0, 256, p.tile_t}) {     // stream kernel: default width, widest, one tile per CTA
-        a.variant = 3; a.bn = bn; a.stages = 0;
-        if ((bn == 0 || bn != p.tile_t || bn < 128) && nmhost::stream_plan_ok(p, &a)) out.push_back(a);
+    std::vector<int> listed;
+    for (int bn : {0, 256, p.tile_t, nmhost::stream_width(p, nullptr)}) {   // stream kernel: default width, widest, one tile per CTA, and the one
+        a.variant = 3; a.bn = bn; a.stages = 0;                             // that a call without a plan takes
+        const int width = nmhost::stream_width(p, &a);
+        if (width == 0 || std::find(listed.begin(), listed.end(), width) != listed.end()) continue;
+        listed.push_back(width);
+        out.push_back(a);
     }
     std::memset(&a, 0, sizeof(a));
     for (int bn : {0, p.tile_t}) {          // default (as many tiles as fit) and one tile per CTA

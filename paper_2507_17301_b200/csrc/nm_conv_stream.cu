@@ -504,28 +504,29 @@ bool make_cfg(const ConvParams& p, const nm_plan_t* plan, StreamCfg* cfg)
     // im2col maps of very small tensors are left to the other kernels
     if (static_cast<long long>(p.batch) * p.h * p.w * p.c_in * 4 < 131072) return false;
     if (p.pixels >= (1ll << 31) - BM) return false;
-    int g;
+    int g = 0;
     if (plan && plan->bn > 0) {
         if (plan->bn % T != 0) return false;
         g = plan->bn / T;
-    } else {
+    } else if (plan) {
         // largest group of up to 128 channels that divides the tiles
-        g = 1;
-        for (int cand = 4; cand >= 1; --cand)
-            if (cand * T <= 128 && p.n_tiles % cand == 0 && (cand * T) % 32 == 0) { g = cand; break; }
+        for (int cand = 4; cand >= 1 && g == 0; --cand)
+            if (cand * T <= 128 && p.n_tiles % cand == 0 && (cand * T) % 32 == 0) g = cand;
+        if (g == 0 && T > 128) g = 1;
+    }
+    if (g == 0) {
         // The library default deals tiles out in groups that need not divide them, by an estimate of the time (a
         // chunk takes 0.24 us and 0.12-0.17 per tile): 128 -> 128, 3x3 at 28x28, batch 4, T = 32 19.1 us in the gather kernel, 12.0 with
         // a tile per CTA, 21.9 with four; 96 -> 80, T = 16 (five tiles) at 31x38, batch 5 21.6 in the gather kernel, 15.9 with two.
-        if (!plan) {
-            double best = 0.0;
-            for (int cand = 4; cand >= 1; --cand) {
-                if (cand * T > 128 || (cand * T) % 32 != 0) continue;
-                const double t = item_rounds(p, (p.n_tiles + cand - 1) / cand) * (0.25 + 0.15 * cand);
-                if (best == 0.0 || t < best) { best = t; g = cand; }
-            }
+        g = 1;
+        double best = 0.0;
+        for (int cand = 4; cand >= 1; --cand) {
+            if (cand * T > 128 || (cand * T) % 32 != 0) continue;
+            const double t = item_rounds(p, (p.n_tiles + cand - 1) / cand) * (0.25 + 0.15 * cand);
+            if (best == 0.0 || t < best) { best = t; g = cand; }
         }
     }
-    if (g < 1 || g > 4 || g * T > 256 || (plan && p.n_tiles % g != 0) || (g * T) % 32 != 0) return false;
+    if (g < 1 || g > 4 || g * T > 256 || (g * T) % 32 != 0) return false;
     cfg->g = g;
     cfg->bn = g * T;
     cfg->n_slices = (p.n_tiles + g - 1) / g;
@@ -585,6 +586,12 @@ bool stream_plan_ok(const ConvParams& p, const nm_plan_t* plan)
 {
     StreamCfg cfg;
     return make_cfg(p, plan, &cfg);
+}
+
+int stream_width(const ConvParams& p, const nm_plan_t* plan)
+{
+    StreamCfg cfg;
+    return make_cfg(p, plan, &cfg) ? cfg.bn : 0;
 }
 
 bool stream_leaves_sms_idle(const ConvParams& p)

@@ -259,6 +259,7 @@ nm_status_t launch_conv_pair(const ConvParams& p, const nm_plan_t* plan, cudaStr
 
 // nm_conv_stream.cu — variant 3
 bool stream_plan_ok(const ConvParams& p, const nm_plan_t* plan);
+int stream_width(const ConvParams& p, const nm_plan_t* plan);   // channels per work item, 0: the kernel does not take the layer / plan
 bool stream_leaves_sms_idle(const ConvParams& p);   // few work items, each with a long reduction: the gather kernel splits it
 nm_status_t launch_conv_stream(const ConvParams& p, const nm_plan_t* plan, cudaStream_t st);
 
