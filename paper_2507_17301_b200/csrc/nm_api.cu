@@ -156,7 +156,7 @@ nm_status_t run_plan(const ConvParams& p, const nm_plan_t* plan, cudaStream_t st
     switch (variant) {
         case 0:
             // (the row-run and plane kernels truncate activations and multiply zeros for pruned columns, the others do neither)
-            if (nmhost::stream_plan_ok(p, nullptr) && !nmhost::stream_leaves_sms_idle(p)) return nmhost::launch_conv_stream(p, nullptr, st);
+            if (nmhost::stream_beats_gather(p)) return nmhost::launch_conv_stream(p, nullptr, st);
             if (nmhost::planes_plan_ok(p, nullptr)) return nmhost::launch_conv_planes(p, nullptr, st);
             // Channel counts that are no multiple of 32: runs of rows where there is enough work for their set-up.  Units of a pixel
             // block, tile and chunk, and us against the gather's: 2352 (8x112x112, 16->32) 18.4 / 20.6, 1568 (32x56x56, 8->64 by

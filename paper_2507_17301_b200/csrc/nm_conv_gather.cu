@@ -422,6 +422,41 @@ __global__ void __launch_bounds__(THREADS, 2) k_conv_gather(const ConvParams p, 
 
 namespace nmhost {
 
+// Ranges of the chunks (CTAs of a cluster) for a launch of `items` (pixel block, tile) pairs.
+static int ranges_of(long long items, int chunks)
+{
+    // By an estimate of the time from the costs above: a chunk takes a CTA 0.95 us, 0.70 us where it has its
+    // SM to itself; a wave has about 3 us of its own and 4 more with the exchange (clusters do not fit on every last SM).
+    // Measured, us: 7 blocks x 5 tiles, 95 chunks, one range 69, two 42, four 28, eight (a second wave) 49; 55 blocks x 8 tiles, 54 chunks,
+    // one range 68, two 83; 15 blocks x 8 tiles, 5 chunks, one range 14, two 16.
+    const long long sms = sm_count();
+    double best = 1e30;
+    int ranges = 1;
+    for (int cs = 1; cs <= 8 && (cs == 1 || chunks >= 2 * cs); cs *= 2) {
+        const long long ctas = items * cs, slots = 2 * sms - (cs > 1 ? 32 : 0);
+        const long long full = ctas / slots, rest = ctas - full * slots;
+        const int range = (chunks + cs - 1) / cs;
+        const double wave = cs > 1 ? 7.0 : 3.0;
+        const double t = full * (range * 0.95 + wave) + (rest == 0 ? 0.0 : range * (rest <= sms ? 0.70 : 0.95) + wave);
+        if (t < best * 0.95) { best = t; ranges = cs; }
+    }
+    return ranges;
+}
+
+// The time over all sizes, fitted to 900 layers that the stream kernel takes as well (c_in 32-512, c_out 16-1024, 1x1 to 5x5, T 16-128; 12 % rms).  A row
+// of a chunk reads as many sectors more as there are source columns to a kept one.
+double gather_estimate_us(const ConvParams& p)
+{
+    const int chunks = p.kk_pad / NM_KCHUNK;
+    const long long items = (p.pixels + BM - 1) / BM * p.n_tiles, sms = sm_count();
+    const int cs = ranges_of(items, chunks);
+    const long long ctas = items * cs, slots = 2 * sms - (cs > 1 ? 32 : 0), full = ctas / slots, rest = ctas - full * slots;
+    const double range = (chunks + cs - 1) / cs, spread = static_cast<double>(p.m_group) / p.n_keep, width = p.tile_t / 32.0;
+    const double wave = (cs > 1 ? 4.8 : 2.6) + 1.0 * width;
+    const double beside = range * (0.675 + 0.08 * spread + 0.084 * width) + wave, alone = range * (0.475 + 0.023 * spread + 0.072 * width) + wave;
+    return full * beside + (rest == 0 ? 0.0 : rest <= sms ? alone : beside);
+}
+
 double gather_time_us(const ConvParams& p)
 {
     const double chunks = p.kk_pad / NM_KCHUNK, channels = std::min(p.tile_t, p.c_out);
@@ -435,20 +470,7 @@ nm_status_t launch_conv_gather(const ConvParams& p, cudaStream_t st)
     if (cfg.n > 256) return fail(NM_ERR_UNSUPPORTED, "nm_conv2d: tile_t %d exceeds 256", p.tile_t);
     cfg.chunks = p.kk_pad / NM_KCHUNK;
     const long long blocks = (p.pixels + BM - 1) / BM;
-    // Ranges of the chunks, by an estimate of the time from the costs above: a chunk takes a CTA 0.95 us, 0.70 us where it has its
-    // SM to itself; a wave has about 3 us of its own and 4 more with the exchange (clusters do not fit on every last SM).
-    // Measured, us: 7 blocks x 5 tiles, 95 chunks, one range 69, two 42, four 28, eight (a second wave) 49; 55 blocks x 8 tiles, 54 chunks,
-    // one range 68, two 83; 15 blocks x 8 tiles, 5 chunks, one range 14, two 16.
-    const long long sms = nmhost::sm_count();
-    double best = 1e30;
-    for (int cs = 1; cs <= 8 && (cs == 1 || cfg.chunks >= 2 * cs); cs *= 2) {
-        const long long ctas = blocks * p.n_tiles * cs, slots = 2 * sms - (cs > 1 ? 32 : 0);
-        const long long full = ctas / slots, rest = ctas - full * slots;
-        const int range = (cfg.chunks + cs - 1) / cs;
-        const double wave = cs > 1 ? 7.0 : 3.0;
-        const double t = full * (range * 0.95 + wave) + (rest == 0 ? 0.0 : range * (rest <= sms ? 0.70 : 0.95) + wave);
-        if (t < best * 0.95) { best = t; cfg.cs = cs; }
-    }
+    cfg.cs = ranges_of(blocks * p.n_tiles, cfg.chunks);
     cfg.rps = BM / cfg.cs;
     cfg.tmem_cols = 32;
     while (cfg.tmem_cols < cfg.n) cfg.tmem_cols <<= 1;

@@ -475,11 +475,19 @@ bool layout_matches(const ConvParams& p)
     return p.v2_s == Pattern<NK, MG>::S && p.v2_kc == Pattern<NK, MG>::KC;
 }
 
-// Rounds of the SMs that the work items of `slices` slices take.
-double item_rounds(const ConvParams& p, int slices)
+// Two teams from four chunks and 24 kept columns of a CTA's tiles per chunk on; below that the selection is short beside the loads, and what
+// a second team costs (80 registers a thread instead of 128, another stage held) shows.  Of 900 layer and width pairs the choice is 0.2 % behind
+// the better of the two in the middle, more than 2 % for 41, 8 % at worst; always two is behind by more than 2 % for 272, always one for 407.
+int teams_for(const ConvParams& p, int g) { return p.v2_chunks >= 4 && g * p.v2_kc >= 24 ? 2 : 1; }
+
+// Time with `g` tiles per CTA, fitted to 1900 measured layer and width pairs (c_in 32-512, c_out 16-1024, 1x1 to 5x5, 1 to 12 tiles of 16-128; 17 %
+// rms): rounds of the SMs, each the chunks' chain or the epilogue, whichever is longer.
+double stream_time_us(const ConvParams& p, int g)
 {
-    const long long items = (p.pixels + BM - 1) / BM * slices, sms = nmhost::sm_count();
-    return static_cast<double>((items + sms - 1) / sms);
+    const long long items = (p.pixels + BM - 1) / BM * ((p.n_tiles + g - 1) / g), sms = nmhost::sm_count();
+    const double kept = g * p.v2_kc, segs = p.v2_s / 32, epilogue = 0.01 * g * p.tile_t;
+    const double chunk = teams_for(p, g) == 2 ? 0.24 + 0.0019 * kept + 0.11 * segs : 0.26 + 0.0028 * kept + 0.076 * segs;
+    return 1.95 + epilogue + static_cast<double>((items + sms - 1) / sms) * std::max(p.v2_chunks * chunk + 0.87, epilogue);
 }
 
 bool make_cfg(const ConvParams& p, const nm_plan_t* plan, StreamCfg* cfg)
@@ -515,14 +523,14 @@ bool make_cfg(const ConvParams& p, const nm_plan_t* plan, StreamCfg* cfg)
         if (g == 0 && T > 128) g = 1;
     }
     if (g == 0) {
-        // The library default deals tiles out in groups that need not divide them, by an estimate of the time (a
-        // chunk takes 0.24 us and 0.12-0.17 per tile): 128 -> 128, 3x3 at 28x28, batch 4, T = 32 19.1 us in the gather kernel, 12.0 with
-        // a tile per CTA, 21.9 with four; 96 -> 80, T = 16 (five tiles) at 31x38, batch 5 21.6 in the gather kernel, 15.9 with two.
+        // The library default deals tiles out in groups that need not divide them, by the estimate: 128 -> 128, 3x3 at 28x28, batch 4, T = 32
+        // 19.1 us in the gather kernel, 12.0 with a tile per CTA, 21.9 with four; 96 -> 80, T = 16 (five tiles) at 31x38, batch 5 21.6 in the gather
+        // kernel, 15.9 with two.
         g = 1;
         double best = 0.0;
         for (int cand = 4; cand >= 1; --cand) {
             if (cand * T > 128 || (cand * T) % 32 != 0) continue;
-            const double t = item_rounds(p, (p.n_tiles + cand - 1) / cand) * (0.25 + 0.15 * cand);
+            const double t = stream_time_us(p, cand);
             if (best == 0.0 || t < best) { best = t; g = cand; }
         }
     }
@@ -532,10 +540,7 @@ bool make_cfg(const ConvParams& p, const nm_plan_t* plan, StreamCfg* cfg)
     cfg->n_slices = (p.n_tiles + g - 1) / g;
     cfg->n_acc = cfg->bn <= 128 ? 2 : 1;
     cfg->set_cols = g * 32;
-    // Two teams from four chunks and 24 kept columns of a CTA's tiles per chunk on; below that the selection is short beside the loads, and what
-    // a second team costs (80 registers a thread instead of 128, another stage held) shows.  Of 900 layer and width pairs the choice is 0.2 % behind
-    // the better of the two in the middle, more than 2 % for 41, 8 % at worst; always two is behind by more than 2 % for 272, always one for 407.
-    cfg->teams = p.v2_chunks >= 4 && g * p.v2_kc >= 24 ? 2 : 1;
+    cfg->teams = teams_for(p, g);
     cfg->n_sets = cfg->teams == 2 && 4 * cfg->set_cols <= 512 - A_COL0 ? 4 : 2;
     cfg->b_bytes = ((cfg->bn * 128 + 1023) / 1024) * 1024;   // whole swizzle atoms
     cfg->stage_bytes = cfg->b_bytes + (p.v2_s / 32) * SUB_BYTES + 1024;  // offsets area padded to keep stages aligned
@@ -594,15 +599,16 @@ int stream_width(const ConvParams& p, const nm_plan_t* plan)
     return make_cfg(p, plan, &cfg) ? cfg.bn : 0;
 }
 
-bool stream_leaves_sms_idle(const ConvParams& p)
+bool stream_beats_gather(const ConvParams& p)
 {
-    // Work items on less than half of the SMs and sixteen chunks or more each, or on less than a quarter and twelve, us here and in the gather
-    // kernel, which splits the chunks over a cluster: 3x3 256 -> 256 at 14x14, batch 4 (28 items, 36 chunks) 20.3, 10.9; 128 -> 128 at 28x28, batch
-    // 4 (50, 18) 12.1, 10.5; 96 -> 96 at 20x20, batch 2 (21, 14) 9.9, 7.1; 1x1 512 -> 64 at 14x14, batch 4 (7, 8) 7.4, 9.2.
+    // The gather kernel gathers a pixel block once per tile, but has two CTAs on an SM, and splits the chunks over a cluster where there are
+    // few: one tile, or few pixel blocks with long reductions, are its own.  By both estimates, with a margin for small layers.  Measured, us, here and
+    // there: one tile of 16, 192 -> 16, 3x3 at 76x25, batch 23, 1:8 37.4, 19.5; one of 48, 64 -> 48, 5x5 at 21x44, batch 22, 1:4 27.0, 16.8; 3x3 256 -> 256 at
+    // 14x14, batch 4 20.3, 10.9; 448 -> 64, 5x5 at 40x69, batch 2, 2:8 83, 56; but 1x1 512 -> 64 at 14x14, batch 4 7.4, 9.2; five tiles of 16, 96 -> 80 at
+    // 31x38, batch 5, 3:4 15.9, 21.6.  Of 900 layers (a third of them one tile of 16 or 48; half of them not among the fitted
+    // ones) the choice is 1.6 % behind the better of the two in the middle, 46 % at worst.
     StreamCfg cfg;
-    if (!make_cfg(p, nullptr, &cfg)) return false;
-    const long long sms = nmhost::sm_count();
-    return (2 * cfg.n_work < sms && p.v2_chunks >= 16) || (4 * cfg.n_work < sms && p.v2_chunks >= 12);
+    return make_cfg(p, nullptr, &cfg) && stream_time_us(p, cfg.g) < 0.97 * gather_estimate_us(p) - 0.3;
 }
 
 nm_status_t launch_conv_stream(const ConvParams& p, const nm_plan_t* plan, cudaStream_t st)

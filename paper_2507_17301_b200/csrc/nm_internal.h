@@ -227,6 +227,7 @@ nm_status_t build_from_compressed(const float* values, const uint16_t* indices, 
 inline int gather_width(int tile_t, int c_out) { return ((tile_t < c_out ? tile_t : c_out) + 15) / 16 * 16; }
 nm_status_t launch_conv_gather(const ConvParams& p, cudaStream_t st);
 double gather_time_us(const ConvParams& p);   // estimate, one range of the chunks
+double gather_estimate_us(const ConvParams& p);   // the same where the stream kernel takes the layer, over all sizes
 
 // nm_conv_slab.cu — variant 2
 bool slab_plan_ok(const ConvParams& p, const nm_plan_t* plan);
@@ -260,7 +261,7 @@ nm_status_t launch_conv_pair(const ConvParams& p, const nm_plan_t* plan, cudaStr
 // nm_conv_stream.cu — variant 3
 bool stream_plan_ok(const ConvParams& p, const nm_plan_t* plan);
 int stream_width(const ConvParams& p, const nm_plan_t* plan);   // channels per work item, 0: the kernel does not take the layer / plan
-bool stream_leaves_sms_idle(const ConvParams& p);   // few work items, each with a long reduction: the gather kernel splits it
+bool stream_beats_gather(const ConvParams& p);   // (and takes the layer)
 nm_status_t launch_conv_stream(const ConvParams& p, const nm_plan_t* plan, cudaStream_t st);
 
 // nm_conv_select.cu — variant 8

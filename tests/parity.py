@@ -1,5 +1,7 @@
 """Shared helpers for the GPU parity tests: run one layer through the C-ABI binding and through
 the CPU oracle on the same seeded inputs and compare (helpers only; no method arithmetic)."""
+import re
+
 import numpy as np
 import torch
 
@@ -55,3 +57,13 @@ def assert_conv_close(y_gpu, y_ref):
     rel_fro, max_abs, ref_max = errors(y_gpu, y_ref)
     assert rel_fro <= REL_FRO_TOL, f"relative Frobenius error {rel_fro:.3e} above {REL_FRO_TOL}"
     assert max_abs <= MAX_ABS_TOL * ref_max, f"max-abs error {max_abs:.3e} above {MAX_ABS_TOL} * {ref_max:.3e}"
+
+
+def kernels_of(call):
+    """Names of this library's kernels that `call` launches, in order."""
+    from torch.profiler import ProfilerActivity, profile
+    torch.cuda.synchronize()
+    with profile(activities=[ProfilerActivity.CUDA]) as prof:
+        call()
+        torch.cuda.synchronize()
+    return [m for e in prof.events() for m in re.findall(r"\bk_[a-z0-9_]+", e.name)]
