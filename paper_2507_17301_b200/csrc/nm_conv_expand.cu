@@ -852,10 +852,11 @@ bool make_cfg(const ConvParams& p, const nm_plan_t* plan, ExpandCfg* cfg)
     cfg->w_stages = nw;
     cfg->n_work = tiles * cfg->n_slices * splits;
     if (cfg->n_work >= (1ll << 31)) return false;
-    // A pointwise layer that reads more than it writes walks its pixels backwards: its input is as a rule the layer before's output,
-    // written front to back, and of one that does not fit the L2 it is the end that is still there (ResNet-101 at batch 128 5276 -> 5128 us, with the pooling layer).
-    cfg->last_tile = pointwise && splits == 1 && !balanced && static_cast<double>(p.batch) * p.h * p.w * p.c_in > static_cast<double>(p.pixels) * p.c_out
-                         ? static_cast<int>(tiles) - 1 : -1;
+    // A pointwise layer that reads more than it writes walks its pixels backwards: its input is as a rule the layer before's output, written
+    // front to back, and the end of it is what the L2 still holds most of.  By itself (us, forwards and backwards): ResNet-101 at batch 128, 2:8 5155,
+    // 5023; ResNet-50 at batch 64, 2:4 1857, 1827; MobileNet-V2's pointwise layers, each on an input of its own, 310, 310.  Only for maps beyond
+    // the L2's 126 MB 5118 and 1846: a smaller one shares it with the shortcut and the outputs since.
+    cfg->last_tile = pointwise && splits == 1 && !balanced && nm_pointwise_reads_more(p) ? static_cast<int>(tiles) - 1 : -1;
     cfg->balanced = 0;
     if (balanced) {
         // one range per SM; needs at least one (item, stage) unit per CTA and the per-CTA slots + flags in the scratch

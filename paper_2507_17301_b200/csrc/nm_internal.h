@@ -106,6 +106,9 @@ struct ConvParams {
     const float* ws;
 };
 
+// Pointwise layers (no padding): a stride passes pixels by, so what is read is what is computed from.
+inline bool nm_pointwise_reads_more(const ConvParams& p) { return p.pixels * p.c_in > p.pixels * p.c_out; }
+
 #ifdef __CUDACC__
 // Shortcut input of one output pixel from channel `channel` on, as float4s (NULL without a residual or past the end).
 __device__ __forceinline__ const float4* nm_residual_row(const ConvParams& p, long long pixel, int channel)

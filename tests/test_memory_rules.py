@@ -55,3 +55,16 @@ def test_shared_arrays_read_as_vectors_are_aligned_for_them():
                         found += 1
                         assert int(align or 4) >= vectors[vector], (name, array, vector)
     assert found >= 2
+
+
+def test_which_pointwise_layers_read_more_than_they_write(tmp_path):
+    """A strided layer reads the pixels it computes from, not its whole input: 256 -> 512 by 2 reads half of what it writes."""
+    out = _run(tmp_path,
+               "    for (int stride : {1, 2})\n"
+               "        for (int c_out : {128, 256, 512}) {\n"
+               "            ConvParams p = {};\n"
+               "            p.batch = 2; p.h = p.w = 56; p.c_in = 256; p.c_out = c_out; p.stride_h = p.stride_w = stride;\n"
+               "            p.ho = p.wo = (56 + stride - 1) / stride; p.pixels = 2ll * p.ho * p.wo;\n"
+               '            std::printf("%d", nm_pointwise_reads_more(p) ? 1 : 0);\n'
+               "        }\n")
+    assert out == "100100"
