@@ -713,8 +713,10 @@ k_conv_expand(const ConvParams p, const ExpandCfg cfg, const __grid_constant__ C
 }
 
 // Second pass of a split-K plan: y[p][c] = act(sum over splits of partial[s][p][c] + bias[c] + residual[p][c]), the sums in the order of the
-// splits.  It is bound by latency (19 MB of sums that are still in the L2 for 6272 x 256 outputs in three ranges), so the number of splits and
-// the index type are compile-time and every load of an output is in flight at once (256 -> 256, 3x3 at 14x14, batch 32, with its first pass 19.9 -> 18.4 us).  S = 0: any number; I: index type.
+// splits.  It is bound by latency (19 MB of sums that are still in the L2 for 6272 x 256 outputs in three ranges): it lets the next kernel start early,
+// and with the number of splits and the index type known at compile time every load of an output is in flight at once.  By itself, over 360 pairs
+// of layer and split plan, the launch takes 4.3 % less than with a loop that does neither (256 -> 256, 3x3 at 14x14, batch 32, 2:8, three ranges of variant 4
+// 18.3 -> 17.7 us); the instances are 2 % of it for two and four splits, 0.3 % for three.  S = 0: any number; I: index type.
 template <int S, typename I>
 __global__ void __launch_bounds__(256) k_splitk_reduce(const float4* __restrict__ part, int splits, size_t split_stride4, size_t n4, int c_out4,
                                                        const float4* __restrict__ bias, const float4* __restrict__ residual, int relu,
