@@ -919,7 +919,7 @@ namespace nmhost {
 
 bool select_layout_dims(const nm_weights* h, int* s, int* kc)
 {
-    return pattern_dims(h->n_keep, h->m_group, s, kc) && h->kk > 0 && h->k % h->m_group == 0 && h->c_in % *s == 0 && h->tile_t % 16 == 0 &&
+    return pattern_dims(h->n_keep, h->m_group, s, kc) && h->k % h->m_group == 0 && h->c_in % *s == 0 && h->tile_t % 16 == 0 &&
            h->c_out % h->tile_t == 0;
 }
 

@@ -12,8 +12,9 @@
 // With groups of at most 128 columns a handle is built by ONE kernel (k_compress): a block owns a span of whole groups of one tile
 // (up to 64 of its rows), reads that piece of the dense weights (import: of the retained values) once into shared memory, selects
 // the columns there, and writes the piece's part of every layout, zeros of the expanded one included.  Wider groups are
-// selected by the kernels of nm_prune.cu, and k_build_layouts writes the layouts from the index array after a memset.
-// Both are bound by the writes (28 MB for 512 x 3 x 3 x 512 at 2:4).
+// selected by the kernels of nm_prune.cu, and k_build_layouts writes the layouts from the index array after a memset; the layouts' rules
+// are functions that both share.  k_compress writes 28 MB for 512 x 3 x 3 x 512 at 2:4 in 12 us, 2.3 TB/s: its blocks fit one wave and go
+// through loading, scoring, placing and writing in step, so memory idles while they score.
 #include <algorithm>
 #include <mutex>
 #include <vector>
@@ -141,9 +142,54 @@ __device__ int select_place(const uint16_t* idx, int kc, int e)
     return 0;   // (not reached: as many free places as columns left over)
 }
 
-constexpr int ROWS = 8;   // output channels per thread: a column is decoded and placed once for all of them (512 x 3 x 3 x 512: 106 us with one, 85 with 4, 82)
+// Tap and channel of column k of a row of weights.
+struct Column {
+    int tap, c, kh, kw;
+};
+__device__ __forceinline__ Column column_of(const LayoutArgs& a, int k)
+{
+    Column at;
+    at.tap = div_by(k, a.by_c_in);
+    at.c = k - at.tap * a.c_in;
+    at.kh = div_by(at.tap, a.by_kw);
+    at.kw = at.tap - at.kh * a.kw;
+    return at;
+}
+__device__ __forceinline__ uint32_t tap_word(const Column& at)
+{
+    return (static_cast<uint32_t>(at.kh) << 24) | (static_cast<uint32_t>(at.kw) << 16) | static_cast<uint32_t>(at.c);
+}
+// Float of column k in a 128-byte row whose 16-byte pieces are XOR-ed with (row % 8), the 128-byte swizzle.
+__device__ __forceinline__ int swizzled(int row, int k) { return (((k >> 2) ^ (row & 7)) << 2) | (k & 3); }
+// Gather layout: per (tile, chunk of 32 retained columns) the shared-memory image of the tile's rows; as many rows as the tile has, so it is as
+// large as the values whatever the tile width (padded to the MMA's 16 rows, 512 x 3 x 3 x 512 at 2:4 and T = 1 took 75 MB here
+// instead of 4.7).  The image of retained column j's chunk:
+__device__ __forceinline__ float* gather_image(const LayoutArgs& a, int row0, int tile_rows, int j)
+{
+    return a.wt + static_cast<size_t>(row0) * a.kk_pad + static_cast<size_t>(j / NM_KCHUNK) * tile_rows * NM_KCHUNK;
+}
+__device__ __forceinline__ int gather_cell(int row_of_tile, int j) { return row_of_tile * NM_KCHUNK + swizzled(row_of_tile, j & (NM_KCHUNK - 1)); }
+// Slab layout: retained column j (source column k) lies in chunk k / S at position j - chunk * KC (every group before the last is full, so a
+// chunk of whole groups holds exactly KC kept columns); `rel`: its offset in the chunk's source columns.
+__device__ __forceinline__ int slab_place(const LayoutArgs& a, int k, int j, uint8_t* rel)
+{
+    const int chunk = div_by(k, a.by_v2_s);
+    *rel = static_cast<uint8_t>(k - chunk * a.v2_s);
+    return chunk * 32 + (j - chunk * a.v2_kc);
+}
+// Expanded layout: the shared-memory image the tensor core reads: blocks of 32 columns, inside a block one swizzled row per output channel, so
+// that any run of channels starting at a multiple of 8 is one contiguous bulk copy.
+__device__ __forceinline__ float* expanded_cell(const LayoutArgs& a, int o, int k)
+{
+    return a.wx + (static_cast<size_t>(k >> 5) * a.wx_rows + o) * 32 + swizzled(o, k & 31);
+}
+// Plane layout: ws[kh][c_out][32]: a row holds the taps of one kernel row as (kw, c), c padded to 4 and kw to 8, swizzled.
+__device__ __forceinline__ float* plane_cell(const LayoutArgs& a, int o, int kh, int kw_c) { return a.ws + (static_cast<size_t>(kh) * a.c_out + o) * 32 + swizzled(o, kw_c); }
 
-// One thread per (retained column or padding column, ROWS output channels of a tile).
+constexpr int ROWS = 8;   // output channels per thread: a column is decoded and placed once for all of them (512 x 3 x 3 x 512 in groups of 600: 8.2 us with one, 6.1 with four, 5.6)
+
+// Groups wider than a block of k_compress (the select layout has none): one thread per (retained column or padding column, ROWS output
+// channels of a tile).
 __global__ void k_build_layouts(const LayoutArgs a)
 {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -165,64 +211,26 @@ __global__ void k_build_layouts(const LayoutArgs a)
         if (first_row) a.indices[static_cast<size_t>(r) * a.kk + j] = static_cast<uint16_t>(col);
         if (bad) return;
     }
-    const int tap = col / a.c_in, c = col - tap * a.c_in;
-    if (first_row)
-        a.taps[static_cast<size_t>(r) * a.kk_pad + j] =
-            (static_cast<uint32_t>(tap / a.kw) << 24) | (static_cast<uint32_t>(tap % a.kw) << 16) | static_cast<uint32_t>(c);
-
-    // slab layout: kept column j lies in chunk col / S at position j - chunk * KC (every group before the last is
-    // full, so a chunk of whole groups holds exactly KC kept columns)
+    const Column at = column_of(a, col);
+    if (first_row) a.taps[static_cast<size_t>(r) * a.kk_pad + j] = tap_word(at);
     const size_t pitch2 = static_cast<size_t>(a.v2_chunks) * 32;
-    size_t at2 = 0;
+    int at2 = 0;
     if (a.wt2) {
-        const int chunk = col / a.v2_s, jj = j - chunk * a.v2_kc;
-        at2 = static_cast<size_t>(chunk) * 32 + jj;
-        if (first_row) a.rel2[static_cast<size_t>(r) * pitch2 + at2] = static_cast<uint8_t>(col - chunk * a.v2_s);
+        uint8_t rel;
+        at2 = slab_place(a, col, j, &rel);
+        if (first_row) a.rel2[static_cast<size_t>(r) * pitch2 + at2] = rel;
     }
-    // select layout: w3[chunk][o][32], a chunk being as many steps (one tap of S source columns, of which KC are kept) as fit,
-    // the steps ordered by block of S channels, then tap; swizzled like wx.  The
-    // column tables hold, per chunk and tile, the byte offset of each column in its 128-byte row (and its 32-channel block in
-    // bit 7 and up), in the order in which a thread reads them: [step][place in a quad][quad].
-    int chunk3 = 0, k3 = 0;
-    if (a.w3) {
-        const int spc = 32 / a.sel_kc, cb = c / a.sel_s, cc = c - cb * a.sel_s, n_cb = a.c_in / a.sel_s;
-        const int step = cb * a.kh * a.kw + tap, sub = step % spc;
-        chunk3 = step / spc;
-        const int js = (tap * n_cb + cb) * a.sel_kc;   // the step's first retained column
-        const int place = select_place(idx + js, a.sel_kc, j - js);
-        k3 = sub * a.sel_kc + (place >> 3) * 8 + (place & 3) * 2 + (place >> 2 & 1);   // (a thread's columns of two quads are neighbours)
-        if (first_row) {
-            reinterpret_cast<uint32_t*>(a.sel3)[(static_cast<size_t>(chunk3) * a.n_tiles + r) * 32 + sub * a.sel_kc + (place & 3) * (a.sel_kc / 4) + (place >> 2)] =
-                static_cast<uint32_t>((cc & 31) * 4 | (cc >> 5) << 7);
-        }
-    }
-    // plane layout: ws[kh][c_out][32]: a row holds the taps of one kernel row as (kw, c), c padded to 4 and kw to 8,
-    // its 16-byte pieces (one tap each) XOR-ed with (o % 8)
-    const int khi = tap / a.kw, kwi = tap - khi * a.kw;
-
-    for (int rr = rr0; rr < min(rr0 + ROWS, a.tile_t); ++rr) {
-        const int o = r * a.tile_t + rr;
-        if (o >= a.c_out) break;
+    const int row0 = r * a.tile_t, tile_rows = min(a.tile_t, a.c_out - row0);
+    float* const wt = gather_image(a, row0, tile_rows, j);
+    for (int rr = rr0; rr < min(rr0 + ROWS, tile_rows); ++rr) {
+        const int o = row0 + rr;
         const float v = a.import ? a.src[static_cast<size_t>(o) * a.kk + j] : a.src[static_cast<size_t>(o) * a.k + col];
         const float t = nmk::to_tf32(v);
         a.values[static_cast<size_t>(o) * a.kk + j] = v;
-        {
-            // gather layout: per (tile, chunk of 32 retained columns) the shared-memory image of the tile's rows, swizzled like wx;
-            // as many rows as the tile has, so it is as large as the values whatever the tile width (padded to the MMA's 16 rows,
-            // 512 x 3 x 3 x 512 at 2:4 and T = 1 took 75 MB here instead of 4.7)
-            const int jj = j & (NM_KCHUNK - 1), rows = min(a.tile_t, a.c_out - r * a.tile_t);
-            a.wt[static_cast<size_t>(r) * a.tile_t * a.kk_pad + (static_cast<size_t>(j / NM_KCHUNK) * rows + rr) * NM_KCHUNK + ((((jj >> 2) ^ (rr & 7)) << 2) | (jj & 3))] = t;
-        }
+        wt[gather_cell(rr, j)] = t;
         if (a.wt2) a.wt2[static_cast<size_t>(o) * pitch2 + at2] = t;
-        if (a.wx) {
-            // expanded layout: the shared-memory image the tensor core reads: blocks of 32 columns, inside a block one
-            // 128-byte row per output channel whose 16-byte pieces are XOR-ed with (o % 8) (the 128-byte swizzle), so that
-            // any run of channels starting at a multiple of 8 is one contiguous bulk copy
-            const int blk = col >> 5, kc = col & 31;
-            a.wx[(static_cast<size_t>(blk) * a.wx_rows + o) * 32 + ((((kc >> 2) ^ (o & 7)) << 2) | (kc & 3))] = t;
-        }
-        if (a.w3) a.w3[(static_cast<size_t>(chunk3) * a.c_out + o) * 32 + ((((k3 >> 2) ^ (o & 7)) << 2) | (k3 & 3))] = t;
-        if (a.ws) a.ws[(static_cast<size_t>(khi) * a.c_out + o) * 32 + ((kwi ^ (o & 7)) << 2) + c] = t;
+        if (a.wx) *expanded_cell(a, o, col) = t;
+        if (a.ws) *plane_cell(a, o, at.kh, at.kw << 2 | at.c) = t;
     }
 }
 
@@ -383,17 +391,16 @@ __global__ void __launch_bounds__(544) k_compress(const LayoutArgs a, int span, 
     if (tid < SPAN) {
         const int jj = j0 + tid, col = tid < nk ? s_idx[tid] : 0xFFFF;
         if (col != 0xFFFF) {
-            const int tap = div_by(col, a.by_c_in), c = col - tap * a.c_in, khi = div_by(tap, a.by_kw), kwi = tap - khi * a.kw;
+            const Column at = column_of(a, col);
             if (first) {
                 a.indices[static_cast<size_t>(r) * a.kk + jj] = static_cast<uint16_t>(col);
-                a.taps[static_cast<size_t>(r) * a.kk_pad + jj] = (static_cast<uint32_t>(khi) << 24) | (static_cast<uint32_t>(kwi) << 16) | static_cast<uint32_t>(c);
+                a.taps[static_cast<size_t>(r) * a.kk_pad + jj] = tap_word(at);
             }
-            // slab layout: kept column jj lies in chunk col / S at position jj - chunk * KC (every group before the last is
-            // full, so a chunk of whole groups holds exactly KC kept columns)
             if (a.wt2) {
-                const int chunk = div_by(col, a.by_v2_s), at = chunk * 32 + (jj - chunk * a.v2_kc);
-                s_at2[tid] = static_cast<uint32_t>(at);
-                if (first) a.rel2[static_cast<size_t>(r) * pitch2 + at] = static_cast<uint8_t>(col - chunk * a.v2_s);
+                uint8_t rel;
+                const int place = slab_place(a, col, jj, &rel);
+                s_at2[tid] = static_cast<uint32_t>(place);
+                if (first) a.rel2[static_cast<size_t>(r) * pitch2 + place] = rel;
             }
             // select layout: w3[chunk][o][32], a chunk being as many steps (one tap of S source columns, of which KC are kept) as fit,
             // the steps ordered by block of S channels, then tap; swizzled like wx.  The
@@ -401,8 +408,8 @@ __global__ void __launch_bounds__(544) k_compress(const LayoutArgs a, int span, 
             // bit 7 and up), in the order in which a thread reads them: [step][place in a quad][quad].  (A span is whole steps.)
             if (a.w3) {
                 // (steps of 32 or 64 columns; four, two or one of them in a chunk as 8, 16 or 24 columns stay; a step's columns begin at its column's)
-                const int shift_s = a.sel_s == 64 ? 6 : 5, shift_c = a.sel_kc == 8 ? 2 : a.sel_kc == 16 ? 1 : 0, cb = c >> shift_s, cc = c - (cb << shift_s);
-                const int step = cb * a.kh * a.kw + tap, chunk = step >> shift_c, sub = step - (chunk << shift_c), js = ((col - c0) >> shift_s) * a.sel_kc;
+                const int shift_s = a.sel_s == 64 ? 6 : 5, shift_c = a.sel_kc == 8 ? 2 : a.sel_kc == 16 ? 1 : 0, cb = at.c >> shift_s, cc = at.c - (cb << shift_s);
+                const int step = cb * a.kh * a.kw + at.tap, chunk = step >> shift_c, sub = step - (chunk << shift_c), js = ((col - c0) >> shift_s) * a.sel_kc;
                 const int place = select_place(s_idx + js, a.sel_kc, tid - js);
                 // (a thread's columns of two quads are neighbours)
                 s_at3[tid] = static_cast<uint32_t>(chunk * 32 + sub * a.sel_kc + (place >> 3) * 8 + (place & 3) * 2 + (place >> 2 & 1));
@@ -410,37 +417,28 @@ __global__ void __launch_bounds__(544) k_compress(const LayoutArgs a, int span, 
                     reinterpret_cast<uint32_t*>(a.sel3)[(static_cast<size_t>(chunk) * a.n_tiles + r) * 32 + sub * a.sel_kc + (place & 3) * (a.sel_kc / 4) + (place >> 2)] =
                         static_cast<uint32_t>((cc & 31) * 4 | (cc >> 5) << 7);
             }
-            if (a.ws) s_ats[tid] = static_cast<uint32_t>(khi << 5 | kwi << 2 | c);
+            if (a.ws) s_ats[tid] = static_cast<uint32_t>(at.kh << 5 | at.kw << 2 | at.c);
         }
         if (first && blockIdx.x + 1 == gridDim.x)
             for (int i = a.kk + tid; i < a.kk_pad; i += SPAN) a.taps[static_cast<size_t>(r) * a.kk_pad + i] = NM_TAP_PAD;
     } else if (a.wx) {
-        // expanded layout: the shared-memory image the tensor core reads: blocks of 32 columns, inside a block one
-        // 128-byte row per output channel whose 16-byte pieces are XOR-ed with (o % 8) (the 128-byte swizzle), so that
-        // any run of channels starting at a multiple of 8 is one contiguous bulk copy
-        auto cell = [&](int o, int col) {
-            const int kc = col & 31;
-            return a.wx + (static_cast<size_t>(col >> 5) * a.wx_rows + o) * 32 + ((((kc >> 2) ^ (o & 7)) << 2) | (kc & 3));
-        };
         const int at = tid - SPAN, n = threads - SPAN, t = at & (SPAN - 1);
         if (t < cols) {
             const int pos = s_pos[t], from = IMPORT ? pos : t;
-            for (int rr = at / SPAN; rr < rows; rr += n / SPAN) *cell(row0 + p0 + rr, c0 + t) = pos >= 0 ? nmk::to_tf32(s_tile[rr][from]) : 0.f;
+            for (int rr = at / SPAN; rr < rows; rr += n / SPAN) *expanded_cell(a, row0 + p0 + rr, c0 + t) = pos >= 0 ? nmk::to_tf32(s_tile[rr][from]) : 0.f;
         }
         // zeros: columns up to the last block's 32nd, rows up to the last 32nd
         const int pad_cols = blockIdx.x + 1 == gridDim.x ? (32 - (a.k & 31)) & 31 : 0;
-        for (int i = at; i < rows * pad_cols; i += n) *cell(row0 + p0 + i / pad_cols, a.k + i % pad_cols) = 0.f;
+        for (int i = at; i < rows * pad_cols; i += n) *expanded_cell(a, row0 + p0 + i / pad_cols, a.k + i % pad_cols) = 0.f;
         if (r + 1 == static_cast<int>(gridDim.y) && first)
-            for (int i = at; i < (a.wx_rows - a.c_out) * (cols + pad_cols); i += n) *cell(a.c_out + i / (cols + pad_cols), c0 + i % (cols + pad_cols)) = 0.f;
+            for (int i = at; i < (a.wx_rows - a.c_out) * (cols + pad_cols); i += n) *expanded_cell(a, a.c_out + i / (cols + pad_cols), c0 + i % (cols + pad_cols)) = 0.f;
     }
     asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory");
 
     const int col = j < nk ? s_idx[j] : 0xFFFF;
     if (col == 0xFFFF) return;
-    // gather layout: per (tile, chunk of 32 retained columns) the shared-memory image of the tile's rows, swizzled like wx; as many
-    // rows as the tile has, so it is as large as the values whatever the tile width
-    const int jj = j0 + j, w = jj & (NM_KCHUNK - 1), from = IMPORT ? j : col - c0;
-    float* const wt = a.wt + static_cast<size_t>(row0) * a.kk_pad + static_cast<size_t>(jj / NM_KCHUNK) * tile_rows * NM_KCHUNK;
+    const int jj = j0 + j, from = IMPORT ? j : col - c0;
+    float* const wt = gather_image(a, row0, tile_rows, jj);
     float* const wt2 = a.wt2 ? a.wt2 + s_at2[j] : nullptr;
     const int k3 = a.w3 ? s_at3[j] & 31 : 0;
     float* const w3 = a.w3 ? a.w3 + static_cast<size_t>(s_at3[j] >> 5) * a.c_out * 32 : nullptr;
@@ -448,12 +446,10 @@ __global__ void __launch_bounds__(544) k_compress(const LayoutArgs a, int span, 
         const int tr = p0 + rr, o = row0 + tr;
         const float v = s_tile[rr][from], t = nmk::to_tf32(v);
         a.values[static_cast<size_t>(o) * a.kk + jj] = v;
-        wt[tr * NM_KCHUNK + ((((w >> 2) ^ (tr & 7)) << 2) | (w & 3))] = t;
+        wt[gather_cell(tr, jj)] = t;
         if (wt2) wt2[static_cast<size_t>(o) * pitch2] = t;
-        if (w3) w3[static_cast<size_t>(o) * 32 + ((((k3 >> 2) ^ (o & 7)) << 2) | (k3 & 3))] = t;
-        // plane layout: ws[kh][c_out][32]: a row holds the taps of one kernel row as (kw, c), c padded to 4 and kw to 8,
-        // its 16-byte pieces (one tap each) XOR-ed with (o % 8)
-        if (a.ws) a.ws[(static_cast<size_t>(s_ats[j] >> 5) * a.c_out + o) * 32 + (((s_ats[j] >> 2 & 7) ^ (o & 7)) << 2) + (s_ats[j] & 3)] = t;
+        if (w3) w3[static_cast<size_t>(o) * 32 + swizzled(o, k3)] = t;
+        if (a.ws) *plane_cell(a, o, static_cast<int>(s_ats[j] >> 5), static_cast<int>(s_ats[j] & 31)) = t;
     }
 }
 
@@ -541,7 +537,7 @@ void device_block_free(void* ptr, size_t bytes, int device, bool idle)
     while (!g_cache.empty() && (g_cached > kCacheBytes || g_cache.front().stamp + kCacheAge < g_frees)) drop(0);
 }
 
-bool compressed_in_one(const nm_weights* h) { return h->m_group <= SPAN && h->kk > 0; }
+bool compressed_in_one(const nm_weights* h) { return h->m_group <= SPAN; }
 
 // Which layouts this layer's kernels can read, and their dimensions (no device work).
 static void plan_layouts(nm_weights* h)
@@ -550,7 +546,7 @@ static void plan_layouts(nm_weights* h)
     // columns number a multiple of 8 up to 32 and whose source columns number <= 64
     const int n = h->n_keep == h->m_group ? 1 : h->n_keep;
     const int m = h->n_keep == h->m_group ? 1 : h->m_group;
-    for (int g = 32 / n; g >= 1 && h->kk > 0; --g)
+    for (int g = 32 / n; g >= 1; --g)
         if ((g * n) % 8 == 0 && g * m <= 64) {
             h->v2_ok = 1;
             h->v2_g = g; h->v2_kc = g * n; h->v2_s = g * m;
@@ -560,7 +556,7 @@ static void plan_layouts(nm_weights* h)
     // expanded layout: only shapes the kernels that read it take: output channels in whole float4s (rows are padded
     // with zeros to blocks of 32), and either whole 32-column slabs (expanded-operand kernel) or a short reduction axis
     // (row-run kernel, pointwise layers)
-    if (h->c_out % 4 == 0 && h->kk > 0 && (h->c_in % 32 == 0 || h->k <= 512)) h->wx_rows = (h->c_out + 31) / 32 * 32;
+    if (h->c_out % 4 == 0 && (h->c_in % 32 == 0 || h->k <= 512)) h->wx_rows = (h->c_out + 31) / 32 * 32;
     int s = 0, kc = 0;
     if (select_layout_dims(h, &s, &kc)) {
         const int spc = 32 / kc, steps = h->c_in / s * h->kh * h->kw;
@@ -573,7 +569,7 @@ static void plan_layouts(nm_weights* h)
 nm_status_t alloc_handle_memory(nm_weights* h, const char* who)
 {
     plan_layouts(h);
-    const bool planes = h->c_in <= 4 && h->kw <= 8 && h->c_out % 32 == 0 && h->c_out <= 256 && h->kk > 0 &&
+    const bool planes = h->c_in <= 4 && h->kw <= 8 && h->c_out % 32 == 0 && h->c_out <= 256 &&
                         h->kh * h->c_out * 128 < (1 << 20);
     size_t total = 0;
     auto place = [&total](size_t bytes) {
@@ -581,14 +577,14 @@ nm_status_t alloc_handle_memory(nm_weights* h, const char* who)
         total += (std::max<size_t>(bytes, 16) + 255) / 256 * 256;
         return at;
     };
-    const size_t kk1 = static_cast<size_t>(std::max(h->kk, 1));
+    const size_t kk1 = static_cast<size_t>(h->kk);
     const size_t pitch2 = static_cast<size_t>(h->v2_chunks) * 32;
     const size_t chunks3 = static_cast<size_t>(h->sel_chunks);
     const size_t at_values = place(h->c_out * kk1 * sizeof(float));
     const size_t at_indices = place(h->n_tiles * kk1 * sizeof(uint16_t));
     const size_t at_taps = place(static_cast<size_t>(h->n_tiles) * h->kk_pad * sizeof(uint32_t));
     // Layouts that every word of is written come before the part of the block that the creating call clears (status, sums and layouts with
-    // padding or zeros in the pruned columns): 512 x 3 x 3 x 512 at 2:4 has 9 of 24 MB to clear, 58 -> 51 us.
+    // padding or zeros in the pruned columns).  512 x 3 x 3 x 512 at 2:4 has nothing to clear (with 9 of its 28 MB cleared it took 7 us more).
     const int spc = h->sel_s ? 32 / h->sel_kc : 1;
     const bool full_wx = compressed_in_one(h);
     const bool full_wt = h->kk % NM_KCHUNK == 0;
@@ -662,11 +658,9 @@ nm_status_t build_layouts(nm_weights* h, const float* src, const uint16_t* idx, 
 {
     const LayoutArgs a = layout_args(h, src, idx, import);
     if (h->c_out > 65535) return fail(NM_ERR_CUDA, "weight layout kernel: more than 65535 output channels");   // bounds grid.y
-    if (h->kk_pad > 0) {
-        const dim3 grid((h->kk_pad + 127) / 128, h->n_tiles * ((h->tile_t + ROWS - 1) / ROWS));
-        k_build_layouts<<<grid, 128, 0, st>>>(a);
-        count_launch(1);
-    }
+    const dim3 grid((h->kk_pad + 127) / 128, h->n_tiles * ((h->tile_t + ROWS - 1) / ROWS));
+    k_build_layouts<<<grid, 128, 0, st>>>(a);
+    count_launch(1);
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? NM_OK : fail(NM_ERR_CUDA, "weight layout kernel: %s", cudaGetErrorString(e));
 }

@@ -19,6 +19,10 @@ SHAPES = [
     (64, 1, 1, 128, 1, 8, 64),      # select layout with steps of 64 columns
     (68, 1, 1, 63, 1, 3, 16),       # spans of 126 columns; a tail group; a last tile of 4 rows
     (32, 7, 7, 3, 1, 1, 32),        # plane layout
+    # groups wider than a block: selected and laid out by kernels of their own
+    (64, 1, 1, 256, 256, 256, 32),  # slab layout (everything kept)
+    (32, 7, 7, 3, 100, 147, 32),    # plane layout with zeros
+    (100, 3, 3, 64, 100, 192, 48),  # expanded layout with zeros; a last tile of 4 rows
 ]
 
 
@@ -55,22 +59,31 @@ def test_layouts_from_dense_weights_and_from_the_compressed_form(c_out, kh, kw, 
 
 
 def test_more_creating_calls_at_once_than_slots():
+    """48 calls wait for their streams at once, each behind a kernel that spins for a while; the 32 that have a slot get their sums through
+    it, the others by a copy."""
+    from torch.profiler import ProfilerActivity, profile
+
     from paper_2507_17301_b200 import nm
     weights = [torch.randint(-4, 5, (48, 3, 3, 32), generator=torch.Generator().manual_seed(s)).float().cuda() for s in range(48)]
+    nm.nm_prune(weights[0], 2, 4, 16)
     torch.cuda.synchronize()
-    got = [None] * len(weights)
+    handles = [None] * len(weights)
     go = threading.Barrier(len(weights))
 
     def create(i):
         with torch.cuda.stream(torch.cuda.Stream()):
             go.wait()
-            hnd = nm.nm_prune(weights[i], 2, 4, 16)
-            got[i] = (nm.nm_weights_retained_l1(hnd), nm.nm_weights_export(hnd)[0].double().abs().sum().item())
+            torch.cuda._sleep(400_000_000)   # 0.2 s
+            handles[i] = nm.nm_prune(weights[i], 2, 4, 16)
 
     threads = [threading.Thread(target=create, args=(i,)) for i in range(len(weights))]
-    for th in threads:
-        th.start()
-    for th in threads:
-        th.join()
-    for w, ((kept, total), values) in zip(weights, got):
-        assert kept == values and total == w.double().abs().sum().item()
+    with profile(activities=[ProfilerActivity.CUDA]) as prof:
+        for th in threads:
+            th.start()
+        for th in threads:
+            th.join()
+    copies = sum("memcpy dtoh" in e.name.lower() for e in prof.events())
+    assert 1 <= copies <= 16, copies
+    for w, hnd in zip(weights, handles):
+        kept, total = nm.nm_weights_retained_l1(hnd)
+        assert kept == nm.nm_weights_export(hnd)[0].double().abs().sum().item() and total == w.double().abs().sum().item()
