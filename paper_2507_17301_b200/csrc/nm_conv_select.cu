@@ -530,9 +530,11 @@ k_conv_select(const ConvParams p, const SelCfg cfg, const __grid_constant__ CUte
                 }
                 const uint32_t box = my_staging + bx * BOX_BYTES;
                 const uint32_t stage_row = box + lane * 128;
-                // (all shuffles and loads before the first store: they are ordered statements, one would wait for the other's result.  With
-                // this and the bias fetched ahead 256 -> 256, 3x3 at 14x14, batch 64, 2:4 takes 30.6 us for 30.9, 512 -> 512 at 7x7 29.9 for 30.8, batch 8,
-                // 1:4, 64 -> 64 at 56x56 with shortcut 9.4 for 9.8; 64 -> 64 at 56x56, batch 128, 2:8 59.6 for 58.8)
+                // (All shuffles and loads before the first store: they are ordered statements, one would wait for the other's result.  With this and
+                // the bias fetched ahead 82 pairs of layer and plan take 0.979 of the time in the middle, split ones 0.93: 256 -> 256, 3x3 at 14x14, batch 64,
+                // 2:4 30.9 -> 30.6 us, 64 -> 256, 1x1 at 56x56, batch 64 59.7 -> 48.5.  64 -> 64, 3x3 at 56x56, batch 128 got slower: 2:8 58.6 -> 59.5, 1:4
+                // in one group of two tiles 66.8 -> 70.4.  So it did with the bias through shared memory, loaded a block ahead or after the wait,
+                // with four loads at a time, and with a load through L2 as the only change: the selecting warps' schedule, not the epilogue.)
                 float4 o8[8];
 #pragma unroll
                 for (int qq = 0; qq < 8; ++qq) {

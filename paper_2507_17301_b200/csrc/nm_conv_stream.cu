@@ -547,7 +547,8 @@ bool make_cfg(const ConvParams& p, const nm_plan_t* plan, StreamCfg* cfg)
     const int budget = 227 * 1024 - 1024 - 1024;         // alignment slack, static shared
     const int asked = plan && plan->stages > 0 ? plan->stages : 0;
     auto most = [&](int boxes) { return std::min((budget - 4 * boxes * BOX_BYTES) / cfg->stage_bytes, NSTAGE_MAX); };
-    // (64 -> 256, one chunk of 64 columns, at 56x56, batch 4: 7.2 us with two boxes, 8.5 with one; 256 -> 256, 3x3 at 14x14, batch 32: 35.1, 25.9)
+    // Two boxes and three stages, one box and four, us: 64 -> 256, 1x1 (one chunk) at 56x56, batch 4 6.6, 7.5; 128 -> 512, 1x1 (two) at 28x28, batch 32 15.0,
+    // 15.6; 384 -> 128, 1x1 (six) at 28x28 12.8, 12.8; 256 -> 256, 3x3 (36) at 14x14, batch 32 27.5, 26.1.
     cfg->boxes = asked ? (asked > most(2) ? 1 : 2) : p.v2_chunks > 4 && most(1) > most(2) ? 1 : 2;
     const int stages = asked ? asked : most(cfg->boxes);
     if (stages < (asked ? 1 : 2) || stages > most(cfg->boxes)) return false;

@@ -43,7 +43,8 @@ template <int ROWS>
 __global__ void __launch_bounds__(256) k_maxpool_3x3s2(const float4* __restrict__ x, int h, int w, int c4, int pad_h, int pad_w, int ho, int wo,
                                                        int row_blocks, unsigned total, float4* __restrict__ y)
 {
-    // from the end: of an input that does not fit the L2, the part the kernel before wrote last is still there
+    // from the end: of an input that does not fit the L2, the part the kernel before wrote last is still there (7x7 / 2 stem and this at batch 64
+    // 116.9 -> 109.2 us, at batch 128 216.4 -> 208.6)
     const unsigned id = (gridDim.x - 1u - blockIdx.x) * 256u + threadIdx.x;
     nmk::pdl_wait();
     if (id >= total) return;
