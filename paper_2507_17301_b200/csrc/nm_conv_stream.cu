@@ -480,7 +480,7 @@ bool layout_matches(const ConvParams& p)
 // the better of the two in the middle, more than 2 % for 41, 8 % at worst; always two is behind by more than 2 % for 272, always one for 407.
 int teams_for(const ConvParams& p, int g) { return p.v2_chunks >= 4 && g * p.v2_kc >= 24 ? 2 : 1; }
 
-// Time with `g` tiles per CTA, fitted to 1900 measured layer and width pairs (c_in 32-512, c_out 16-1024, 1x1 to 5x5, 1 to 12 tiles of 16-128; 17 %
+// Time with `g` tiles per CTA, fitted to 2200 measured layer and width pairs (c_in 32-512, c_out 16-1024, 1x1 to 5x5, 1 to 12 tiles of 16-128; 17 %
 // rms): rounds of the SMs, each the chunks' chain or the epilogue, whichever is longer.
 double stream_time_us(const ConvParams& p, int g)
 {
@@ -587,12 +587,6 @@ nm_status_t launch(const ConvParams& p, const StreamCfg& cfg, cudaStream_t st)
 }  // namespace
 
 namespace nmhost {
-
-bool stream_plan_ok(const ConvParams& p, const nm_plan_t* plan)
-{
-    StreamCfg cfg;
-    return make_cfg(p, plan, &cfg);
-}
 
 int stream_width(const ConvParams& p, const nm_plan_t* plan)
 {

@@ -262,7 +262,6 @@ bool pair_plan_ok(const ConvParams& p, const nm_plan_t* plan);
 nm_status_t launch_conv_pair(const ConvParams& p, const nm_plan_t* plan, cudaStream_t st);
 
 // nm_conv_stream.cu — variant 3
-bool stream_plan_ok(const ConvParams& p, const nm_plan_t* plan);
 int stream_width(const ConvParams& p, const nm_plan_t* plan);   // channels per work item, 0: the kernel does not take the layer / plan
 bool stream_beats_gather(const ConvParams& p);   // (and takes the layer)
 nm_status_t launch_conv_stream(const ConvParams& p, const nm_plan_t* plan, cudaStream_t st);
