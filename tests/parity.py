@@ -1,5 +1,6 @@
 """Shared helpers for the GPU parity tests: run one layer through the C-ABI binding and through
 the CPU oracle on the same seeded inputs and compare (helpers only; no method arithmetic)."""
+import ctypes
 import re
 
 import numpy as np
@@ -59,11 +60,27 @@ def assert_conv_close(y_gpu, y_ref):
     assert max_abs <= MAX_ABS_TOL * ref_max, f"max-abs error {max_abs:.3e} above {MAX_ABS_TOL} * {ref_max:.3e}"
 
 
+class _KernelNode(ctypes.Structure):   # CUDA_KERNEL_NODE_PARAMS_v2
+    _fields_ = [("func", ctypes.c_void_p), ("launch", ctypes.c_uint * 7), ("kernel_params", ctypes.c_void_p), ("extra", ctypes.c_void_p),
+                ("kern", ctypes.c_void_p), ("ctx", ctypes.c_void_p)]
+
+
 def kernels_of(call):
-    """Names of this library's kernels that `call` launches, in order."""
-    from torch.profiler import ProfilerActivity, profile
+    """The library's kernels among the nodes of a graph that `call` is recorded into."""
+    call()                                   # (what a first call allocates cannot be recorded)
     torch.cuda.synchronize()
-    with profile(activities=[ProfilerActivity.CUDA]) as prof:
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
         call()
-        torch.cuda.synchronize()
-    return [m for e in prof.events() for m in re.findall(r"\bk_[a-z0-9_]+", e.name)]
+    cuda, raw, n = ctypes.CDLL("libcuda.so.1"), ctypes.c_void_p(graph.raw_cuda_graph()), ctypes.c_size_t()
+    assert cuda.cuGraphGetNodes(raw, None, ctypes.byref(n)) == 0
+    nodes = (ctypes.c_void_p * n.value)()
+    assert cuda.cuGraphGetNodes(raw, nodes, ctypes.byref(n)) == 0
+    names = []
+    for node in nodes:
+        params, name = _KernelNode(), ctypes.c_char_p()
+        if cuda.cuGraphKernelNodeGetParams_v2(ctypes.c_void_p(node), ctypes.byref(params)) == 0:   # (other nodes are no kernels)
+            handle, get = (params.func, cuda.cuFuncGetName) if params.func else (params.kern, cuda.cuKernelGetName)
+            assert get(ctypes.byref(name), ctypes.c_void_p(handle)) == 0
+            names += re.findall(r"k_[a-z0-9_]+", name.value.decode())
+    return names
